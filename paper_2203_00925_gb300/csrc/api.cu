@@ -108,9 +108,11 @@ void order_slice_for_banks(int16_t* lid, int width) {
   }
 }
 
-int build_grad_tiles(int64_t N, const std::vector<int64_t>& sptr, const std::vector<int32_t>& sidx,
-                     std::vector<int32_t>& tptr, std::vector<int32_t>& tidx, std::vector<int16_t>& lidx) {
-  const int64_t ntile = (N + kGradTile - 1) / kGradTile;
+// Tiles are the row ranges [start[t], start[t + 1]) (at most kGradTile rows each).
+int build_grad_tiles(int64_t N, const std::vector<int64_t>& start, const std::vector<int64_t>& sptr,
+                     const std::vector<int32_t>& sidx, std::vector<int32_t>& tptr, std::vector<int32_t>& tidx,
+                     std::vector<int16_t>& lidx) {
+  const int64_t ntile = (int64_t)start.size() - 1;
   std::vector<std::vector<int32_t>> lists(ntile);
   lidx.assign(sidx.size(), 0);
   int max_len = 0;
@@ -119,21 +121,24 @@ int build_grad_tiles(int64_t N, const std::vector<int64_t>& sptr, const std::vec
     std::vector<int32_t> stamp(N, -1), pos(N, 0);
 #pragma omp for schedule(dynamic, 64)
     for (int64_t t = 0; t < ntile; ++t) {
-      const int64_t r0 = t * kGradTile, r1 = std::min<int64_t>(N, r0 + kGradTile);
+      const int64_t r0 = start[t], r1 = start[t + 1];
       std::vector<int32_t>& L = lists[t];
       for (int64_t r = r0; r < r1; ++r) { stamp[r] = (int32_t)t; L.push_back((int32_t)r); }
-      const int64_t s0 = r0 / 32, s1 = (r1 + 31) / 32;
       const size_t own = L.size();
-      for (int64_t q = sptr[s0]; q < sptr[s1]; ++q) {
-        const int32_t j = sidx[q];
-        if (stamp[j] != (int32_t)t) { stamp[j] = (int32_t)t; L.push_back(j); }
-      }
+      for (int64_t r = r0; r < r1; ++r)
+        for (int64_t q = sptr[r / 32] + r % 32; q < sptr[r / 32 + 1]; q += 32) {
+          const int32_t j = sidx[q];
+          if (stamp[j] != (int32_t)t) { stamp[j] = (int32_t)t; L.push_back(j); }
+        }
       std::sort(L.begin() + own, L.end());
       for (size_t k = 0; k < L.size(); ++k) pos[L[k]] = (int32_t)k;
       if (L.size() <= 32767) {
-        for (int64_t q = sptr[s0]; q < sptr[s1]; ++q) lidx[q] = (int16_t)pos[sidx[q]];
-        for (int64_t sl = s0; sl < s1; ++sl)
-          order_slice_for_banks(lidx.data() + sptr[sl], (int)((sptr[sl + 1] - sptr[sl]) / 32));
+        for (int64_t r = r0; r < r1; ++r)
+          for (int64_t q = sptr[r / 32] + r % 32; q < sptr[r / 32 + 1]; q += 32) lidx[q] = (int16_t)pos[sidx[q]];
+        // the slices whose lanes are this tile's warps
+        if (r0 % 32 == 0)
+          for (int64_t sl = r0 / 32; sl < (r1 == N ? (r1 + 31) / 32 : r1 / 32); ++sl)
+            order_slice_for_banks(lidx.data() + sptr[sl], (int)((sptr[sl + 1] - sptr[sl]) / 32));
       }
       max_len = std::max(max_len, (int)L.size());
     }
@@ -143,6 +148,95 @@ int build_grad_tiles(int64_t N, const std::vector<int64_t>& sptr, const std::vec
   tidx.resize(tptr[ntile]);
   for (int64_t t = 0; t < ntile; ++t) std::copy(lists[t].begin(), lists[t].end(), tidx.begin() + tptr[t]);
   return max_len;
+}
+
+// What k_gradient_fixed needs beside the tiles (FP64 meshes; tiles do not cross parts, so that
+// a mesh gives the same bits alone and in an ensemble):
+//  - centres as integers in units of 2^-scale (|x| 2^scale < 2^61: exact for every coordinate
+//    of at least 2^-9 of the largest);
+//  - per tile bits = 62 - ceil(log2(w + 1)), w the longest neighbour list of its part, so
+//    that a sum over a list stays below 2^62, and the right shift (negative: left) that brings
+//    its coordinate differences from the first own centre below 2^bits;
+//  - per cell D = sum_j (y_j - y_i) of those shifted differences over its neighbours, and the
+//    padding entries of its list.
+// A tile keeps the FP64 sums (bits = 0) in a part of less than one tile, with lists above 511
+// entries, or when its extent is more than kFixedSpread times the smallest neighbourhood in it
+// (a strongly graded mesh): the tile's unit would be coarse for those cells.
+constexpr double kFixedSpread = 8.0;
+
+void build_fixed_tiles(const HostMesh& h, const std::vector<int64_t>& start, const std::vector<int32_t>& tptr,
+                       const std::vector<int32_t>& tidx, std::vector<longlong4_16a>& xfix,
+                       std::vector<int4>& tile, std::vector<int64_t>& dsum, int& scale) {
+  const int64_t N = h.N;
+  const std::vector<double>& cen = h.cen;
+  double top = 0.0;
+  for (double c : cen) top = std::max(top, std::fabs(c));
+  int e = 0;
+  std::frexp(top, &e);                       // top < 2^e
+  scale = 61 - e;
+  const bool usable = top > 0.0 && std::isfinite(top) && scale > -900 && scale < 900;
+  xfix.resize(N);
+#pragma omp parallel for
+  for (int64_t i = 0; i < N; ++i) {
+    auto fix = [&](double c) { return usable ? std::llrint(std::ldexp(c, scale)) : 0ll; };
+    xfix[i] = longlong4_16a{fix(cen[i]), fix(cen[N + i]), fix(cen[2 * N + i]), 0};
+  }
+  const int64_t ntile = (int64_t)start.size() - 1;
+  const int P = (int)h.part_cell_begin.size() - 1;
+  std::vector<int> part_bits(P, 0);
+#pragma omp parallel for
+  for (int p = 0; p < P; ++p) {
+    const int64_t lo = h.part_cell_begin[p], hi = h.part_cell_begin[p + 1];
+    int64_t most = 1;
+    for (int64_t i = lo; i < hi; ++i) most = std::max<int64_t>(most, h.nptr[i + 1] - h.nptr[i]);
+    int w = 0;
+    while ((int64_t(1) << w) < most + 1) ++w;
+    if (usable && hi - lo >= kGradTile && w <= 9) part_bits[p] = 62 - w;
+  }
+  tile.resize(ntile);
+  dsum.assign((size_t)3 * N, 0);
+#pragma omp parallel for schedule(dynamic, 64)
+  for (int64_t t = 0; t < ntile; ++t) {
+    const int64_t r0 = start[t], r1 = start[t + 1];
+    const int p = (int)(std::upper_bound(h.part_cell_begin.begin(), h.part_cell_begin.end(), r0) -
+                        h.part_cell_begin.begin()) - 1;
+    const int bits = part_bits[p];
+    tile[t] = int4{(int)r0, (int)(r1 - r0), 0, 0};
+    if (bits == 0) continue;
+    const longlong4_16a o = xfix[r0];
+    auto diff = [&](int64_t j, const longlong4_16a& q, long long* d) {
+      d[0] = xfix[j].x - q.x; d[1] = xfix[j].y - q.y; d[2] = xfix[j].z - q.z;
+    };
+    long long d[3], most = 1;
+    for (int32_t k = tptr[t]; k < tptr[t + 1]; ++k) {
+      diff(tidx[k], o, d);
+      for (int a = 0; a < 3; ++a) most = std::max(most, d[a] < 0 ? -d[a] : d[a]);
+    }
+    long long least = most;
+    for (int64_t i = r0; i < r1; ++i) {
+      long long m = 0;
+      for (int32_t q = h.nptr[i]; q < h.nptr[i + 1]; ++q) {
+        diff(h.nidx[q], xfix[i], d);
+        for (int a = 0; a < 3; ++a) m = std::max(m, d[a] < 0 ? -d[a] : d[a]);
+      }
+      least = std::min(least, m);
+    }
+    if ((double)most > kFixedSpread * (double)least) continue;
+    int sh = 0;
+    while (most < (1ll << (bits - 1 + sh))) --sh;     // room to the left
+    while (most >= (1ll << (bits + sh)) && bits + sh < 62) ++sh;  // or cut to the right
+    tile[t].z = sh;
+    tile[t].w = bits;
+    auto cut = [&](long long v) { return sh >= 0 ? v >> sh : (long long)((unsigned long long)v << -sh); };
+    for (int64_t i = r0; i < r1; ++i) {
+      diff(i, o, d);
+      const long long yi[3] = {cut(d[0]), cut(d[1]), cut(d[2])};
+      for (int32_t q = h.nptr[i]; q < h.nptr[i + 1]; ++q) {
+        diff(h.nidx[q], o, d);
+        for (int a = 0; a < 3; ++a) dsum[a * N + i] += cut(d[a]) - yi[a];
+      }
+    }
+  }
 }
 
 template <typename T>
@@ -768,12 +862,33 @@ static fvgb_status upload_impl(int32_t dim, int64_t n_vert, const double* xyz, i
   build_sell(h.nptr, h.nidx, nullptr, h.N, true, sptr, sidx, nullptr);
   if ((e = dupload(m, &t.nsell.ptr, sptr, s))) return fail(e, "upload");
   if ((e = dupload(m, &t.nsell.idx, sidx, s))) return fail(e, "upload");
-  if (prec != FVGB_FP64 && h.dim == 3 && h.N >= kGradTile &&
-      (int64_t)h.nptr[h.N] < (int64_t)INT32_MAX / 2) {   // the FP32 shared-memory gradient
+  if (h.dim == 3 && h.N >= kGradTile &&
+      (int64_t)h.nptr[h.N] < (int64_t)INT32_MAX / 2) {   // the shared-memory gradients
     std::vector<int32_t> tptr, tidx;
     std::vector<int16_t> lidx;
-    const int mx = build_grad_tiles(h.N, sptr, sidx, tptr, tidx, lidx);
-    if (mx <= kGradTileMaxHalo) {
+    std::vector<int64_t> start;                  // tiles; in FP64 they do not cross parts
+    for (int p = 0; p < (prec == FVGB_FP64 ? n_part : 1); ++p)
+      for (int64_t r = h.part_cell_begin[p]; r < (prec == FVGB_FP64 ? h.part_cell_begin[p + 1] : h.N); r += kGradTile)
+        start.push_back(r);
+    start.push_back(h.N);
+    const int mx = build_grad_tiles(h.N, start, sptr, sidx, tptr, tidx, lidx);
+    const bool tiled = mx <= kGradTileMaxHalo;
+    if (tiled && prec == FVGB_FP64) {
+      std::vector<longlong4_16a> xfix;
+      std::vector<int4> tile;
+      std::vector<int64_t> dsum;
+      build_fixed_tiles(h, start, tptr, tidx, xfix, tile, dsum, t.fix_scale);
+      std::vector<int16_t> pad(h.N);
+      for (int64_t i = 0; i < h.N; ++i)
+        pad[i] = (int16_t)std::min<int64_t>(INT16_MAX, (sptr[i / 32 + 1] - sptr[i / 32]) / 32 - (h.nptr[i + 1] - h.nptr[i]));
+      t.n_tile = (int)tile.size();
+      if ((e = dupload(m, &t.tile_pad, pad, s))) return fail(e, "upload");
+      if ((e = dupload(m, &t.xfix, xfix, s))) return fail(e, "upload");
+      if ((e = dupload(m, &t.tile_fix, tile, s))) return fail(e, "upload");
+      if ((e = dupload(m, &t.tile_dsum, dsum, s))) return fail(e, "upload");
+      if ((e = prepare_gradient_fixed())) return fail(e, "shared memory limit");
+    }
+    if (tiled) {
       t.tile_max = mx;
       if ((e = dupload(m, &t.tile_ptr, tptr, s))) return fail(e, "upload");
       if ((e = dupload(m, &t.tile_idx, tidx, s))) return fail(e, "upload");

@@ -74,10 +74,19 @@ struct TopoDev {
   int32_t* tile_idx = nullptr;   // halo lists
   int16_t* tile_lidx = nullptr;  // [size of nsell.idx]
   int tile_max = 0;              // longest halo list (0: tiles not built)
+  // FP64 meshes (k_gradient_fixed): integer centres, and per tile and cell what its
+  // fixed-point sums need (see build_fixed_tiles)
+  longlong4_16a* xfix = nullptr; // [N] {x, y, z, 0} in units of 2^-fix_scale
+  int4* tile_fix = nullptr;      // [n_tile] {first row, rows, right shift of the coordinate
+                                 // differences, magnitude bits (0: the tile keeps FP64 sums)}
+  int64_t* tile_dsum = nullptr;  // [3][N] sum of the cell's shifted neighbour differences
+  int16_t* tile_pad = nullptr;   // [N] padding entries of the cell's list (the cell itself)
+  int fix_scale = 0;
+  int n_tile = 0;
 };
 
 constexpr int kGradTile = 128;      // cells per tile of the shared-memory gradient
-constexpr int kGradTileMaxHalo = 3072;  // longest halo list the FP32 tiled kernel stages (48 KB)
+constexpr int kGradTileMaxHalo = 3072;  // longest halo list a tiled kernel stages (FP32 48 KB, FP64 96 KB)
 
 // Scratch of one precision.
 template <typename T>
@@ -216,6 +225,7 @@ void set_error(const std::string& msg);
 fvgb_status cuda_status(cudaError_t e, const char* what);
 
 // ops.cu -------------------------------------------------------------------------------
+cudaError_t prepare_gradient_fixed();   // allow its shared memory (longest halo list)
 template <typename T>
 cudaError_t launch_gradient(fvgb_mesh_s* m, int bcset, const T* u, T* grad, cudaStream_t s);
 // multiplicity-weighted (vertex-factorised) variant of the least-squares gradient

@@ -248,6 +248,170 @@ k_gradient_tiled(int64_t N, int64_t F, int64_t Fi, const int64_t* __restrict__ s
   grad[2 * N + i] = m2 * J[0] + m4 * J[1] + m5 * J[2];
 }
 
+// FP64, 3D, shared-memory form of k_gradient in fixed point. GB300 issues FP64 at 1/64 of
+// the FP32 rate and the direct sum takes seven FP64 operations per neighbour, so the sum over
+// the neighbours runs on the integer pipe instead, exactly: with the tile's first cell o,
+//   y_j = x_j - x_o,  v_j = u_j - u_o,  z_j = y_j v_j   (once per record of the halo list)
+//   J_i = sum_j (y_j - y_i)(v_j - v_i) = sum_j z_j - y_i sum_j v_j - v_i D_i,
+// D_i = sum_j (y_j - y_i) being geometry (tile_dsum). y is the difference of integer centres,
+// v the FP64 difference converted with the tile's largest exponent, z the 128-bit product cut
+// back; all keep ``bits`` (53..61) magnitude bits relative to the tile's range, the sums are
+// exact in 64 bits and the last line is formed in 128. Per neighbour entry that leaves four
+// 64-bit additions and two 16-byte shared-memory reads (the records, in two arrays so that the
+// lists' bank-aware order serves both).
+// The unit is relative to the tile's range R of v: a cell whose own neighbours differ by less
+// than R / 16 (a steep field in the tile), and every cell of a tile whose u is not finite or
+// nearly denormal, or that has no bits, takes the FP64 sum (grad_sum_direct), in the order
+// of k_gradient.
+__device__ __noinline__ void grad_sum_direct(int64_t N, int64_t i, int width, const int32_t* __restrict__ col,
+                                             const double* __restrict__ u, const double* __restrict__ cen,
+                                             double* J) {
+  const double ui = u[i], x = cen[i], y = cen[N + i], z = cen[2 * N + i];
+  double j0 = 0.0, j1 = 0.0, j2 = 0.0;
+  for (int c = 0; c < width; ++c) {
+    const int64_t j = col[32 * c];
+    const double du = u[j] - ui;
+    j0 += (cen[j] - x) * du;
+    j1 += (cen[N + j] - y) * du;
+    j2 += (cen[2 * N + j] - z) * du;
+  }
+  J[0] = j0; J[1] = j1; J[2] = j2;
+}
+
+// round(y v / 2^bits)
+__device__ __forceinline__ long long fixed_mul(long long y, long long v, int bits) {
+  const unsigned long long lo = (unsigned long long)y * (unsigned long long)v;
+  const long long hi = __mul64hi(y, v);
+  const unsigned long long half = 1ull << (bits - 1);
+  const unsigned long long l = lo + half;
+  const long long h = hi + (l < lo ? 1 : 0);
+  return (long long)(((unsigned long long)h << (64 - bits)) | (l >> bits));
+}
+
+__global__ void __launch_bounds__(kGradTile)
+k_gradient_fixed(int64_t N, int64_t F, int64_t Fi, const int64_t* __restrict__ sptr,
+                 const int32_t* __restrict__ sidx, const int16_t* __restrict__ lidx,
+                 const int32_t* __restrict__ tptr, const int32_t* __restrict__ tidx,
+                 const int4* __restrict__ tfix, const longlong4_16a* __restrict__ xfix,
+                 const int64_t* __restrict__ dsum, const int16_t* __restrict__ pad, int scale, int max_halo, const double* __restrict__ u, const double* __restrict__ cen,
+                 const double* __restrict__ xf, const double* __restrict__ minv,
+                 const int32_t* __restrict__ gptr, const int32_t* __restrict__ gface,
+                 const double* __restrict__ bval, double* __restrict__ grad) {
+  extern __shared__ longlong2 frec[];
+  longlong2* ra = frec;                 // {v, z_x}
+  longlong2* rb = frec + max_halo;      // {z_y, z_z}
+  __shared__ int s_top[kGradTile / 32];
+  const int4 td = tfix[blockIdx.x];
+  const int64_t r0 = td.x;
+  const int shift = td.z, bits = td.w;
+  const int32_t h0 = tptr[blockIdx.x], nh = tptr[blockIdx.x + 1] - h0;
+  const bool own = (int)threadIdx.x < td.y;
+  const int64_t i = own ? r0 + threadIdx.x : r0;
+  const int64_t b0 = sptr[i >> 5];
+  const int width = own ? (int)((sptr[(i >> 5) + 1] - b0) >> 5) : 0;
+  const int16_t* col = lidx + b0 + (i & 31);
+  const int32_t* halo = tidx + h0;
+  double J[3] = {0.0, 0.0, 0.0};
+  bool direct = bits == 0;
+  if (!direct) {                        // uniform over the block
+    // the halo's differences from the first own cell; largest exponent of those of u
+    const longlong2* X = reinterpret_cast<const longlong2*>(xfix);
+    const double uo = u[r0];
+    const longlong2 oa = X[2 * r0];
+    const long long oz = X[2 * r0 + 1].x;
+    int top = 0;
+    long long yi[3] = {0, 0, 0};
+    for (int k = threadIdx.x; k < nh; k += kGradTile) {
+      const int64_t j = __ldg(halo + k);
+      const longlong2 a = __ldg(X + 2 * j);
+      const long long az = __ldg(&X[2 * j + 1].x);
+      const long long du = __double_as_longlong(u[j] - uo);
+      long long y[3] = {a.x - oa.x, a.y - oa.y, az - oz};
+#pragma unroll
+      for (int c = 0; c < 3; ++c) y[c] = shift >= 0 ? y[c] >> shift : y[c] << -shift;
+      if (k < kGradTile) { yi[0] = y[0]; yi[1] = y[1]; yi[2] = y[2]; }   // the thread's own cell
+      ra[k] = make_longlong2(du, y[0]);
+      rb[k] = make_longlong2(y[1], y[2]);
+      const int e = (int)((unsigned long long)du >> 52) & 0x7ff;
+      top = max(top, e > 0 ? e : ((du & 0x7fffffffffffffffll) != 0 ? 1 : 0));
+    }
+    top = __reduce_max_sync(0xffffffffu, top);
+    if ((threadIdx.x & 31) == 0) s_top[threadIdx.x >> 5] = top;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < kGradTile / 32; ++w) top = max(top, s_top[w]);
+    // not finite, or so small that the scaled sums could leave the normal range
+    direct = top == 0x7ff || (top < 256 && top > 0);
+    if (!direct && top > 0) {
+      for (int k = threadIdx.x; k < nh; k += kGradTile) {   // the entries this thread staged
+        const longlong2 a = ra[k], b = rb[k];
+        const int e = (int)((unsigned long long)a.x >> 52) & 0x7ff;
+        const int cut = top - e;
+        unsigned long long mag = e > 0 ? (((unsigned long long)a.x & 0xfffffffffffffull) | (1ull << 52)) << (bits - 53) : 0;
+        mag = cut == 0 ? mag : (cut < 63 ? (mag + (1ull << (cut - 1))) >> cut : 0);
+        const long long v = a.x < 0 ? -(long long)mag : (long long)mag;
+        ra[k] = make_longlong2(v, fixed_mul(a.y, v, bits));
+        rb[k] = make_longlong2(fixed_mul(b.x, v, bits), fixed_mul(b.y, v, bits));
+      }
+      __syncthreads();
+      const longlong2 ai = ra[own ? threadIdx.x : 0], bi = rb[own ? threadIdx.x : 0];
+      const long long vi = ai.x;
+      // the padding entries (the cell itself) are taken out again
+      const long long np = own ? pad[i] : 0;
+      long long V = -np * vi, Z0 = -np * ai.y, Z1 = -np * bi.x, Z2 = -np * bi.y;
+      int least = (int)(vi >> 32), most = least;
+      int c = 0;
+      for (; c + 4 <= width; c += 4) {
+        const int e0 = __ldg(col + 32 * c), e1 = __ldg(col + 32 * (c + 1)), e2 = __ldg(col + 32 * (c + 2)),
+                  e3 = __ldg(col + 32 * (c + 3));
+        const longlong2 a[4] = {ra[e0], ra[e1], ra[e2], ra[e3]};
+        const longlong2 b[4] = {rb[e0], rb[e1], rb[e2], rb[e3]};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          V += a[q].x; Z0 += a[q].y; Z1 += b[q].x; Z2 += b[q].y;
+          const int hi = (int)(a[q].x >> 32);
+          least = min(least, hi);
+          most = max(most, hi);
+        }
+      }
+      for (; c < width; ++c) {
+        const int e = __ldg(col + 32 * c);
+        const longlong2 a = ra[e], b = rb[e];
+        V += a.x; Z0 += a.y; Z1 += b.x; Z2 += b.y;
+        const int hi = (int)(a.x >> 32);
+        least = min(least, hi);
+        most = max(most, hi);
+      }
+      direct = most - least < (1 << (bits - 33 - 4));      // R is at least 2^(bits - 1) units
+      if (!direct && own) {
+        const long long Z[3] = {Z0, Z1, Z2};
+        // J = Jint 2^(bits + unit of y + unit of v), in two factors of normal size
+        const double uy = __longlong_as_double((long long)(1023 + bits + shift - scale) << 52);
+        const double uv = __longlong_as_double((long long)(top + 1 - bits) << 52);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          const __int128 t = (__int128)yi[k] * V + (__int128)vi * dsum[k * N + i] + ((__int128)1 << (bits - 1));
+          J[k] = (double)(Z[k] - (long long)(t >> bits)) * uy * uv;
+        }
+      }
+    }
+  }
+  if (!own) return;
+  if (direct) grad_sum_direct(N, i, width, sidx + b0 + (i & 31), u, cen, J);
+  const double ui = u[i];
+  for (int32_t t = gptr[i]; t < gptr[i + 1]; ++t) {
+    const int32_t f = gface[t];
+    const double du = bval[f - Fi] - ui;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) J[a] += (xf[a * F + f] - cen[a * N + i]) * du;
+  }
+  const double m0 = minv[i], m1 = minv[N + i], m2 = minv[2 * N + i], m3 = minv[3 * N + i], m4 = minv[4 * N + i],
+               m5 = minv[5 * N + i];
+  grad[i] = m0 * J[0] + m1 * J[1] + m2 * J[2];
+  grad[N + i] = m1 * J[0] + m3 * J[1] + m4 * J[2];
+  grad[2 * N + i] = m2 * J[0] + m4 * J[1] + m5 * J[2];
+}
+
 // ---- multiplicity-weighted least-squares gradient (vertex-factorised variant) ---------------
 // grad u_i = Mv_i^{-1} J_i, J_i = sum over the vertices A of T_i, over the cells c around A,
 // of (x_c - x_i)(u_c - u_i), plus each Dirichlet ghost point once per shared vertex. Per
@@ -766,6 +930,11 @@ __global__ void k_nonfinite(const double* __restrict__ x, int64_t n, int* flag) 
 
 }  // namespace
 
+cudaError_t prepare_gradient_fixed() {
+  return cudaFuncSetAttribute((const void*)k_gradient_fixed, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)(2 * kGradTileMaxHalo * sizeof(longlong2)));
+}
+
 // ---- launchers -------------------------------------------------------------------------------
 template <typename T>
 cudaError_t launch_gradient(fvgb_mesh_s* m, int bcset, const T* u, T* grad, cudaStream_t s) {
@@ -777,6 +946,16 @@ cudaError_t launch_gradient(fvgb_mesh_s* m, int bcset, const T* u, T* grad, cuda
   const unsigned gg = shape_grid(m, kTuneGrad, t.N);
   const int tg = m->tune[kTuneGrad].threads;
   if (t.dim == 3) {
+    if constexpr (sizeof(T) == 8) {
+      if (t.tile_max > 0) {      // FP64: fixed-point sums in shared memory
+        k_gradient_fixed<<<(unsigned)t.n_tile, kGradTile, 2 * t.tile_max * sizeof(longlong2), s>>>(
+            t.N, t.F, t.Fi, t.nsell.ptr, t.nsell.idx, t.tile_lidx, t.tile_ptr, t.tile_idx, t.tile_fix, t.xfix,
+            t.tile_dsum, t.tile_pad, t.fix_scale, t.tile_max, (const double*)u, (const double*)g.cen, (const double*)g.xf,
+            (const double*)b.minv, b.gptr, b.gface, (const double*)b.bval, (double*)grad);
+        count_launch();
+        return cudaGetLastError();
+      }
+    }
     k_grad_pack<3><<<gp, kThreads, 0, s>>>(t.N, g.cen, g.cen_lo, u, rec);
     if constexpr (sizeof(T) == 4) {
       if (t.tile_max > 0) {      // FP32: the shared-memory form
