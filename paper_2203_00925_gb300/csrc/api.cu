@@ -68,29 +68,30 @@ void build_sell(const std::vector<int32_t>& ptr, const std::vector<int32_t>& idx
   }
 }
 
-// Halo lists of the shared-memory gradient (see TopoDev): per tile of kGradTile rows, its
-// own rows, then every other cell met in the rows' padded node-neighbour lists (sorted);
-// lidx[pos] is the position of sidx[pos] in its row's tile list. Returns the longest list.
-// Order each lane's neighbour entries of a SELL-32 slice so that, column by column, the
+// Order each lane's neighbour entries of a warp's 32 rows so that, column by column, the
 // eight lanes of a quarter warp read records in different shared-memory bank groups
 // (record k of 16 bytes sits in group k % 8; a quarter warp's 16-byte reads are served in
 // one pass when their groups differ, or when they read the same record). Greedy: per
 // column and quarter, each lane takes an entry of the least used group it still has. The
-// least-squares sum is the same set of terms in another order.
-void order_slice_for_banks(int16_t* lid, int width) {
-  thread_local std::vector<int16_t> bucket[32][8];   // reused across slices
+// least-squares sum is the same set of terms in another order. row[lane]: the lane's first
+// entry (stride 32), width[lane] its entries (0: no row).
+void order_rows_for_banks(int16_t* const* row, const int* width) {
+  thread_local std::vector<int16_t> bucket[32][8];   // reused across warps
+  int most = 0;
   for (int lane = 0; lane < 32; ++lane) {
     for (int g = 0; g < 8; ++g) bucket[lane][g].clear();
-    for (int c = width - 1; c >= 0; --c) {            // popped from the back: original order
-      const int16_t v = lid[32 * c + lane];
+    for (int c = width[lane] - 1; c >= 0; --c) {      // popped from the back: original order
+      const int16_t v = row[lane][32 * c];
       bucket[lane][v & 7].push_back(v);
     }
+    most = std::max(most, width[lane]);
   }
-  for (int c = 0; c < width; ++c) {
+  for (int c = 0; c < most; ++c) {
     for (int qw = 0; qw < 4; ++qw) {
       int cnt[8] = {0, 0, 0, 0, 0, 0, 0, 0};          // distinct records read in each group
       int first[8] = {-1, -1, -1, -1, -1, -1, -1, -1};
       for (int lane = 8 * qw; lane < 8 * qw + 8; ++lane) {
+        if (c >= width[lane]) continue;
         int best = -1, best_cost = 1 << 30;
         for (int g = 0; g < 8; ++g) {
           if (bucket[lane][g].empty()) continue;
@@ -102,12 +103,15 @@ void order_slice_for_banks(int16_t* lid, int width) {
         bucket[lane][best].pop_back();
         if (first[best] < 0) first[best] = v;
         if (best_cost > 0) cnt[best] += 1;
-        lid[32 * c + lane] = v;
+        row[lane][32 * c] = v;
       }
     }
   }
 }
 
+// Halo lists of the shared-memory gradient (see TopoDev): per tile its own rows, then every
+// other cell met in the rows' padded node-neighbour lists (sorted); lidx[pos] is the position
+// of sidx[pos] in its row's tile list. Returns the longest list.
 // Tiles are the row ranges [start[t], start[t + 1]) (at most kGradTile rows each).
 int build_grad_tiles(int64_t N, const std::vector<int64_t>& start, const std::vector<int64_t>& sptr,
                      const std::vector<int32_t>& sidx, std::vector<int32_t>& tptr, std::vector<int32_t>& tidx,
@@ -135,10 +139,16 @@ int build_grad_tiles(int64_t N, const std::vector<int64_t>& start, const std::ve
       if (L.size() <= 32767) {
         for (int64_t r = r0; r < r1; ++r)
           for (int64_t q = sptr[r / 32] + r % 32; q < sptr[r / 32 + 1]; q += 32) lidx[q] = (int16_t)pos[sidx[q]];
-        // the slices whose lanes are this tile's warps
-        if (r0 % 32 == 0)
-          for (int64_t sl = r0 / 32; sl < (r1 == N ? (r1 + 31) / 32 : r1 / 32); ++sl)
-            order_slice_for_banks(lidx.data() + sptr[sl], (int)((sptr[sl + 1] - sptr[sl]) / 32));
+        for (int64_t w0 = r0; w0 < r1; w0 += 32) {      // the tile's warps
+          int16_t* row[32];
+          int width[32];
+          for (int lane = 0; lane < 32; ++lane) {
+            const int64_t r = w0 + lane;
+            width[lane] = r < r1 ? (int)((sptr[r / 32 + 1] - sptr[r / 32]) / 32) : 0;
+            row[lane] = r < r1 ? lidx.data() + sptr[r / 32] + r % 32 : nullptr;
+          }
+          order_rows_for_banks(row, width);
+        }
       }
       max_len = std::max(max_len, (int)L.size());
     }
@@ -150,90 +160,120 @@ int build_grad_tiles(int64_t N, const std::vector<int64_t>& start, const std::ve
   return max_len;
 }
 
-// What k_gradient_fixed needs beside the tiles (FP64 meshes; tiles do not cross parts, so that
-// a mesh gives the same bits alone and in an ensemble):
+// What the FP64 gradient's fixed-point sums (k_gradient_fixed) need beside the halo lists.
+// Tiles do not cross parts, so that a mesh gives the same bits alone and in an ensemble.
 //  - centres as integers in units of 2^-scale (|x| 2^scale < 2^61: exact for every coordinate
 //    of at least 2^-9 of the largest);
+//  - tiles: up to kGradTile consecutive rows, ended early where the next row would stretch
+//    the halo to more than kFixedSpread times the smallest neighbourhood (a jump of the Morton
+//    curve, a graded mesh): the tile's unit would be coarse for those cells;
 //  - per tile bits = 62 - ceil(log2(w + 1)), w the longest neighbour list of its part, so
-//    that a sum over a list stays below 2^62, and the right shift (negative: left) that brings
-//    its coordinate differences from the first own centre below 2^bits;
+//    that a sum over a list stays below 2^62 (0, FP64 sums, in a part of less than one tile
+//    and with lists above 511), and the right shifts (negative: left) that bring its centre
+//    differences below 2^bits;
 //  - per cell D = sum_j (y_j - y_i) of those shifted differences over its neighbours, and the
 //    padding entries of its list.
-// A tile keeps the FP64 sums (bits = 0) in a part of less than one tile, with lists above 511
-// entries, or when its extent is more than kFixedSpread times the smallest neighbourhood in it
-// (a strongly graded mesh): the tile's unit would be coarse for those cells.
 constexpr double kFixedSpread = 8.0;
 
-void build_fixed_tiles(const HostMesh& h, const std::vector<int64_t>& start, const std::vector<int32_t>& tptr,
-                       const std::vector<int32_t>& tidx, std::vector<longlong4_16a>& xfix,
-                       std::vector<int4>& tile, std::vector<int64_t>& dsum, int& scale) {
+struct FixedHost {
+  std::vector<longlong4_16a> xfix;
+  std::vector<int64_t> start;
+  std::vector<GradTileFix> tile;
+  std::vector<int64_t> dsum;
+  std::vector<int16_t> pad;
+  int scale = 0;
+};
+
+// largest component of x_j - x_i
+long long fixed_distance(const longlong4_16a& p, const longlong4_16a& q) {
+  auto mag = [](long long v) { return v < 0 ? -v : v; };
+  return std::max(mag(p.x - q.x), std::max(mag(p.y - q.y), mag(p.z - q.z)));
+}
+
+// integer centres and tiles
+void build_fixed_start(const HostMesh& h, FixedHost& o) {
   const int64_t N = h.N;
   const std::vector<double>& cen = h.cen;
   double top = 0.0;
   for (double c : cen) top = std::max(top, std::fabs(c));
   int e = 0;
   std::frexp(top, &e);                       // top < 2^e
-  scale = 61 - e;
-  const bool usable = top > 0.0 && std::isfinite(top) && scale > -900 && scale < 900;
-  xfix.resize(N);
+  o.scale = 61 - e;
+  const bool usable = top > 0.0 && std::isfinite(top) && o.scale > -200 && o.scale < 260;
+  o.xfix.resize(N);
+  std::vector<long long> near(N, 0);         // extent of each neighbourhood
 #pragma omp parallel for
   for (int64_t i = 0; i < N; ++i) {
-    auto fix = [&](double c) { return usable ? std::llrint(std::ldexp(c, scale)) : 0ll; };
-    xfix[i] = longlong4_16a{fix(cen[i]), fix(cen[N + i]), fix(cen[2 * N + i]), 0};
+    auto fix = [&](double c) { return usable ? std::llrint(std::ldexp(c, o.scale)) : 0ll; };
+    o.xfix[i] = longlong4_16a{fix(cen[i]), fix(cen[N + i]), fix(cen[2 * N + i]), 0};
   }
-  const int64_t ntile = (int64_t)start.size() - 1;
-  const int P = (int)h.part_cell_begin.size() - 1;
-  std::vector<int> part_bits(P, 0);
 #pragma omp parallel for
-  for (int p = 0; p < P; ++p) {
+  for (int64_t i = 0; i < N; ++i)
+    for (int32_t q = h.nptr[i]; q < h.nptr[i + 1]; ++q)
+      near[i] = std::max(near[i], fixed_distance(o.xfix[h.nidx[q]], o.xfix[i]));
+  for (size_t p = 0; p + 1 < h.part_cell_begin.size(); ++p) {
     const int64_t lo = h.part_cell_begin[p], hi = h.part_cell_begin[p + 1];
-    int64_t most = 1;
-    for (int64_t i = lo; i < hi; ++i) most = std::max<int64_t>(most, h.nptr[i + 1] - h.nptr[i]);
+    int64_t widest = 1;
+    for (int64_t i = lo; i < hi; ++i) widest = std::max<int64_t>(widest, h.nptr[i + 1] - h.nptr[i]);
     int w = 0;
-    while ((int64_t(1) << w) < most + 1) ++w;
-    if (usable && hi - lo >= kGradTile && w <= 9) part_bits[p] = 62 - w;
-  }
-  tile.resize(ntile);
-  dsum.assign((size_t)3 * N, 0);
-#pragma omp parallel for schedule(dynamic, 64)
-  for (int64_t t = 0; t < ntile; ++t) {
-    const int64_t r0 = start[t], r1 = start[t + 1];
-    const int p = (int)(std::upper_bound(h.part_cell_begin.begin(), h.part_cell_begin.end(), r0) -
-                        h.part_cell_begin.begin()) - 1;
-    const int bits = part_bits[p];
-    tile[t] = int4{(int)r0, (int)(r1 - r0), 0, 0};
-    if (bits == 0) continue;
-    const longlong4_16a o = xfix[r0];
-    auto diff = [&](int64_t j, const longlong4_16a& q, long long* d) {
-      d[0] = xfix[j].x - q.x; d[1] = xfix[j].y - q.y; d[2] = xfix[j].z - q.z;
-    };
-    long long d[3], most = 1;
-    for (int32_t k = tptr[t]; k < tptr[t + 1]; ++k) {
-      diff(tidx[k], o, d);
-      for (int a = 0; a < 3; ++a) most = std::max(most, d[a] < 0 ? -d[a] : d[a]);
-    }
-    long long least = most;
-    for (int64_t i = r0; i < r1; ++i) {
-      long long m = 0;
-      for (int32_t q = h.nptr[i]; q < h.nptr[i + 1]; ++q) {
-        diff(h.nidx[q], xfix[i], d);
-        for (int a = 0; a < 3; ++a) m = std::max(m, d[a] < 0 ? -d[a] : d[a]);
+    while ((int64_t(1) << w) < widest + 1) ++w;
+    const int bits = usable && hi - lo >= kGradTile && w <= 9 ? 62 - w : 0;
+    for (int64_t r = lo; r < hi;) {
+      long long reach = 0, least = near[r];
+      int64_t end = r;
+      for (; end < hi && end < r + kGradTile; ++end) {
+        const long long to = std::max(reach, fixed_distance(o.xfix[end], o.xfix[r]) + near[end]);
+        const long long small = std::min(least, near[end]);
+        if (bits > 0 && end > r && (double)to > kFixedSpread * (double)small) break;
+        reach = to;
+        least = small;
       }
-      least = std::min(least, m);
+      o.start.push_back(r);
+      o.tile.push_back(GradTileFix{(int32_t)r, (int32_t)(end - r), (int16_t)bits, 0, 0, 0});
+      r = end;
     }
-    if ((double)most > kFixedSpread * (double)least) continue;
-    int sh = 0;
-    while (most < (1ll << (bits - 1 + sh))) --sh;     // room to the left
-    while (most >= (1ll << (bits + sh)) && bits + sh < 62) ++sh;  // or cut to the right
-    tile[t].z = sh;
-    tile[t].w = bits;
+  }
+  o.start.push_back(N);
+}
+
+// shifts, sums of differences and padding counts, once the halo lists are known
+void build_fixed_sums(const HostMesh& h, const std::vector<int64_t>& sptr, const std::vector<int32_t>& tptr,
+                      const std::vector<int32_t>& tidx, FixedHost& o) {
+  const int64_t N = h.N;
+  o.dsum.assign((size_t)3 * N, 0);
+  o.pad.resize(N);
+#pragma omp parallel for schedule(dynamic, 64)
+  for (int64_t t = 0; t < (int64_t)o.tile.size(); ++t) {
+    GradTileFix& tile = o.tile[t];
+    const int64_t r0 = tile.row0, r1 = r0 + tile.rows;
+    const int bits = tile.bits;
+    for (int64_t i = r0; i < r1; ++i)
+      o.pad[i] = (int16_t)std::min<int64_t>(INT16_MAX, (sptr[i / 32 + 1] - sptr[i / 32]) / 32 - (h.nptr[i + 1] - h.nptr[i]));
+    if (bits == 0) continue;
+    const longlong4_16a at = o.xfix[r0];
+    long long most = 1, widest = 1;
+    for (int32_t k = tptr[t]; k < tptr[t + 1]; ++k) most = std::max(most, fixed_distance(o.xfix[tidx[k]], at));
+    for (int64_t i = r0; i < r1; ++i)
+      for (int32_t q = h.nptr[i]; q < h.nptr[i + 1]; ++q)
+        widest = std::max(widest, fixed_distance(o.xfix[h.nidx[q]], o.xfix[i]));
+    auto shift_for = [&](long long top) {
+      int sh = 0;
+      while (top < (1ll << (bits - 1 + sh))) --sh;     // room to the left
+      while (bits + sh < 62 && top >= (1ll << (bits + sh))) ++sh;  // or cut to the right
+      return sh;
+    };
+    const int sh = shift_for(most);
+    tile.shift = (int16_t)sh;
+    tile.own_shift = (int16_t)shift_for(widest);
     auto cut = [&](long long v) { return sh >= 0 ? v >> sh : (long long)((unsigned long long)v << -sh); };
     for (int64_t i = r0; i < r1; ++i) {
-      diff(i, o, d);
-      const long long yi[3] = {cut(d[0]), cut(d[1]), cut(d[2])};
+      const longlong4_16a& x = o.xfix[i];
+      const long long yi[3] = {cut(x.x - at.x), cut(x.y - at.y), cut(x.z - at.z)};
       for (int32_t q = h.nptr[i]; q < h.nptr[i + 1]; ++q) {
-        diff(h.nidx[q], o, d);
-        for (int a = 0; a < 3; ++a) dsum[a * N + i] += cut(d[a]) - yi[a];
+        const longlong4_16a& y = o.xfix[h.nidx[q]];
+        o.dsum[i] += cut(y.x - at.x) - yi[0];
+        o.dsum[N + i] += cut(y.y - at.y) - yi[1];
+        o.dsum[2 * N + i] += cut(y.z - at.z) - yi[2];
       }
     }
   }
@@ -866,26 +906,28 @@ static fvgb_status upload_impl(int32_t dim, int64_t n_vert, const double* xyz, i
       (int64_t)h.nptr[h.N] < (int64_t)INT32_MAX / 2) {   // the shared-memory gradients
     std::vector<int32_t> tptr, tidx;
     std::vector<int16_t> lidx;
-    std::vector<int64_t> start;                  // tiles; in FP64 they do not cross parts
-    for (int p = 0; p < (prec == FVGB_FP64 ? n_part : 1); ++p)
-      for (int64_t r = h.part_cell_begin[p]; r < (prec == FVGB_FP64 ? h.part_cell_begin[p + 1] : h.N); r += kGradTile)
-        start.push_back(r);
-    start.push_back(h.N);
-    const int mx = build_grad_tiles(h.N, start, sptr, sidx, tptr, tidx, lidx);
-    const bool tiled = mx <= kGradTileMaxHalo;
+    FixedHost fx;
+    if (prec == FVGB_FP64) {
+      build_fixed_start(h, fx);
+    } else {
+      for (int64_t r = 0; r < h.N; r += kGradTile) fx.start.push_back(r);
+      fx.start.push_back(h.N);
+    }
+    // tiles much shorter than their room (a mesh in no local order) gain nothing
+    bool tiled = (int64_t)fx.start.size() - 1 <= h.N / 32 + n_part;
+    const int mx = tiled ? build_grad_tiles(h.N, fx.start, sptr, sidx, tptr, tidx, lidx) : 0;
+    tiled = tiled && mx <= kGradTileMaxHalo;
     if (tiled && prec == FVGB_FP64) {
-      std::vector<longlong4_16a> xfix;
-      std::vector<int4> tile;
-      std::vector<int64_t> dsum;
-      build_fixed_tiles(h, start, tptr, tidx, xfix, tile, dsum, t.fix_scale);
-      std::vector<int16_t> pad(h.N);
-      for (int64_t i = 0; i < h.N; ++i)
-        pad[i] = (int16_t)std::min<int64_t>(INT16_MAX, (sptr[i / 32 + 1] - sptr[i / 32]) / 32 - (h.nptr[i + 1] - h.nptr[i]));
-      t.n_tile = (int)tile.size();
-      if ((e = dupload(m, &t.tile_pad, pad, s))) return fail(e, "upload");
-      if ((e = dupload(m, &t.xfix, xfix, s))) return fail(e, "upload");
-      if ((e = dupload(m, &t.tile_fix, tile, s))) return fail(e, "upload");
-      if ((e = dupload(m, &t.tile_dsum, dsum, s))) return fail(e, "upload");
+      build_fixed_sums(h, sptr, tptr, tidx, fx);
+      t.n_tile = (int)fx.tile.size();
+      t.fix_scale = fx.scale;
+      t.fix_bits = fx.tile[0].bits;
+      for (const GradTileFix& q : fx.tile)
+        if (q.bits != t.fix_bits) t.fix_bits = 0;
+      if ((e = dupload(m, &t.tile_pad, fx.pad, s))) return fail(e, "upload");
+      if ((e = dupload(m, &t.xfix, fx.xfix, s))) return fail(e, "upload");
+      if ((e = dupload(m, &t.tile_fix, fx.tile, s))) return fail(e, "upload");
+      if ((e = dupload(m, &t.tile_dsum, fx.dsum, s))) return fail(e, "upload");
       if ((e = prepare_gradient_fixed())) return fail(e, "shared memory limit");
     }
     if (tiled) {

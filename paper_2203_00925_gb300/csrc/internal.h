@@ -12,6 +12,15 @@
 
 namespace fvgb {
 
+// Tile of the FP64 gradient's fixed-point sums (k_gradient_fixed).
+struct GradTileFix {
+  int32_t row0, rows;
+  int16_t bits;       // magnitude bits of its integers (0: FP64 sums)
+  int16_t shift;      // right shift of centre differences from its first cell
+  int16_t own_shift;  // right shift of centre differences from a cell to its neighbours
+  int16_t spare;
+};
+
 // Sliced-ELL (SELL-32) list: rows grouped in slices of 32 consecutive rows; slice s
 // stores its entries column-major from ptr[s], width ptr[s+1]-ptr[s] over 32, so one
 // warp reads 128 contiguous bytes per column.
@@ -77,11 +86,11 @@ struct TopoDev {
   // FP64 meshes (k_gradient_fixed): integer centres, and per tile and cell what its
   // fixed-point sums need (see build_fixed_tiles)
   longlong4_16a* xfix = nullptr; // [N] {x, y, z, 0} in units of 2^-fix_scale
-  int4* tile_fix = nullptr;      // [n_tile] {first row, rows, right shift of the coordinate
-                                 // differences, magnitude bits (0: the tile keeps FP64 sums)}
+  GradTileFix* tile_fix = nullptr;  // [n_tile]
   int64_t* tile_dsum = nullptr;  // [3][N] sum of the cell's shifted neighbour differences
   int16_t* tile_pad = nullptr;   // [N] padding entries of the cell's list (the cell itself)
-  int fix_scale = 0;
+  int fix_scale = 0;             // see xfix
+  int fix_bits = 0;              // the tiles' bits where all have the same, else 0
   int n_tile = 0;
 };
 

@@ -259,13 +259,54 @@ k_gradient_tiled(int64_t N, int64_t F, int64_t Fi, const int64_t* __restrict__ s
 // exact in 64 bits and the last line is formed in 128. Per neighbour entry that leaves four
 // 64-bit additions and two 16-byte shared-memory reads (the records, in two arrays so that the
 // lists' bank-aware order serves both).
-// The unit is relative to the tile's range R of v: a cell whose own neighbours differ by less
-// than R / 16 (a steep field in the tile), and every cell of a tile whose u is not finite or
-// nearly denormal, or that has no bits, takes the FP64 sum (grad_sum_direct), in the order
-// of k_gradient.
-__device__ __noinline__ void grad_sum_direct(int64_t N, int64_t i, int width, const int32_t* __restrict__ col,
-                                             const double* __restrict__ u, const double* __restrict__ cen,
-                                             double* J) {
+// The unit is relative to the tile's range R of v. A cell whose own neighbours differ by less
+// than R / 16 (a steep field in the tile) sums its own products (x_j - x_i)(u_j - u_i) instead,
+// also as integers but with the cell's own unit (own_scale_sum). Where u is not finite or beyond 2^+-600, and in
+// parts of less than a tile, the sum stays in FP64, in the order of k_gradient.
+constexpr int kFixTopMin = 400, kFixTopMax = 1600;   // biased exponents the scaled sums stay normal for
+
+__device__ __forceinline__ int exp_bits(long long v) { return (int)((unsigned long long)v >> 52) & 0x7ff; }
+// biased exponent of a nonzero value (1 for a subnormal), 0 for zero
+__device__ __forceinline__ int exp_of(long long v) {
+  const int e = exp_bits(v);
+  return e > 0 ? e : ((v & 0x7fffffffffffffffll) != 0 ? 1 : 0);
+}
+
+// the value of the FP64 bits a as an integer, in units of 2^(top - 1022 - bits) (its exponent
+// at most top): bits magnitude bits, rounded to nearest
+__device__ __forceinline__ long long to_fixed(long long a, int top, int bits) {
+  const int e = exp_bits(a), cut = top - e;
+  unsigned long long mag = e > 0 ? ((a & 0xfffffffffffffull) | (1ull << 52)) << (bits - 53) : 0;
+  mag = cut == 0 ? mag : (cut < 63 ? (mag + (1ull << (cut - 1))) >> cut : 0);
+  return a < 0 ? -(long long)mag : (long long)mag;
+}
+
+// round(y v / 2^bits)
+__device__ __forceinline__ long long fixed_mul(long long y, long long v, int bits) {
+  const unsigned long long lo = (unsigned long long)y * (unsigned long long)v;
+  const long long hi = __mul64hi(y, v);
+  const unsigned long long l = lo + (1ull << (bits - 1));
+  const long long h = hi + (l < lo ? 1 : 0);
+  return (long long)(((unsigned long long)h << (64 - bits)) | (l >> bits));
+}
+
+// v 2^e as FP64, rounded to nearest even (the result is in the normal range), without the
+// FP64 pipe
+__device__ __forceinline__ double from_fixed(long long v, int e) {
+  if (v == 0) return 0.0;
+  unsigned long long m = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+  const int lz = __clzll(m);
+  m <<= lz;
+  const unsigned long long rest = m & 0x7ff;
+  m >>= 11;
+  m += rest > 0x400 || (rest == 0x400 && (m & 1)) ? 1 : 0;
+  const unsigned long long w = ((unsigned long long)(1022 + 63 - lz + e) << 52) + m;   // m holds the leading one
+  return __longlong_as_double((long long)(w | (v < 0 ? 1ull << 63 : 0)));
+}
+
+// J of one cell in FP64, neighbours' values and centres from memory
+__device__ __noinline__ void direct_sum(int64_t N, int64_t i, int width, const int32_t* __restrict__ col,
+                                        const double* __restrict__ u, const double* __restrict__ cen, double* J) {
   const double ui = u[i], x = cen[i], y = cen[N + i], z = cen[2 * N + i];
   double j0 = 0.0, j1 = 0.0, j2 = 0.0;
   for (int c = 0; c < width; ++c) {
@@ -278,42 +319,99 @@ __device__ __noinline__ void grad_sum_direct(int64_t N, int64_t i, int width, co
   J[0] = j0; J[1] = j1; J[2] = j2;
 }
 
-// round(y v / 2^bits)
-__device__ __forceinline__ long long fixed_mul(long long y, long long v, int bits) {
-  const unsigned long long lo = (unsigned long long)y * (unsigned long long)v;
-  const long long hi = __mul64hi(y, v);
-  const unsigned long long half = 1ull << (bits - 1);
-  const unsigned long long l = lo + half;
-  const long long h = hi + (l < lo ? 1 : 0);
-  return (long long)(((unsigned long long)h << (64 - bits)) | (l >> bits));
+// J of one cell from its own integer products: differences of the integer centres shifted to
+// ``bits`` bits, u_j - u_i converted with the exponent top (0: the largest, found first).
+// False where the exponents leave the range.
+template <int BITS>
+__device__ __noinline__ bool own_scale_sum(int64_t i, int width, const int32_t* __restrict__ col,
+                                           const longlong4_16a* __restrict__ xfix, const double* __restrict__ u,
+                                           int tile_bits, int shift, int scale, int top, double* J) {
+  const int bits = BITS > 0 ? BITS : tile_bits;
+  const longlong2* X = reinterpret_cast<const longlong2*>(xfix);
+  constexpr int U = 4;                  // neighbours in flight
+  const double ui = u[i];
+  if (top == 0) {
+    for (int c0 = 0; c0 < width; c0 += U) {
+      double uj[U];
+#pragma unroll
+      for (int q = 0; q < U; ++q) uj[q] = c0 + q < width ? u[col[32 * (c0 + q)]] : ui;
+#pragma unroll
+      for (int q = 0; q < U; ++q) top = max(top, exp_of(__double_as_longlong(uj[q] - ui)));
+    }
+    if (top == 0) { J[0] = J[1] = J[2] = 0.0; return true; }
+  }
+  if (top < kFixTopMin || top > kFixTopMax) return false;
+  const longlong2 xi = X[2 * i];
+  const long long zi = X[2 * i + 1].x;
+  long long s[3] = {0, 0, 0};
+  for (int c0 = 0; c0 < width; c0 += U) {
+    int64_t j[U];
+    longlong2 a[U];
+    long long az[U];
+    double uj[U];
+#pragma unroll
+    for (int q = 0; q < U; ++q) j[q] = c0 + q < width ? col[32 * (c0 + q)] : i;   // the cell itself adds 0
+#pragma unroll
+    for (int q = 0; q < U; ++q) {
+      a[q] = __ldg(X + 2 * j[q]);
+      az[q] = __ldg(&X[2 * j[q] + 1].x);
+      uj[q] = u[j[q]];
+    }
+#pragma unroll
+    for (int q = 0; q < U; ++q) {
+      const long long v = to_fixed(__double_as_longlong(uj[q] - ui), top, bits);
+      const long long d[3] = {a[q].x - xi.x, a[q].y - xi.y, az[q] - zi};
+#pragma unroll
+      for (int k = 0; k < 3; ++k) s[k] += fixed_mul(shift >= 0 ? d[k] >> shift : d[k] << -shift, v, bits);
+    }
+  }
+  const int e = shift - scale + top - 1022;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) J[k] = from_fixed(s[k], e);
+  return true;
 }
 
-__global__ void __launch_bounds__(kGradTile)
+// Two threads a cell, each summing half of its list (the second half's partial sums are
+// exact integers, so the split changes no bit): the tile's chain of dependent loads, not the
+// issue rate, bounds the block. BITS: the tiles' bits where all have the same (0: per tile).
+constexpr int kFixBitsUsual = 55;       // neighbour lists of 64 to 127 cells
+constexpr int kFixThreads = 2 * kGradTile;
+constexpr int kFixBatch = 4;            // halo records in flight per thread
+
+template <int BITS>
+__global__ void __launch_bounds__(kFixThreads, 4)
 k_gradient_fixed(int64_t N, int64_t F, int64_t Fi, const int64_t* __restrict__ sptr,
                  const int32_t* __restrict__ sidx, const int16_t* __restrict__ lidx,
                  const int32_t* __restrict__ tptr, const int32_t* __restrict__ tidx,
-                 const int4* __restrict__ tfix, const longlong4_16a* __restrict__ xfix,
-                 const int64_t* __restrict__ dsum, const int16_t* __restrict__ pad, int scale, int max_halo, const double* __restrict__ u, const double* __restrict__ cen,
+                 const GradTileFix* __restrict__ tfix, const longlong4_16a* __restrict__ xfix,
+                 const int64_t* __restrict__ dsum, const int16_t* __restrict__ pad, int scale, int max_halo,
+                 const double* __restrict__ u, const double* __restrict__ cen,
                  const double* __restrict__ xf, const double* __restrict__ minv,
                  const int32_t* __restrict__ gptr, const int32_t* __restrict__ gface,
                  const double* __restrict__ bval, double* __restrict__ grad) {
   extern __shared__ longlong2 frec[];
   longlong2* ra = frec;                 // {v, z_x}
   longlong2* rb = frec + max_halo;      // {z_y, z_z}
-  __shared__ int s_top[kGradTile / 32];
-  const int4 td = tfix[blockIdx.x];
-  const int64_t r0 = td.x;
-  const int shift = td.z, bits = td.w;
-  const int32_t h0 = tptr[blockIdx.x], nh = tptr[blockIdx.x + 1] - h0;
-  const bool own = (int)threadIdx.x < td.y;
-  const int64_t i = own ? r0 + threadIdx.x : r0;
+  __shared__ int s_top[kFixThreads / 32];
+  __shared__ longlong2 s_sum[2][kGradTile];   // the second halves' sums
+  __shared__ int2 s_range[kGradTile];
+  const GradTileFix td = tfix[blockIdx.x];
+  const int64_t r0 = td.row0;
+  const int bits = BITS > 0 ? BITS : td.bits, shift = td.shift;
+  const int row = threadIdx.x & (kGradTile - 1), half = threadIdx.x / kGradTile;
+  const bool own = row < td.rows;
+  const int64_t i = own ? r0 + row : r0;
   const int64_t b0 = sptr[i >> 5];
   const int width = own ? (int)((sptr[(i >> 5) + 1] - b0) >> 5) : 0;
-  const int16_t* col = lidx + b0 + (i & 31);
-  const int32_t* halo = tidx + h0;
+  const int32_t* gcol = sidx + b0 + (i & 31);
   double J[3] = {0.0, 0.0, 0.0};
-  bool direct = bits == 0;
-  if (!direct) {                        // uniform over the block
+  // how the cell sums: 0 done, 1 its own unit, 2 FP64
+  int todo = bits == 0 ? 2 : 1;
+  int otop = 0;                         // known exponent of the cell's own differences
+  if (bits > 0) {                       // uniform over the block
+    const int32_t h0 = tptr[blockIdx.x], nh = tptr[blockIdx.x + 1] - h0;
+    const int32_t* halo = tidx + h0;
+    const int16_t* col = lidx + b0 + (i & 31);
     // the halo's differences from the first own cell; largest exponent of those of u
     const longlong2* X = reinterpret_cast<const longlong2*>(xfix);
     const double uo = u[r0];
@@ -321,47 +419,60 @@ k_gradient_fixed(int64_t N, int64_t F, int64_t Fi, const int64_t* __restrict__ s
     const long long oz = X[2 * r0 + 1].x;
     int top = 0;
     long long yi[3] = {0, 0, 0};
-    for (int k = threadIdx.x; k < nh; k += kGradTile) {
-      const int64_t j = __ldg(halo + k);
-      const longlong2 a = __ldg(X + 2 * j);
-      const long long az = __ldg(&X[2 * j + 1].x);
-      const long long du = __double_as_longlong(u[j] - uo);
-      long long y[3] = {a.x - oa.x, a.y - oa.y, az - oz};
+    for (int k0 = threadIdx.x; k0 < nh; k0 += kFixBatch * kFixThreads) {
+      int32_t j[kFixBatch];
+      longlong2 a[kFixBatch];
+      long long az[kFixBatch];
+      double uj[kFixBatch];
 #pragma unroll
-      for (int c = 0; c < 3; ++c) y[c] = shift >= 0 ? y[c] >> shift : y[c] << -shift;
-      if (k < kGradTile) { yi[0] = y[0]; yi[1] = y[1]; yi[2] = y[2]; }   // the thread's own cell
-      ra[k] = make_longlong2(du, y[0]);
-      rb[k] = make_longlong2(y[1], y[2]);
-      const int e = (int)((unsigned long long)du >> 52) & 0x7ff;
-      top = max(top, e > 0 ? e : ((du & 0x7fffffffffffffffll) != 0 ? 1 : 0));
+      for (int q = 0; q < kFixBatch; ++q) j[q] = k0 + q * kFixThreads < nh ? __ldg(halo + k0 + q * kFixThreads) : (int32_t)r0;
+#pragma unroll
+      for (int q = 0; q < kFixBatch; ++q) {
+        a[q] = __ldg(X + 2 * (int64_t)j[q]);
+        az[q] = __ldg(&X[2 * (int64_t)j[q] + 1].x);
+        uj[q] = u[j[q]];
+      }
+#pragma unroll
+      for (int q = 0; q < kFixBatch; ++q) {
+        const int k = k0 + q * kFixThreads;
+        if (k >= nh) break;
+        const long long du = __double_as_longlong(uj[q] - uo);
+        long long y[3] = {a[q].x - oa.x, a[q].y - oa.y, az[q] - oz};
+#pragma unroll
+        for (int c = 0; c < 3; ++c) y[c] = shift >= 0 ? y[c] >> shift : y[c] << -shift;
+        if (k < kGradTile) { yi[0] = y[0]; yi[1] = y[1]; yi[2] = y[2]; }   // the thread's own cell
+        ra[k] = make_longlong2(du, y[0]);
+        rb[k] = make_longlong2(y[1], y[2]);
+        top = max(top, exp_of(du));
+      }
     }
     top = __reduce_max_sync(0xffffffffu, top);
     if ((threadIdx.x & 31) == 0) s_top[threadIdx.x >> 5] = top;
     __syncthreads();
 #pragma unroll
-    for (int w = 0; w < kGradTile / 32; ++w) top = max(top, s_top[w]);
-    // not finite, or so small that the scaled sums could leave the normal range
-    direct = top == 0x7ff || (top < 256 && top > 0);
-    if (!direct && top > 0) {
-      for (int k = threadIdx.x; k < nh; k += kGradTile) {   // the entries this thread staged
+    for (int w = 0; w < kFixThreads / 32; ++w) top = max(top, s_top[w]);
+    if (top == 0) {
+      todo = 0;                         // every difference is zero
+    } else if (top < kFixTopMin || top > kFixTopMax) {
+      todo = 2;
+    } else {
+      for (int k = threadIdx.x; k < nh; k += kFixThreads) {   // the entries this thread staged
         const longlong2 a = ra[k], b = rb[k];
-        const int e = (int)((unsigned long long)a.x >> 52) & 0x7ff;
-        const int cut = top - e;
-        unsigned long long mag = e > 0 ? (((unsigned long long)a.x & 0xfffffffffffffull) | (1ull << 52)) << (bits - 53) : 0;
-        mag = cut == 0 ? mag : (cut < 63 ? (mag + (1ull << (cut - 1))) >> cut : 0);
-        const long long v = a.x < 0 ? -(long long)mag : (long long)mag;
+        const long long v = to_fixed(a.x, top, bits);
         ra[k] = make_longlong2(v, fixed_mul(a.y, v, bits));
         rb[k] = make_longlong2(fixed_mul(b.x, v, bits), fixed_mul(b.y, v, bits));
       }
       __syncthreads();
-      const longlong2 ai = ra[own ? threadIdx.x : 0], bi = rb[own ? threadIdx.x : 0];
+      const longlong2 ai = ra[own ? row : 0], bi = rb[own ? row : 0];
       const long long vi = ai.x;
       // the padding entries (the cell itself) are taken out again
-      const long long np = own ? pad[i] : 0;
+      const long long np = own && half == 0 ? pad[i] : 0;
       long long V = -np * vi, Z0 = -np * ai.y, Z1 = -np * bi.x, Z2 = -np * bi.y;
       int least = (int)(vi >> 32), most = least;
-      int c = 0;
-      for (; c + 4 <= width; c += 4) {
+      const int mid = (width + 1) >> 1;
+      int c = half == 0 ? 0 : mid;
+      const int end = half == 0 ? mid : width;
+      for (; c + 4 <= end; c += 4) {
         const int e0 = __ldg(col + 32 * c), e1 = __ldg(col + 32 * (c + 1)), e2 = __ldg(col + 32 * (c + 2)),
                   e3 = __ldg(col + 32 * (c + 3));
         const longlong2 a[4] = {ra[e0], ra[e1], ra[e2], ra[e3]};
@@ -374,7 +485,7 @@ k_gradient_fixed(int64_t N, int64_t F, int64_t Fi, const int64_t* __restrict__ s
           most = max(most, hi);
         }
       }
-      for (; c < width; ++c) {
+      for (; c < end; ++c) {
         const int e = __ldg(col + 32 * c);
         const longlong2 a = ra[e], b = rb[e];
         V += a.x; Z0 += a.y; Z1 += b.x; Z2 += b.y;
@@ -382,22 +493,36 @@ k_gradient_fixed(int64_t N, int64_t F, int64_t Fi, const int64_t* __restrict__ s
         least = min(least, hi);
         most = max(most, hi);
       }
-      direct = most - least < (1 << (bits - 33 - 4));      // R is at least 2^(bits - 1) units
-      if (!direct && own) {
-        const long long Z[3] = {Z0, Z1, Z2};
-        // J = Jint 2^(bits + unit of y + unit of v), in two factors of normal size
-        const double uy = __longlong_as_double((long long)(1023 + bits + shift - scale) << 52);
-        const double uv = __longlong_as_double((long long)(top + 1 - bits) << 52);
+      if (half == 1) {
+        s_sum[0][row] = make_longlong2(V, Z0);
+        s_sum[1][row] = make_longlong2(Z1, Z2);
+        s_range[row] = make_int2(least, most);
+      }
+      __syncthreads();
+      if (half == 0) {
+        const longlong2 p = s_sum[0][row], q = s_sum[1][row];
+        const int2 r = s_range[row];
+        V += p.x; Z0 += p.y; Z1 += q.x; Z2 += q.y;
+        const int m = max(most, r.y) - min(least, r.x);
+        if (m >= 1 << (bits - 33 - 4)) {      // R is at least 2^(bits - 1) units
+          todo = 0;
+          const long long Z[3] = {Z0, Z1, Z2};
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          const __int128 t = (__int128)yi[k] * V + (__int128)vi * dsum[k * N + i] + ((__int128)1 << (bits - 1));
-          J[k] = (double)(Z[k] - (long long)(t >> bits)) * uy * uv;
+          for (int k = 0; k < 3; ++k) {
+            const __int128 t = (__int128)yi[k] * V + (__int128)vi * dsum[k * N + i] + ((__int128)1 << (bits - 1));
+            J[k] = from_fixed(Z[k] - (long long)(t >> bits), shift - scale + top - 1022);
+          }
+        } else if (m >= 2) {
+          // (m - 1) 2^32 < range of the u_j < (m + 1) 2^32 units: the largest |u_j - u_i| has
+          // at most this exponent (one spare bit for the units' rounding), and two less at least
+          otop = 33 + (31 - __clz(m + 1)) + top - bits + 1;
         }
       }
     }
   }
-  if (!own) return;
-  if (direct) grad_sum_direct(N, i, width, sidx + b0 + (i & 31), u, cen, J);
+  if (!own || half == 1) return;
+  if (todo == 1 && own_scale_sum<BITS>(i, width, gcol, xfix, u, bits, td.own_shift, scale, otop, J)) todo = 0;
+  if (todo != 0) direct_sum(N, i, width, gcol, u, cen, J);
   const double ui = u[i];
   for (int32_t t = gptr[i]; t < gptr[i + 1]; ++t) {
     const int32_t f = gface[t];
@@ -931,8 +1056,12 @@ __global__ void k_nonfinite(const double* __restrict__ x, int64_t n, int* flag) 
 }  // namespace
 
 cudaError_t prepare_gradient_fixed() {
-  return cudaFuncSetAttribute((const void*)k_gradient_fixed, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)(2 * kGradTileMaxHalo * sizeof(longlong2)));
+  const int most = (int)(2 * kGradTileMaxHalo * sizeof(longlong2));
+  cudaError_t e = cudaFuncSetAttribute((const void*)k_gradient_fixed<kFixBitsUsual>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute((const void*)k_gradient_fixed<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  return e;
 }
 
 // ---- launchers -------------------------------------------------------------------------------
@@ -948,10 +1077,11 @@ cudaError_t launch_gradient(fvgb_mesh_s* m, int bcset, const T* u, T* grad, cuda
   if (t.dim == 3) {
     if constexpr (sizeof(T) == 8) {
       if (t.tile_max > 0) {      // FP64: fixed-point sums in shared memory
-        k_gradient_fixed<<<(unsigned)t.n_tile, kGradTile, 2 * t.tile_max * sizeof(longlong2), s>>>(
+        auto* k = t.fix_bits == kFixBitsUsual ? k_gradient_fixed<kFixBitsUsual> : k_gradient_fixed<0>;
+        k<<<(unsigned)t.n_tile, kFixThreads, 2 * t.tile_max * sizeof(longlong2), s>>>(
             t.N, t.F, t.Fi, t.nsell.ptr, t.nsell.idx, t.tile_lidx, t.tile_ptr, t.tile_idx, t.tile_fix, t.xfix,
-            t.tile_dsum, t.tile_pad, t.fix_scale, t.tile_max, (const double*)u, (const double*)g.cen, (const double*)g.xf,
-            (const double*)b.minv, b.gptr, b.gface, (const double*)b.bval, (double*)grad);
+            t.tile_dsum, t.tile_pad, t.fix_scale, t.tile_max, (const double*)u, (const double*)g.cen,
+            (const double*)g.xf, (const double*)b.minv, b.gptr, b.gface, (const double*)b.bval, (double*)grad);
         count_launch();
         return cudaGetLastError();
       }
