@@ -125,7 +125,7 @@ struct PartsDev {
   int64_t* sc_begin = nullptr;  // [n_sc+1] first row of each sub-chunk
   int32_t* sc_part = nullptr;   // [n_sc] part of each sub-chunk
   int32_t* part_sc = nullptr;   // [P+1] first sub-chunk of each part
-  double* buf = nullptr;        // [2][2][n_sc] partial sums
+  double* buf = nullptr;        // [4][n_sc] partial sums
   int* active = nullptr;        // [P] parts the inner solve works on
   int* out_inner = nullptr;     // [P] inner iterations of the last CG launch
   double* norms = nullptr;      // [P] per-part sums of squares

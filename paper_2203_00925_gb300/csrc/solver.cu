@@ -33,35 +33,33 @@ __device__ __forceinline__ unsigned long long global_ns() {
 
 // Grid barrier on a monotone arrival counter with a bounded wait: the r-th barrier of a
 // launch is passed once the counter (zeroed before the launch) reaches r * nblocks, so
-// the last arrival itself releases the waiting blocks (no reset, no second word).
-// ``target`` is the caller's running count. Returns false when any block gave up
-// (status set), in which case the caller leaves. ``skip`` (test hook only) leaves out this
-// block's arrival, so that the other blocks' waits run out.
-__device__ bool grid_barrier(Barrier* bar, unsigned nblocks, unsigned& target, bool skip,
-                             unsigned long long limit_ns) {
-  __shared__ int ok;
-  __syncthreads();
-  target += nblocks;
-  if (threadIdx.x == 0) {
-    volatile unsigned* vcount = &bar->count;
-    volatile int* vstatus = &bar->status;
-    __threadfence();
-    if (!skip) atomicAdd(&bar->count, 1u);
-    int good = 1;
-    if ((int)(*vcount - target) < 0) {
-      const unsigned long long t0 = global_ns();
-      while ((int)(*vcount - target) < 0) {
-        if (*vstatus != 0) { good = 0; break; }
-        if (global_ns() - t0 > limit_ns) { atomicExch(&bar->status, 1); good = 0; break; }
-        __nanosleep(32);
-      }
+// the last arrival itself releases the waiting blocks (no reset, no second word). One thread
+// of the block arrives (release: what the block wrote before the preceding __syncthreads is
+// visible with it), one warp waits (acquire). Measured over 152 blocks: 2,280 cycles a
+// barrier; slots polled by every block instead of the counter 3,400 (one to a 128-byte line)
+// to 10,900 (packed): stores to a line that is being polled are slow.
+__device__ __forceinline__ void grid_arrive(Barrier* bar) {
+  asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&bar->count) : "memory");
+}
+__device__ __forceinline__ unsigned count_acquire(const Barrier* bar) {
+  unsigned v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&bar->count) : "memory");
+  return v;
+}
+// False when the wait ran out, here or (status word) in another block; a whole warp calls.
+__device__ __forceinline__ bool grid_wait(Barrier* bar, unsigned target, unsigned long long limit_ns) {
+  if ((int)(count_acquire(bar) - target) >= 0) return true;
+  const unsigned long long t0 = global_ns();
+  for (int spin = 1;; ++spin) {
+    if ((int)(count_acquire(bar) - target) >= 0) return true;
+    if ((spin & 15) != 0) continue;
+    bool late = *(volatile int*)&bar->status != 0;
+    if (!late && global_ns() - t0 > limit_ns) {
+      late = true;
+      if ((threadIdx.x & 31) == 0) atomicExch(&bar->status, 1);
     }
-    if (*vstatus != 0) good = 0;
-    __threadfence();
-    ok = good;
+    if (__any_sync(0xffffffffu, late)) return false;
   }
-  __syncthreads();
-  return ok != 0;
 }
 
 // Block-wide FP64 sum in a fixed order, valid in thread 0. Every thread's value goes to
@@ -108,11 +106,6 @@ __device__ __forceinline__ double block_sum_tree(double v, double* sh) {
   return t;
 }
 
-// the block sum of the CG kernel: by part count (uniform over the grid)
-__device__ __forceinline__ double cg_block_sum(double v, double* sh, bool many_parts) {
-  return many_parts ? block_sum_tree(v, sh) : block_sum(v, sh);
-}
-
 template <typename T>
 struct SolveArgs {
   int64_t N;
@@ -133,7 +126,7 @@ struct SolveArgs {
   const int32_t* sc_part;   // [n_sc]
   const int32_t* part_sc;   // [P+1]
   const int* active;        // [P] parts to solve
-  double* buf;              // [2][2][n_sc] partial sums
+  double* buf;              // [2][n_sc] partial sums, used in turn
   Barrier* bar;
   double inner_tol2;
   int maxit_inner;
@@ -143,48 +136,93 @@ struct SolveArgs {
   unsigned long long barrier_ns;  // limit of a barrier wait
 };
 
-// Sum the per-sub-chunk partials of K quantities into per-part totals (shared memory
-// tot[k * P + p]), every part in sub-chunk order. Call after a grid barrier. The partials
-// are first staged in shared memory with one load per thread (one L2 round trip). A part
-// of at most kSeqSubChunks sub-chunks is summed by one thread, left to right; a longer
-// one by one warp: lanes stride 32 over its sub-chunks, then a shuffle tree. (A warp-wide
-// FP64 add costs the same whatever its active lanes, so the few adds of the short parts
-// of an ensemble are cheaper in one thread than in a five-level shuffle tree.)
+// One exchange of a launch over many parts: the grid's barrier behind the blocks' partial
+// sums (buf[sc], written by thread 0 of each block), then the per-part totals (shared memory
+// tot[p]), every part in sub-chunk order. A part of at most kSeqSubChunks sub-chunks is summed
+// by one thread, left to right; a longer one by one warp: lanes stride 32 over its sub-chunks,
+// then a shuffle tree. (A warp-wide FP64 add costs the same whatever its active lanes, so the
+// few adds of the short parts of an ensemble are cheaper in one thread than in a five-level
+// shuffle tree.) False when a wait ran out.
 constexpr int kSeqSubChunks = 8;
+constexpr int kLaneSlots = 5;        // partial sums a lane loads at once (160 blocks)
 
-template <typename T, int K>
-__device__ void part_totals(const SolveArgs<T>& a, const double* buf, double* tot,
-                            double (*stage)[kCgThreads]) {
+template <typename T>
+__device__ bool exchange(const SolveArgs<T>& a, const double* buf, unsigned& target, bool arrive, double* tot,
+                         double* stage) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  const bool staged = a.n_sc <= (int)blockDim.x;
-  if (staged) {
-#pragma unroll
-    for (int k = 0; k < K; ++k)
-      if ((int)threadIdx.x < a.n_sc) stage[k][threadIdx.x] = __ldcg(buf + (size_t)k * a.n_sc + threadIdx.x);
-    __syncthreads();
+  bool ok = true;
+  target += gridDim.x;
+  if (warp == 0) {
+    if (lane == 0 && arrive) grid_arrive(a.bar);
+    __syncwarp();
+    ok = grid_wait(a.bar, target, a.barrier_ns);
+    if (ok)
+      for (int sc = lane; sc < a.n_sc; sc += 32) stage[sc] = __ldcg(buf + sc);
   }
+  if (!__syncthreads_and(ok)) return false;
   for (int p = threadIdx.x; p < a.n_part; p += blockDim.x) {
     const int s0 = a.part_sc[p], s1 = a.part_sc[p + 1];
     if (s1 - s0 > kSeqSubChunks) continue;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-      double t = 0.0;
-      for (int sc = s0; sc < s1; ++sc) t += staged ? stage[k][sc] : __ldcg(buf + (size_t)k * a.n_sc + sc);
-      tot[k * a.n_part + p] = t;
-    }
+    double t = 0.0;
+    for (int sc = s0; sc < s1; ++sc) t += stage[sc];
+    tot[p] = t;
   }
   for (int p = warp; p < a.n_part; p += nw) {
     if (a.part_sc[p + 1] - a.part_sc[p] <= kSeqSubChunks) continue;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-      double t = 0.0;
-      for (int sc = a.part_sc[p] + lane; sc < a.part_sc[p + 1]; sc += 32)
-        t += staged ? stage[k][sc] : __ldcg(buf + (size_t)k * a.n_sc + sc);
-      for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-      if (lane == 0) tot[k * a.n_part + p] = t;
-    }
+    double t = 0.0;
+    for (int sc = a.part_sc[p] + lane; sc < a.part_sc[p + 1]; sc += 32) t += stage[sc];
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+    if (lane == 0) tot[p] = t;
   }
   __syncthreads();
+  return true;
+}
+
+// The same for a single mesh (at most one sub-chunk a block), with the block's sum before it
+// and the scalars after it: acc of every thread -> block sum (four warps, one per SM
+// sub-partition, a quarter each: GB300 issues FP64 adds at a small fraction of the FP32 rate,
+// so the FP64 instructions on the critical path are few and spread) -> buf; warp 0 waits,
+// sums the partials from registers and hands the total to use(total) (every lane of warp 0);
+// one block barrier at the end. False when a wait ran out.
+template <typename T, typename F>
+__device__ __forceinline__ bool exchange_one(const SolveArgs<T>& a, double* buf, unsigned& target, int sc0, int sc1,
+                                             bool arrive, double acc, double* sh, int* s_ok, F use) {
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  const int quarter = blockDim.x >> 2;
+  target += gridDim.x;
+  sh[threadIdx.x] = acc;
+  __syncthreads();                   // and every row of the phase is written before the arrival
+  if (w < 4) {
+    const double* q = sh + w * quarter;
+    double t = q[l];
+    for (int j = l + 32; j < quarter; j += 32) t += q[j];
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+    if (l == 0) sh[blockDim.x + w] = t;
+    asm volatile("bar.sync 1, 128;" ::: "memory");
+  }
+  if (w == 0) {
+    if (l == 0) {
+      const double* q = sh + blockDim.x;
+      if (sc1 > sc0) __stcg(buf + sc0, (q[0] + q[1]) + (q[2] + q[3]));
+      if (arrive) grid_arrive(a.bar);
+    }
+    __syncwarp();
+    const bool ok = grid_wait(a.bar, target, a.barrier_ns);
+    double t = 0.0;
+    if (ok) {
+      double v[kLaneSlots];
+#pragma unroll
+      for (int q = 0; q < kLaneSlots; ++q) v[q] = l + 32 * q < a.n_sc ? __ldcg(buf + l + 32 * q) : 0.0;
+#pragma unroll
+      for (int q = 0; q < kLaneSlots; ++q) t += v[q];
+      for (int sc = l + 32 * kLaneSlots; sc < a.n_sc; sc += 32) t += __ldcg(buf + sc);
+      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      use(t);
+    }
+    if (l == 0) *s_ok = ok;
+  }
+  __syncthreads();
+  return *s_ok != 0;
 }
 
 // Four operator coefficients of one row, loaded with vector loads.
@@ -317,26 +355,82 @@ __device__ __forceinline__ T cg_phase_pq(const SolveArgs<T>& a, int64_t lo, int6
   return acc;
 }
 
-// One 512-thread block per SM (measured faster than two smaller-register blocks: fewer
-// grid-barrier arrivals and partial sums, more rows in flight per thread).
+// The kernel for a single mesh: scalars in shared memory, one exchange per phase.
 template <typename T>
-__global__ void __launch_bounds__(kCgThreads, kCgBlocksPerSm) k_cg(SolveArgs<T> a) {
+__device__ void cg_one(const SolveArgs<T>& a) {
+  __shared__ double sh[kCgThreads + 4];
+  __shared__ T s_alpha, s_beta;
+  __shared__ int s_state;              // 0 running, 1 converged, 2 breakdown, 3 idle
+  __shared__ int s_ok;
+  const int sc0 = a.blk_sc[blockIdx.x], sc1 = a.blk_sc[blockIdx.x + 1];
+  const int64_t lo = a.sc_begin[sc0], hi = sc1 > sc0 ? a.sc_begin[sc1] : lo;
+  const bool arrive = a.skip_block != (int)blockIdx.x;   // test hook
+  const bool act = a.active[0] != 0;
+  unsigned target = 0;
+  int its = 0;
+  double* const buf0 = a.buf;
+  double* const buf1 = a.buf + a.n_sc;
+  bool pending = false, ok;
+  double rr = 0.0, rr0 = 0.0;          // warp 0's
+  T acc = T(0);
+  // r = D^-1/2 rhs, p = q = x = 0; the first p/q phase (beta = 0) then gives p = r, q = S r
+  for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) {
+    const T ri = act ? (T)(a.r_in[i] * (double)__ldg(a.at_isd + i)) : T(0);
+    a.cr[i] = ri;
+    a.cp[i] = T(0);
+    a.cq[i] = T(0);
+    a.cx[i] = T(0);
+    acc += ri * ri;
+  }
+  ok = exchange_one(a, buf0, target, sc0, sc1, arrive, (double)acc, sh, &s_ok, [&](double t) {
+    rr = rr0 = t;
+    s_state = !act || t == 0.0 ? 3 : (t > 0.0 ? 0 : 2);
+    s_alpha = s_beta = T(0);
+  });
+  while (ok && s_state == 0) {
+    acc = cg_phase_pq<T>(a, lo, hi, s_beta, s_alpha);
+    pending = false;                   // x += alpha p of the last r phase is applied
+    ok = exchange_one(a, buf1, target, sc0, sc1, arrive, (double)acc, sh, &s_ok, [&](double pq) {
+      if (!(pq > 0.0) || !isfinite(pq)) s_state = 2;
+      else s_alpha = (T)(rr / pq);
+    });
+    if (!ok || s_state != 0 || its >= a.maxit_inner) break;
+    acc = cg_phase_r<T>(a, lo, hi, s_alpha);
+    pending = true;
+    ++its;
+    ok = exchange_one(a, buf0, target, sc0, sc1, arrive, (double)acc, sh, &s_ok, [&](double rrn) {
+      if (!isfinite(rrn)) s_state = 2;
+      else if (rrn <= a.inner_tol2 * rr0) s_state = 1;
+      else s_beta = (T)(rrn / rr);
+      rr = rrn;
+    });
+    if (its >= a.maxit_inner) break;
+  }
+  if (ok) cg_phase_x<T>(a, lo, hi, pending, s_alpha);
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    a.out_inner[0] = its;
+    a.out_status[0] = ok && s_state == 2 ? 6 : 0;
+    a.out_status[1] = its;
+  }
+}
+
+// Many parts (an ensemble): per-part scalars and stopping tests.
+template <typename T>
+__device__ void cg_many(const SolveArgs<T>& a) {
   __shared__ double sh[kCgThreads];
-  __shared__ double stage[2][kCgThreads];
-  __shared__ double tot[2 * kMaxParts];
+  __shared__ double stage[kCgThreads];
+  __shared__ double tot[kMaxParts];
   __shared__ double s_rr[kMaxParts], s_rr0[kMaxParts];
   __shared__ T s_alpha[kMaxParts], s_beta[kMaxParts];
   __shared__ int s_cg[kMaxParts];      // 0 running, 1 converged, 2 breakdown, 3 idle
   __shared__ int s_inner[kMaxParts];
   __shared__ int s_pend[kMaxParts];    // x += alpha p of the part's last phase 1 not yet applied
   __shared__ int s_flag, s_status;
-  const unsigned G = gridDim.x;
   const int P = a.n_part;
-  const bool many = P > 1;
   const int sc0 = a.blk_sc[blockIdx.x], sc1 = a.blk_sc[blockIdx.x + 1];
-  int parity = 0;
-  int total_its = 0;
+  const bool arrive = a.skip_block != (int)blockIdx.x;   // test hook
   unsigned target = 0;
+  int total_its = 0;
   if (threadIdx.x == 0) s_status = 0;
   for (int p = threadIdx.x; p < P; p += blockDim.x) { s_inner[p] = 0; s_pend[p] = 0; }
 
@@ -344,35 +438,33 @@ __global__ void __launch_bounds__(kCgThreads, kCgBlocksPerSm) k_cg(SolveArgs<T> 
   // (beta = 0) then gives p = r, q = S r
   for (int sc = sc0; sc < sc1; ++sc) {
     const bool act = a.active[a.sc_part[sc]] != 0;
+    T l0 = T(0);
     for (int64_t i = a.sc_begin[sc] + threadIdx.x; i < a.sc_begin[sc + 1]; i += blockDim.x) {
-      a.cr[i] = act ? (T)(a.r_in[i] * (double)__ldg(a.at_isd + i)) : T(0);
+      const T ri = act ? (T)(a.r_in[i] * (double)__ldg(a.at_isd + i)) : T(0);
+      a.cr[i] = ri;
       a.cp[i] = T(0);
       a.cq[i] = T(0);
       a.cx[i] = T(0);
+      l0 += ri * ri;
     }
+    const double t0 = act ? block_sum_tree((double)l0, sh) : 0.0;
+    __syncthreads();                  // the block's rows are written before it arrives
+    if (threadIdx.x == 0) __stcg(a.buf + sc, t0);
   }
-  if (!grid_barrier(a.bar, G, target, a.skip_block == (int)blockIdx.x, a.barrier_ns)) goto done;
+  if (!exchange<T>(a, a.buf, target, arrive, tot, stage)) goto done;
+  for (int p = threadIdx.x; p < P; p += blockDim.x) s_rr[p] = s_rr0[p] = tot[p];
   for (int sc = sc0; sc < sc1; ++sc) {
     const int p = a.sc_part[sc];
-    T l0 = T(0), l1 = T(0);
-    if (a.active[p]) {
-      for (int64_t i = a.sc_begin[sc] + threadIdx.x; i < a.sc_begin[sc + 1]; i += blockDim.x) {
-        const T ri = a.cr[i];
-        l0 += ri * ri;
-      }
-      l1 = cg_phase_pq<T>(a, a.sc_begin[sc], a.sc_begin[sc + 1], T(0), T(0));
-    }
-    const double t0 = cg_block_sum((double)l0, sh, many);
-    const double t1 = cg_block_sum((double)l1, sh, many);
-    if (threadIdx.x == 0) { a.buf[sc] = t0; a.buf[a.n_sc + sc] = t1; }
+    double t1 = 0.0;
+    if (a.active[p])
+      t1 = block_sum_tree((double)cg_phase_pq<T>(a, a.sc_begin[sc], a.sc_begin[sc + 1], T(0), T(0)), sh);
+    if (threadIdx.x == 0) __stcg(a.buf + a.n_sc + sc, t1);
   }
-  if (!grid_barrier(a.bar, G, target, a.skip_block == (int)blockIdx.x, a.barrier_ns)) goto done;
-  part_totals<T, 2>(a, a.buf, tot, stage);
+  if (!exchange<T>(a, a.buf + a.n_sc, target, arrive, tot, stage)) goto done;
   if (threadIdx.x == 0) s_flag = 0;
   __syncthreads();
   for (int p = threadIdx.x; p < P; p += blockDim.x) {
-    const double rr0 = tot[p], pq = tot[P + p];
-    s_rr[p] = s_rr0[p] = rr0;
+    const double rr0 = s_rr0[p], pq = tot[p];
     int st = 3;
     if (a.active[p]) {
       if (!(rr0 > 0.0)) st = rr0 == 0.0 ? 3 : 2;
@@ -384,19 +476,15 @@ __global__ void __launch_bounds__(kCgThreads, kCgBlocksPerSm) k_cg(SolveArgs<T> 
   }
   __syncthreads();
   for (int its = 0; s_flag != 0 && its < a.maxit_inner; ++its) {
-    parity ^= 1;
-    double* buf = a.buf + (size_t)parity * 2 * a.n_sc;
+    double* buf = a.buf;
     for (int sc = sc0; sc < sc1; ++sc) {
       const int p = a.sc_part[sc];
-      if (s_cg[p] == 0) {             // uniform in the block
-        const double t = cg_block_sum((double)cg_phase_r<T>(a, a.sc_begin[sc], a.sc_begin[sc + 1], s_alpha[p]), sh, many);
-        if (threadIdx.x == 0) buf[sc] = t;
-      } else if (threadIdx.x == 0) {
-        buf[sc] = 0.0;
-      }
+      double t = 0.0;
+      if (s_cg[p] == 0)               // uniform in the block
+        t = block_sum_tree((double)cg_phase_r<T>(a, a.sc_begin[sc], a.sc_begin[sc + 1], s_alpha[p]), sh);
+      if (threadIdx.x == 0) __stcg(buf + sc, t);
     }
-    if (!grid_barrier(a.bar, G, target, a.skip_block == (int)blockIdx.x, a.barrier_ns)) goto done;
-    part_totals<T, 1>(a, buf, tot, stage);
+    if (!exchange<T>(a, buf, target, arrive, tot, stage)) goto done;
     ++total_its;
     if (threadIdx.x == 0) s_flag = 0;
     __syncthreads();
@@ -413,20 +501,15 @@ __global__ void __launch_bounds__(kCgThreads, kCgBlocksPerSm) k_cg(SolveArgs<T> 
     }
     __syncthreads();
     if (s_flag == 0) break;
-    parity ^= 1;
-    buf = a.buf + (size_t)parity * 2 * a.n_sc;
+    buf = a.buf + a.n_sc;
     for (int sc = sc0; sc < sc1; ++sc) {
       const int p = a.sc_part[sc];
-      if (s_cg[p] == 0) {             // uniform in the block
-        const double t = cg_block_sum((double)cg_phase_pq<T>(a, a.sc_begin[sc], a.sc_begin[sc + 1], s_beta[p],
-                                                             s_alpha[p]), sh, many);
-        if (threadIdx.x == 0) buf[sc] = t;
-      } else if (threadIdx.x == 0) {
-        buf[sc] = 0.0;
-      }
+      double t = 0.0;
+      if (s_cg[p] == 0)               // uniform in the block
+        t = block_sum_tree((double)cg_phase_pq<T>(a, a.sc_begin[sc], a.sc_begin[sc + 1], s_beta[p], s_alpha[p]), sh);
+      if (threadIdx.x == 0) __stcg(buf + sc, t);
     }
-    if (!grid_barrier(a.bar, G, target, a.skip_block == (int)blockIdx.x, a.barrier_ns)) goto done;
-    part_totals<T, 1>(a, buf, tot, stage);
+    if (!exchange<T>(a, buf, target, arrive, tot, stage)) goto done;
     for (int p = threadIdx.x; p < P; p += blockDim.x) {
       if (s_cg[p] != 0) continue;
       s_pend[p] = 0;                  // phase 2 applied the pending x update
@@ -454,6 +537,14 @@ done:
       a.out_status[1] = total_its;
     }
   }
+}
+
+// One 512-thread block per SM (measured faster than two smaller-register blocks: fewer
+// exchanges and partial sums, more rows in flight per thread).
+template <typename T, bool kMany>
+__global__ void __launch_bounds__(kCgThreads, kCgBlocksPerSm) k_cg(SolveArgs<T> a) {
+  if constexpr (kMany) cg_many<T>(a);
+  else cg_one<T>(a);
 }
 
 // Per-part sum of squares of an FP64 vector over the same sub-chunks (one block per
@@ -514,14 +605,15 @@ __global__ void __launch_bounds__(kCgThreads) k_part_dots_partial(const double* 
 }  // namespace
 
 int solve_grid_size(fvgb_mesh_s* m) {
-  int a = 0, b = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, (const void*)k_cg<float>, kCgThreads, 0) != cudaSuccess)
-    return 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, (const void*)k_cg<double>, kCgThreads, 0) != cudaSuccess)
-    return 0;
-  const int per_sm = a < b ? a : b;
-  if (per_sm < 1) return 0;
-  return (per_sm < kCgBlocksPerSm ? per_sm : kCgBlocksPerSm) * m->num_sms;
+  const void* kernels[] = {(const void*)k_cg<float, false>, (const void*)k_cg<float, true>,
+                           (const void*)k_cg<double, false>, (const void*)k_cg<double, true>};
+  int per_sm = kCgBlocksPerSm;
+  for (const void* k : kernels) {
+    int n = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, kCgThreads, 0) != cudaSuccess) return 0;
+    per_sm = n < per_sm ? n : per_sm;
+  }
+  return per_sm < 1 ? 0 : per_sm * m->num_sms;
 }
 
 cudaError_t launch_part_sumsq(fvgb_mesh_s* m, const double* v, double* out, cudaStream_t s) {
@@ -562,11 +654,13 @@ cudaError_t launch_cg(fvgb_mesh_s* m, int bcset, const double* r, double inner_r
   a.out_status = m->d_cg_info;
   a.skip_block = m->test_skip_block;
   a.barrier_ns = m->test_barrier_ns > 0 ? m->test_barrier_ns : kBarrierTimeoutNs;
+  if (pd.n_sc > kCgThreads) return cudaErrorInvalidConfiguration;   // their staging
   cudaError_t e = cudaMemsetAsync(m->barrier, 0, sizeof(Barrier), s);
   if (e != cudaSuccess) return e;
   void* args[] = {&a};
   count_launch();
-  return cudaLaunchCooperativeKernel((const void*)k_cg<T>, dim3(m->solve_grid), dim3(kCgThreads),
+  const void* k = pd.n_part > 1 ? (const void*)k_cg<T, true> : (const void*)k_cg<T, false>;
+  return cudaLaunchCooperativeKernel(k, dim3(m->solve_grid), dim3(kCgThreads),
                                      args, 0, s);
 }
 
