@@ -882,6 +882,7 @@ static fvgb_status upload_impl(int32_t dim, int64_t n_vert, const double* xyz, i
   cudaError_t e;
   if ((e = cudaGetDevice(&m->device))) return fail(e, "cudaGetDevice");
   if ((e = cudaDeviceGetAttribute(&m->num_sms, cudaDevAttrMultiProcessorCount, m->device))) return fail(e, "device attribute");
+  if ((e = cudaDeviceGetAttribute(&m->l2_bytes, cudaDevAttrL2CacheSize, m->device))) return fail(e, "device attribute");
   TopoDev& t = m->topo;
   t.dim = h.dim; t.N = h.N; t.V = h.V; t.F = h.F; t.Fi = h.Fi; t.n_nbr = h.nptr[h.N];
   m->cell_perm_host = h.cell_perm;

@@ -152,6 +152,7 @@ enum TuneKernel { kTuneGrad = 0, kTuneVertex = 1, kTuneFace = 2, kTuneUpdate = 3
 struct fvgb_mesh_s {
   int device = 0;
   int num_sms = 0;
+  int l2_bytes = 0;
   fvgb_prec prec = FVGB_FP64;
   fvgb::TopoDev topo;
   fvgb::GeoDev<double> g64;

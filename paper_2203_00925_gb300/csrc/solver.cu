@@ -225,20 +225,53 @@ __device__ __forceinline__ bool exchange_one(const SolveArgs<T>& a, double* buf,
   return *s_ok != 0;
 }
 
+// Loads of the operator and of the vectors in the two phases.
+// kStream (a working set well above L2): what an iteration reads once (operator) or reads and
+// writes once without a neighbour's look (x) is marked to leave L2 first, so that r, p and q
+// stay; 6M cells FP32 84.6 -> 70.3 us an iteration. Smaller sets live in L2 as they are and
+// the marks cost them (750,000 cells 13.4 -> 14.5 us), and in FP64 the phase waits for the
+// FP64 pipe more than for memory (6M cells 145 us without, 159 with the marks).
+template <bool kStream>
+__device__ __forceinline__ int4 load_op(const int4* p) {
+  if constexpr (!kStream) return __ldg(p);
+  unsigned long long pol;
+  int4 v;
+  asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
+  asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.v4.s32 {%0, %1, %2, %3}, [%4], %5;"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p), "l"(pol));
+  return v;
+}
+// r, own rows and neighbours': a plain load that may hit L1 (an acquire in every grid barrier
+// orders it behind the other blocks' stores). Neighbours are mostly rows of the same warps, so
+// L1 takes most of the gathers' traffic: 6M cells FP32 68.5 -> 64.5 us, 750,000 cells 13.4 ->
+// 11.8 us an iteration against loads that pass L1 by.
+__device__ __forceinline__ float load_r(const float* p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ double load_r(const double* p) {
+  double v;
+  asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p) : "memory");
+  return v;
+}
+
 // Four operator coefficients of one row, loaded with vector loads.
 template <typename T>
 struct Coef4;
 template <>
 struct Coef4<float> {
   float c[4];
+  template <bool kStream>
   __device__ __forceinline__ void load(const float* p, int64_t i) {
-    const float4 v = __ldg(reinterpret_cast<const float4*>(p) + i);
-    c[0] = v.x; c[1] = v.y; c[2] = v.z; c[3] = v.w;
+    const int4 v = load_op<kStream>(reinterpret_cast<const int4*>(p) + i);
+    c[0] = __int_as_float(v.x); c[1] = __int_as_float(v.y); c[2] = __int_as_float(v.z); c[3] = __int_as_float(v.w);
   }
 };
 template <>
 struct Coef4<double> {
   double c[4];
+  template <bool kStream>
   __device__ __forceinline__ void load(const double* p, int64_t i) {
     const double2 v0 = __ldg(reinterpret_cast<const double2*>(p) + 2 * i);
     const double2 v1 = __ldg(reinterpret_cast<const double2*>(p) + 2 * i + 1);
@@ -246,39 +279,46 @@ struct Coef4<double> {
   }
 };
 
-// Rows per thread per trip: all loads of a trip are issued before any store so that the
-// gathers of several rows are in flight together.
+// Rows per thread per trip. Both phases load the next trip's rows before they work on this
+// one's, so that the loads of one trip are always in flight: two FP32 rows of 48 bytes or one
+// FP64 row of 80 for each of 512 threads. 6M cells FP64 168 -> 146 us an iteration, 750,000
+// cells 23.1 -> 20.7 us (more rows a trip without the overlap were no faster, and more rows
+// with it spill).
 template <typename T>
-__host__ __device__ constexpr int unroll_rows() { return sizeof(T) == 4 ? 4 : 2; }
-// the x/r phase holds four values a row: more FP64 rows per trip (measured: four FP32 rows
-// a trip beat eight on the 64-mesh ensemble and on the 750,000-cell mixed step)
+__host__ __device__ constexpr int unroll_rows() { return sizeof(T) == 4 ? 2 : 1; }
+// the r phase holds two values a row
 template <typename T>
-__host__ __device__ constexpr int unroll_rows_xr() { return 4; }
+__host__ __device__ constexpr int unroll_rows_r() { return sizeof(T) == 4 ? 8 : 4; }
 
 // CG phase 1 on rows [lo, hi): r -= alpha q; returns the thread's sum of r^2. (The matching
 // x += alpha p is deferred to the next phase 2, which reads p anyway, or to the final pass:
 // the same additions in the same order, without streaming x and p through this phase.)
 template <typename T>
 __device__ __forceinline__ T cg_phase_r(const SolveArgs<T>& a, int64_t lo, int64_t hi, T alpha) {
-  constexpr int U = unroll_rows_xr<T>();
-  T* __restrict__ R = a.cr;
-  const T* __restrict__ Q = a.cq;
-  T acc = T(0);
-  const int64_t bd = blockDim.x;
-  for (int64_t b = lo + threadIdx.x; b < hi; b += U * bd) {
-    T r[U], q[U];
+  constexpr int U = unroll_rows_r<T>();
+  T* R = a.cr + lo;
+  const T* __restrict__ Q = a.cq + lo;
+  const int n = (int)(hi - lo), bd = blockDim.x;
+  T acc = T(0), r[U], q[U];
+  auto load = [&](int b) {
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int64_t i = b + u * bd;
-      if (i < hi) { r[u] = R[i]; q[u] = Q[i]; }
+      const int i = b + u * bd;
+      if (i < n) { r[u] = R[i]; q[u] = Q[i]; }
     }
+  };
+  load(threadIdx.x);
+  for (int b = threadIdx.x; b < n; b += U * bd) {
+    T rn[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) rn[u] = r[u] - alpha * q[u];
+    load(b + U * bd);
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int64_t i = b + u * bd;
-      if (i < hi) {
-        const T rn = r[u] - alpha * q[u];
-        R[i] = rn;
-        acc += rn * rn;
+      const int i = b + u * bd;
+      if (i < n) {
+        R[i] = rn[u];
+        acc += rn[u] * rn[u];
       }
     }
   }
@@ -299,64 +339,88 @@ __device__ __forceinline__ void cg_phase_x(const SolveArgs<T>& a, int64_t lo, in
 
 // CG phase 2 on rows [lo, hi): x += alpha p (the previous phase 1's update, with the old p),
 // p = r + beta p, q = S r + beta q (= S p, S = D^-1/2 A_T D^-1/2 with unit diagonal);
-// returns the thread's sum of p.q. Neighbours' r are read through L2 (other blocks wrote
-// them).
-template <typename T>
+// returns the thread's sum of p.q.
+template <typename T, int U>
+struct CgRows {
+  T r[U], p[U], q[U], x[U];
+  int4 nb[U];
+  Coef4<T> c[U];
+};
+
+template <typename T, bool kStream>
 __device__ __forceinline__ T cg_phase_pq(const SolveArgs<T>& a, int64_t lo, int64_t hi, T beta, T alpha) {
   constexpr int U = unroll_rows<T>();
-  T* __restrict__ P = a.cp;
-  T* __restrict__ Q = a.cq;
-  T* __restrict__ X = a.cx;
-  const T* __restrict__ R = a.cr;
-  const int4* __restrict__ NB = reinterpret_cast<const int4*>(a.at_nbr);
+  T* __restrict__ P = a.cp + lo;
+  T* __restrict__ Q = a.cq + lo;
+  T* __restrict__ X = a.cx + lo;
+  const T* R0 = a.cr;
+  const T* R = a.cr + lo;
+  const int4* __restrict__ NB = reinterpret_cast<const int4*>(a.at_nbr) + lo;
+  const T* __restrict__ C = a.at_scoef + 4 * lo;
+  const int n = (int)(hi - lo), bd = blockDim.x;
   T acc = T(0);
-  const int64_t bd = blockDim.x;
-  for (int64_t b = lo + threadIdx.x; b < hi; b += U * bd) {
-    T r[U], p[U], q[U], x[U], g[U][4];
-    int4 nb[U];
-    Coef4<T> c[U];
+  auto load = [&](CgRows<T, U>& w, int b) {
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int64_t i = b + u * bd;
-      if (i < hi) {
-        nb[u] = __ldg(NB + i);
-        r[u] = R[i]; p[u] = P[i]; q[u] = Q[i]; x[u] = X[i];
-        c[u].load(a.at_scoef, i);
+      const int i = b + u * bd;
+      if (i < n) {
+        w.nb[u] = load_op<kStream>(NB + i);
+        w.c[u].template load<kStream>(C, i);
+        w.r[u] = load_r(R + i);
+        w.p[u] = P[i];
+        w.q[u] = Q[i];
+        w.x[u] = kStream ? __ldcs(X + i) : X[i];
       }
     }
+  };
+  // rows w of trip b; the next trip's go to nx behind this trip's gathers
+  auto work = [&](const CgRows<T, U>& w, CgRows<T, U>& nx, int b) {
+    T g[U][4];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int64_t i = b + u * bd;
-      if (i < hi) {
-        g[u][0] = __ldcg(R + nb[u].x);
-        g[u][1] = __ldcg(R + nb[u].y);
-        g[u][2] = __ldcg(R + nb[u].z);
-        g[u][3] = __ldcg(R + nb[u].w);
+      if (b + u * bd < n) {
+        g[u][0] = load_r(R0 + w.nb[u].x);
+        g[u][1] = load_r(R0 + w.nb[u].y);
+        g[u][2] = load_r(R0 + w.nb[u].z);
+        g[u][3] = load_r(R0 + w.nb[u].w);
       }
     }
+    load(nx, b + U * bd);
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int64_t i = b + u * bd;
-      if (i < hi) {
-        T y = r[u];                     // unit diagonal
-        y -= c[u].c[0] * g[u][0];
-        y -= c[u].c[1] * g[u][1];
-        y -= c[u].c[2] * g[u][2];
-        y -= c[u].c[3] * g[u][3];
-        const T pn = r[u] + beta * p[u];
-        const T qn = y + beta * q[u];
-        X[i] = x[u] + alpha * p[u];
+      const int i = b + u * bd;
+      if (i < n) {
+        T y = w.r[u];                   // unit diagonal
+        y -= w.c[u].c[0] * g[u][0];
+        y -= w.c[u].c[1] * g[u][1];
+        y -= w.c[u].c[2] * g[u][2];
+        y -= w.c[u].c[3] * g[u][3];
+        const T pn = w.r[u] + beta * w.p[u];
+        const T qn = y + beta * w.q[u];
+        const T xn = w.x[u] + alpha * w.p[u];
+        if (kStream) __stcs(X + i, xn);
+        else X[i] = xn;
         P[i] = pn;
         Q[i] = qn;
         acc += pn * qn;
       }
     }
+  };
+  CgRows<T, U> w0, w1;
+  int b = threadIdx.x;
+  load(w0, b);
+  while (b < n) {
+    work(w0, w1, b);
+    b += U * bd;
+    if (b >= n) break;
+    work(w1, w0, b);
+    b += U * bd;
   }
   return acc;
 }
 
 // The kernel for a single mesh: scalars in shared memory, one exchange per phase.
-template <typename T>
+template <typename T, bool kStream>
 __device__ void cg_one(const SolveArgs<T>& a) {
   __shared__ double sh[kCgThreads + 4];
   __shared__ T s_alpha, s_beta;
@@ -388,7 +452,7 @@ __device__ void cg_one(const SolveArgs<T>& a) {
     s_alpha = s_beta = T(0);
   });
   while (ok && s_state == 0) {
-    acc = cg_phase_pq<T>(a, lo, hi, s_beta, s_alpha);
+    acc = cg_phase_pq<T, kStream>(a, lo, hi, s_beta, s_alpha);
     pending = false;                   // x += alpha p of the last r phase is applied
     ok = exchange_one(a, buf1, target, sc0, sc1, arrive, (double)acc, sh, &s_ok, [&](double pq) {
       if (!(pq > 0.0) || !isfinite(pq)) s_state = 2;
@@ -415,7 +479,7 @@ __device__ void cg_one(const SolveArgs<T>& a) {
 }
 
 // Many parts (an ensemble): per-part scalars and stopping tests.
-template <typename T>
+template <typename T, bool kStream>
 __device__ void cg_many(const SolveArgs<T>& a) {
   __shared__ double sh[kCgThreads];
   __shared__ double stage[kCgThreads];
@@ -457,7 +521,7 @@ __device__ void cg_many(const SolveArgs<T>& a) {
     const int p = a.sc_part[sc];
     double t1 = 0.0;
     if (a.active[p])
-      t1 = block_sum_tree((double)cg_phase_pq<T>(a, a.sc_begin[sc], a.sc_begin[sc + 1], T(0), T(0)), sh);
+      t1 = block_sum_tree((double)cg_phase_pq<T, kStream>(a, a.sc_begin[sc], a.sc_begin[sc + 1], T(0), T(0)), sh);
     if (threadIdx.x == 0) __stcg(a.buf + a.n_sc + sc, t1);
   }
   if (!exchange<T>(a, a.buf + a.n_sc, target, arrive, tot, stage)) goto done;
@@ -506,7 +570,7 @@ __device__ void cg_many(const SolveArgs<T>& a) {
       const int p = a.sc_part[sc];
       double t = 0.0;
       if (s_cg[p] == 0)               // uniform in the block
-        t = block_sum_tree((double)cg_phase_pq<T>(a, a.sc_begin[sc], a.sc_begin[sc + 1], s_beta[p], s_alpha[p]), sh);
+        t = block_sum_tree((double)cg_phase_pq<T, kStream>(a, a.sc_begin[sc], a.sc_begin[sc + 1], s_beta[p], s_alpha[p]), sh);
       if (threadIdx.x == 0) __stcg(buf + sc, t);
     }
     if (!exchange<T>(a, buf, target, arrive, tot, stage)) goto done;
@@ -541,10 +605,21 @@ done:
 
 // One 512-thread block per SM (measured faster than two smaller-register blocks: fewer
 // exchanges and partial sums, more rows in flight per thread).
-template <typename T, bool kMany>
+template <typename T, bool kMany, bool kStream>
 __global__ void __launch_bounds__(kCgThreads, kCgBlocksPerSm) k_cg(SolveArgs<T> a) {
-  if constexpr (kMany) cg_many<T>(a);
-  else cg_one<T>(a);
+  if constexpr (kMany) cg_many<T, kStream>(a);
+  else cg_one<T, kStream>(a);
+}
+
+// The variant for a mesh of N cells in n_part parts: kStream in FP32 once an iteration's
+// operator and vectors (48 bytes a cell) are beyond L2.
+template <typename T>
+const void* cg_kernel(int64_t N, int n_part, int64_t l2_bytes) {
+  if constexpr (sizeof(T) == 4) {
+    if (48 * N > l2_bytes)
+      return n_part > 1 ? (const void*)k_cg<T, true, true> : (const void*)k_cg<T, false, true>;
+  }
+  return n_part > 1 ? (const void*)k_cg<T, true, false> : (const void*)k_cg<T, false, false>;
 }
 
 // Per-part sum of squares of an FP64 vector over the same sub-chunks (one block per
@@ -605,8 +680,9 @@ __global__ void __launch_bounds__(kCgThreads) k_part_dots_partial(const double* 
 }  // namespace
 
 int solve_grid_size(fvgb_mesh_s* m) {
-  const void* kernels[] = {(const void*)k_cg<float, false>, (const void*)k_cg<float, true>,
-                           (const void*)k_cg<double, false>, (const void*)k_cg<double, true>};
+  const void* kernels[] = {(const void*)k_cg<float, false, false>, (const void*)k_cg<float, true, false>,
+                           (const void*)k_cg<float, false, true>, (const void*)k_cg<float, true, true>,
+                           (const void*)k_cg<double, false, false>, (const void*)k_cg<double, true, false>};
   int per_sm = kCgBlocksPerSm;
   for (const void* k : kernels) {
     int n = 0;
@@ -659,8 +735,7 @@ cudaError_t launch_cg(fvgb_mesh_s* m, int bcset, const double* r, double inner_r
   if (e != cudaSuccess) return e;
   void* args[] = {&a};
   count_launch();
-  const void* k = pd.n_part > 1 ? (const void*)k_cg<T, true> : (const void*)k_cg<T, false>;
-  return cudaLaunchCooperativeKernel(k, dim3(m->solve_grid), dim3(kCgThreads),
+  return cudaLaunchCooperativeKernel(cg_kernel<T>(a.N, a.n_part, m->l2_bytes), dim3(m->solve_grid), dim3(kCgThreads),
                                      args, 0, s);
 }
 
