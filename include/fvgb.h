@@ -34,8 +34,9 @@
  *   at the end of a graph-mode fvgb_streamer_step call, each of which returns
  *   FVGB_ENONFINITE and clears it. Grid-wide waits inside the persistent CG kernel are
  *   bounded (1 s) and give FVGB_ETIMEOUT instead of hanging; a wait of the network's
- *   tensor-core kernels for its matrix products (also bounded, 1 s) latches a timeout
- *   in the same status word, reported as FVGB_ETIMEOUT.
+ *   tensor-core kernels for its matrix products, or of the steps of fvgb_fv_step on a small
+ *   mesh for one another (also bounded, 1 s), latches a timeout in the same status word,
+ *   reported as FVGB_ETIMEOUT.
  * - Sizes are int64_t; element indices inside the library are int32 (meshes up to
  *   2^31 - 1 cells, faces and neighbour entries).
  */
@@ -508,8 +509,7 @@ fvgb_status fvgb_mpnn_train_step(fvgb_mpnn net, const double* dq_dev, const doub
                                  void* stream);
 
 /* Synchronise the stream and report the latched asynchronous status of the mesh (see the
- * conventions above), then clear it: FVGB_ETIMEOUT when a tensor-core wait of the network
- * kernels ran out, FVGB_ENONFINITE when a transport update wrote a non-finite value since
+ * conventions above), then clear it: FVGB_ETIMEOUT when a bounded wait on the device ran out, FVGB_ENONFINITE when a transport update wrote a non-finite value since
  * the last report, FVGB_OK otherwise. */
 fvgb_status fvgb_sync(fvgb_mesh m, void* stream);
 

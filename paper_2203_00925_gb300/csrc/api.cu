@@ -449,6 +449,8 @@ fvgb_status step_T(fvgb_mesh m, const fvgb_tcoef* tc, T* u, double dt, int nstep
                    const double* alpha, int nstage, T* ni_out, cudaStream_t s) {
   Work<T>& w = work_of<T>(m);
   const bool diff = tc->diff != 0.0;
+  if (!tc->recon && !ni_out && step_small_ok<T>(m, (int64_t)nsteps * nstage))
+    return cuda_status(launch_small_steps<T>(m, tc, u, dt, nsteps, alpha, nstage, s), "step kernel");
   for (int n = 0; n < nsteps; ++n) {
     const T* in = u;
     for (int k = 0; k < nstage; ++k) {
@@ -545,7 +547,7 @@ fvgb_status solve_impl(fvgb_mesh m, int bcset, const double* f, double* phi,
     FVGB_TRY(cudaMemsetAsync(m->d_status, 0, sizeof(int), s), "memset");
     if (info) *info = loc;
     if (hst[3] & 2) {
-      set_error("a tensor-core wait of the learned start timed out (latched status)");
+      set_error("a bounded wait on the device (tensor cores, grid barrier) timed out (latched status)");
       return FVGB_ETIMEOUT;
     }
     set_error("an earlier transport call produced a non-finite value (latched status)");
@@ -940,6 +942,7 @@ static fvgb_status upload_impl(int32_t dim, int64_t n_vert, const double* xyz, i
   }
   std::vector<double> sw;
   build_sell(h.vptr, h.vcell, &h.valpha, h.V, false, sptr, sidx, &sw);
+  for (size_t q = 0; q + 1 < sptr.size(); ++q) t.star_max = std::max(t.star_max, (int)((sptr[q + 1] - sptr[q]) / 32));
   if ((e = dupload(m, &t.vsell.ptr, sptr, s))) return fail(e, "upload");
   if ((e = dupload(m, &t.vsell.idx, sidx, s))) return fail(e, "upload");
   if ((e = upload_geo<double>(m, h, sw, m->g64, s))) return fail(e, "upload");
@@ -971,6 +974,7 @@ static fvgb_status upload_impl(int32_t dim, int64_t n_vert, const double* xyz, i
     return FVGB_EUNSUPPORTED;
   }
   if ((e = setup_parts(m, h.part_cell_begin, s))) return fail(e, "parts setup");
+  if ((e = prepare_small(m))) return fail(e, "step kernel setup");
   if ((e = cudaStreamSynchronize(s))) return fail(e, "synchronize");
   *out = m;
   return FVGB_OK;
@@ -1265,7 +1269,7 @@ fvgb_status fvgb_sync(fvgb_mesh m, void* stream) {
     FVGB_TRY(cudaMemsetAsync(m->d_status, 0, sizeof(int), s), "memset");
     FVGB_TRY(cudaStreamSynchronize(s), "synchronize");
     if (v & 2) {
-      set_error("a tensor-core wait of the network kernels timed out (latched status, now cleared)");
+      set_error("a bounded wait on the device (tensor cores, grid barrier) timed out (latched status, now cleared)");
       return FVGB_ETIMEOUT;
     }
     set_error("a transport call produced a non-finite value (latched status, now cleared)");

@@ -76,6 +76,7 @@ struct TopoDev {
   int32_t* vcount = nullptr;     // [V] cells around each vertex
   Sell nsell;                    // node neighbours of each cell (padded with the cell)
   Sell vsell;                    // cells around each vertex (padded, weight 0)
+  int star_max = 0;              // longest (padded) star
   // Tiles of kGradTile consecutive cells for the shared-memory gradient: per tile its
   // halo list (the tile's own cells in order, then the other node neighbours of its cells,
   // sorted) and, aligned with nsell.idx, each entry's position in its tile's list.
@@ -175,6 +176,7 @@ struct fvgb_mesh_s {
   int test_skip_block = -1;             // test hook of the CG barrier (fvgb_test_barrier)
   unsigned long long test_barrier_ns = 0;  // barrier wait limit (0: the default 1 s)
   int solve_grid = 0;                   // cooperative grid of the Poisson kernel
+  bool small_ok = false;                // time steps can run as one launch (small.cu)
   fvgb::PartsDev parts;
   std::vector<int64_t> part_cell_begin; // [P+1] internal cell range of each part
   std::vector<int32_t> last_outer, last_inner;  // per-part results of the last solve
@@ -343,6 +345,14 @@ fvgb_status warm_start(fvgb_mesh m, const fvgb_streamer_params* p, void* ne, voi
 bool warm_requested(const fvgb_streamer_params* p);
 fvgb_status streamer_transport(fvgb_mesh m, const fvgb_streamer_params* p, void* ne, void* ni,
                                const double* phi, void* E, cudaStream_t s);
+
+// small.cu: all steps and stages of a call on a small mesh in one launch
+cudaError_t prepare_small(fvgb_mesh_s* m);
+template <typename T>
+bool step_small_ok(const fvgb_mesh_s* m, int64_t stages);
+template <typename T>
+cudaError_t launch_small_steps(fvgb_mesh_s* m, const fvgb_tcoef* tc, T* u, double dt, int nsteps,
+                               const double* alpha, int nstage, cudaStream_t s);
 
 // graph.cu -----------------------------------------------------------------------------
 fvgb_status streamer_graph_steps(fvgb_mesh m, const fvgb_streamer_params* p, void* ne, void* ni,
