@@ -507,6 +507,52 @@ fvgb_status poisson_rhs_impl(fvgb_mesh m, int bcset, const double* f, double* b,
 }
 
 namespace {
+// The latched status of an earlier call, met by a solve: cleared and reported.
+fvgb_status report_latched(fvgb_mesh m, int latched, cudaStream_t s) {
+  FVGB_TRY(cudaMemsetAsync(m->d_status, 0, sizeof(int), s), "memset");
+  if (latched & 2) {
+    set_error("a bounded wait on the device (tensor cores, grid barrier) timed out (latched status)");
+    return FVGB_ETIMEOUT;
+  }
+  set_error("an earlier transport call produced a non-finite value (latched status)");
+  return FVGB_ENONFINITE;
+}
+
+// The refinement loop of a single mesh as one launch (solver.cu), with one host
+// synchronisation for its result.
+fvgb_status solve_one(fvgb_mesh m, int bcset, const double* b, double* r, double* phi, bool primed,
+                      const fvgb_solve_opts* o, fvgb_solve_info* info, cudaStream_t s) {
+  SolveInfoDev* d = (SolveInfoDev*)(m->h_scal + 8);
+  int* hwarm = (int*)(d + 1);
+  const bool count_warm = m->warm_check_pending;
+  m->warm_check_pending = false;
+  FVGB_TRY(launch_solve_one(m, bcset, b, phi, r, primed, o, true, m->d_solve, nullptr, nullptr, nullptr, s), "solve kernel");
+  FVGB_TRY(cudaMemcpyAsync(d, m->d_solve, sizeof(SolveInfoDev), cudaMemcpyDeviceToHost, s), "copy");
+  if (count_warm) FVGB_TRY(cudaMemcpyAsync(hwarm, m->warm_used, sizeof(int), cudaMemcpyDeviceToHost, s), "copy");
+  FVGB_TRY(cudaStreamSynchronize(s), "synchronize");
+  if (count_warm) {
+    m->stats.learned_starts += 1;
+    m->stats.learned_kept += *hwarm ? 1 : 0;
+  }
+  if (info) *info = fvgb_solve_info{d->outer, d->inner, d->rel, std::sqrt(d->bn2)};
+  if (d->latched) {
+    if (info) *info = fvgb_solve_info{0, 0, 0.0, 0.0};
+    return report_latched(m, d->latched, s);
+  }
+  m->last_outer.assign(1, d->outer);
+  m->last_inner.assign(1, d->inner);
+  m->last_rel.assign(1, d->rel);
+  m->stats.outer_its += d->outer;
+  m->stats.cg_launches += d->outer;
+  m->stats.cg_iterations += d->inner;
+  switch (d->status) {
+    case 0: return FVGB_OK;
+    case 5: set_error("Poisson refinement did not reach rtol within maxit_outer"); return FVGB_ENOCONV;
+    case 7: set_error("a grid barrier of the CG kernel timed out"); return FVGB_ETIMEOUT;
+    default: set_error("non-finite value or CG breakdown in the Poisson solve"); return FVGB_ENONFINITE;
+  }
+}
+
 // Outer FP64 refinement loop, per part: r = b - A phi, stop a part when
 // ||r_p|| <= rtol ||b_p||, otherwise one inner CG solve of A_T delta = r on the parts
 // still active and phi += delta. One host synchronisation per outer step.
@@ -526,6 +572,7 @@ fvgb_status solve_impl(fvgb_mesh m, int bcset, const double* f, double* phi,
   if (o->inner > 0) FVGB_TRY_ST(amg_ensure(m, bcset, fp32, s));
   fvgb_status st = primed ? FVGB_OK : poisson_rhs_impl(m, bcset, f, b, s);
   if (st) return st;
+  if (solve_one_ok(m, o)) return solve_one(m, bcset, b, r, phi, primed, o, info, s);
   // host staging in pinned memory: [0, P) norms, [P, 2P) ints (active flags, inner its)
   double* hn = m->h_scal + 8;
   int* hact = (int*)(m->h_scal + 8 + P);
@@ -544,14 +591,8 @@ fvgb_status solve_impl(fvgb_mesh m, int bcset, const double* f, double* phi,
     for (int p = 0; p < P; ++p) m->stats.learned_kept += hact[p] ? 1 : 0;
   }
   if (hst[3] != 0) {
-    FVGB_TRY(cudaMemsetAsync(m->d_status, 0, sizeof(int), s), "memset");
     if (info) *info = loc;
-    if (hst[3] & 2) {
-      set_error("a bounded wait on the device (tensor cores, grid barrier) timed out (latched status)");
-      return FVGB_ETIMEOUT;
-    }
-    set_error("an earlier transport call produced a non-finite value (latched status)");
-    return FVGB_ENONFINITE;
+    return report_latched(m, hst[3], s);
   }
   std::vector<double> bn2(hn, hn + P);
   double bsum = 0.0;
@@ -962,6 +1003,7 @@ static fvgb_status upload_impl(int32_t dim, int64_t n_vert, const double* xyz, i
   if ((e = cudaMemsetAsync(m->barrier, 0, sizeof(Barrier), s))) return fail(e, "memset");
   if ((e = dalloc(m, &m->d_cg_info, 4))) return fail(e, "allocation");
   if ((e = cudaMemsetAsync(m->d_cg_info, 0, 4 * sizeof(int), s))) return fail(e, "memset");
+  if ((e = dalloc(m, &m->d_solve, 1))) return fail(e, "allocation");
   if ((e = dalloc(m, &m->d_status, 1))) return fail(e, "allocation");
   if ((e = cudaMemsetAsync(m->d_status, 0, sizeof(int), s))) return fail(e, "memset");
   if ((e = dalloc(m, &m->d_time, 1))) return fail(e, "allocation");

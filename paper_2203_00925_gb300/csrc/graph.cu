@@ -16,14 +16,7 @@
 
 namespace fvgb {
 
-struct StepInfoDev {
-  int outer;      // outer steps (max over parts)
-  int inner;      // inner CG iterations (max over parts)
-  int status;     // 0 ok, 5 not converged, 6 non-finite / breakdown, 7 barrier timeout
-  int pad;
-  double rel;     // final relative residual (max over parts)
-  double bn2;     // sum over parts of ||b_p||^2
-};
+using StepInfoDev = SolveInfoDev;
 
 struct GraphState {
   cudaGraphExec_t exec = nullptr;
@@ -97,6 +90,7 @@ __global__ void k_decide(int P, const double* __restrict__ norms, const double* 
     info->outer = mo;
     info->inner = mi;
     info->status = ctl[1];
+    info->latched = 0;
     info->rel = mr;
     info->bn2 = b2;
   }
@@ -158,8 +152,10 @@ fvgb_status build_graph(fvgb_mesh m, GraphState& g, const fvgb_streamer_params* 
   const long long k0 = g_kernel_launches.load();
   cudaGraph_t graph = nullptr;
   FVGB_TRY(cudaGraphCreate(&graph, 0), "graph create");
-  cudaGraphConditionalHandle handle;
-  FVGB_TRY(cudaGraphConditionalHandleCreate(&handle, graph, 0, 0), "conditional handle");
+  // a mesh whose whole solve is one launch needs no loop node
+  const bool whole = solve_one_ok(m, &p->solve);
+  cudaGraphConditionalHandle handle{};
+  if (!whole) FVGB_TRY(cudaGraphConditionalHandleCreate(&handle, graph, 0, 0), "conditional handle");
   FVGB_TRY(cudaStreamBeginCaptureToGraph(g.cs, graph, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed),
            "begin capture");
   fvgb_status st = FVGB_OK;
@@ -180,38 +176,46 @@ fvgb_status build_graph(fvgb_mesh m, GraphState& g, const fvgb_streamer_params* 
     if ((st = cuda_status(launch_poisson_source(m, ne, ni, is_fp32(m), f, g.cs), "source kernel"))) return bail(st);
     if ((st = poisson_rhs_impl(m, p->bcset_phi, f, b, g.cs))) return bail(st);
   }
-  if ((st = cuda_status(launch_part_sumsq(m, b, g.bn2, g.cs), "norm kernel"))) return bail(st);
-  k_graph_init<<<1, 128, 0, g.cs>>>(P, g.ctl, g.outer, g.inner);
-  k_zero_parts<<<part_grid(m), 256, 0, g.cs>>>(g.bn2, m->parts.part_sc, m->parts.sc_begin, phi,
-                                               primed ? r : nullptr);
-  count_launch(2);
-  if (!primed && (st = poisson_residual(m, p->bcset_phi, phi, b, r, g.cs))) return bail(st);
-  if ((st = cuda_status(launch_part_sumsq(m, r, m->parts.norms, g.cs), "norm kernel"))) return bail(st);
-  k_decide<<<1, 128, 0, g.cs>>>(P, m->parts.norms, g.bn2, p->solve.rtol, p->solve.maxit_outer, 0,
-                                m->parts.out_inner, m->d_cg_info, m->barrier, g.ctl, m->parts.active,
-                                g.outer, g.inner, g.rel, g.info, handle);
-  count_launch();
-  const long long k1 = g_kernel_launches.load();
-  // ---- the conditional WHILE node
-  cudaStreamCaptureStatus cst;
-  const cudaGraphNode_t* deps = nullptr;
-  size_t ndeps = 0;
-  if ((st = cuda_status(cudaStreamGetCaptureInfo(g.cs, &cst, nullptr, nullptr, &deps, nullptr, &ndeps),
-                        "capture info"))) return bail(st);
-  alignas(cudaGraphNodeParams) unsigned char cp_mem[sizeof(cudaGraphNodeParams)];
-  std::memset(cp_mem, 0, sizeof(cp_mem));
-  cudaGraphNodeParams& cp = *reinterpret_cast<cudaGraphNodeParams*>(cp_mem);
-  cp.type = cudaGraphNodeTypeConditional;
-  cp.conditional.handle = handle;
-  cp.conditional.type = cudaGraphCondTypeWhile;
-  cp.conditional.size = 1;
-  cudaGraphNode_t cnode;
-  if ((st = cuda_status(cudaGraphAddNode(&cnode, graph, deps, nullptr, ndeps, &cp), "conditional node")))
-    return bail(st);
-  cudaGraph_t body = cp.conditional.phGraph_out[0];
-  if ((st = cuda_status(cudaStreamUpdateCaptureDependencies(g.cs, &cnode, nullptr, 1,
-                                                            cudaStreamSetCaptureDependencies),
-                        "capture dependencies"))) return bail(st);
+  long long k1 = 0;
+  cudaGraph_t body = nullptr;
+  if (whole) {
+    if ((st = cuda_status(launch_solve_one(m, p->bcset_phi, b, phi, r, primed, &p->solve, false, g.info, g.rel, g.outer,
+                                           g.inner, g.cs), "solve kernel"))) return bail(st);
+    k1 = g_kernel_launches.load();
+  } else {
+    if ((st = cuda_status(launch_part_sumsq(m, b, g.bn2, g.cs), "norm kernel"))) return bail(st);
+    k_graph_init<<<1, 128, 0, g.cs>>>(P, g.ctl, g.outer, g.inner);
+    k_zero_parts<<<part_grid(m), 256, 0, g.cs>>>(g.bn2, m->parts.part_sc, m->parts.sc_begin, phi,
+                                                 primed ? r : nullptr);
+    count_launch(2);
+    if (!primed && (st = poisson_residual(m, p->bcset_phi, phi, b, r, g.cs))) return bail(st);
+    if ((st = cuda_status(launch_part_sumsq(m, r, m->parts.norms, g.cs), "norm kernel"))) return bail(st);
+    k_decide<<<1, 128, 0, g.cs>>>(P, m->parts.norms, g.bn2, p->solve.rtol, p->solve.maxit_outer, 0,
+                                  m->parts.out_inner, m->d_cg_info, m->barrier, g.ctl, m->parts.active,
+                                  g.outer, g.inner, g.rel, g.info, handle);
+    count_launch();
+    k1 = g_kernel_launches.load();
+    // ---- the conditional WHILE node
+    cudaStreamCaptureStatus cst;
+    const cudaGraphNode_t* deps = nullptr;
+    size_t ndeps = 0;
+    if ((st = cuda_status(cudaStreamGetCaptureInfo(g.cs, &cst, nullptr, nullptr, &deps, nullptr, &ndeps),
+                          "capture info"))) return bail(st);
+    alignas(cudaGraphNodeParams) unsigned char cp_mem[sizeof(cudaGraphNodeParams)];
+    std::memset(cp_mem, 0, sizeof(cp_mem));
+    cudaGraphNodeParams& cp = *reinterpret_cast<cudaGraphNodeParams*>(cp_mem);
+    cp.type = cudaGraphNodeTypeConditional;
+    cp.conditional.handle = handle;
+    cp.conditional.type = cudaGraphCondTypeWhile;
+    cp.conditional.size = 1;
+    cudaGraphNode_t cnode;
+    if ((st = cuda_status(cudaGraphAddNode(&cnode, graph, deps, nullptr, ndeps, &cp), "conditional node")))
+      return bail(st);
+    body = cp.conditional.phGraph_out[0];
+    if ((st = cuda_status(cudaStreamUpdateCaptureDependencies(g.cs, &cnode, nullptr, 1,
+                                                              cudaStreamSetCaptureDependencies),
+                          "capture dependencies"))) return bail(st);
+  }
   // ---- after the loop: field, cell physics, transport
   if ((st = streamer_transport(m, p, ne, ni, phi, E, g.cs))) return bail(st);
   if (p->n_spot > 0 && (st = cuda_status(launch_time(m, false, p->dt, g.cs), "time kernel"))) return bail(st);
@@ -219,35 +223,37 @@ fvgb_status build_graph(fvgb_mesh m, GraphState& g, const fvgb_streamer_params* 
   cudaGraph_t out = nullptr;
   if ((st = cuda_status(cudaStreamEndCapture(g.cs, &out), "end capture"))) { cudaGraphDestroy(graph); return st; }
   // ---- the loop body
-  if ((st = cuda_status(cudaStreamBeginCaptureToGraph(g.cs2, body, nullptr, nullptr, 0,
-                                                      cudaStreamCaptureModeRelaxed), "begin body capture"))) {
-    cudaGraphDestroy(graph);
-    return st;
+  if (!whole) {
+    if ((st = cuda_status(cudaStreamBeginCaptureToGraph(g.cs2, body, nullptr, nullptr, 0,
+                                                        cudaStreamCaptureModeRelaxed), "begin body capture"))) {
+      cudaGraphDestroy(graph);
+      return st;
+    }
+    auto bail2 = [&](fvgb_status s2) {
+      cudaGraph_t dummy = nullptr;
+      cudaStreamEndCapture(g.cs2, &dummy);
+      cudaGraphDestroy(graph);
+      cudaGetLastError();
+      return s2;
+    };
+    const int64_t N = m->topo.N;
+    if (fp32_solve) {
+      if ((st = cuda_status(launch_inner<float>(m, p->bcset_phi, r, &p->solve, g.cs2), "inner solve"))) return bail2(st);
+      if ((st = cuda_status(launch_add_to_double(m->w32.cg_x, true, phi, N, g.cs2), "update"))) return bail2(st);
+    } else {
+      if ((st = cuda_status(launch_inner<double>(m, p->bcset_phi, r, &p->solve, g.cs2), "inner solve"))) return bail2(st);
+      if ((st = cuda_status(launch_add_to_double(m->w64.cg_x, false, phi, N, g.cs2), "update"))) return bail2(st);
+    }
+    if ((st = poisson_residual(m, p->bcset_phi, phi, b, r, g.cs2))) return bail2(st);
+    if ((st = cuda_status(launch_part_sumsq(m, r, m->parts.norms, g.cs2), "norm kernel"))) return bail2(st);
+    k_decide<<<1, 128, 0, g.cs2>>>(P, m->parts.norms, g.bn2, p->solve.rtol, p->solve.maxit_outer, 1,
+                                   m->parts.out_inner, m->d_cg_info, m->barrier, g.ctl, m->parts.active,
+                                   g.outer, g.inner, g.rel, g.info, handle);
+    count_launch();
+    cudaGraph_t body_out = nullptr;
+    if ((st = cuda_status(cudaStreamEndCapture(g.cs2, &body_out), "end body capture"))) { cudaGraphDestroy(graph); return st; }
   }
-  auto bail2 = [&](fvgb_status s2) {
-    cudaGraph_t dummy = nullptr;
-    cudaStreamEndCapture(g.cs2, &dummy);
-    cudaGraphDestroy(graph);
-    cudaGetLastError();
-    return s2;
-  };
-  const int64_t N = m->topo.N;
-  if (fp32_solve) {
-    if ((st = cuda_status(launch_inner<float>(m, p->bcset_phi, r, &p->solve, g.cs2), "inner solve"))) return bail2(st);
-    if ((st = cuda_status(launch_add_to_double(m->w32.cg_x, true, phi, N, g.cs2), "update"))) return bail2(st);
-  } else {
-    if ((st = cuda_status(launch_inner<double>(m, p->bcset_phi, r, &p->solve, g.cs2), "inner solve"))) return bail2(st);
-    if ((st = cuda_status(launch_add_to_double(m->w64.cg_x, false, phi, N, g.cs2), "update"))) return bail2(st);
-  }
-  if ((st = poisson_residual(m, p->bcset_phi, phi, b, r, g.cs2))) return bail2(st);
-  if ((st = cuda_status(launch_part_sumsq(m, r, m->parts.norms, g.cs2), "norm kernel"))) return bail2(st);
-  k_decide<<<1, 128, 0, g.cs2>>>(P, m->parts.norms, g.bn2, p->solve.rtol, p->solve.maxit_outer, 1,
-                                 m->parts.out_inner, m->d_cg_info, m->barrier, g.ctl, m->parts.active,
-                                 g.outer, g.inner, g.rel, g.info, handle);
-  count_launch();
   const long long k3 = g_kernel_launches.load();
-  cudaGraph_t body_out = nullptr;
-  if ((st = cuda_status(cudaStreamEndCapture(g.cs2, &body_out), "end body capture"))) { cudaGraphDestroy(graph); return st; }
   cudaGraphExec_t exec = nullptr;
   cudaError_t e = cudaGraphInstantiate(&exec, graph, 0);
   cudaGraphDestroy(graph);

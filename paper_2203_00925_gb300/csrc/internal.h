@@ -133,9 +133,19 @@ struct PartsDev {
 };
 
 struct Barrier {
-  unsigned int count;  // arrivals since the launch (zeroed before every launch)
-  int status;          // 0 ok, 1 timeout
-  int pad[2];
+  unsigned int count = 0;  // arrivals since the launch (zeroed before every launch)
+  int status = 0;          // 0 ok, 1 timeout
+  int pad[2] = {0, 0};
+};
+
+// Result of a whole solve run on the device (single mesh).
+struct SolveInfoDev {
+  int outer;      // outer steps (max over parts)
+  int inner;      // inner CG iterations (max over parts)
+  int status;     // 0 ok, 5 not converged, 6 non-finite / breakdown, 7 barrier timeout
+  int latched;    // nonzero: an earlier error was latched, nothing was solved
+  double rel;     // final relative residual (max over parts)
+  double bn2;     // sum over parts of ||b_p||^2
 };
 
 struct GraphState;
@@ -169,6 +179,7 @@ struct fvgb_mesh_s {
   double* dzero = nullptr;              // [N] zeros
   fvgb::Barrier* barrier = nullptr;
   int* d_cg_info = nullptr;             // [4] iterations, status
+  fvgb::SolveInfoDev* d_solve = nullptr;  // result of the last solve in one launch
   int* d_status = nullptr;              // latched asynchronous errors, cleared when reported:
                                         // bit 0 (1) non-finite transport output, bit 1 (2) a
                                         // tensor-core wait of the network kernels timed out
@@ -363,6 +374,7 @@ void graph_invalidate(fvgb_mesh m);
 
 // solver.cu ----------------------------------------------------------------------------
 int solve_grid_size(fvgb_mesh_s* m);
+cudaError_t launch_barrier_reset(fvgb_mesh_s* m, cudaStream_t s);   // before every cooperative launch
 template <typename T>
 cudaError_t launch_cg(fvgb_mesh_s* m, int bcset, const double* r, double inner_rtol, int maxit,
                       cudaStream_t s);
@@ -375,6 +387,15 @@ cudaError_t launch_inner(fvgb_mesh_s* m, int bcset, const double* r, const fvgb_
   if (o->inner > 0) return launch_amg_inner<T>(m, bcset, r, o->inner, s);
   return launch_cg<T>(m, bcset, r, o->inner_rtol, o->maxit_inner, s);
 }
+
+// A whole solve of the refinement loop with the CG inner solve in one cooperative launch, for
+// a single mesh: from b (and, when primed, the start's residual r) to phi; parts.norms,
+// parts.out_inner and *info are written. rel / outer / inner: optional per-part results.
+bool solve_one_ok(const fvgb_mesh_s* m, const fvgb_solve_opts* o);
+// check_latched: solve nothing when an earlier error is latched (info->latched then holds it).
+cudaError_t launch_solve_one(fvgb_mesh_s* m, int bcset, const double* b, double* phi, double* r, bool primed,
+                             const fvgb_solve_opts* o, bool check_latched, SolveInfoDev* info, double* rel,
+                             int* outer, int* inner, cudaStream_t s);
 
 cudaError_t launch_part_sumsq(fvgb_mesh_s* m, const double* v, double* out, cudaStream_t s);
 // per part <r0, r0 - r1>, ||r0 - r1||^2, ||r0||^2, ||r1||^2 into out[k P, (k + 1) P), k = 0..3

@@ -292,7 +292,7 @@ cudaError_t launch_small_steps(fvgb_mesh_s* m, const fvgb_tcoef* tc, T* u, doubl
   a.barrier_ns = kBarrierTimeoutNs;
   a.status = m->d_status;
   const int threads = small_threads<T>(m);
-  cudaError_t e = cudaMemsetAsync(m->barrier, 0, sizeof(Barrier), s);
+  cudaError_t e = launch_barrier_reset(m, s);
   if (e != cudaSuccess) return e;
   void* args[] = {&a};
   count_launch();

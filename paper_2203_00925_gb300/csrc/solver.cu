@@ -140,6 +140,25 @@ __device__ bool exchange(const SolveArgs<T>& a, const double* buf, unsigned& tar
   return true;
 }
 
+// This block's rows in a single mesh, and its grid barriers.
+struct OneBlock {
+  int sc0, sc1;
+  int64_t lo, hi;
+  bool arrive;                         // test hook: false leaves out this block's arrivals
+  unsigned target;
+};
+template <typename T>
+__device__ OneBlock one_block(const SolveArgs<T>& a) {
+  OneBlock k;
+  k.sc0 = a.blk_sc[blockIdx.x];
+  k.sc1 = a.blk_sc[blockIdx.x + 1];
+  k.lo = a.sc_begin[k.sc0];
+  k.hi = k.sc1 > k.sc0 ? a.sc_begin[k.sc1] : k.lo;
+  k.arrive = a.skip_block != (int)blockIdx.x;
+  k.target = 0;
+  return k;
+}
+
 // The same for a single mesh (at most one sub-chunk a block), with the block's sum before it
 // and the scalars after it: acc of every thread -> block sum (four warps, one per SM
 // sub-partition, a quarter each: GB300 issues FP64 adds at a small fraction of the FP32 rate,
@@ -147,11 +166,11 @@ __device__ bool exchange(const SolveArgs<T>& a, const double* buf, unsigned& tar
 // sums the partials from registers and hands the total to use(total) (every lane of warp 0);
 // one block barrier at the end. False when a wait ran out.
 template <typename T, typename F>
-__device__ __forceinline__ bool exchange_one(const SolveArgs<T>& a, double* buf, unsigned& target, int sc0, int sc1,
-                                             bool arrive, double acc, double* sh, int* s_ok, F use) {
+__device__ __forceinline__ bool exchange_one(const SolveArgs<T>& a, double* buf, OneBlock& k, double acc, double* sh,
+                                             int* s_ok, F use) {
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
   const int quarter = blockDim.x >> 2;
-  target += gridDim.x;
+  k.target += gridDim.x;
   sh[threadIdx.x] = acc;
   __syncthreads();                   // and every row of the phase is written before the arrival
   if (w < 4) {
@@ -165,11 +184,11 @@ __device__ __forceinline__ bool exchange_one(const SolveArgs<T>& a, double* buf,
   if (w == 0) {
     if (l == 0) {
       const double* q = sh + blockDim.x;
-      if (sc1 > sc0) __stcg(buf + sc0, (q[0] + q[1]) + (q[2] + q[3]));
-      if (arrive) grid_arrive(a.bar);
+      if (k.sc1 > k.sc0) __stcg(buf + k.sc0, (q[0] + q[1]) + (q[2] + q[3]));
+      if (k.arrive) grid_arrive(a.bar);
     }
     __syncwarp();
-    const bool ok = grid_wait(a.bar, target, a.barrier_ns);
+    const bool ok = grid_wait(a.bar, k.target, a.barrier_ns);
     double t = 0.0;
     if (ok) {
       double v[kLaneSlots];
@@ -288,14 +307,16 @@ __device__ __forceinline__ T cg_phase_r(const SolveArgs<T>& a, int64_t lo, int64
 }
 
 // The final pass on rows [lo, hi): the deferred x += alpha p of the part's last phase 1
-// (pending), then back from the scaled unknowns, x = D^-1/2 x.
+// (pending), then back from the scaled unknowns, x = D^-1/2 x, or with phi phi += D^-1/2 x.
 template <typename T>
-__device__ __forceinline__ void cg_phase_x(const SolveArgs<T>& a, int64_t lo, int64_t hi, bool pending, T alpha) {
+__device__ __forceinline__ void cg_phase_x(const SolveArgs<T>& a, int64_t lo, int64_t hi, bool pending, T alpha,
+                                           double* phi) {
   T* __restrict__ X = a.cx;
   const T* __restrict__ P = a.cp;
   for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) {
-    const T x = pending ? X[i] + alpha * P[i] : X[i];
-    X[i] = x * __ldg(a.at_isd + i);
+    const T x = (pending ? X[i] + alpha * P[i] : X[i]) * __ldg(a.at_isd + i);
+    if (phi) phi[i] += (double)x;
+    else X[i] = x;
   }
 }
 
@@ -381,19 +402,22 @@ __device__ __forceinline__ T cg_phase_pq(const SolveArgs<T>& a, int64_t lo, int6
   return acc;
 }
 
-// The kernel for a single mesh: scalars in shared memory, one exchange per phase.
+// Shared memory of the single-mesh kernels.
+template <typename T>
+struct OneShared {
+  double sh[kCgThreads + 4];
+  double total;
+  T alpha, beta;
+  int state;                           // 0 running, 1 converged, 2 breakdown, 3 idle
+  int ok;
+};
+
+// CG on a single mesh: scalars in shared memory, one exchange per phase. The correction
+// goes to a.cx, or with phi onto phi. Returns false when a wait ran out; its: iterations.
 template <typename T, bool kStream>
-__device__ void cg_one(const SolveArgs<T>& a) {
-  __shared__ double sh[kCgThreads + 4];
-  __shared__ T s_alpha, s_beta;
-  __shared__ int s_state;              // 0 running, 1 converged, 2 breakdown, 3 idle
-  __shared__ int s_ok;
-  const int sc0 = a.blk_sc[blockIdx.x], sc1 = a.blk_sc[blockIdx.x + 1];
-  const int64_t lo = a.sc_begin[sc0], hi = sc1 > sc0 ? a.sc_begin[sc1] : lo;
-  const bool arrive = a.skip_block != (int)blockIdx.x;   // test hook
-  const bool act = a.active[0] != 0;
-  unsigned target = 0;
-  int its = 0;
+__device__ bool cg_one(const SolveArgs<T>& a, OneBlock& k, OneShared<T>& s, bool act, double* phi, int& its) {
+  const int64_t lo = k.lo, hi = k.hi;
+  its = 0;
   double* const buf0 = a.buf;
   double* const buf1 = a.buf + a.n_sc;
   bool pending = false, ok;
@@ -408,36 +432,32 @@ __device__ void cg_one(const SolveArgs<T>& a) {
     a.cx[i] = T(0);
     acc += ri * ri;
   }
-  ok = exchange_one(a, buf0, target, sc0, sc1, arrive, (double)acc, sh, &s_ok, [&](double t) {
+  ok = exchange_one(a, buf0, k, (double)acc, s.sh, &s.ok, [&](double t) {
     rr = rr0 = t;
-    s_state = !act || t == 0.0 ? 3 : (t > 0.0 ? 0 : 2);
-    s_alpha = s_beta = T(0);
+    s.state = !act || t == 0.0 ? 3 : (t > 0.0 ? 0 : 2);
+    s.alpha = s.beta = T(0);
   });
-  while (ok && s_state == 0) {
-    acc = cg_phase_pq<T, kStream>(a, lo, hi, s_beta, s_alpha);
+  while (ok && s.state == 0) {
+    acc = cg_phase_pq<T, kStream>(a, lo, hi, s.beta, s.alpha);
     pending = false;                   // x += alpha p of the last r phase is applied
-    ok = exchange_one(a, buf1, target, sc0, sc1, arrive, (double)acc, sh, &s_ok, [&](double pq) {
-      if (!(pq > 0.0) || !isfinite(pq)) s_state = 2;
-      else s_alpha = (T)(rr / pq);
+    ok = exchange_one(a, buf1, k, (double)acc, s.sh, &s.ok, [&](double pq) {
+      if (!(pq > 0.0) || !isfinite(pq)) s.state = 2;
+      else s.alpha = (T)(rr / pq);
     });
-    if (!ok || s_state != 0 || its >= a.maxit_inner) break;
-    acc = cg_phase_r<T>(a, lo, hi, s_alpha);
+    if (!ok || s.state != 0 || its >= a.maxit_inner) break;
+    acc = cg_phase_r<T>(a, lo, hi, s.alpha);
     pending = true;
     ++its;
-    ok = exchange_one(a, buf0, target, sc0, sc1, arrive, (double)acc, sh, &s_ok, [&](double rrn) {
-      if (!isfinite(rrn)) s_state = 2;
-      else if (rrn <= a.inner_tol2 * rr0) s_state = 1;
-      else s_beta = (T)(rrn / rr);
+    ok = exchange_one(a, buf0, k, (double)acc, s.sh, &s.ok, [&](double rrn) {
+      if (!isfinite(rrn)) s.state = 2;
+      else if (rrn <= a.inner_tol2 * rr0) s.state = 1;
+      else s.beta = (T)(rrn / rr);
       rr = rrn;
     });
     if (its >= a.maxit_inner) break;
   }
-  if (ok) cg_phase_x<T>(a, lo, hi, pending, s_alpha);
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    a.out_inner[0] = its;
-    a.out_status[0] = ok && s_state == 2 ? 6 : 0;
-    a.out_status[1] = its;
-  }
+  if (ok) cg_phase_x<T>(a, lo, hi, pending, s.alpha, phi);
+  return ok;
 }
 
 // Many parts (an ensemble): per-part scalars and stopping tests.
@@ -550,7 +570,7 @@ __device__ void cg_many(const SolveArgs<T>& a) {
   __syncthreads();
   for (int sc = sc0; sc < sc1; ++sc) {
     const int p = a.sc_part[sc];
-    cg_phase_x<T>(a, a.sc_begin[sc], a.sc_begin[sc + 1], s_pend[p] != 0, s_alpha[p]);
+    cg_phase_x<T>(a, a.sc_begin[sc], a.sc_begin[sc + 1], s_pend[p] != 0, s_alpha[p], nullptr);
   }
   for (int p = threadIdx.x; p < P; p += blockDim.x)
     if (s_cg[p] == 2) s_status = 6;
@@ -569,8 +589,208 @@ done:
 // exchanges and partial sums, more rows in flight per thread).
 template <typename T, bool kMany, bool kStream>
 __global__ void __launch_bounds__(kCgThreads, kCgBlocksPerSm) k_cg(SolveArgs<T> a) {
-  if constexpr (kMany) cg_many<T, kStream>(a);
-  else cg_one<T, kStream>(a);
+  if constexpr (kMany) {
+    cg_many<T, kStream>(a);
+  } else {
+    __shared__ OneShared<T> s;
+    OneBlock k = one_block(a);
+    int its = 0;
+    const bool ok = cg_one<T, kStream>(a, k, s, a.active[0] != 0, nullptr, its);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      a.out_inner[0] = its;
+      a.out_status[0] = ok && s.state == 2 ? 6 : 0;
+      a.out_status[1] = its;
+    }
+  }
+}
+
+// ---- a whole solve in one launch (single mesh) -----------------------------------------------
+// The refinement loop of api.cu's solve_impl on the device: r = b - A phi on the full diamond
+// operator, its norm, the stopping test, then the CG above with the correction added to phi
+// in its last pass. An outer step as separate launches is six kernels and a host
+// synchronisation around the CG, some 60 us on 10,000 cells against 60 us of CG; here it is
+// three grid barriers. The operator is applied in two passes: vertex values, then per cell its
+// faces' fluxes (each formed from both sides, the operations and their order those of k_face and
+// k_update, so the residual has the same bits).
+struct ResidualArgs {
+  int64_t N, F, Fi, V;
+  const int64_t* sptr;
+  const int32_t* sidx;
+  const double* alpha;
+  const double* vdir;
+  const int32_t* cell_face;
+  const int4* nbr;                     // the other cell of every face slot (the cell itself on the boundary)
+  const int32_t* fvert;
+  const double* coef;
+  const int8_t* bkind;
+  const double* b;
+  double* phi;
+  double* uv;
+  double* r;
+  double rtol;
+  int maxit_outer;
+  int primed;                          // r holds b - A phi already
+  const int* latched;                  // status word to check first, or null
+  SolveInfoDev* info;
+  double* rel;                         // optional per-part results
+  int* outer;
+  int* inner;
+};
+
+// an FP64 value other blocks wrote before the last grid barrier
+__device__ __forceinline__ double load_shared(const double* p) { return load_r(p); }
+
+__device__ __forceinline__ void residual_vertices(const ResidualArgs& g) {
+  constexpr int U = 8;
+  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < g.V; v += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t b0 = g.sptr[v >> 5];
+    const int width = (int)((g.sptr[(v >> 5) + 1] - b0) >> 5);
+    const int32_t* col = g.sidx + b0 + (v & 31);
+    const double* wcol = g.alpha + b0 + (v & 31);
+    double s = 0.0;
+    for (int c = 0; c < width; c += U) {
+      int32_t j[U];
+      double w[U], x[U];
+#pragma unroll
+      for (int q = 0; q < U; ++q) j[q] = c + q < width ? __ldg(col + 32 * (c + q)) : -1;
+#pragma unroll
+      for (int q = 0; q < U; ++q) {
+        w[q] = j[q] >= 0 ? __ldg(wcol + 32 * (c + q)) : 0.0;
+        x[q] = j[q] >= 0 ? load_shared(g.phi + j[q]) : 0.0;
+      }
+#pragma unroll
+      for (int q = 0; q < U; ++q)
+        if (j[q] >= 0) s = __fma_rn(w[q], x[q], s);
+    }
+    const double d = g.vdir[v];
+    g.uv[v] = d == d ? 0.0 : s;
+  }
+}
+
+// r = b - A phi on the block's rows; returns the thread's sum of r^2
+template <int D>
+__device__ __forceinline__ double residual_rows(const ResidualArgs& g, int64_t lo, int64_t hi) {
+  double sum = 0.0;
+  for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) {
+    int32_t e[D + 1], vx[D + 1][3];
+    double c[D + 1][3], o[D + 1], uvx[D + 1][3];
+    bool on[D + 1], bnd[D + 1];
+#pragma unroll
+    for (int k = 0; k <= D; ++k) e[k] = g.cell_face[k * g.N + i];
+    const int4 nb4 = __ldg(g.nbr + i);
+    const int nb[4] = {nb4.x, nb4.y, nb4.z, nb4.w};
+    const double me = load_shared(g.phi + i);
+#pragma unroll
+    for (int k = 0; k <= D; ++k) {
+      const int64_t f = e[k] >= 0 ? e[k] : ~e[k];
+      bnd[k] = f >= g.Fi;
+      on[k] = !bnd[k] || g.bkind[f - g.Fi] == FVGB_BC_DIRICHLET;
+      o[k] = bnd[k] ? 0.0 : load_shared(g.phi + nb[k]);
+#pragma unroll
+      for (int q = 0; q < D; ++q) {
+        c[k][q] = __ldg(g.coef + q * g.F + f);
+        vx[k][q] = __ldg(g.fvert + q * g.F + f);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k <= D; ++k)
+#pragma unroll
+      for (int q = 0; q < D; ++q) uvx[k][q] = on[k] ? load_shared(g.uv + vx[k][q]) : 0.0;
+    double acc = 0.0;
+#pragma unroll
+    for (int k = 0; k <= D; ++k) {
+      const bool left = e[k] >= 0;
+      const double ul = left ? me : o[k], ur = left ? o[k] : me;
+      double q = __dmul_rn(c[k][0], __dsub_rn(ur, ul));
+      if constexpr (D == 3) {
+        q = __fma_rn(c[k][1], __dsub_rn(uvx[k][0], uvx[k][2]), q);
+        q = __fma_rn(c[k][2], __dsub_rn(uvx[k][1], uvx[k][2]), q);
+      } else {
+        q = __fma_rn(c[k][1], __dsub_rn(uvx[k][1], uvx[k][0]), q);
+      }
+      if (on[k]) acc += left ? -q : q;
+    }
+    const double r = g.b[i] - acc;
+    g.r[i] = r;
+    sum += r * r;
+  }
+  return sum;
+}
+
+// grid barrier without sums; false when the wait ran out
+template <typename T>
+__device__ bool one_barrier(const SolveArgs<T>& a, OneBlock& k) {
+  bool ok = true;
+  k.target += gridDim.x;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    if (threadIdx.x == 0 && k.arrive) grid_arrive(a.bar);
+    __syncwarp();
+    ok = grid_wait(a.bar, k.target, a.barrier_ns);
+  }
+  return __syncthreads_and(ok) != 0;
+}
+
+template <typename T, int D>
+__global__ void __launch_bounds__(kCgThreads, kCgBlocksPerSm) k_solve_one(SolveArgs<T> a, ResidualArgs g) {
+  __shared__ OneShared<T> s;
+  OneBlock k = one_block(a);
+  SolveInfoDev out{0, 0, 0, 0, 0.0, 0.0};
+  double* const buf0 = a.buf + 2 * (size_t)a.n_sc;   // the CG uses the first two
+  double* const buf1 = buf0 + a.n_sc;
+  auto total = [&](double t) { s.total = t; };
+  bool ok = true, run = true;
+  double sum = 0.0, rel = 0.0;
+  const int latched = g.latched ? *g.latched : 0;
+  if (latched != 0) {                       // uniform over the grid: nothing writes it meanwhile
+    out.latched = latched;
+    run = false;
+  } else {
+    for (int64_t i = k.lo + threadIdx.x; i < k.hi; i += blockDim.x) sum += g.b[i] * g.b[i];
+    ok = exchange_one(a, buf1, k, sum, s.sh, &s.ok, total);
+    out.bn2 = ok ? s.total : 0.0;
+    if (!isfinite(out.bn2)) { out.status = 6; run = false; }
+  }
+  const double bn2 = out.bn2;
+  if (ok && run && bn2 == 0.0) {            // the solution is 0 (and then the residual 0)
+    for (int64_t i = k.lo + threadIdx.x; i < k.hi; i += blockDim.x) {
+      g.phi[i] = 0.0;
+      g.r[i] = 0.0;
+    }
+    run = false;
+  }
+  for (int outer = 0; ok && run; ++outer) {
+    sum = 0.0;
+    if (outer == 0 && g.primed) {
+      for (int64_t i = k.lo + threadIdx.x; i < k.hi; i += blockDim.x) sum += g.r[i] * g.r[i];
+    } else {
+      if (outer > 0 && !(ok = one_barrier(a, k))) break;      // phi of every block
+      residual_vertices(g);
+      if (!(ok = one_barrier(a, k))) break;                    // vertex values of every block
+      sum = residual_rows<D>(g, k.lo, k.hi);
+    }
+    if (!(ok = exchange_one(a, outer & 1 ? buf1 : buf0, k, sum, s.sh, &s.ok, total))) break;
+    rel = sqrt(s.total / bn2);
+    out.outer = outer;
+    out.rel = rel;
+    if (!isfinite(rel)) { out.status = 6; break; }
+    if (!(rel > g.rtol)) break;
+    if (outer >= g.maxit_outer) { out.status = 5; break; }
+    int its = 0;
+    ok = cg_one<T, false>(a, k, s, true, g.phi, its);
+    out.inner += its;
+    if (ok && s.state == 2) { out.outer = outer + 1; out.status = 6; break; }
+  }
+  if (!ok) out.status = 7;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    *g.info = out;
+    a.out_inner[0] = out.inner;
+    if (g.rel) {
+      g.rel[0] = out.rel;
+      g.outer[0] = out.outer;
+      g.inner[0] = out.inner;
+    }
+  }
 }
 
 // The variant for a mesh of N cells in n_part parts: kStream in FP32 once an iteration's
@@ -582,6 +802,11 @@ const void* cg_kernel(int64_t N, int n_part, int64_t l2_bytes) {
       return n_part > 1 ? (const void*)k_cg<T, true, true> : (const void*)k_cg<T, false, true>;
   }
   return n_part > 1 ? (const void*)k_cg<T, true, false> : (const void*)k_cg<T, false, false>;
+}
+
+// a kernel, not a memset: the same engine as its neighbours in the stream or graph
+__global__ void k_barrier_reset(Barrier* bar) {
+  if (threadIdx.x == 0) *bar = Barrier{};
 }
 
 // Per-part sum of squares of an FP64 vector over the same sub-chunks (one block per
@@ -641,11 +866,24 @@ __global__ void __launch_bounds__(kCgThreads) k_part_dots_partial(const double* 
 
 }  // namespace
 
+cudaError_t launch_barrier_reset(fvgb_mesh_s* m, cudaStream_t s) {
+  k_barrier_reset<<<1, 32, 0, s>>>(m->barrier);
+  count_launch();
+  return cudaGetLastError();
+}
+
 int solve_grid_size(fvgb_mesh_s* m) {
   const void* kernels[] = {(const void*)k_cg<float, false, false>, (const void*)k_cg<float, true, false>,
                            (const void*)k_cg<float, false, true>, (const void*)k_cg<float, true, true>,
                            (const void*)k_cg<double, false, false>, (const void*)k_cg<double, true, false>};
   int per_sm = kCgBlocksPerSm;
+  const void* whole[] = {(const void*)k_solve_one<float, 2>, (const void*)k_solve_one<float, 3>,
+                         (const void*)k_solve_one<double, 2>, (const void*)k_solve_one<double, 3>};
+  for (const void* k : whole) {
+    int n = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, kCgThreads, 0) != cudaSuccess) return 0;
+    per_sm = n < per_sm ? n : per_sm;
+  }
   for (const void* k : kernels) {
     int n = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, kCgThreads, 0) != cudaSuccess) return 0;
@@ -671,9 +909,9 @@ cudaError_t launch_part_dots(fvgb_mesh_s* m, const double* r0, const double* r1,
   return cudaGetLastError();
 }
 
+namespace {
 template <typename T>
-cudaError_t launch_cg(fvgb_mesh_s* m, int bcset, const double* r, double inner_rtol, int maxit,
-                      cudaStream_t s) {
+SolveArgs<T> solve_args(fvgb_mesh_s* m, int bcset, const double* r, double inner_rtol, int maxit) {
   GeoDev<T>& g = geo_of<T>(m);
   Work<T>& w = work_of<T>(m);
   SolveArgs<T> a;
@@ -692,13 +930,64 @@ cudaError_t launch_cg(fvgb_mesh_s* m, int bcset, const double* r, double inner_r
   a.out_status = m->d_cg_info;
   a.skip_block = m->test_skip_block;
   a.barrier_ns = m->test_barrier_ns > 0 ? m->test_barrier_ns : kBarrierTimeoutNs;
-  if (pd.n_sc > kCgThreads) return cudaErrorInvalidConfiguration;   // their staging
-  cudaError_t e = cudaMemsetAsync(m->barrier, 0, sizeof(Barrier), s);
+  return a;
+}
+
+template <typename T>
+cudaError_t launch_whole(fvgb_mesh_s* m, int bcset, ResidualArgs& g, const double* r, const fvgb_solve_opts* o,
+                         cudaStream_t s) {
+  SolveArgs<T> a = solve_args<T>(m, bcset, r, o->inner_rtol, o->maxit_inner);
+  cudaError_t e = launch_barrier_reset(m, s);
+  if (e != cudaSuccess) return e;
+  void* args[] = {&a, &g};
+  const void* k = m->topo.dim == 3 ? (const void*)k_solve_one<T, 3> : (const void*)k_solve_one<T, 2>;
+  count_launch();
+  return cudaLaunchCooperativeKernel(k, dim3(m->solve_grid), dim3(kCgThreads), args, 0, s);
+}
+}  // namespace
+
+template <typename T>
+cudaError_t launch_cg(fvgb_mesh_s* m, int bcset, const double* r, double inner_rtol, int maxit,
+                      cudaStream_t s) {
+  SolveArgs<T> a = solve_args<T>(m, bcset, r, inner_rtol, maxit);
+  if (a.n_sc > kCgThreads) return cudaErrorInvalidConfiguration;   // their staging
+  cudaError_t e = launch_barrier_reset(m, s);
   if (e != cudaSuccess) return e;
   void* args[] = {&a};
   count_launch();
   return cudaLaunchCooperativeKernel(cg_kernel<T>(a.N, a.n_part, m->l2_bytes), dim3(m->solve_grid), dim3(kCgThreads),
                                      args, 0, s);
+}
+
+// The whole solve in one launch up to kSolveOneMax cells. A solve to 1e-8 against separate
+// launches: 10,368 cells FP64 3.46 -> 2.38 ms, 384,000 13.4 -> 12.3 (mixed 9.7 -> 8.8); 750,000
+// equal; 1.3M 38.8 -> 43.1: one 512-thread block an SM streams the operator's passes slower than
+// their own kernels. (CUDA-event timing of the CG wants its own launches.)
+constexpr int64_t kSolveOneMax = 600000;
+
+bool solve_one_ok(const fvgb_mesh_s* m, const fvgb_solve_opts* o) {
+  return m->parts.n_part == 1 && o->inner == 0 && !m->time_cg && m->topo.N <= kSolveOneMax;
+}
+
+cudaError_t launch_solve_one(fvgb_mesh_s* m, int bcset, const double* b, double* phi, double* r, bool primed,
+                             const fvgb_solve_opts* o, bool check_latched, SolveInfoDev* info, double* rel,
+                             int* outer, int* inner, cudaStream_t s) {
+  const TopoDev& t = m->topo;
+  const BCDev<double>& bc = m->g64.bc[bcset];
+  ResidualArgs g;
+  g.N = t.N; g.F = t.F; g.Fi = t.Fi; g.V = t.V;
+  g.sptr = t.vsell.ptr; g.sidx = t.vsell.idx;
+  g.alpha = m->g64.valpha; g.vdir = bc.vdir;
+  g.cell_face = t.cell_face; g.nbr = reinterpret_cast<const int4*>(bc.at_nbr);
+  g.fvert = t.fvert; g.coef = m->g64.coef; g.bkind = bc.bkind;
+  g.b = b; g.phi = phi; g.uv = m->w64.uv; g.r = r;
+  g.rtol = o->rtol; g.maxit_outer = o->maxit_outer;
+  g.primed = primed ? 1 : 0;
+  g.latched = check_latched ? m->d_status : nullptr;
+  g.info = info;
+  g.rel = rel; g.outer = outer; g.inner = inner;
+  const bool fp32 = o->prec == FVGB_FP32 || o->prec == FVGB_MIXED;
+  return fp32 ? launch_whole<float>(m, bcset, g, r, o, s) : launch_whole<double>(m, bcset, g, r, o, s);
 }
 
 template cudaError_t launch_cg<double>(fvgb_mesh_s*, int, const double*, double, int, cudaStream_t);
