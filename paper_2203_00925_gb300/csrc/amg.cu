@@ -13,6 +13,7 @@
 #include <cuda_runtime.h>
 
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "amg_host.h"
@@ -47,9 +48,7 @@ struct AmgDev {
   T* cinv = nullptr;
   T* cb = nullptr;
   T* cx = nullptr;
-  T* t0 = nullptr;   // level-0 scratch: masked right-hand side
-  T* t1 = nullptr;   // level-0 scratch: residual of the current correction
-  T* t2 = nullptr;   // level-0 scratch: one cycle's correction
+  T* t0 = nullptr;   // level 0: masked right-hand side
 };
 
 struct AmgState {
@@ -112,21 +111,65 @@ k_amg_dense(int64_t n, const T* __restrict__ inv, const T* __restrict__ b, T* __
   if (lane == 0) x[i] = s;
 }
 
-// right-hand side in T, zero on the parts that are not active (one block per sub-chunk)
+// Start of the first cycle: the right-hand side in T, zero on the parts that are not active,
+// and the first smoothing step from zero, x = w D^-1 b (blockIdx.y pieces of sub-chunk
+// blockIdx.x)
 template <typename T>
-__global__ void k_amg_rhs(const double* __restrict__ r, const int64_t* __restrict__ sc_begin,
-                          const int32_t* __restrict__ sc_part, const int* __restrict__ active,
-                          T* __restrict__ b) {
+__global__ void __launch_bounds__(kAmgThreads)
+k_amg_start(const double* __restrict__ r, const int64_t* __restrict__ sc_begin, const int32_t* __restrict__ sc_part,
+            const int* __restrict__ active, const T* __restrict__ dinv, T w, T* __restrict__ b, T* __restrict__ x) {
   const int sc = blockIdx.x;
   const bool act = active[sc_part[sc]] != 0;
-  for (int64_t i = sc_begin[sc] + threadIdx.x; i < sc_begin[sc + 1]; i += blockDim.x)
-    b[i] = act ? (T)r[i] : T(0);
+  for (int64_t i = sc_begin[sc] + blockIdx.y * (int64_t)blockDim.x + threadIdx.x; i < sc_begin[sc + 1];
+       i += (int64_t)gridDim.y * blockDim.x) {
+    const T v = act ? (T)r[i] : T(0);
+    b[i] = v;
+    if (x) x[i] = w * dinv[i] * v;
+  }
+}
+
+// Finest level, on the operator as the mesh stores it (four neighbours and coefficients a row
+// by vector loads; the CSR form took 60 bytes a row with its row pointers and indices of the
+// diagonal): mode 0 y = b - A x; 1 y = x + w D^-1 (b - A x); 2 the same added to phi.
+template <typename T> struct FineCoef;
+template <> struct FineCoef<float> {
+  static __device__ __forceinline__ void load(const float* p, int64_t i, float (&c)[4]) {
+    const float4 v = __ldg(reinterpret_cast<const float4*>(p) + i);
+    c[0] = v.x; c[1] = v.y; c[2] = v.z; c[3] = v.w;
+  }
+};
+template <> struct FineCoef<double> {
+  static __device__ __forceinline__ void load(const double* p, int64_t i, double (&c)[4]) {
+    const double2 v = __ldg(reinterpret_cast<const double2*>(p) + 2 * i), w = __ldg(reinterpret_cast<const double2*>(p) + 2 * i + 1);
+    c[0] = v.x; c[1] = v.y; c[2] = w.x; c[3] = w.y;
+  }
+};
+template <typename T, int MODE>
+__global__ void __launch_bounds__(kAmgThreads)
+k_amg_fine(int64_t n, const int4* __restrict__ nbr, const T* __restrict__ coef, const T* __restrict__ diag,
+           const T* __restrict__ dinv, T w, const T* __restrict__ x, const T* __restrict__ b, T* __restrict__ y,
+           double* __restrict__ phi) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const int4 nb = __ldg(nbr + i);
+  T c[4];
+  FineCoef<T>::load(coef, i, c);
+  const T xi = x[i], g0 = x[nb.x], g1 = x[nb.y], g2 = x[nb.z], g3 = x[nb.w];
+  T s = diag[i] * xi;
+  s -= c[0] * g0;
+  s -= c[1] * g1;
+  s -= c[2] * g2;
+  s -= c[3] * g3;
+  const T res = b[i] - s;
+  if (MODE == 0) y[i] = res;
+  else if (MODE == 1) y[i] = xi + w * dinv[i] * res;
+  else phi[i] += (double)(xi + w * dinv[i] * res);
 }
 
 template <typename T>
-__global__ void k_amg_add(int64_t n, const T* __restrict__ a, T* __restrict__ y) {
+__global__ void k_amg_add(int64_t n, const T* __restrict__ a, double* __restrict__ phi) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i < n) y[i] += a[i];
+  if (i < n) phi[i] += (double)a[i];
 }
 
 // inner-solve bookkeeping read by the outer loop: cycles per active part, status ok
@@ -178,7 +221,8 @@ fvgb_status amg_upload(fvgb_mesh m, const AmgHost& H, AmgDev<T>& a, cudaStream_t
   for (int l = 0; l < L; ++l) {
     const AmgHostLevel& h = H.levels[l];
     AmgLevelDev<T>& d = a.lv[l];
-    FVGB_TRY(upload_csr<T>(m, h.A, d.A, s), "upload");
+    if (l > 0) FVGB_TRY(upload_csr<T>(m, h.A, d.A, s), "upload");
+    else d.A.n = d.A.m = h.A.n;          // level 0 works on the mesh's own arrays (k_amg_fine)
     FVGB_TRY(upload_csr<T>(m, h.P, d.P, s), "upload");
     FVGB_TRY(upload_csr<T>(m, h.R, d.R, s), "upload");
     FVGB_TRY(dupload(m, &d.dinv, std::vector<T>(h.dinv.begin(), h.dinv.end()), s), "upload");
@@ -194,13 +238,11 @@ fvgb_status amg_upload(fvgb_mesh m, const AmgHost& H, AmgDev<T>& a, cudaStream_t
   FVGB_TRY(dalloc(m, &a.cx, a.nco), "allocation");
   const int64_t N = m->topo.N;
   FVGB_TRY(dalloc(m, &a.t0, N), "allocation");
-  FVGB_TRY(dalloc(m, &a.t1, N), "allocation");
-  FVGB_TRY(dalloc(m, &a.t2, N), "allocation");
   a.built = true;
   return FVGB_OK;
 }
 
-// One V-cycle on level l: b -> out (zero initial guess).
+// One V-cycle on level l >= 1: b -> out (zero initial guess).
 template <typename T>
 cudaError_t vcycle(AmgDev<T>& a, int l, const T* b, T* out, cudaStream_t s) {
   const T w = T(2.0 / 3.0);
@@ -271,33 +313,58 @@ int amg_levels(fvgb_mesh m, int bcset, bool fp32, int64_t* sizes, int cap) {
   return fp32 ? fill(m->amg->d32[bcset]) : fill(m->amg->d64[bcset]);
 }
 
-// delta (work_of<T>(m).cg_x) = `cycles` V-cycles on A_T delta = r (masked to the active
-// parts); the outer loop's inner bookkeeping is filled as for the CG.
+// phi += `cycles` V-cycles on A_T delta = r (masked to the active parts); the outer loop's
+// inner bookkeeping is filled as for the CG. Cycles after the first go on from the iterate
+// (smooth, coarse correction, smooth) instead of solving for a correction of it, which needs no
+// pass to form that residual, to add it back, or to start it.
 template <typename T>
-cudaError_t launch_amg_inner(fvgb_mesh_s* m, int bcset, const double* r, int cycles, cudaStream_t s) {
+cudaError_t launch_amg_inner(fvgb_mesh_s* m, int bcset, const double* r, int cycles, double* phi, cudaStream_t s) {
   AmgDev<T>& a = amg_of<T>(m->amg)[bcset];
+  const BCDev<T>& bc = geo_of<T>(m).bc[bcset];
   Work<T>& w = work_of<T>(m);
   const PartsDev& pd = m->parts;
   const int64_t N = m->topo.N;
+  const T om = T(2.0 / 3.0);
+  const bool dense = a.lv.empty();     // at most kAmgCoarseMax cells: the dense solve is exact
+  const unsigned rows = blocks_for(N, kAmgThreads);
   cudaError_t e;
-  k_amg_rhs<T><<<pd.n_sc, 256, 0, s>>>(r, pd.sc_begin, pd.sc_part, pd.active, a.t0);
+  const dim3 pieces((unsigned)pd.n_sc, (unsigned)pd.split);
+  k_amg_start<T><<<pieces, kAmgThreads, 0, s>>>(r, pd.sc_begin, pd.sc_part, pd.active, dense ? nullptr : a.lv[0].dinv,
+                                                om, a.t0, dense ? nullptr : a.lv[0].x);
   count_launch();
   if ((e = cudaGetLastError())) return e;
-  if ((e = vcycle(a, 0, a.t0, w.cg_x, s))) return e;
-  // with no levels (a mesh of at most kAmgCoarseMax cells) the dense solve is exact
-  for (int c = 1; c < cycles && !a.lv.empty(); ++c) {
-    if ((e = csr_launch(a.lv[0].A, w.cg_x, a.t0, a.lv[0].dinv, T(0), 2, a.t1, s))) return e;
-    if ((e = vcycle(a, 0, a.t1, a.t2, s))) return e;
-    k_amg_add<T><<<blocks_for(N, kAmgThreads), kAmgThreads, 0, s>>>(N, a.t2, w.cg_x);
+  if (dense) {
+    if ((e = vcycle(a, 0, a.t0, w.cg_x, s))) return e;
+    k_amg_add<T><<<rows, kAmgThreads, 0, s>>>(N, w.cg_x, phi);
     count_launch();
-    if ((e = cudaGetLastError())) return e;
+  } else {
+    AmgLevelDev<T>& L = a.lv[0];
+    const bool last = a.lv.size() == 1;
+    T* nb = last ? a.cb : a.lv[1].b;
+    T* nx = last ? a.cx : a.lv[1].xo;
+    auto fine = [&](auto mode, const T* x, T* y) {
+      k_amg_fine<T, decltype(mode)::value><<<rows, kAmgThreads, 0, s>>>(
+          N, reinterpret_cast<const int4*>(bc.at_nbr), bc.at_coef, bc.at_diag, L.dinv, om, x, a.t0, y, phi);
+      count_launch();
+      return cudaGetLastError();
+    };
+    for (int c = 0; c < cycles; ++c) {
+      if (c > 0 && (e = fine(std::integral_constant<int, 1>{}, L.xo, L.x))) return e;          // smoothing
+      if ((e = fine(std::integral_constant<int, 0>{}, L.x, L.r))) return e;                    // r = b - A x
+      if ((e = csr_launch(L.R, L.r, (const T*)nullptr, L.dinv, om, 0, nb, s))) return e;      // b' = R r
+      if ((e = vcycle(a, 1, nb, nx, s))) return e;
+      if ((e = csr_launch(L.P, nx, (const T*)nullptr, L.dinv, om, 1, L.x, s))) return e;      // x += P x'
+      if (c + 1 < cycles) e = fine(std::integral_constant<int, 1>{}, L.x, L.xo);               // smoothing
+      else e = fine(std::integral_constant<int, 2>{}, L.x, (T*)nullptr);
+      if (e) return e;
+    }
   }
   k_amg_info<<<1, 128, 0, s>>>(pd.n_part, pd.active, cycles, pd.out_inner, m->d_cg_info);
   count_launch();
   return cudaGetLastError();
 }
 
-template cudaError_t launch_amg_inner<float>(fvgb_mesh_s*, int, const double*, int, cudaStream_t);
-template cudaError_t launch_amg_inner<double>(fvgb_mesh_s*, int, const double*, int, cudaStream_t);
+template cudaError_t launch_amg_inner<float>(fvgb_mesh_s*, int, const double*, int, double*, cudaStream_t);
+template cudaError_t launch_amg_inner<double>(fvgb_mesh_s*, int, const double*, int, double*, cudaStream_t);
 
 }  // namespace fvgb

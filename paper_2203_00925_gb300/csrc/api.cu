@@ -391,6 +391,9 @@ cudaError_t setup_parts(fvgb_mesh_s* m, const std::vector<int64_t>& part_begin, 
   if ((e = dalloc(m, &pd.active, P))) return e;
   if ((e = dalloc(m, &pd.out_inner, P))) return e;
   if ((e = dalloc(m, &pd.norms, P))) return e;
+  // the norm kernels' blocks: up to eight an SM, of at least four rows a thread
+  pd.split = (int)std::max<int64_t>(1, std::min<int64_t>(8, N / (1024 * (int64_t)n_sc)));
+  if ((e = dalloc(m, &pd.norm_buf, (size_t)n_sc * pd.split))) return e;
   return cudaSuccess;
 }
 
@@ -489,10 +492,14 @@ fvgb_status transport_stage(fvgb_mesh m, const fvgb_tcoef* tc, const T* base, T*
 
 // FP64 full diamond operator pieces
 fvgb_status poisson_residual(fvgb_mesh m, int bcset, const double* x, const double* b, double* r,
-                             cudaStream_t s) {
+                             cudaStream_t s, double* norms) {
   Work<double>& w = m->w64;
   FVGB_TRY(launch_vertex<double>(m, bcset, x, w.uv, true, s), "vertex kernel");
   FVGB_TRY(launch_face<double>(m, bcset, x, w.uv, nullptr, nullptr, false, -1.0, true, w.flux, s), "face kernel");
+  if (norms) {
+    FVGB_TRY(launch_residual_norm(m, w.flux, b, r, norms, s), "residual kernel");
+    return FVGB_OK;
+  }
   FVGB_TRY(launch_update<double>(m, b ? kPoissonResidual : kPoissonApply, w.flux, nullptr, nullptr,
                                  0.0, b, r, nullptr, s), "update kernel");
   return FVGB_OK;
@@ -560,7 +567,6 @@ fvgb_status solve_impl(fvgb_mesh m, int bcset, const double* f, double* phi,
                        const fvgb_solve_opts* o, fvgb_solve_info* info, cudaStream_t s) {
   fvgb_solve_info loc{0, 0, 0.0, 0.0};
   m->stats.solves++;
-  const int64_t N = m->topo.N;
   const int P = m->parts.n_part;
   const bool fp32 = o->prec == FVGB_FP32 || o->prec == FVGB_MIXED;
   if (fp32 && !is_fp32(m)) { set_error("FP32 inner solve needs a mesh uploaded with FVGB_FP32 or FVGB_MIXED"); return FVGB_EINVAL; }
@@ -615,11 +621,8 @@ fvgb_status solve_impl(fvgb_mesh m, int bcset, const double* f, double* phi,
   m->last_inner.assign(P, 0);
   m->last_rel.assign(P, 0.0);
   for (int outer = 0;; ++outer) {
-    if (!(primed && outer == 0)) {
-      st = poisson_residual(m, bcset, phi, b, r, s);
-      if (st) return st;
-    }
-    FVGB_TRY(launch_part_sumsq(m, r, m->parts.norms, s), "norm kernel");
+    if (primed && outer == 0) FVGB_TRY(launch_part_sumsq(m, r, m->parts.norms, s), "norm kernel");
+    else if ((st = poisson_residual(m, bcset, phi, b, r, s, m->parts.norms))) return st;
     FVGB_TRY(cudaMemcpyAsync(hn, m->parts.norms, P * sizeof(double), cudaMemcpyDeviceToHost, s), "copy");
     if (outer > 0) {
       FVGB_TRY(cudaMemcpyAsync(hinner, m->parts.out_inner, P * sizeof(int), cudaMemcpyDeviceToHost, s), "copy");
@@ -664,15 +667,13 @@ fvgb_status solve_impl(fvgb_mesh m, int bcset, const double* f, double* phi,
     m->stats.outer_its++;
     FVGB_TRY(cudaMemcpyAsync(m->parts.active, hact, P * sizeof(int), cudaMemcpyHostToDevice, s), "copy");
     if (m->time_cg) FVGB_TRY(cudaEventRecord(m->ev_cg0, s), "event");
-    if (fp32) FVGB_TRY(launch_inner<float>(m, bcset, r, o, s), "inner solve");
-    else FVGB_TRY(launch_inner<double>(m, bcset, r, o, s), "inner solve");
+    if (fp32) FVGB_TRY(launch_inner<float>(m, bcset, r, o, phi, s), "inner solve");
+    else FVGB_TRY(launch_inner<double>(m, bcset, r, o, phi, s), "inner solve");
     if (m->time_cg) {
       FVGB_TRY(cudaEventRecord(m->ev_cg1, s), "event");
       m->cg_pending = true;
     }
     m->stats.cg_launches++;
-    if (fp32) FVGB_TRY(launch_add_to_double(m->w32.cg_x, true, phi, N, s), "update");
-    else FVGB_TRY(launch_add_to_double(m->w64.cg_x, false, phi, N, s), "update");
   }
   if (info) *info = loc;
   return FVGB_OK;

@@ -188,8 +188,9 @@ fvgb_status build_graph(fvgb_mesh m, GraphState& g, const fvgb_streamer_params* 
     k_zero_parts<<<part_grid(m), 256, 0, g.cs>>>(g.bn2, m->parts.part_sc, m->parts.sc_begin, phi,
                                                  primed ? r : nullptr);
     count_launch(2);
-    if (!primed && (st = poisson_residual(m, p->bcset_phi, phi, b, r, g.cs))) return bail(st);
-    if ((st = cuda_status(launch_part_sumsq(m, r, m->parts.norms, g.cs), "norm kernel"))) return bail(st);
+    if (primed) st = cuda_status(launch_part_sumsq(m, r, m->parts.norms, g.cs), "norm kernel");
+    else st = poisson_residual(m, p->bcset_phi, phi, b, r, g.cs, m->parts.norms);
+    if (st) return bail(st);
     k_decide<<<1, 128, 0, g.cs>>>(P, m->parts.norms, g.bn2, p->solve.rtol, p->solve.maxit_outer, 0,
                                   m->parts.out_inner, m->d_cg_info, m->barrier, g.ctl, m->parts.active,
                                   g.outer, g.inner, g.rel, g.info, handle);
@@ -236,16 +237,10 @@ fvgb_status build_graph(fvgb_mesh m, GraphState& g, const fvgb_streamer_params* 
       cudaGetLastError();
       return s2;
     };
-    const int64_t N = m->topo.N;
-    if (fp32_solve) {
-      if ((st = cuda_status(launch_inner<float>(m, p->bcset_phi, r, &p->solve, g.cs2), "inner solve"))) return bail2(st);
-      if ((st = cuda_status(launch_add_to_double(m->w32.cg_x, true, phi, N, g.cs2), "update"))) return bail2(st);
-    } else {
-      if ((st = cuda_status(launch_inner<double>(m, p->bcset_phi, r, &p->solve, g.cs2), "inner solve"))) return bail2(st);
-      if ((st = cuda_status(launch_add_to_double(m->w64.cg_x, false, phi, N, g.cs2), "update"))) return bail2(st);
-    }
-    if ((st = poisson_residual(m, p->bcset_phi, phi, b, r, g.cs2))) return bail2(st);
-    if ((st = cuda_status(launch_part_sumsq(m, r, m->parts.norms, g.cs2), "norm kernel"))) return bail2(st);
+    if (fp32_solve) st = cuda_status(launch_inner<float>(m, p->bcset_phi, r, &p->solve, phi, g.cs2), "inner solve");
+    else st = cuda_status(launch_inner<double>(m, p->bcset_phi, r, &p->solve, phi, g.cs2), "inner solve");
+    if (!st) st = poisson_residual(m, p->bcset_phi, phi, b, r, g.cs2, m->parts.norms);
+    if (st) return bail2(st);
     k_decide<<<1, 128, 0, g.cs2>>>(P, m->parts.norms, g.bn2, p->solve.rtol, p->solve.maxit_outer, 1,
                                    m->parts.out_inner, m->d_cg_info, m->barrier, g.ctl, m->parts.active,
                                    g.outer, g.inner, g.rel, g.info, handle);

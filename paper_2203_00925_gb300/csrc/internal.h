@@ -130,6 +130,8 @@ struct PartsDev {
   int* active = nullptr;        // [P] parts the inner solve works on
   int* out_inner = nullptr;     // [P] inner iterations of the last CG launch
   double* norms = nullptr;      // [P] per-part sums of squares
+  int split = 1;                // pieces a sub-chunk is cut into by the norm kernels
+  double* norm_buf = nullptr;   // [n_sc * split] their sums
 };
 
 struct Barrier {
@@ -300,7 +302,11 @@ cudaError_t launch_scale_start(fvgb_mesh_s* m, const double* dots, const double*
                                double* phi, int* used, double* scale, double* r0, const double* r1,
                                cudaStream_t s);
 cudaError_t launch_axpy_d(const double* x, double a, double* y, int64_t n, cudaStream_t s);
-cudaError_t launch_add_to_double(const void* x, bool fp32, double* y, int64_t n, cudaStream_t s);
+// per-part sums of squares of an FP64 vector; the Poisson residual r = b - (gathered fluxes)
+// with its sums
+cudaError_t launch_part_sumsq(fvgb_mesh_s* m, const double* v, double* out, cudaStream_t s);
+cudaError_t launch_residual_norm(fvgb_mesh_s* m, const double* flux, const double* b, double* r, double* out,
+                                 cudaStream_t s);
 cudaError_t launch_convert(const double* x, float* y, int64_t n, cudaStream_t s);
 cudaError_t launch_convert_back(const float* x, double* y, int64_t n, cudaStream_t s);
 cudaError_t launch_permute(const void* src, void* dst, const int32_t* perm, int64_t n, int ncomp,
@@ -343,10 +349,11 @@ fvgb_status amg_ensure(fvgb_mesh m, int bcset, bool fp32, cudaStream_t s);
 void amg_release(fvgb_mesh m);
 int amg_levels(fvgb_mesh m, int bcset, bool fp32, int64_t* sizes, int cap);
 template <typename T>
-cudaError_t launch_amg_inner(fvgb_mesh_s* m, int bcset, const double* r, int cycles, cudaStream_t s);
+cudaError_t launch_amg_inner(fvgb_mesh_s* m, int bcset, const double* r, int cycles, double* phi, cudaStream_t s);
 
+// y = A x (b null), or r = b - A x, with norms (optional) its per-part sums of squares
 fvgb_status poisson_residual(fvgb_mesh m, int bcset, const double* x, const double* b, double* r,
-                             cudaStream_t s);
+                             cudaStream_t s, double* norms = nullptr);
 fvgb_status poisson_rhs_impl(fvgb_mesh m, int bcset, const double* f, double* b, cudaStream_t s);
 template <typename T>
 fvgb_status step_T(fvgb_mesh m, const fvgb_tcoef* tc, T* u, double dt, int nsteps,
@@ -376,16 +383,16 @@ void graph_invalidate(fvgb_mesh m);
 int solve_grid_size(fvgb_mesh_s* m);
 cudaError_t launch_barrier_reset(fvgb_mesh_s* m, cudaStream_t s);   // before every cooperative launch
 template <typename T>
-cudaError_t launch_cg(fvgb_mesh_s* m, int bcset, const double* r, double inner_rtol, int maxit,
+cudaError_t launch_cg(fvgb_mesh_s* m, int bcset, const double* r, double inner_rtol, int maxit, double* phi,
                       cudaStream_t s);
 
-// the inner solve of the Poisson refinement loop selected by o->inner (result in
-// work_of<T>(m).cg_x, bookkeeping in parts.out_inner / d_cg_info)
+// the inner solve of the Poisson refinement loop selected by o->inner: phi += the correction
+// (bookkeeping in parts.out_inner / d_cg_info)
 template <typename T>
-cudaError_t launch_inner(fvgb_mesh_s* m, int bcset, const double* r, const fvgb_solve_opts* o,
+cudaError_t launch_inner(fvgb_mesh_s* m, int bcset, const double* r, const fvgb_solve_opts* o, double* phi,
                          cudaStream_t s) {
-  if (o->inner > 0) return launch_amg_inner<T>(m, bcset, r, o->inner, s);
-  return launch_cg<T>(m, bcset, r, o->inner_rtol, o->maxit_inner, s);
+  if (o->inner > 0) return launch_amg_inner<T>(m, bcset, r, o->inner, phi, s);
+  return launch_cg<T>(m, bcset, r, o->inner_rtol, o->maxit_inner, phi, s);
 }
 
 // A whole solve of the refinement loop with the CG inner solve in one cooperative launch, for
@@ -397,7 +404,6 @@ cudaError_t launch_solve_one(fvgb_mesh_s* m, int bcset, const double* b, double*
                              const fvgb_solve_opts* o, bool check_latched, SolveInfoDev* info, double* rel,
                              int* outer, int* inner, cudaStream_t s);
 
-cudaError_t launch_part_sumsq(fvgb_mesh_s* m, const double* v, double* out, cudaStream_t s);
 // per part <r0, r0 - r1>, ||r0 - r1||^2, ||r0||^2, ||r1||^2 into out[k P, (k + 1) P), k = 0..3
 cudaError_t launch_part_dots(fvgb_mesh_s* m, const double* r0, const double* r1, double* out, cudaStream_t s);
 

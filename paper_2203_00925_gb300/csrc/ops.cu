@@ -862,11 +862,30 @@ k_face(int64_t F, int64_t Fi, int64_t N, const int32_t* __restrict__ fL,
         } else {
           q = fma_rn(c1[k], sub_rn(ub[k], ua[k]), q);
         }
-        Ff = fma_rn(-Dcoef, q, Ff);
+        Ff = CONV ? fma_rn(-Dcoef, q, Ff) : q;   // without convection: the Poisson flux q (D = -1)
       }
       flux[f] = Ff;
     }
   }
+}
+
+// Sum over a block of kNormThreads in a fixed order, valid in thread 0: four warps (one per SM
+// sub-partition) take a quarter each.
+constexpr int kNormThreads = 256;
+__device__ __forceinline__ double norm_block_sum(double v, double* sh) {
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  sh[threadIdx.x] = v;
+  __syncthreads();
+  double t = 0.0;
+  if (w < 4) {
+    const double* q = sh + w * (kNormThreads / 4);
+    t = q[l] + q[l + 32];
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+  }
+  __syncthreads();
+  if (w < 4 && l == 0) sh[w] = t;
+  __syncthreads();
+  return (sh[0] + sh[1]) + (sh[2] + sh[3]);
 }
 
 // ---- gather of the face fluxes of every cell (eq. 4) and what follows from it ---------------
@@ -905,6 +924,88 @@ k_update(int64_t N, const int32_t* __restrict__ cell_face, const T* __restrict__
     } else {
       out[i] = -vol[i] * (aux ? aux[i] : T(0)) - acc;   // b = -mu f + mu Lap_h(0; g)
     }
+  }
+}
+
+// The Poisson residual r = b - A x with its sum of squares (k_update<kPoissonResidual> and the
+// norm's pass over r in one): block (sc, j) takes the j-th of ``split`` pieces of sub-chunk sc
+// and leaves its sum in part[sc * split + j]. 6M cells: 106 + 45 us -> see launch_residual_norm.
+template <int NV>
+__global__ void __launch_bounds__(kNormThreads)
+k_residual_norm(int64_t N, const int32_t* __restrict__ cell_face, const double* __restrict__ flux,
+                const double* __restrict__ b, double* __restrict__ r, const int64_t* __restrict__ sc_begin,
+                int split, double* __restrict__ part) {
+  constexpr int U = 2;
+  __shared__ double sh[kNormThreads];
+  const int sc = blockIdx.x / split, j = blockIdx.x % split;
+  const int64_t s0 = sc_begin[sc], n = sc_begin[sc + 1] - s0;
+  const int64_t lo = s0 + n * j / split, hi = s0 + n * (j + 1) / split;
+  double sum = 0.0;
+  for (int64_t i0 = lo + threadIdx.x; i0 < hi; i0 += U * kNormThreads) {
+    int32_t e[U][NV];
+    double bb[U], f[U][NV];
+#pragma unroll
+    for (int q = 0; q < U; ++q) {
+      const int64_t i = i0 + q * kNormThreads;
+      if (i < hi) {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) e[q][k] = __ldg(cell_face + k * N + i);
+        bb[q] = b[i];
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < U; ++q)
+      if (i0 + q * kNormThreads < hi) {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) f[q][k] = __ldg(flux + (e[q][k] >= 0 ? e[q][k] : ~e[q][k]));
+      }
+#pragma unroll
+    for (int q = 0; q < U; ++q) {
+      const int64_t i = i0 + q * kNormThreads;
+      if (i < hi) {
+        double acc = 0.0;
+#pragma unroll
+        for (int k = 0; k < NV; ++k) acc += e[q][k] >= 0 ? -f[q][k] : f[q][k];
+        const double v = bb[q] - acc;
+        r[i] = v;
+        sum += v * v;
+      }
+    }
+  }
+  sum = norm_block_sum(sum, sh);
+  if (threadIdx.x == 0) part[blockIdx.x] = sum;
+}
+
+// the same sums of a vector
+__global__ void __launch_bounds__(kNormThreads)
+k_norm_partial(const double* __restrict__ v, const int64_t* __restrict__ sc_begin, int split,
+               double* __restrict__ part) {
+  constexpr int U = 8;
+  __shared__ double sh[kNormThreads];
+  const int sc = blockIdx.x / split, j = blockIdx.x % split;
+  const int64_t s0 = sc_begin[sc], n = sc_begin[sc + 1] - s0;
+  const int64_t lo = s0 + n * j / split, hi = s0 + n * (j + 1) / split;
+  double sum = 0.0;
+  for (int64_t i0 = lo + threadIdx.x; i0 < hi; i0 += U * kNormThreads) {
+    double x[U];
+#pragma unroll
+    for (int q = 0; q < U; ++q) x[q] = i0 + q * kNormThreads < hi ? v[i0 + q * kNormThreads] : 0.0;
+#pragma unroll
+    for (int q = 0; q < U; ++q) sum += x[q] * x[q];
+  }
+  sum = norm_block_sum(sum, sh);
+  if (threadIdx.x == 0) part[blockIdx.x] = sum;
+}
+
+// per part the sum of its pieces' sums, in order (a warp a part)
+__global__ void __launch_bounds__(512) k_norm_final(const double* __restrict__ part, const int32_t* __restrict__ part_sc,
+                                                    int split, int n_part, double* __restrict__ out) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  for (int p = warp; p < n_part; p += nw) {
+    double t = 0.0;
+    for (int k = part_sc[p] * split + lane; k < part_sc[p + 1] * split; k += 32) t += part[k];
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+    if (lane == 0) out[p] = t;
   }
 }
 
@@ -1018,12 +1119,6 @@ __global__ void __launch_bounds__(1024) k_sum_final(const double* __restrict__ p
 __global__ void k_axpy_d(const double* __restrict__ x, double a, double* __restrict__ y, int64_t n) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i < n) y[i] += a * x[i];
-}
-
-template <typename T>
-__global__ void k_add_to_double(const T* __restrict__ x, double* __restrict__ y, int64_t n) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i < n) y[i] += (double)x[i];
 }
 
 __global__ void k_convert(const double* __restrict__ x, float* __restrict__ y, int64_t n) {
@@ -1424,10 +1519,25 @@ cudaError_t launch_axpy_d(const double* x, double a, double* y, int64_t n, cudaS
   return cudaGetLastError();
 }
 
-cudaError_t launch_add_to_double(const void* x, bool fp32, double* y, int64_t n, cudaStream_t s) {
-  if (fp32) k_add_to_double<float><<<grid_for(n), kThreads, 0, s>>>((const float*)x, y, n);
-  else k_add_to_double<double><<<grid_for(n), kThreads, 0, s>>>((const double*)x, y, n);
-  count_launch();
+cudaError_t launch_part_sumsq(fvgb_mesh_s* m, const double* v, double* out, cudaStream_t s) {
+  const PartsDev& pd = m->parts;
+  k_norm_partial<<<pd.n_sc * pd.split, kNormThreads, 0, s>>>(v, pd.sc_begin, pd.split, pd.norm_buf);
+  k_norm_final<<<1, 512, 0, s>>>(pd.norm_buf, pd.part_sc, pd.split, pd.n_part, out);
+  count_launch(2);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_residual_norm(fvgb_mesh_s* m, const double* flux, const double* b, double* r, double* out,
+                                 cudaStream_t s) {
+  const TopoDev& t = m->topo;
+  const PartsDev& pd = m->parts;
+  const unsigned g = (unsigned)(pd.n_sc * pd.split);
+  if (t.dim == 3)
+    k_residual_norm<4><<<g, kNormThreads, 0, s>>>(t.N, t.cell_face, flux, b, r, pd.sc_begin, pd.split, pd.norm_buf);
+  else
+    k_residual_norm<3><<<g, kNormThreads, 0, s>>>(t.N, t.cell_face, flux, b, r, pd.sc_begin, pd.split, pd.norm_buf);
+  k_norm_final<<<1, 512, 0, s>>>(pd.norm_buf, pd.part_sc, pd.split, pd.n_part, out);
+  count_launch(2);
   return cudaGetLastError();
 }
 

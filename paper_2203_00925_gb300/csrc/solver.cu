@@ -76,6 +76,7 @@ struct SolveArgs {
   const T* at_scoef;
   const T* at_isd;          // [N] D^-1/2: the CG solves for D^1/2 x from D^-1/2 r
   const double* r_in;       // [N] right-hand side (FP64 outer residual)
+  double* phi;              // the correction is added here
   T* cx;
   T* cr;
   T* cp;
@@ -307,16 +308,14 @@ __device__ __forceinline__ T cg_phase_r(const SolveArgs<T>& a, int64_t lo, int64
 }
 
 // The final pass on rows [lo, hi): the deferred x += alpha p of the part's last phase 1
-// (pending), then back from the scaled unknowns, x = D^-1/2 x, or with phi phi += D^-1/2 x.
+// (pending), then back from the scaled unknowns onto the potential, phi += D^-1/2 x.
 template <typename T>
-__device__ __forceinline__ void cg_phase_x(const SolveArgs<T>& a, int64_t lo, int64_t hi, bool pending, T alpha,
-                                           double* phi) {
-  T* __restrict__ X = a.cx;
+__device__ __forceinline__ void cg_phase_x(const SolveArgs<T>& a, int64_t lo, int64_t hi, bool pending, T alpha) {
+  const T* __restrict__ X = a.cx;
   const T* __restrict__ P = a.cp;
   for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) {
-    const T x = (pending ? X[i] + alpha * P[i] : X[i]) * __ldg(a.at_isd + i);
-    if (phi) phi[i] += (double)x;
-    else X[i] = x;
+    const T x = pending ? X[i] + alpha * P[i] : X[i];
+    a.phi[i] += (double)(x * __ldg(a.at_isd + i));
   }
 }
 
@@ -412,10 +411,10 @@ struct OneShared {
   int ok;
 };
 
-// CG on a single mesh: scalars in shared memory, one exchange per phase. The correction
-// goes to a.cx, or with phi onto phi. Returns false when a wait ran out; its: iterations.
+// CG on a single mesh: scalars in shared memory, one exchange per phase. Returns false when a
+// wait ran out; its: iterations.
 template <typename T, bool kStream>
-__device__ bool cg_one(const SolveArgs<T>& a, OneBlock& k, OneShared<T>& s, bool act, double* phi, int& its) {
+__device__ bool cg_one(const SolveArgs<T>& a, OneBlock& k, OneShared<T>& s, bool act, int& its) {
   const int64_t lo = k.lo, hi = k.hi;
   its = 0;
   double* const buf0 = a.buf;
@@ -456,7 +455,7 @@ __device__ bool cg_one(const SolveArgs<T>& a, OneBlock& k, OneShared<T>& s, bool
     });
     if (its >= a.maxit_inner) break;
   }
-  if (ok) cg_phase_x<T>(a, lo, hi, pending, s.alpha, phi);
+  if (ok) cg_phase_x<T>(a, lo, hi, pending, s.alpha);
   return ok;
 }
 
@@ -570,7 +569,7 @@ __device__ void cg_many(const SolveArgs<T>& a) {
   __syncthreads();
   for (int sc = sc0; sc < sc1; ++sc) {
     const int p = a.sc_part[sc];
-    cg_phase_x<T>(a, a.sc_begin[sc], a.sc_begin[sc + 1], s_pend[p] != 0, s_alpha[p], nullptr);
+    cg_phase_x<T>(a, a.sc_begin[sc], a.sc_begin[sc + 1], s_pend[p] != 0, s_alpha[p]);
   }
   for (int p = threadIdx.x; p < P; p += blockDim.x)
     if (s_cg[p] == 2) s_status = 6;
@@ -595,7 +594,7 @@ __global__ void __launch_bounds__(kCgThreads, kCgBlocksPerSm) k_cg(SolveArgs<T> 
     __shared__ OneShared<T> s;
     OneBlock k = one_block(a);
     int its = 0;
-    const bool ok = cg_one<T, kStream>(a, k, s, a.active[0] != 0, nullptr, its);
+    const bool ok = cg_one<T, kStream>(a, k, s, a.active[0] != 0, its);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
       a.out_inner[0] = its;
       a.out_status[0] = ok && s.state == 2 ? 6 : 0;
@@ -777,7 +776,7 @@ __global__ void __launch_bounds__(kCgThreads, kCgBlocksPerSm) k_solve_one(SolveA
     if (!(rel > g.rtol)) break;
     if (outer >= g.maxit_outer) { out.status = 5; break; }
     int its = 0;
-    ok = cg_one<T, false>(a, k, s, true, g.phi, its);
+    ok = cg_one<T, false>(a, k, s, true, its);
     out.inner += its;
     if (ok && s.state == 2) { out.outer = outer + 1; out.status = 6; break; }
   }
@@ -809,20 +808,7 @@ __global__ void k_barrier_reset(Barrier* bar) {
   if (threadIdx.x == 0) *bar = Barrier{};
 }
 
-// Per-part sum of squares of an FP64 vector over the same sub-chunks (one block per
-// range of the persistent grid): partials per sub-chunk, then one block sums each part's
-// sub-chunks in order.
-__global__ void __launch_bounds__(kCgThreads) k_part_sumsq_partial(const double* __restrict__ v,
-    const int32_t* __restrict__ blk_sc, const int64_t* __restrict__ sc_begin, double* __restrict__ buf) {
-  __shared__ double sh[kCgThreads];
-  for (int sc = blk_sc[blockIdx.x]; sc < blk_sc[blockIdx.x + 1]; ++sc) {
-    double l = 0.0;
-    for (int64_t i = sc_begin[sc] + threadIdx.x; i < sc_begin[sc + 1]; i += blockDim.x) l += v[i] * v[i];
-    l = block_sum(l, sh);
-    if (threadIdx.x == 0) buf[sc] = l;
-  }
-}
-
+// Per part the sum of its sub-chunks' partial sums, in order.
 __global__ void __launch_bounds__(kCgThreads) k_part_sumsq_final(const double* __restrict__ buf,
     const int32_t* __restrict__ part_sc, int n_part, double* __restrict__ out) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
@@ -892,14 +878,6 @@ int solve_grid_size(fvgb_mesh_s* m) {
   return per_sm < 1 ? 0 : per_sm * m->num_sms;
 }
 
-cudaError_t launch_part_sumsq(fvgb_mesh_s* m, const double* v, double* out, cudaStream_t s) {
-  const PartsDev& pd = m->parts;
-  k_part_sumsq_partial<<<m->solve_grid, kCgThreads, 0, s>>>(v, pd.blk_sc, pd.sc_begin, pd.buf);
-  k_part_sumsq_final<<<1, kCgThreads, 0, s>>>(pd.buf, pd.part_sc, pd.n_part, out);
-  count_launch(2);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_part_dots(fvgb_mesh_s* m, const double* r0, const double* r1, double* out, cudaStream_t s) {
   const PartsDev& pd = m->parts;
   k_part_dots_partial<<<m->solve_grid, kCgThreads, 0, s>>>(r0, r1, pd.blk_sc, pd.sc_begin, pd.n_sc, pd.buf);
@@ -911,13 +889,14 @@ cudaError_t launch_part_dots(fvgb_mesh_s* m, const double* r0, const double* r1,
 
 namespace {
 template <typename T>
-SolveArgs<T> solve_args(fvgb_mesh_s* m, int bcset, const double* r, double inner_rtol, int maxit) {
+SolveArgs<T> solve_args(fvgb_mesh_s* m, int bcset, const double* r, double inner_rtol, int maxit, double* phi) {
   GeoDev<T>& g = geo_of<T>(m);
   Work<T>& w = work_of<T>(m);
   SolveArgs<T> a;
   a.N = m->topo.N;
   a.at_nbr = g.bc[bcset].at_nbr; a.at_scoef = g.bc[bcset].at_scoef; a.at_isd = g.bc[bcset].at_isd;
   a.r_in = r;
+  a.phi = phi;
   a.cx = w.cg_x; a.cr = w.cg_r; a.cp = w.cg_p; a.cq = w.cg_q;
   const PartsDev& pd = m->parts;
   a.n_part = pd.n_part; a.n_sc = pd.n_sc;
@@ -936,7 +915,7 @@ SolveArgs<T> solve_args(fvgb_mesh_s* m, int bcset, const double* r, double inner
 template <typename T>
 cudaError_t launch_whole(fvgb_mesh_s* m, int bcset, ResidualArgs& g, const double* r, const fvgb_solve_opts* o,
                          cudaStream_t s) {
-  SolveArgs<T> a = solve_args<T>(m, bcset, r, o->inner_rtol, o->maxit_inner);
+  SolveArgs<T> a = solve_args<T>(m, bcset, r, o->inner_rtol, o->maxit_inner, g.phi);
   cudaError_t e = launch_barrier_reset(m, s);
   if (e != cudaSuccess) return e;
   void* args[] = {&a, &g};
@@ -947,9 +926,9 @@ cudaError_t launch_whole(fvgb_mesh_s* m, int bcset, ResidualArgs& g, const doubl
 }  // namespace
 
 template <typename T>
-cudaError_t launch_cg(fvgb_mesh_s* m, int bcset, const double* r, double inner_rtol, int maxit,
+cudaError_t launch_cg(fvgb_mesh_s* m, int bcset, const double* r, double inner_rtol, int maxit, double* phi,
                       cudaStream_t s) {
-  SolveArgs<T> a = solve_args<T>(m, bcset, r, inner_rtol, maxit);
+  SolveArgs<T> a = solve_args<T>(m, bcset, r, inner_rtol, maxit, phi);
   if (a.n_sc > kCgThreads) return cudaErrorInvalidConfiguration;   // their staging
   cudaError_t e = launch_barrier_reset(m, s);
   if (e != cudaSuccess) return e;
@@ -990,7 +969,7 @@ cudaError_t launch_solve_one(fvgb_mesh_s* m, int bcset, const double* b, double*
   return fp32 ? launch_whole<float>(m, bcset, g, r, o, s) : launch_whole<double>(m, bcset, g, r, o, s);
 }
 
-template cudaError_t launch_cg<double>(fvgb_mesh_s*, int, const double*, double, int, cudaStream_t);
-template cudaError_t launch_cg<float>(fvgb_mesh_s*, int, const double*, double, int, cudaStream_t);
+template cudaError_t launch_cg<double>(fvgb_mesh_s*, int, const double*, double, int, double*, cudaStream_t);
+template cudaError_t launch_cg<float>(fvgb_mesh_s*, int, const double*, double, int, double*, cudaStream_t);
 
 }  // namespace fvgb
