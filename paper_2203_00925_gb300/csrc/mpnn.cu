@@ -72,7 +72,7 @@ struct fvgb_mpnn_s {
   __nv_bfloat16* wbf = nullptr;        // [3][64][128]
   float* wn = nullptr;                 // [N][4] message weights
   double* hcell = nullptr;             // [N] mu^(1/3)
-  __nv_bfloat16* Hb[2] = {};           // [N][64] BF16 hidden states of the inference path
+  __nv_bfloat16* Hb[2][2] = {};        // [N][64] BF16 hidden states of the inference path, per evaluation
   // aggregate hierarchy (multilevel architecture; n_lev = 0: the middle layer runs on the
   // faces): level k (0-based) has lev_n[k] nodes, rows [lev_off[k], + lev_n[k]) of the
   // coarse arrays; the nodes below it are the cells (k = 0) or level k - 1's
@@ -98,16 +98,20 @@ struct fvgb_mpnn_s {
   float* Mc[2][fvgb::kHops] = {};
   float* Zc[2][fvgb::kHops] = {};
   float* dout = nullptr;               // [N]
-  float* dH = nullptr;                 // [N][64]
-  float* dHb = nullptr;                // [N][64]
-  float* G = nullptr;                  // [N][64] message part of dz W
-  float* dC = nullptr;                 // [coarse rows][64] gradients of the level outputs
-  float* cP = nullptr;                 // [lev_n[0]][64] gradient ping-pong of the hops
-  float* cQ = nullptr;
+  float* dH[2] = {};                   // [N][64]
+  float* dHb[2] = {};                  // [N][64]
+  float* G[2] = {};                    // [N][64] message part of dz W
+  float* dC[2] = {};                   // [coarse rows][64] gradients of the level outputs
+  float* cP[2] = {};                   // [lev_n[0]][64] gradient ping-pong of the hops
+  float* cQ[2] = {};
   float* part = nullptr;               // [blocks][params] gradient partials
   double* dpart = nullptr;             // [kGradBlocks] loss partials
   double* dloss = nullptr;             // [1]
   double* hloss = nullptr;             // pinned [1]
+  // the second evaluation runs beside the first: the aggregate levels are some twenty launches
+  // that fill a fraction of the SMs each
+  cudaStream_t side = nullptr;
+  cudaEvent_t fork = nullptr, join = nullptr;
   int step = 0;
   bool train_buffers = false;
   std::vector<void*> allocs;
@@ -994,6 +998,9 @@ cudaError_t nalloc(MpnnNet* n, T** p, size_t count) {
 void net_release(MpnnNet* n) {
   for (void* p : n->allocs) cudaFree(p);
   if (n->hloss) cudaFreeHost(n->hloss);
+  if (n->fork) cudaEventDestroy(n->fork);
+  if (n->join) cudaEventDestroy(n->join);
+  if (n->side) cudaStreamDestroy(n->side);
   delete n;
 }
 
@@ -1008,7 +1015,6 @@ cudaError_t alloc_train(MpnnNet* n) {
   const size_t NH = (size_t)n->N * kHid, CH = (size_t)n->n_coarse * kHid;
   cudaError_t e;
   for (int set = 0; set < 2; ++set) {
-    if (set == 1 && (e = nalloc(n, &n->F[1], (size_t)n->N * 2))) return e;
     if ((e = nalloc(n, &n->Z0[set], NH))) return e;
     for (int l = 0; l < kLayers; l += n->n_lev > 0 ? 2 : 1) {   // the fine layers
       if ((e = nalloc(n, &n->M[set][l], NH))) return e;
@@ -1020,17 +1026,14 @@ cudaError_t alloc_train(MpnnNet* n) {
       if ((e = nalloc(n, &n->Mc[set][j], CH))) return e;
       if ((e = nalloc(n, &n->Zc[set][j], CH))) return e;
     }
-    if (set == 1 && n->n_lev > 0)
-      for (int j = 0; j <= kHops; ++j)
-        if ((e = nalloc(n, &n->Hc[1][j], CH))) return e;
-  }
-  if ((e = nalloc(n, &n->dH, NH))) return e;
-  if ((e = nalloc(n, &n->dHb, NH))) return e;
-  if ((e = nalloc(n, &n->G, NH))) return e;
-  if (n->n_lev > 0) {
-    if ((e = nalloc(n, &n->dC, CH))) return e;
-    if ((e = nalloc(n, &n->cP, (size_t)n->lev_n[0] * kHid))) return e;
-    if ((e = nalloc(n, &n->cQ, (size_t)n->lev_n[0] * kHid))) return e;
+    if ((e = nalloc(n, &n->dH[set], NH))) return e;
+    if ((e = nalloc(n, &n->dHb[set], NH))) return e;
+    if ((e = nalloc(n, &n->G[set], NH))) return e;
+    if (n->n_lev > 0) {
+      if ((e = nalloc(n, &n->dC[set], CH))) return e;
+      if ((e = nalloc(n, &n->cP[set], (size_t)n->lev_n[0] * kHid))) return e;
+      if ((e = nalloc(n, &n->cQ[set], (size_t)n->lev_n[0] * kHid))) return e;
+    }
   }
   if ((e = nalloc(n, &n->dout, n->N))) return e;
   if ((e = nalloc(n, &n->part, (size_t)2 * kGradBlocks * kNParams))) return e;
@@ -1289,53 +1292,75 @@ cudaError_t forward(MpnnNet* n, int set, const double* dq, const double* phi, bo
   return cudaGetLastError();
 }
 
-// One inference evaluation, decoded into pred (mode 0: pred = V s2 N(f); mode 1: pred -=
-// V s2 N(f)). The encoder runs inside layer 0's gathers, the cells' copy back of the
-// hierarchy inside layer 2's, and the decoder in layer 2's epilogue: the cells' hidden
-// states are written once, as BF16 (h1; h2 too for the local architecture).
-cudaError_t forward_infer(MpnnNet* n, const double* dq, const double* phi, bool zero_charge, double* pred,
-                          int mode, cudaStream_t s) {
+// One inference evaluation up to its last layer (set 0: N(f), set 1: N(f0 = 0)). The encoder
+// runs inside layer 0's gathers, the cells' copy back of the hierarchy inside layer 2's, and
+// the decoder in layer 2's epilogue: the cells' hidden states are written once, as BF16 (h1;
+// h2 too for the local architecture).
+void infer_layers(MpnnNet* n, int set, const double* dq, const double* phi, cudaStream_t s) {
   fvgb_mesh m = n->m;
   const int64_t N = n->N;
   constexpr double kEoverEps0 = 1.602176634e-19 / 8.8541878128e-12;
   k_features<<<grid_n(N), 256, 0, s>>>(N, dq, phi, n->hcell, kEoverEps0 / (n->V * n->s0),
-                                       1.0 / (n->V * n->s1), zero_charge ? 1 : 0, n->F[0]);
+                                       1.0 / (n->V * n->s1), set, n->F[set]);
   count_launch();
   const int4* nbr = reinterpret_cast<const int4*>(m->g64.bc[n->bcset].at_nbr);
-  __nv_bfloat16* h1 = n->Hb[0];
   LayerArgs a0;
-  a0.F = n->F[0];
+  a0.F = n->F[set];
   a0.enc = n->theta + kOffWenc;
-  a0.Houtb = h1;
+  a0.Houtb = n->Hb[set][0];
   launch_layer<false, kInEncode>(n, 0, N, a0, nbr, s);
+  if (n->n_lev == 0) {
+    LayerArgs a1;
+    a1.Hb = n->Hb[set][0];
+    a1.Houtb = n->Hb[set][1];
+    launch_layer<false, kInHb>(n, 1, N, a1, nbr, s);
+  } else {
+    levels_forward(n, nullptr, n->Hb[set][0], n->Hc[set], nullptr, nullptr, s);
+  }
+}
+
+// its last layer, decoded into pred (set 0: pred = V s2 N(f); set 1: pred -= V s2 N(f))
+void infer_decode(MpnnNet* n, int set, double* pred, cudaStream_t s) {
+  const int4* nbr = reinterpret_cast<const int4*>(n->m->g64.bc[n->bcset].at_nbr);
   LayerArgs a2;
   a2.dec = n->theta + kOffWdec;
   a2.scale = n->V * n->s2;
-  a2.mode = mode;
+  a2.mode = set;
   a2.pred = pred;
   if (n->n_lev == 0) {
-    LayerArgs a1;
-    a1.Hb = h1;
-    a1.Houtb = n->Hb[1];
-    launch_layer<false, kInHb>(n, 1, N, a1, nbr, s);
-    a2.Hb = n->Hb[1];
-    launch_layer<false, kInHb>(n, 2, N, a2, nbr, s);
+    a2.Hb = n->Hb[set][1];
+    launch_layer<false, kInHb>(n, 2, n->N, a2, nbr, s);
   } else {
-    levels_forward(n, nullptr, h1, n->Hc[0], nullptr, nullptr, s);
-    a2.Hb = h1;
-    a2.U = rows_at(n->Hc[0][kHops], n, 0);
+    a2.Hb = n->Hb[set][0];
+    a2.U = rows_at(n->Hc[set][kHops], n, 0);
     a2.parent = lev_parent(n, 0);
     a2.nparent = reinterpret_cast<const int4*>(n->nparent);
-    launch_layer<false, kInParentB>(n, 2, N, a2, nbr, s);
+    launch_layer<false, kInParentB>(n, 2, n->N, a2, nbr, s);
   }
-  return cudaGetLastError();
+}
+
+// The second evaluation's work on the network's own stream, between two events of s: it is
+// behind what s holds when it forks, and s waits for it when it joins (a capture of s takes
+// both in).
+cudaError_t fork_side(MpnnNet* n, cudaStream_t s) {
+  cudaError_t e = cudaEventRecord(n->fork, s);
+  return e == cudaSuccess ? cudaStreamWaitEvent(n->side, n->fork, 0) : e;
+}
+cudaError_t join_side(MpnnNet* n, cudaStream_t s) {
+  cudaError_t e = cudaEventRecord(n->join, n->side);
+  return e == cudaSuccess ? cudaStreamWaitEvent(s, n->join, 0) : e;
 }
 
 // prediction dphi = V s2 (N(f) - N(f0 = 0))
 cudaError_t predict(MpnnNet* n, const double* dq, const double* phi, double* dphi, cudaStream_t s) {
   cudaError_t e;
-  if ((e = forward_infer(n, dq, phi, false, dphi, 0, s))) return e;
-  return forward_infer(n, dq, phi, true, dphi, 1, s);
+  if ((e = fork_side(n, s))) return e;
+  infer_layers(n, 0, dq, phi, s);
+  infer_layers(n, 1, dq, phi, n->side);
+  infer_decode(n, 0, dphi, s);
+  if ((e = join_side(n, s))) return e;
+  infer_decode(n, 1, dphi, s);
+  return cudaGetLastError();
 }
 
 // backward of sum_i dout_i sign N_set(f)_i through the layers, the hierarchy and the encoder
@@ -1349,52 +1374,52 @@ void backward_set(MpnnNet* n, int set, float sign, int row0, cudaStream_t s) {
   auto layer_back = [&](int l, int64_t rows, const float* dHn, const float* Z, const float* Hin, const float* Min,
                         float* dHo, bool coarse, const int4* nb) {
     k_layer_bwd<<<bwd_grid(rows), kTileThreads, kBwdSmem, s>>>(rows, dHn, Z, Hin, Min, n->wbf + (size_t)l * kHid * kIn,
-                                                               dHo, n->G, part + kOffLayer0 + l * kLayerSize, err);
-    if (coarse) k_msg_add<true><<<grid_n(rows * 32), 256, 0, s>>>(rows, n->G, nb, nullptr, dHo);
-    else k_msg_add<false><<<grid_n(rows * 32), 256, 0, s>>>(rows, n->G, nb, wn, dHo);
+                                                               dHo, n->G[set], part + kOffLayer0 + l * kLayerSize, err);
+    if (coarse) k_msg_add<true><<<grid_n(rows * 32), 256, 0, s>>>(rows, n->G[set], nb, nullptr, dHo);
+    else k_msg_add<false><<<grid_n(rows * 32), 256, 0, s>>>(rows, n->G[set], nb, wn, dHo);
     count_launch(2);
   };
-  k_head_dh<<<grid_n(N * kHid), 256, 0, s>>>(N, n->dout, n->theta, sign, n->dH);
+  k_head_dh<<<grid_n(N * kHid), 256, 0, s>>>(N, n->dout, n->theta, sign, n->dH[set]);
   count_launch();
   // layer 2: d h3 (dH) -> d h2 (dHb)
-  layer_back(2, N, n->dH, n->Z[set][2], n->H[set][2], n->M[set][2], n->dHb, false, nbr);
-  float* X = n->dHb;
+  layer_back(2, N, n->dH[set], n->Z[set][2], n->H[set][2], n->M[set][2], n->dHb[set], false, nbr);
+  float* X = n->dHb[set];
   if (n->n_lev == 0) {
     // local: layer 1, d h2 (dHb) -> d h1 (dH); layer 0, -> d h0 (dHb)
-    layer_back(1, N, X, n->Z[set][1], n->H[set][1], n->M[set][1], n->dH, false, nbr);
-    layer_back(0, N, n->dH, n->Z[set][0], n->H[set][0], n->M[set][0], n->dHb, false, nbr);
-    k_encode_grad<<<kGradBlocks, kRowGroups * kHid, 0, s>>>(N, n->dHb, n->Z0[set], n->F[set], part);
+    layer_back(1, N, X, n->Z[set][1], n->H[set][1], n->M[set][1], n->dH[set], false, nbr);
+    layer_back(0, N, n->dH[set], n->Z[set][0], n->H[set][0], n->M[set][0], n->dHb[set], false, nbr);
+    k_encode_grad<<<kGradBlocks, kRowGroups * kHid, 0, s>>>(N, n->dHb[set], n->Z0[set], n->F[set], part);
     count_launch();
     return;
   }
   // adjoint of the way up: the output of level k receives the sum over its nodes of theirs
   const int L = n->n_lev;
   k_child_sum<float><<<row16_grid(n->lev_n[0]), 256, 0, s>>>(n->lev_n[0], lev_child_ptr(n, 0), lev_child_idx(n, 0), X,
-                                                      nullptr, rows_at(n->dC, n, 0));
+                                                      nullptr, rows_at(n->dC[set], n, 0));
   count_launch();
   for (int k = 1; k < L; ++k) {
     k_child_sum<float><<<row16_grid(n->lev_n[k]), 256, 0, s>>>(n->lev_n[k], lev_child_ptr(n, k), lev_child_idx(n, k),
-                                                        rows_at(n->dC, n, k - 1), nullptr, rows_at(n->dC, n, k));
+                                                        rows_at(n->dC[set], n, k - 1), nullptr, rows_at(n->dC[set], n, k));
     count_launch();
   }
   // adjoint of the way down, coarsest level first: the hops in reverse, then the mean
   for (int k = L - 1; k >= 0; --k) {
     const int64_t nk = n->lev_n[k];
-    const float* cur = rows_at(n->dC, n, k);
+    const float* cur = rows_at(n->dC[set], n, k);
     for (int j = kHops - 1; j >= 0; --j) {
-      float* nxt = (j % 2 == (kHops - 1) % 2) ? n->cP : n->cQ;
+      float* nxt = (j % 2 == (kHops - 1) % 2) ? n->cP[set] : n->cQ[set];
       layer_back(1, nk, cur, rows_at(n->Zc[set][j], n, k), rows_at(n->Hc[set][j], n, k), rows_at(n->Mc[set][j], n, k),
                  nxt, true, lev_nbr(n, k));
       cur = nxt;
     }
-    float* down = k > 0 ? rows_at(n->dC, n, k - 1) : X;
+    float* down = k > 0 ? rows_at(n->dC[set], n, k - 1) : X;
     const int64_t nb = k > 0 ? n->lev_n[k - 1] : N;
     k_add_parent<<<parent_grid(n, nb), 256, 0, s>>>(nb, down, cur, lev_parent(n, k), lev_inv(n, k), down);
     count_launch();
   }
   // layer 0: d h1 (dHb) -> d h0 (dH)
-  layer_back(0, N, X, n->Z[set][0], n->H[set][0], n->M[set][0], n->dH, false, nbr);
-  k_encode_grad<<<kGradBlocks, kRowGroups * kHid, 0, s>>>(N, n->dH, n->Z0[set], n->F[set], part);
+  layer_back(0, N, X, n->Z[set][0], n->H[set][0], n->M[set][0], n->dH[set], false, nbr);
+  k_encode_grad<<<kGradBlocks, kRowGroups * kHid, 0, s>>>(N, n->dH[set], n->Z0[set], n->F[set], part);
   count_launch();
 }
 
@@ -1402,18 +1427,22 @@ void backward_set(MpnnNet* n, int set, float sign, int row0, cudaStream_t s) {
 cudaError_t loss_grad(MpnnNet* n, const double* dq, const double* phi, const double* target, cudaStream_t s) {
   cudaError_t e;
   if ((e = alloc_train(n))) return e;
-  if ((e = forward(n, 0, dq, phi, false, s))) return e;
-  if ((e = forward(n, 1, dq, phi, true, s))) return e;
   const int64_t N = n->N;
   const int G = kGradBlocks;
   if ((e = cudaMemsetAsync(n->part, 0, (size_t)2 * G * kNParams * sizeof(float), s))) return e;
+  if ((e = fork_side(n, s))) return e;
+  if ((e = forward(n, 0, dq, phi, false, s))) return e;
+  if ((e = forward(n, 1, dq, phi, true, n->side))) return e;
+  if ((e = join_side(n, s))) return e;
   k_head_train<<<G, 256, 0, s>>>(N, n->H[0][kLayers], n->H[1][kLayers], n->theta, n->V * n->s2, target,
                                  n->dout, n->dpart);
   k_reduce_loss<<<1, 32, 0, s>>>(G, n->dpart, n->dloss);
   k_decode_grad<<<G, kRowGroups * kHid, 0, s>>>(N, n->H[0][kLayers], n->H[1][kLayers], n->dout, n->part);
   count_launch(3);
+  if ((e = fork_side(n, s))) return e;
   backward_set(n, 0, 1.0f, 0, s);
-  backward_set(n, 1, -1.0f, G, s);
+  backward_set(n, 1, -1.0f, G, n->side);
+  if ((e = join_side(n, s))) return e;
   k_reduce_grad<<<grid_n(kNParams), 256, 0, s>>>(2 * G, n->part, n->grad);
   count_launch();
   return cudaGetLastError();
@@ -1450,10 +1479,15 @@ fvgb_status fvgb_mpnn_create(fvgb_mesh m, int32_t bcset, int32_t multilevel, fvg
   if ((e = nalloc(n, &n->grad, kNParams))) return fail("allocation");
   if ((e = nalloc(n, &n->wbf, (size_t)kLayers * kHid * kIn))) return fail("allocation");
   if ((e = nalloc(n, &n->wn, (size_t)n->N * 4))) return fail("allocation");
-  if ((e = nalloc(n, &n->F[0], (size_t)n->N * 2))) return fail("allocation");
+  for (int set = 0; set < 2; ++set) {
+    if ((e = nalloc(n, &n->F[set], (size_t)n->N * 2))) return fail("allocation");
+    if ((e = nalloc(n, &n->Hb[set][0], NH))) return fail("allocation");
+    if (!multilevel && (e = nalloc(n, &n->Hb[set][1], NH))) return fail("allocation");
+  }
+  if ((e = cudaStreamCreateWithFlags(&n->side, cudaStreamNonBlocking))) return fail("stream create");
+  if ((e = cudaEventCreateWithFlags(&n->fork, cudaEventDisableTiming))) return fail("event create");
+  if ((e = cudaEventCreateWithFlags(&n->join, cudaEventDisableTiming))) return fail("event create");
   if ((e = nalloc(n, &n->hcell, (size_t)n->N))) return fail("allocation");
-  if ((e = nalloc(n, &n->Hb[0], NH))) return fail("allocation");
-  if (!multilevel && (e = nalloc(n, &n->Hb[1], NH))) return fail("allocation");
   k_cell_size<<<grid_n(n->N), 256>>>(n->N, m->g64.vol, n->hcell);
   count_launch();
   if (multilevel) {
@@ -1464,7 +1498,8 @@ fvgb_status fvgb_mpnn_create(fvgb_mesh m, int32_t bcset, int32_t multilevel, fvg
       return fail("aggregate hierarchy");
   }
   for (int j = 0; j <= kHops && n->n_lev > 0; ++j)
-    if ((e = nalloc(n, &n->Hc[0][j], (size_t)n->n_coarse * kHid))) return fail("allocation");
+    for (int set = 0; set < 2; ++set)
+      if ((e = nalloc(n, &n->Hc[set][j], (size_t)n->n_coarse * kHid))) return fail("allocation");
   if (n->n_lev > 0) {
     if ((e = nalloc(n, &n->nparent, (size_t)4 * n->N))) return fail("allocation");
     k_neighbour_parents<<<grid_n(n->N), 256>>>(n->N, reinterpret_cast<const int4*>(m->g64.bc[bcset].at_nbr),
