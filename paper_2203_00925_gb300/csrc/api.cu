@@ -914,9 +914,9 @@ static fvgb_status upload_impl(int32_t dim, int64_t n_vert, const double* xyz, i
   cudaStream_t s = (cudaStream_t)stream;
   fvgb_mesh_s* m = new fvgb_mesh_s();
   m->prec = (fvgb_prec)prec;
-  // default launch shapes (measured on 6M-cell tetrahedral meshes): FP32 face fluxes two
-  // faces per thread in 128-thread blocks; everything else one element per thread
-  if (m->prec != FVGB_FP64) m->tune[kTuneFace] = LaunchShape{128, 2};
+  // default launch shapes (measured on 6M-cell tetrahedral meshes): FP32 face fluxes and
+  // updates two per thread in 128-thread blocks; everything else one element per thread
+  if (m->prec != FVGB_FP64) m->tune[kTuneFace] = m->tune[kTuneUpdate] = LaunchShape{128, 2};
   fvgb_status st = FVGB_OK;
   auto fail = [&](cudaError_t e, const char* what) {
     st = cuda_status(e, what);
@@ -974,6 +974,22 @@ static fvgb_status upload_impl(int32_t dim, int64_t n_vert, const double* xyz, i
       if ((e = dupload(m, &t.tile_fix, fx.tile, s))) return fail(e, "upload");
       if ((e = dupload(m, &t.tile_dsum, fx.dsum, s))) return fail(e, "upload");
       if ((e = prepare_gradient_fixed())) return fail(e, "shared memory limit");
+    }
+    if (tiled && prec != FVGB_FP64) {
+      std::vector<float4> xa(h.N);
+      std::vector<float2> xb(h.N);
+#pragma omp parallel for
+      for (int64_t i = 0; i < h.N; ++i) {
+        float hi[3], lo[3];
+        for (int a = 0; a < 3; ++a) {
+          hi[a] = (float)h.cen[a * h.N + i];
+          lo[a] = (float)(h.cen[a * h.N + i] - (double)hi[a]);
+        }
+        xa[i] = make_float4(hi[0], hi[1], hi[2], lo[0]);
+        xb[i] = make_float2(lo[1], lo[2]);
+      }
+      if ((e = dupload(m, &t.tile_xa, xa, s))) return fail(e, "upload");
+      if ((e = dupload(m, &t.tile_xb, xb, s))) return fail(e, "upload");
     }
     if (tiled) {
       t.tile_max = mx;

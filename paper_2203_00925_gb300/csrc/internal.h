@@ -84,6 +84,9 @@ struct TopoDev {
   int32_t* tile_idx = nullptr;   // halo lists
   int16_t* tile_lidx = nullptr;  // [size of nsell.idx]
   int tile_max = 0;              // longest halo list (0: tiles not built)
+  // FP32 meshes (k_gradient_tiled): centres as high and low parts, {x, y, z, x_lo}, {y_lo, z_lo}
+  float4* tile_xa = nullptr;     // [N]
+  float2* tile_xb = nullptr;     // [N]
   // FP64 meshes (k_gradient_fixed): integer centres, and per tile and cell what its
   // fixed-point sums need (see build_fixed_tiles)
   longlong4_16a* xfix = nullptr; // [N] {x, y, z, 0} in units of 2^-fix_scale

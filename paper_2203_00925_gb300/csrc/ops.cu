@@ -188,7 +188,8 @@ k_gradient(int64_t N, int64_t F, int64_t Fi, const int64_t* __restrict__ sptr,
 __global__ void __launch_bounds__(kGradTile)
 k_gradient_tiled(int64_t N, int64_t F, int64_t Fi, const int64_t* __restrict__ sptr,
                  const int16_t* __restrict__ lidx, const int32_t* __restrict__ tptr,
-                 const int32_t* __restrict__ tidx, const float* __restrict__ rec,
+                 const int32_t* __restrict__ tidx, const float4* __restrict__ xa, const float2* __restrict__ xb,
+                 const float* __restrict__ u,
                  const float* __restrict__ cen, const float* __restrict__ cen_lo, const float* __restrict__ xf,
                  const float* __restrict__ xf_lo, const float* __restrict__ minv,
                  const int32_t* __restrict__ gptr, const int32_t* __restrict__ gface,
@@ -197,12 +198,23 @@ k_gradient_tiled(int64_t N, int64_t F, int64_t Fi, const int64_t* __restrict__ s
   const int64_t tile = blockIdx.x;
   const int64_t r0 = tile * kGradTile;
   const int32_t h0 = tptr[tile], nh = tptr[tile + 1] - h0;
-  const float4* R = reinterpret_cast<const float4*>(rec);
-  const float4 oa = __ldg(R + 2 * r0), ob = __ldg(R + 2 * r0 + 1);   // origin: the first own centre
-  for (int k = threadIdx.x; k < nh; k += blockDim.x) {
-    const int32_t j = __ldg(tidx + h0 + k);
-    const float4 a = __ldg(R + 2 * (int64_t)j), b = __ldg(R + 2 * (int64_t)j + 1);
-    hrec[k] = make_float4(a.x, (a.y - oa.y) + (b.x - ob.x), (a.z - oa.z) + (b.y - ob.y), (a.w - oa.w) + (b.z - ob.z));
+  const float4 oa = __ldg(xa + r0);      // origin: the first own centre
+  const float2 ob = __ldg(xb + r0);
+  constexpr int U = 4;                   // records in flight
+  for (int k0 = threadIdx.x; k0 < nh; k0 += U * kGradTile) {
+    int32_t j[U];
+    float4 a[U];
+    float2 b[U];
+    float v[U];
+#pragma unroll
+    for (int q = 0; q < U; ++q) j[q] = k0 + q * kGradTile < nh ? __ldg(tidx + h0 + k0 + q * kGradTile) : (int32_t)r0;
+#pragma unroll
+    for (int q = 0; q < U; ++q) { a[q] = __ldg(xa + j[q]); b[q] = __ldg(xb + j[q]); v[q] = __ldg(u + j[q]); }
+#pragma unroll
+    for (int q = 0; q < U; ++q)
+      if (k0 + q * kGradTile < nh)
+        hrec[k0 + q * kGradTile] = make_float4(v[q], (a[q].x - oa.x) + (a[q].w - oa.w), (a[q].y - oa.y) + (b[q].x - ob.x),
+                                               (a[q].z - oa.z) + (b[q].y - ob.y));
   }
   __syncthreads();
   const int64_t i = r0 + threadIdx.x;
@@ -666,16 +678,30 @@ k_vertex(int64_t V, const int64_t* __restrict__ sptr, const int32_t* __restrict_
     const T* wcol = alpha + b0 + lane;
     T s = T(0);
     int c = 0;
-    for (; c + 4 <= width; c += 4) {      // four independent gathers in flight
-      const int32_t j0 = __ldg(col + 32 * c), j1 = __ldg(col + 32 * (c + 1)),
-                    j2 = __ldg(col + 32 * (c + 2)), j3 = __ldg(col + 32 * (c + 3));
-      const T w0 = wcol[32 * c], w1 = wcol[32 * (c + 1)], w2 = wcol[32 * (c + 2)],
-              w3 = wcol[32 * (c + 3)];
-      const T u0 = u[j0], u1 = u[j1], u2 = u[j2], u3 = u[j3];
-      s = fma_rn(w0, u0, s);
-      s = fma_rn(w1, u1, s);
-      s = fma_rn(w2, u2, s);
-      s = fma_rn(w3, u3, s);
+    if constexpr (sizeof(T) == 4) {       // FP32: eight independent gathers in flight
+      constexpr int U = 8;
+      for (; c + U <= width; c += U) {
+        int32_t j[U];
+        T w[U], x[U];
+#pragma unroll
+        for (int q = 0; q < U; ++q) { j[q] = __ldg(col + 32 * (c + q)); w[q] = __ldg(wcol + 32 * (c + q)); }
+#pragma unroll
+        for (int q = 0; q < U; ++q) x[q] = u[j[q]];
+#pragma unroll
+        for (int q = 0; q < U; ++q) s = fma_rn(w[q], x[q], s);
+      }
+    } else {
+      for (; c + 4 <= width; c += 4) {      // FP64: four (eight were slower)
+        const int32_t j0 = __ldg(col + 32 * c), j1 = __ldg(col + 32 * (c + 1)),
+                      j2 = __ldg(col + 32 * (c + 2)), j3 = __ldg(col + 32 * (c + 3));
+        const T w0 = wcol[32 * c], w1 = wcol[32 * (c + 1)], w2 = wcol[32 * (c + 2)],
+                w3 = wcol[32 * (c + 3)];
+        const T u0 = u[j0], u1 = u[j1], u2 = u[j2], u3 = u[j3];
+        s = fma_rn(w0, u0, s);
+        s = fma_rn(w1, u1, s);
+        s = fma_rn(w2, u2, s);
+        s = fma_rn(w3, u3, s);
+      }
     }
     for (; c < width; ++c) s = fma_rn(wcol[32 * c], u[__ldg(col + 32 * c)], s);
     const T g = vdir[v];
@@ -889,40 +915,76 @@ __device__ __forceinline__ double norm_block_sum(double v, double* sh) {
 }
 
 // ---- gather of the face fluxes of every cell (eq. 4) and what follows from it ---------------
-template <typename T, int NV, int MODE>
+// One cell, from its gathered fluxes f (already signed: entering minus leaving).
+template <typename T, int MODE>
+__device__ __forceinline__ void update_cell(int64_t i, T acc, const T* __restrict__ inv_vol, const T* __restrict__ vol,
+                                            const T* __restrict__ src, const T* base, T adt,
+                                            const T* __restrict__ aux, T* out, T* out2, int* __restrict__ status) {
+  if constexpr (MODE == kResidual) {
+    const T r = acc * inv_vol[i] + (src ? src[i] : T(0));
+    out[i] = r;
+    if (!isfinite(r)) atomicOr(status, 1);     // latched for fvgb_sync
+  } else if constexpr (MODE == kStep) {
+    const T s = src ? src[i] : T(0);
+    const T r = acc * inv_vol[i] + s;
+    const T v = base[i] + adt * r;
+    out[i] = v;
+    if (out2) {
+      const T w = out2[i] + adt * s;
+      out2[i] = w;
+      if (!isfinite(w)) atomicOr(status, 1);
+    }
+    if (!isfinite(v)) atomicOr(status, 1);
+  } else if constexpr (MODE == kPoissonApply) {
+    out[i] = acc;                       // A x = -mu Lap_h x
+  } else if constexpr (MODE == kPoissonResidual) {
+    out[i] = aux[i] - acc;              // r = b - A x
+  } else {
+    out[i] = -vol[i] * (aux ? aux[i] : T(0)) - acc;   // b = -mu f + mu Lap_h(0; g)
+  }
+}
+
+// Each thread takes K cells (block-contiguous, stride blockDim): the cells' face lists first, then
+// all their fluxes, so that K cells' gathers are in flight together (FP32; an FP64 update waits
+// for the FP64 pipe and takes K = 1). The arithmetic of a cell does not depend on K.
+template <typename T, int NV, int MODE, int K>
 __global__ void __launch_bounds__(1024)
 k_update(int64_t N, const int32_t* __restrict__ cell_face, const T* __restrict__ flux,
          const T* __restrict__ inv_vol, const T* __restrict__ vol, const T* __restrict__ src,
          const T* base, T adt, const T* __restrict__ aux, T* out, T* out2, int* __restrict__ status) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    T acc = T(0);  // sum over faces entering i minus faces leaving i
+  if constexpr (K == 1) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N;
+         i += (int64_t)gridDim.x * blockDim.x) {
+      T acc = T(0);  // sum over faces entering i minus faces leaving i
 #pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      const int32_t e = cell_face[k * N + i];
-      acc += e >= 0 ? -flux[e] : flux[~e];
-    }
-    if constexpr (MODE == kResidual) {
-      const T r = acc * inv_vol[i] + (src ? src[i] : T(0));
-      out[i] = r;
-      if (!isfinite(r)) atomicOr(status, 1);     // latched for fvgb_sync
-    } else if constexpr (MODE == kStep) {
-      const T s = src ? src[i] : T(0);
-      const T r = acc * inv_vol[i] + s;
-      const T v = base[i] + adt * r;
-      out[i] = v;
-      if (out2) {
-        const T w = out2[i] + adt * s;
-        out2[i] = w;
-        if (!isfinite(w)) atomicOr(status, 1);
+      for (int k = 0; k < NV; ++k) {
+        const int32_t e = cell_face[k * N + i];
+        acc += e >= 0 ? -flux[e] : flux[~e];
       }
-      if (!isfinite(v)) atomicOr(status, 1);
-    } else if constexpr (MODE == kPoissonApply) {
-      out[i] = acc;                       // A x = -mu Lap_h x
-    } else if constexpr (MODE == kPoissonResidual) {
-      out[i] = aux[i] - acc;              // r = b - A x
-    } else {
-      out[i] = -vol[i] * (aux ? aux[i] : T(0)) - acc;   // b = -mu f + mu Lap_h(0; g)
+      update_cell<T, MODE>(i, acc, inv_vol, vol, src, base, adt, aux, out, out2, status);
+    }
+  } else {
+    const int64_t per_block = (int64_t)blockDim.x * K;
+    for (int64_t i0 = blockIdx.x * per_block + threadIdx.x; i0 < N; i0 += (int64_t)gridDim.x * per_block) {
+      int32_t e[K][NV];
+      T f[K][NV];
+#pragma unroll
+      for (int q = 0; q < K; ++q)               // in bounds: clamped
+#pragma unroll
+        for (int k = 0; k < NV; ++k) e[q][k] = cell_face[k * N + min(i0 + (int64_t)q * blockDim.x, N - 1)];
+#pragma unroll
+      for (int q = 0; q < K; ++q)
+#pragma unroll
+        for (int k = 0; k < NV; ++k) f[q][k] = flux[e[q][k] >= 0 ? e[q][k] : ~e[q][k]];
+#pragma unroll
+      for (int q = 0; q < K; ++q) {
+        const int64_t i = i0 + (int64_t)q * blockDim.x;
+        if (i >= N) break;
+        T acc = T(0);
+#pragma unroll
+        for (int k = 0; k < NV; ++k) acc += e[q][k] >= 0 ? -f[q][k] : f[q][k];
+        update_cell<T, MODE>(i, acc, inv_vol, vol, src, base, adt, aux, out, out2, status);
+      }
     }
   }
 }
@@ -1181,18 +1243,18 @@ cudaError_t launch_gradient(fvgb_mesh_s* m, int bcset, const T* u, T* grad, cuda
         return cudaGetLastError();
       }
     }
-    k_grad_pack<3><<<gp, kThreads, 0, s>>>(t.N, g.cen, g.cen_lo, u, rec);
     if constexpr (sizeof(T) == 4) {
       if (t.tile_max > 0) {      // FP32: the shared-memory form
         const int64_t ntile = (t.N + kGradTile - 1) / kGradTile;
         k_gradient_tiled<<<(unsigned)ntile, kGradTile, t.tile_max * sizeof(float4), s>>>(
-            t.N, t.F, t.Fi, t.nsell.ptr, t.tile_lidx, t.tile_ptr, t.tile_idx, (const float*)rec,
+            t.N, t.F, t.Fi, t.nsell.ptr, t.tile_lidx, t.tile_ptr, t.tile_idx, t.tile_xa, t.tile_xb, (const float*)u,
             (const float*)g.cen, (const float*)g.cen_lo, (const float*)g.xf, (const float*)g.xf_lo,
             (const float*)b.minv, b.gptr, b.gface, (const float*)b.bval, (float*)grad);
-        count_launch(2);
+        count_launch();
         return cudaGetLastError();
       }
     }
+    k_grad_pack<3><<<gp, kThreads, 0, s>>>(t.N, g.cen, g.cen_lo, u, rec);
     k_gradient<T, 3><<<gg, tg, 0, s>>>(t.N, t.F, t.Fi, t.nsell.ptr, t.nsell.idx, rec, g.cen,
         g.cen_lo, g.xf, g.xf_lo, u, b.minv, b.gptr, b.gface, b.bval, grad);
   } else {
@@ -1319,11 +1381,24 @@ cudaError_t launch_update(fvgb_mesh_s* m, int mode, const T* flux, const T* src,
                           double adt, const T* aux, T* out, T* out2, cudaStream_t s) {
   const TopoDev& t = m->topo;
   GeoDev<T>& g = geo_of<T>(m);
-  const unsigned gr = shape_grid(m, kTuneUpdate, t.N);
+  // FP32 step and residual: K cells per thread from the launch shape (1, 2 or 4 and more); the
+  // other modes one
   const int tb = m->tune[kTuneUpdate].threads;
-#define FVGB_UPD(NV, MD)                                                                 \
-  k_update<T, NV, MD><<<gr, tb, 0, s>>>(t.N, t.cell_face, flux, g.inv_vol, g.vol, src, \
-                                              base, (T)adt, aux, out, out2, m->d_status)
+  const int K = sizeof(T) == 4 && (mode == kResidual || mode == kStep) ? std::min(m->tune[kTuneUpdate].ipt, 4) : 1;
+#define FVGB_UPD_K(NV, MD, KK)                                                              \
+  do {                                                                                      \
+    const unsigned gr_ = (unsigned)std::max<int64_t>(1, (t.N + (int64_t)tb * KK - 1) / ((int64_t)tb * KK)); \
+    k_update<T, NV, MD, KK><<<gr_, tb, 0, s>>>(t.N, t.cell_face, flux, g.inv_vol, g.vol, src, \
+                                               base, (T)adt, aux, out, out2, m->d_status);  \
+  } while (0)
+#define FVGB_UPD(NV, MD)                                                                    \
+  do {                                                                                      \
+    if constexpr (sizeof(T) == 4 && (MD == kResidual || MD == kStep)) {                     \
+      if (K >= 4) { FVGB_UPD_K(NV, MD, 4); break; }                                         \
+      if (K >= 2) { FVGB_UPD_K(NV, MD, 2); break; }                                         \
+    }                                                                                       \
+    FVGB_UPD_K(NV, MD, 1);                                                                  \
+  } while (0)
 #define FVGB_UPD_MODES(NV)                                       \
   switch (mode) {                                                \
     case kResidual: FVGB_UPD(NV, kResidual); break;              \
@@ -1335,6 +1410,7 @@ cudaError_t launch_update(fvgb_mesh_s* m, int mode, const T* flux, const T* src,
   if (t.dim == 3) { FVGB_UPD_MODES(4) } else { FVGB_UPD_MODES(3) }
 #undef FVGB_UPD_MODES
 #undef FVGB_UPD
+#undef FVGB_UPD_K
   count_launch();
   return cudaGetLastError();
 }
