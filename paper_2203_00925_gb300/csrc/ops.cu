@@ -53,6 +53,29 @@ __device__ __forceinline__ double sub_rn(double a, double b) { return __dsub_rn(
 __device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
 
+// Tests on the bits. A comparison in FP64 takes the FP64 pipe as long as an addition (64 cycles
+// a warp), and these are asked of every face or cell.
+__device__ __forceinline__ bool is_finite(float v) { return isfinite(v); }
+__device__ __forceinline__ bool is_finite(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
+// v < 0 (false for -0; a NaN counts by its sign)
+__device__ __forceinline__ bool is_negative(float v) { return v < 0.0f; }
+__device__ __forceinline__ bool is_negative(double v) {
+  const int hi = __double2hiint(v);
+  return hi < 0 && ((hi & 0x7fffffff) | __double2loint(v)) != 0;
+}
+__device__ __forceinline__ bool is_zero(float v) { return v == 0.0f; }
+__device__ __forceinline__ bool is_zero(double v) {
+  return ((__double2hiint(v) & 0x7fffffff) | __double2loint(v)) == 0;
+}
+// a > b for finite values and infinities (order of the bits, sign and magnitude)
+__device__ __forceinline__ bool is_above(float a, float b) { return a > b; }
+__device__ __forceinline__ bool is_above(double a, double b) {
+  long long x = __double_as_longlong(a), y = __double_as_longlong(b);
+  x ^= (long long)((unsigned long long)(x >> 63) >> 1);
+  y ^= (long long)((unsigned long long)(y >> 63) >> 1);
+  return x > y;
+}
+
 // ---- Algorithm "grad": grad u_i = M_i^{-1} sum_j d_ij (u_j - u_i) ------------------------
 // The neighbour loop reads, per neighbour j, one packed 32-byte record (one memory sector)
 // holding u_j and the centre of j, written by k_grad_pack for this call:
@@ -734,18 +757,20 @@ k_bj_limit(int64_t N, int64_t F, int64_t Fi, const int32_t* __restrict__ cell_fa
     fc[k] = f;
     if (f < Fi) {
       const T uj = u[e >= 0 ? fR[f] : fL[f]];
-      umax = fmax(umax, uj);
-      umin = fmin(umin, uj);
+      umax = is_above(uj, umax) ? uj : umax;
+      umin = is_above(umin, uj) ? uj : umin;
     } else if (bkind[f - Fi] == FVGB_BC_DIRICHLET) {
       const T g = bval[f - Fi];
-      umax = fmax(umax, g);
-      umin = fmin(umin, g);
+      umax = is_above(g, umax) ? g : umax;
+      umin = is_above(umin, g) ? g : umin;
     }
   }
   // psi = min(1, min over faces of (bound - u_i) / d_f). The smallest ratio is tracked as
   // a fraction num / den (both >= 0); in FP64 (costly division) the comparison is by
   // cross-multiplication and the winner is divided once.
   T num = T(1), den = T(1);
+  bool one = true;                       // num / den = 1
+  const T above = umax - ui, below = ui - umin;
 #pragma unroll
   for (int k = 0; k <= D; ++k) {
     const int32_t f = fc[k];
@@ -754,17 +779,17 @@ k_bj_limit(int64_t N, int64_t F, int64_t Fi, const int32_t* __restrict__ cell_fa
     if (D == 3)
       d = fma_rn(gi[2], cdiff(xf + 2 * F, xf_lo ? xf_lo + 2 * F : nullptr, f, cen + 2 * N,
                               cen_lo ? cen_lo + 2 * N : nullptr, i), d);
-    if (d != T(0)) {
-      const T a = d > T(0) ? umax - ui : ui - umin;   // >= 0
+    if (!is_zero(d)) {
+      const T a = is_negative(d) ? below : above;        // >= 0
       const T b = fabs(d);
       if constexpr (sizeof(T) == 8) {
-        if (a * den < num * b) { num = a; den = b; }
+        if (is_above(num * b, a * den)) { num = a; den = b; one = false; }
       } else {                                           // FP32: products could overflow
-        if (a / b < num / den) { num = a; den = b; }
+        if (a / b < num / den) { num = a; den = b; one = false; }
       }
     }
   }
-  const T psi = num == T(1) && den == T(1) ? T(1) : num / den;
+  const T psi = one ? T(1) : num / den;
 #pragma unroll
   for (int a = 0; a < D; ++a) grad[a * N + i] = mul_rn(psi, gi[a]);
 }
@@ -807,7 +832,7 @@ k_face(int64_t F, int64_t Fi, int64_t N, const int32_t* __restrict__ fL,
        const T* __restrict__ S, const T* __restrict__ coef, const T* __restrict__ u,
        const T* __restrict__ uv, const T* __restrict__ vel, T vc0, T vc1, T vc2, T Dcoef,
        const int8_t* __restrict__ bkind, const T* __restrict__ bval, int homog,
-       T* __restrict__ flux, Recon rc) {
+       T* __restrict__ flux, Recon rc, int diffuse) {
   constexpr int kInterior = 3;
   const int64_t per_block = (int64_t)blockDim.x * K;
   for (int64_t base = blockIdx.x * per_block + threadIdx.x; base < F;
@@ -838,7 +863,7 @@ k_face(int64_t F, int64_t Fi, int64_t N, const int32_t* __restrict__ fL,
       vC[k] = D == 3 ? fvert[2 * F + f] : 0;
     }
     T uL[K], uR[K], ua[K], ub[K], uc[K], vl[K][3], vr[K][3];
-    const bool diff = Dcoef != T(0);
+    const bool diff = diffuse != 0;
 #pragma unroll
     for (int k = 0; k < K; ++k) {           // gathers
       uL[k] = u[L[k]];
@@ -867,15 +892,22 @@ k_face(int64_t F, int64_t Fi, int64_t N, const int32_t* __restrict__ fL,
         T vf[3];
         if (VFIELD) {
 #pragma unroll
-          for (int a = 0; a < D; ++a) vf[a] = mul_rn(T(0.5), add_rn(vl[k][a], vr[k][a]));
+          for (int a = 0; a < D; ++a) {
+            vf[a] = add_rn(vl[k][a], vr[k][a]);
+            if (sizeof(T) == 4) vf[a] = mul_rn(T(0.5), vf[a]);
+          }
         } else {
           vf[0] = vc0; vf[1] = vc1; vf[2] = vc2;
         }
         T vn = fma_rn(vf[1], s1[k], mul_rn(vf[0], s0[k]));
         if (D == 3) vn = fma_rn(vf[2], s2[k], vn);
-        T up = vn >= T(0) ? ul : ur;
+        // the mean velocity's half: exact on the sum as on each term, and in FP64 one product
+        // instead of three on the pipe that bounds the kernel
+        if (VFIELD && sizeof(T) == 8) vn = mul_rn(T(0.5), vn);
+        const bool from_left = !is_negative(vn);
+        T up = from_left ? ul : ur;
         if (RECON) {
-          if (vn >= T(0)) up = recon_value<T, D>(rc, N, F, f, L[k], ul);
+          if (from_left) up = recon_value<T, D>(rc, N, F, f, L[k], ul);
           else if (kind[k] == kInterior) up = recon_value<T, D>(rc, N, F, f, R[k], ur);
         }
         Ff = mul_rn(vn, up);
@@ -923,7 +955,7 @@ __device__ __forceinline__ void update_cell(int64_t i, T acc, const T* __restric
   if constexpr (MODE == kResidual) {
     const T r = acc * inv_vol[i] + (src ? src[i] : T(0));
     out[i] = r;
-    if (!isfinite(r)) atomicOr(status, 1);     // latched for fvgb_sync
+    if (!is_finite(r)) atomicOr(status, 1);    // latched for fvgb_sync
   } else if constexpr (MODE == kStep) {
     const T s = src ? src[i] : T(0);
     const T r = acc * inv_vol[i] + s;
@@ -932,9 +964,9 @@ __device__ __forceinline__ void update_cell(int64_t i, T acc, const T* __restric
     if (out2) {
       const T w = out2[i] + adt * s;
       out2[i] = w;
-      if (!isfinite(w)) atomicOr(status, 1);
+      if (!is_finite(w)) atomicOr(status, 1);
     }
-    if (!isfinite(v)) atomicOr(status, 1);
+    if (!is_finite(v)) atomicOr(status, 1);
   } else if constexpr (MODE == kPoissonApply) {
     out[i] = acc;                       // A x = -mu Lap_h x
   } else if constexpr (MODE == kPoissonResidual) {
@@ -959,7 +991,8 @@ k_update(int64_t N, const int32_t* __restrict__ cell_face, const T* __restrict__
 #pragma unroll
       for (int k = 0; k < NV; ++k) {
         const int32_t e = cell_face[k * N + i];
-        acc += e >= 0 ? -flux[e] : flux[~e];
+        const T f = e >= 0 ? -flux[e] : flux[~e];
+        acc = k == 0 ? f : acc + f;
       }
       update_cell<T, MODE>(i, acc, inv_vol, vol, src, base, adt, aux, out, out2, status);
     }
@@ -1027,7 +1060,10 @@ k_residual_norm(int64_t N, const int32_t* __restrict__ cell_face, const double* 
       if (i < hi) {
         double acc = 0.0;
 #pragma unroll
-        for (int k = 0; k < NV; ++k) acc += e[q][k] >= 0 ? -f[q][k] : f[q][k];
+        for (int k = 0; k < NV; ++k) {
+          const double x = e[q][k] >= 0 ? -f[q][k] : f[q][k];
+          acc = k == 0 ? x : acc + x;
+        }
         const double v = bb[q] - acc;
         r[i] = v;
         sum += v * v;
@@ -1338,13 +1374,13 @@ cudaError_t launch_face(fvgb_mesh_s* m, int bcset, const T* u, const T* uv, cons
     const unsigned gr_ = face_grid(KK, tb);                                                 \
     k_face<T, DD, CV, VF, KK><<<gr_, tb, 0, s>>>(t.F, t.Fi, t.N, t.fL, t.fR, t.fvert, g.S,  \
                                                  g.coef, u, uv, vel, v0, v1, v2, (T)D,      \
-                                                 b.bkind, b.bval, homog ? 1 : 0, flux, rc); \
+                                                 b.bkind, b.bval, homog ? 1 : 0, flux, rc, D != 0.0 ? 1 : 0); \
   } while (0)
 #define FVGB_FACE_RECON(DD, VF)                                                            \
   do {                                                                                     \
     const unsigned gr_ = face_grid(1, tb);                                                 \
     k_face<T, DD, true, VF, 1, true><<<gr_, tb, 0, s>>>(t.F, t.Fi, t.N, t.fL, t.fR, t.fvert, \
-        g.S, g.coef, u, uv, vel, v0, v1, v2, (T)D, b.bkind, b.bval, homog ? 1 : 0, flux, rc); \
+        g.S, g.coef, u, uv, vel, v0, v1, v2, (T)D, b.bkind, b.bval, homog ? 1 : 0, flux, rc, D != 0.0 ? 1 : 0); \
   } while (0)
 #define FVGB_FACE(DD, CV, VF)                                          \
   do {                                                                 \
