@@ -46,6 +46,7 @@ void build_sell(const std::vector<int32_t>& ptr, const std::vector<int32_t>& idx
     int64_t width = 0;
     for (int64_t r = s * 32; r < std::min(nrows, s * 32 + 32); ++r)
       width = std::max<int64_t>(width, ptr[r + 1] - ptr[r]);
+    if (pad_self) width += width & 1;        // the gradient tiles read two entries at once
     sptr[s + 1] = sptr[s] + width * 32;
   }
   sidx.assign(sptr[ns], 0);
@@ -995,7 +996,14 @@ static fvgb_status upload_impl(int32_t dim, int64_t n_vert, const double* xyz, i
       t.tile_max = mx;
       if ((e = dupload(m, &t.tile_ptr, tptr, s))) return fail(e, "upload");
       if ((e = dupload(m, &t.tile_idx, tidx, s))) return fail(e, "upload");
-      if ((e = dupload(m, &t.tile_lidx, lidx, s))) return fail(e, "upload");
+      // two consecutive entries of a row in one word
+      std::vector<uint32_t> pairs(lidx.size() / 2);
+#pragma omp parallel for
+      for (int64_t sl = 0; sl < (int64_t)sptr.size() - 1; ++sl)
+        for (int64_t q = sptr[sl]; q < sptr[sl + 1]; q += 64)
+          for (int lane = 0; lane < 32; ++lane)
+            pairs[q / 2 + lane] = (uint32_t)(uint16_t)lidx[q + lane] | (uint32_t)(uint16_t)lidx[q + 32 + lane] << 16;
+      if ((e = dupload(m, &t.tile_lidx, pairs, s))) return fail(e, "upload");
     }
   }
   std::vector<double> sw;

@@ -82,7 +82,7 @@ struct TopoDev {
   // sorted) and, aligned with nsell.idx, each entry's position in its tile's list.
   int32_t* tile_ptr = nullptr;   // [n_tile + 1]
   int32_t* tile_idx = nullptr;   // halo lists
-  int16_t* tile_lidx = nullptr;  // [size of nsell.idx]
+  uint32_t* tile_lidx = nullptr; // [half the size of nsell.idx] two consecutive entries of a row a word
   int tile_max = 0;              // longest halo list (0: tiles not built)
   // FP32 meshes (k_gradient_tiled): centres as high and low parts, {x, y, z, x_lo}, {y_lo, z_lo}
   float4* tile_xa = nullptr;     // [N]

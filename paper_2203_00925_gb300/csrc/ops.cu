@@ -210,7 +210,7 @@ k_gradient(int64_t N, int64_t F, int64_t Fi, const int64_t* __restrict__ sptr,
 // position instead of a 32-byte gather from L1/L2. Same sum order as k_gradient.
 __global__ void __launch_bounds__(kGradTile)
 k_gradient_tiled(int64_t N, int64_t F, int64_t Fi, const int64_t* __restrict__ sptr,
-                 const int16_t* __restrict__ lidx, const int32_t* __restrict__ tptr,
+                 const uint32_t* __restrict__ lidx, const int32_t* __restrict__ tptr,
                  const int32_t* __restrict__ tidx, const float4* __restrict__ xa, const float2* __restrict__ xb,
                  const float* __restrict__ u,
                  const float* __restrict__ cen, const float* __restrict__ cen_lo, const float* __restrict__ xf,
@@ -246,28 +246,25 @@ k_gradient_tiled(int64_t N, int64_t F, int64_t Fi, const int64_t* __restrict__ s
   const int lane = (int)(i & 31);
   const int64_t b0 = sptr[sl];
   const int width = (int)((sptr[sl + 1] - b0) >> 5);
-  const int16_t* col = lidx + b0 + lane;
+  const uint32_t* col = lidx + (b0 >> 1) + lane;      // two entries a word, width even
   const float4 me = hrec[threadIdx.x];
   float J[3] = {0.0f, 0.0f, 0.0f};
+  auto add = [&](const float4& n) {
+    const float du = n.x - me.x;
+    J[0] += (n.y - me.y) * du;
+    J[1] += (n.z - me.z) * du;
+    J[2] += (n.w - me.w) * du;
+  };
   int c = 0;
   for (; c + 4 <= width; c += 4) {
-    const float4 n0 = hrec[__ldg(col + 32 * c)], n1 = hrec[__ldg(col + 32 * (c + 1))],
-                 n2 = hrec[__ldg(col + 32 * (c + 2))], n3 = hrec[__ldg(col + 32 * (c + 3))];
-    const float4 nn[4] = {n0, n1, n2, n3};
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const float du = nn[q].x - me.x;
-      J[0] += (nn[q].y - me.y) * du;
-      J[1] += (nn[q].z - me.z) * du;
-      J[2] += (nn[q].w - me.w) * du;
-    }
+    const uint32_t e0 = __ldg(col + 16 * c), e1 = __ldg(col + 16 * c + 32);
+    const float4 n0 = hrec[e0 & 0xffff], n1 = hrec[e0 >> 16], n2 = hrec[e1 & 0xffff], n3 = hrec[e1 >> 16];
+    add(n0); add(n1); add(n2); add(n3);
   }
-  for (; c < width; ++c) {
-    const float4 nq = hrec[__ldg(col + 32 * c)];
-    const float du = nq.x - me.x;
-    J[0] += (nq.y - me.y) * du;
-    J[1] += (nq.z - me.z) * du;
-    J[2] += (nq.w - me.w) * du;
+  if (c < width) {
+    const uint32_t e0 = __ldg(col + 16 * c);
+    const float4 n0 = hrec[e0 & 0xffff], n1 = hrec[e0 >> 16];
+    add(n0); add(n1);
   }
   const float ui = me.x;
   for (int32_t t = gptr[i]; t < gptr[i + 1]; ++t) {
@@ -316,13 +313,13 @@ __device__ __forceinline__ long long to_fixed(long long a, int top, int bits) {
   return a < 0 ? -(long long)mag : (long long)mag;
 }
 
-// round(y v / 2^bits)
-__device__ __forceinline__ long long fixed_mul(long long y, long long v, int bits) {
-  const unsigned long long lo = (unsigned long long)y * (unsigned long long)v;
-  const long long hi = __mul64hi(y, v);
-  const unsigned long long l = lo + (1ull << (bits - 1));
-  const long long h = hi + (l < lo ? 1 : 0);
-  return (long long)(((unsigned long long)h << (64 - bits)) | (l >> bits));
+// floor(y v / 2^bits) as one high product: the operands are shifted up by 64 - bits in all,
+// y here and v by the caller (v_up). The missing half unit of every product is added to the
+// sums (half the number of terms).
+__device__ __forceinline__ int y_up(int bits) { return (64 - bits) / 2; }
+__device__ __forceinline__ int v_up(int bits) { return 64 - bits - y_up(bits); }
+__device__ __forceinline__ long long fixed_mul(long long y, long long v_shifted, int bits) {
+  return __mul64hi((long long)((unsigned long long)y << y_up(bits)), v_shifted);
 }
 
 // v 2^e as FP64, rounded to nearest even (the result is in the normal range), without the
@@ -354,38 +351,41 @@ __device__ __noinline__ void direct_sum(int64_t N, int64_t i, int width, const i
   J[0] = j0; J[1] = j1; J[2] = j2;
 }
 
-// J of one cell from its own integer products: differences of the integer centres shifted to
-// ``bits`` bits, u_j - u_i converted with the exponent top (0: the largest, found first).
-// False where the exponents leave the range.
+// Largest exponent of u_j - u_i over entries [c, end) of a cell's list.
+__device__ __forceinline__ int own_top(int c, int end, double ui, const int32_t* __restrict__ col,
+                                       const double* __restrict__ u) {
+  constexpr int U = 4;                  // neighbours in flight
+  int top = 0;
+  for (; c < end; c += U) {
+    double uj[U];
+#pragma unroll
+    for (int q = 0; q < U; ++q) uj[q] = c + q < end ? u[col[32 * (c + q)]] : ui;
+#pragma unroll
+    for (int q = 0; q < U; ++q) top = max(top, exp_of(__double_as_longlong(uj[q] - ui)));
+  }
+  return top;
+}
+
+// A cell's own integer products over entries [c, end): differences of the integer centres
+// shifted to ``bits`` bits, u_j - u_i converted with the exponent top. (Padding entries, the
+// cell itself, add 0.)
 template <int BITS>
-__device__ __noinline__ bool own_scale_sum(int64_t i, int width, const int32_t* __restrict__ col,
+__device__ __noinline__ void own_scale_sum(int64_t i, int c, int end, double ui, const int32_t* __restrict__ col,
                                            const longlong4_16a* __restrict__ xfix, const double* __restrict__ u,
-                                           int tile_bits, int shift, int scale, int top, double* J) {
+                                           int tile_bits, int shift, int top, long long* s) {
+  constexpr int U = 4;
   const int bits = BITS > 0 ? BITS : tile_bits;
   const longlong2* X = reinterpret_cast<const longlong2*>(xfix);
-  constexpr int U = 4;                  // neighbours in flight
-  const double ui = u[i];
-  if (top == 0) {
-    for (int c0 = 0; c0 < width; c0 += U) {
-      double uj[U];
-#pragma unroll
-      for (int q = 0; q < U; ++q) uj[q] = c0 + q < width ? u[col[32 * (c0 + q)]] : ui;
-#pragma unroll
-      for (int q = 0; q < U; ++q) top = max(top, exp_of(__double_as_longlong(uj[q] - ui)));
-    }
-    if (top == 0) { J[0] = J[1] = J[2] = 0.0; return true; }
-  }
-  if (top < kFixTopMin || top > kFixTopMax) return false;
   const longlong2 xi = X[2 * i];
   const long long zi = X[2 * i + 1].x;
-  long long s[3] = {0, 0, 0};
-  for (int c0 = 0; c0 < width; c0 += U) {
+  long long s0 = 0, s1 = 0, s2 = 0;
+  for (; c < end; c += U) {
     int64_t j[U];
     longlong2 a[U];
     long long az[U];
     double uj[U];
 #pragma unroll
-    for (int q = 0; q < U; ++q) j[q] = c0 + q < width ? col[32 * (c0 + q)] : i;   // the cell itself adds 0
+    for (int q = 0; q < U; ++q) j[q] = c + q < end ? col[32 * (c + q)] : i;
 #pragma unroll
     for (int q = 0; q < U; ++q) {
       a[q] = __ldg(X + 2 * j[q]);
@@ -394,16 +394,14 @@ __device__ __noinline__ bool own_scale_sum(int64_t i, int width, const int32_t* 
     }
 #pragma unroll
     for (int q = 0; q < U; ++q) {
-      const long long v = to_fixed(__double_as_longlong(uj[q] - ui), top, bits);
+      const long long v = (long long)((unsigned long long)to_fixed(__double_as_longlong(uj[q] - ui), top, bits) << v_up(bits));
       const long long d[3] = {a[q].x - xi.x, a[q].y - xi.y, az[q] - zi};
-#pragma unroll
-      for (int k = 0; k < 3; ++k) s[k] += fixed_mul(shift >= 0 ? d[k] >> shift : d[k] << -shift, v, bits);
+      s0 += fixed_mul(shift >= 0 ? d[0] >> shift : d[0] << -shift, v, bits);
+      s1 += fixed_mul(shift >= 0 ? d[1] >> shift : d[1] << -shift, v, bits);
+      s2 += fixed_mul(shift >= 0 ? d[2] >> shift : d[2] << -shift, v, bits);
     }
   }
-  const int e = shift - scale + top - 1022;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) J[k] = from_fixed(s[k], e);
-  return true;
+  s[0] = s0; s[1] = s1; s[2] = s2;
 }
 
 // Two threads a cell, each summing half of its list (the second half's partial sums are
@@ -411,12 +409,12 @@ __device__ __noinline__ bool own_scale_sum(int64_t i, int width, const int32_t* 
 // issue rate, bounds the block. BITS: the tiles' bits where all have the same (0: per tile).
 constexpr int kFixBitsUsual = 55;       // neighbour lists of 64 to 127 cells
 constexpr int kFixThreads = 2 * kGradTile;
-constexpr int kFixBatch = 4;            // halo records in flight per thread
+constexpr int kFixBatch = 2;            // halo records in flight per thread
 
 template <int BITS>
 __global__ void __launch_bounds__(kFixThreads, 4)
 k_gradient_fixed(int64_t N, int64_t F, int64_t Fi, const int64_t* __restrict__ sptr,
-                 const int32_t* __restrict__ sidx, const int16_t* __restrict__ lidx,
+                 const int32_t* __restrict__ sidx, const uint32_t* __restrict__ lidx,
                  const int32_t* __restrict__ tptr, const int32_t* __restrict__ tidx,
                  const GradTileFix* __restrict__ tfix, const longlong4_16a* __restrict__ xfix,
                  const int64_t* __restrict__ dsum, const int16_t* __restrict__ pad, int scale, int max_halo,
@@ -446,7 +444,7 @@ k_gradient_fixed(int64_t N, int64_t F, int64_t Fi, const int64_t* __restrict__ s
   if (bits > 0) {                       // uniform over the block
     const int32_t h0 = tptr[blockIdx.x], nh = tptr[blockIdx.x + 1] - h0;
     const int32_t* halo = tidx + h0;
-    const int16_t* col = lidx + b0 + (i & 31);
+    const uint32_t* col = lidx + (b0 >> 1) + (i & 31);    // two entries a word, width even
     // the halo's differences from the first own cell; largest exponent of those of u
     const longlong2* X = reinterpret_cast<const longlong2*>(xfix);
     const double uo = u[r0];
@@ -493,9 +491,9 @@ k_gradient_fixed(int64_t N, int64_t F, int64_t Fi, const int64_t* __restrict__ s
     } else {
       for (int k = threadIdx.x; k < nh; k += kFixThreads) {   // the entries this thread staged
         const longlong2 a = ra[k], b = rb[k];
-        const long long v = to_fixed(a.x, top, bits);
-        ra[k] = make_longlong2(v, fixed_mul(a.y, v, bits));
-        rb[k] = make_longlong2(fixed_mul(b.x, v, bits), fixed_mul(b.y, v, bits));
+        const long long v = to_fixed(a.x, top, bits), vu = (long long)((unsigned long long)v << v_up(bits));
+        ra[k] = make_longlong2(v, fixed_mul(a.y, vu, bits));
+        rb[k] = make_longlong2(fixed_mul(b.x, vu, bits), fixed_mul(b.y, vu, bits));
       }
       __syncthreads();
       const longlong2 ai = ra[own ? row : 0], bi = rb[own ? row : 0];
@@ -504,29 +502,25 @@ k_gradient_fixed(int64_t N, int64_t F, int64_t Fi, const int64_t* __restrict__ s
       const long long np = own && half == 0 ? pad[i] : 0;
       long long V = -np * vi, Z0 = -np * ai.y, Z1 = -np * bi.x, Z2 = -np * bi.y;
       int least = (int)(vi >> 32), most = least;
-      const int mid = (width + 1) >> 1;
+      const int mid = ((width >> 1) + 1) & ~1;
       int c = half == 0 ? 0 : mid;
       const int end = half == 0 ? mid : width;
-      for (; c + 4 <= end; c += 4) {
-        const int e0 = __ldg(col + 32 * c), e1 = __ldg(col + 32 * (c + 1)), e2 = __ldg(col + 32 * (c + 2)),
-                  e3 = __ldg(col + 32 * (c + 3));
-        const longlong2 a[4] = {ra[e0], ra[e1], ra[e2], ra[e3]};
-        const longlong2 b[4] = {rb[e0], rb[e1], rb[e2], rb[e3]};
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          V += a[q].x; Z0 += a[q].y; Z1 += b[q].x; Z2 += b[q].y;
-          const int hi = (int)(a[q].x >> 32);
-          least = min(least, hi);
-          most = max(most, hi);
-        }
-      }
-      for (; c < end; ++c) {
-        const int e = __ldg(col + 32 * c);
-        const longlong2 a = ra[e], b = rb[e];
+      auto add = [&](const longlong2& a, const longlong2& b) {
         V += a.x; Z0 += a.y; Z1 += b.x; Z2 += b.y;
         const int hi = (int)(a.x >> 32);
         least = min(least, hi);
         most = max(most, hi);
+      };
+      for (; c + 4 <= end; c += 4) {
+        const uint32_t e0 = __ldg(col + 16 * c), e1 = __ldg(col + 16 * c + 32);
+        const longlong2 a0 = ra[e0 & 0xffff], a1 = ra[e0 >> 16], a2 = ra[e1 & 0xffff], a3 = ra[e1 >> 16];
+        const longlong2 b0 = rb[e0 & 0xffff], b1 = rb[e0 >> 16], b2 = rb[e1 & 0xffff], b3 = rb[e1 >> 16];
+        add(a0, b0); add(a1, b1); add(a2, b2); add(a3, b3);
+      }
+      if (c < end) {
+        const uint32_t e0 = __ldg(col + 16 * c);
+        add(ra[e0 & 0xffff], rb[e0 & 0xffff]);
+        add(ra[e0 >> 16], rb[e0 >> 16]);
       }
       if (half == 1) {
         s_sum[0][row] = make_longlong2(V, Z0);
@@ -541,7 +535,8 @@ k_gradient_fixed(int64_t N, int64_t F, int64_t Fi, const int64_t* __restrict__ s
         const int m = max(most, r.y) - min(least, r.x);
         if (m >= 1 << (bits - 33 - 4)) {      // R is at least 2^(bits - 1) units
           todo = 0;
-          const long long Z[3] = {Z0, Z1, Z2};
+          const long long half_units = (width - np) >> 1;     // of the floored products
+          const long long Z[3] = {Z0 + half_units, Z1 + half_units, Z2 + half_units};
 #pragma unroll
           for (int k = 0; k < 3; ++k) {
             const __int128 t = (__int128)yi[k] * V + (__int128)vi * dsum[k * N + i] + ((__int128)1 << (bits - 1));
@@ -555,10 +550,44 @@ k_gradient_fixed(int64_t N, int64_t F, int64_t Fi, const int64_t* __restrict__ s
       }
     }
   }
-  if (!own || half == 1) return;
-  if (todo == 1 && own_scale_sum<BITS>(i, width, gcol, xfix, u, bits, td.own_shift, scale, otop, J)) todo = 0;
-  if (todo != 0) direct_sum(N, i, width, gcol, u, cen, J);
   const double ui = u[i];
+  // cells that sum in their own unit: again both threads, half of the list each
+  if (half == 0) s_range[row] = make_int2(own ? todo : 0, otop);
+  if (__syncthreads_or(half == 0 && own && todo == 1)) {
+    const int2 r = s_range[row];
+    const bool mine = own && r.x == 1;
+    const int mid = (width + 1) >> 1, c0 = half == 0 ? 0 : mid, c1 = half == 0 ? mid : width;
+    int top = r.y;
+    if (mine && top == 0) top = own_top(c0, c1, ui, gcol, u);
+    int* tops = reinterpret_cast<int*>(s_range);
+    __syncthreads();
+    tops[threadIdx.x] = top;
+    __syncthreads();
+    top = max(tops[row], tops[row + kGradTile]);
+    const bool usable = top >= kFixTopMin && top <= kFixTopMax;
+    long long s[3] = {0, 0, 0};
+    if (mine && usable) own_scale_sum<BITS>(i, c0, c1, ui, gcol, xfix, u, bits, td.own_shift, top, s);
+    if (half == 1) {
+      s_sum[0][row] = make_longlong2(s[0], s[1]);
+      s_sum[1][row].x = s[2];
+    }
+    __syncthreads();
+    if (half == 0 && mine) {
+      if (top == 0) {
+        todo = 0;                       // every difference is zero
+      } else if (usable) {
+        todo = 0;
+        const long long half_units = (width - pad[i]) >> 1;
+        const long long t[3] = {s_sum[0][row].x, s_sum[0][row].y, s_sum[1][row].x};
+#pragma unroll
+        for (int k = 0; k < 3; ++k) J[k] = from_fixed(s[k] + t[k] + half_units, td.own_shift - scale + top - 1022);
+      } else {
+        todo = 2;
+      }
+    }
+  }
+  if (!own || half == 1) return;
+  if (todo != 0) direct_sum(N, i, width, gcol, u, cen, J);
   for (int32_t t = gptr[i]; t < gptr[i + 1]; ++t) {
     const int32_t f = gface[t];
     const double du = bval[f - Fi] - ui;
