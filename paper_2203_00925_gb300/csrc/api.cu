@@ -6,6 +6,7 @@
 #include <cmath>
 #include <cstring>
 #include <limits>
+#include <queue>
 #include <string>
 #include <vector>
 
@@ -352,34 +353,44 @@ cudaError_t alloc_work(fvgb_mesh_s* m, Work<T>& w) {
   return cudaSuccess;
 }
 
-// Sub-chunks of the persistent solve: block b owns rows [b N / G, (b+1) N / G), cut at
-// part boundaries; parts are contiguous ranges of internal cells.
-cudaError_t setup_parts(fvgb_mesh_s* m, const std::vector<int64_t>& part_begin, cudaStream_t s) {
+// Sub-chunks of the persistent solve. Blocks are given to the parts one by one, always to the
+// part with the most cells a block, and a part's blocks share its cells equally; a single
+// mesh: block b owns rows [b N / G, (b+1) N / G). With more parts than blocks a block takes
+// whole parts.
+cudaError_t setup_parts(fvgb_mesh_s* m, const std::vector<int64_t>& part_begin, const HostMesh& h, cudaStream_t s) {
   const int64_t N = m->topo.N;
   const int G = m->solve_grid;
   const int P = (int)part_begin.size() - 1;
   m->part_cell_begin = part_begin;
-  std::vector<int32_t> blk_sc(G + 1, 0), sc_part, part_sc(P + 1, 0);
-  std::vector<int64_t> sc_begin;
-  int p = 0;
-  for (int b = 0; b < G; ++b) {
-    blk_sc[b] = (int32_t)sc_part.size();
-    const int64_t lo = (int64_t)b * N / G, hi = (int64_t)(b + 1) * N / G;
-    int64_t i = lo;
-    while (i < hi) {
-      while (part_begin[p + 1] <= i) ++p;
-      sc_begin.push_back(i);
-      sc_part.push_back(p);
-      i = std::min(hi, part_begin[p + 1]);
+  std::vector<int> blocks(P, 1);
+  {
+    std::priority_queue<std::pair<double, int>> most;
+    for (int p = 0; p < P; ++p) most.push({(double)(part_begin[p + 1] - part_begin[p]), -p});
+    for (int left = G - P; left > 0; --left) {
+      const int p = -most.top().second;
+      most.pop();
+      blocks[p] += 1;
+      most.push({(double)(part_begin[p + 1] - part_begin[p]) / blocks[p], -p});
     }
   }
-  blk_sc[G] = (int32_t)sc_part.size();
+  std::vector<int32_t> blk_sc(G + 1, 0), sc_part, part_sc(P + 1, 0), vert_begin(P + 1, 0);
+  std::vector<int64_t> sc_begin;
+  for (int p = 0; p < P; ++p) {
+    const int64_t lo = part_begin[p], n = part_begin[p + 1] - lo;
+    part_sc[p] = (int32_t)sc_part.size();
+    for (int b = 0; b < blocks[p]; ++b) {
+      sc_begin.push_back(lo + (int64_t)b * n / blocks[p]);
+      sc_part.push_back(p);
+    }
+    // vertices are numbered in the order of the cells that touch them first: a part's are one range
+    const int nv = h.dim + 1;
+    vert_begin[p] = *std::min_element(&h.cells[lo * nv], &h.cells[lo * nv] + nv);
+  }
   sc_begin.push_back(N);
   const int n_sc = (int)sc_part.size();
-  for (int q = 0, sc = 0; q <= P; ++q) {
-    while (sc < n_sc && sc_part[sc] < q) ++sc;
-    part_sc[q] = sc;
-  }
+  part_sc[P] = n_sc;
+  vert_begin[P] = (int32_t)h.V;
+  for (int b = 0; b <= G; ++b) blk_sc[b] = (int32_t)((int64_t)b * n_sc / G);
   PartsDev& pd = m->parts;
   pd.n_part = P;
   pd.n_sc = n_sc;
@@ -389,6 +400,14 @@ cudaError_t setup_parts(fvgb_mesh_s* m, const std::vector<int64_t>& part_begin, 
   if ((e = dupload(m, &pd.sc_part, sc_part, s))) return e;
   if ((e = dupload(m, &pd.part_sc, part_sc, s))) return e;
   if ((e = dalloc(m, &pd.buf, 4 * (size_t)n_sc))) return e;
+  if ((e = dupload(m, &pd.vert_begin, vert_begin, s))) return e;
+  if ((e = dalloc(m, &pd.rel, P))) return e;
+  if ((e = dalloc(m, &pd.bn2, P))) return e;
+  if ((e = dalloc(m, &pd.outer, P))) return e;
+  if ((e = dalloc(m, &pd.inner, P))) return e;
+  if ((e = dalloc(m, &pd.stat, P))) return e;
+  if ((e = dalloc(m, &m->barrier, (size_t)P + 1))) return e;
+  if ((e = cudaMemsetAsync(m->barrier, 0, ((size_t)P + 1) * sizeof(Barrier), s))) return e;
   if ((e = dalloc(m, &pd.active, P))) return e;
   if ((e = dalloc(m, &pd.out_inner, P))) return e;
   if ((e = dalloc(m, &pd.norms, P))) return e;
@@ -526,30 +545,45 @@ fvgb_status report_latched(fvgb_mesh m, int latched, cudaStream_t s) {
   return FVGB_ENONFINITE;
 }
 
-// The refinement loop of a single mesh as one launch (solver.cu), with one host
-// synchronisation for its result.
+// The refinement loop as one launch (solver.cu), with one host synchronisation for its result.
 fvgb_status solve_one(fvgb_mesh m, int bcset, const double* b, double* r, double* phi, bool primed,
                       const fvgb_solve_opts* o, fvgb_solve_info* info, cudaStream_t s) {
+  const int P = m->parts.n_part;
+  // pinned staging: the result, then per part rel, outer, inner, whether a learned start was kept
   SolveInfoDev* d = (SolveInfoDev*)(m->h_scal + 8);
-  int* hwarm = (int*)(d + 1);
+  double* hrel = (double*)(d + 1);
+  int* houter = (int*)(hrel + P);
+  int* hinner = houter + P;
+  int* hwarm = hinner + P;
   const bool count_warm = m->warm_check_pending;
   m->warm_check_pending = false;
-  FVGB_TRY(launch_solve_one(m, bcset, b, phi, r, primed, o, true, m->d_solve, nullptr, nullptr, nullptr, s), "solve kernel");
+  const PartsDev& pd = m->parts;
+  FVGB_TRY(launch_solve_one(m, bcset, b, phi, r, primed, o, true, m->d_solve, pd.rel, pd.outer, pd.inner, s), "solve kernel");
   FVGB_TRY(cudaMemcpyAsync(d, m->d_solve, sizeof(SolveInfoDev), cudaMemcpyDeviceToHost, s), "copy");
-  if (count_warm) FVGB_TRY(cudaMemcpyAsync(hwarm, m->warm_used, sizeof(int), cudaMemcpyDeviceToHost, s), "copy");
+  if (P > 1) {
+    FVGB_TRY(cudaMemcpyAsync(hrel, pd.rel, P * sizeof(double), cudaMemcpyDeviceToHost, s), "copy");
+    FVGB_TRY(cudaMemcpyAsync(houter, pd.outer, P * sizeof(int), cudaMemcpyDeviceToHost, s), "copy");
+    FVGB_TRY(cudaMemcpyAsync(hinner, pd.inner, P * sizeof(int), cudaMemcpyDeviceToHost, s), "copy");
+  }
+  if (count_warm) FVGB_TRY(cudaMemcpyAsync(hwarm, m->warm_used, P * sizeof(int), cudaMemcpyDeviceToHost, s), "copy");
   FVGB_TRY(cudaStreamSynchronize(s), "synchronize");
   if (count_warm) {
-    m->stats.learned_starts += 1;
-    m->stats.learned_kept += *hwarm ? 1 : 0;
+    m->stats.learned_starts += P;
+    for (int p = 0; p < P; ++p) m->stats.learned_kept += hwarm[p] ? 1 : 0;
   }
   if (info) *info = fvgb_solve_info{d->outer, d->inner, d->rel, std::sqrt(d->bn2)};
   if (d->latched) {
     if (info) *info = fvgb_solve_info{0, 0, 0.0, 0.0};
     return report_latched(m, d->latched, s);
   }
-  m->last_outer.assign(1, d->outer);
-  m->last_inner.assign(1, d->inner);
-  m->last_rel.assign(1, d->rel);
+  if (P == 1) {
+    hrel[0] = d->rel;
+    houter[0] = d->outer;
+    hinner[0] = d->inner;
+  }
+  m->last_outer.assign(houter, houter + P);
+  m->last_inner.assign(hinner, hinner + P);
+  m->last_rel.assign(hrel, hrel + P);
   m->stats.outer_its += d->outer;
   m->stats.cg_launches += d->outer;
   m->stats.cg_iterations += d->inner;
@@ -1022,10 +1056,6 @@ static fvgb_status upload_impl(int32_t dim, int64_t n_vert, const double* xyz, i
   if ((e = dalloc(m, &m->dphi_tmp2, h.N))) return fail(e, "allocation");
   if ((e = dalloc(m, &m->dzero, h.N))) return fail(e, "allocation");
   if ((e = cudaMemsetAsync(m->dzero, 0, h.N * sizeof(double), s))) return fail(e, "memset");
-  if ((e = dalloc(m, &m->barrier, 1))) return fail(e, "allocation");
-  // zeroed here: solves whose inner solve is not the CG (which resets it per launch) still
-  // read its status word
-  if ((e = cudaMemsetAsync(m->barrier, 0, sizeof(Barrier), s))) return fail(e, "memset");
   if ((e = dalloc(m, &m->d_cg_info, 4))) return fail(e, "allocation");
   if ((e = cudaMemsetAsync(m->d_cg_info, 0, 4 * sizeof(int), s))) return fail(e, "memset");
   if ((e = dalloc(m, &m->d_solve, 1))) return fail(e, "allocation");
@@ -1040,7 +1070,7 @@ static fvgb_status upload_impl(int32_t dim, int64_t n_vert, const double* xyz, i
     release(m);
     return FVGB_EUNSUPPORTED;
   }
-  if ((e = setup_parts(m, h.part_cell_begin, s))) return fail(e, "parts setup");
+  if ((e = setup_parts(m, h.part_cell_begin, h, s))) return fail(e, "parts setup");
   if ((e = prepare_small(m))) return fail(e, "step kernel setup");
   if ((e = cudaStreamSynchronize(s))) return fail(e, "synchronize");
   *out = m;

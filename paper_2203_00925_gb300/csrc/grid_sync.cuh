@@ -30,17 +30,19 @@ __device__ __forceinline__ unsigned count_acquire(const Barrier* bar) {
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&bar->count) : "memory");
   return v;
 }
-// False when the wait ran out, here or (status word) in another block; a whole warp calls.
-__device__ __forceinline__ bool grid_wait(Barrier* bar, unsigned target, unsigned long long limit_ns) {
+// False when the wait ran out, here or (status, the launch's common word) in another block; a
+// whole warp calls.
+__device__ __forceinline__ bool grid_wait(const Barrier* bar, int* status, unsigned target,
+                                          unsigned long long limit_ns) {
   if ((int)(count_acquire(bar) - target) >= 0) return true;
   const unsigned long long t0 = global_ns();
   for (int spin = 1;; ++spin) {
     if ((int)(count_acquire(bar) - target) >= 0) return true;
     if ((spin & 15) != 0) continue;
-    bool late = *(volatile int*)&bar->status != 0;
+    bool late = *(volatile int*)status != 0;
     if (!late && global_ns() - t0 > limit_ns) {
       late = true;
-      if ((threadIdx.x & 31) == 0) atomicExch(&bar->status, 1);
+      if ((threadIdx.x & 31) == 0) atomicExch(status, 1);
     }
     if (__any_sync(0xffffffffu, late)) return false;
   }

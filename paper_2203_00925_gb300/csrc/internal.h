@@ -120,8 +120,8 @@ struct Work {
 };
 
 // Parts of a mesh (an ensemble of independent meshes packed into one index space) and
-// the sub-chunks of the persistent solve: block b owns rows [b N / G, (b+1) N / G) cut at
-// part boundaries.
+// the sub-chunks of the persistent solve: every block owns one, an equal piece of one part
+// (with more parts than blocks: whole parts in turn).
 struct PartsDev {
   int n_part = 1;
   int n_sc = 0;
@@ -129,7 +129,14 @@ struct PartsDev {
   int64_t* sc_begin = nullptr;  // [n_sc+1] first row of each sub-chunk
   int32_t* sc_part = nullptr;   // [n_sc] part of each sub-chunk
   int32_t* part_sc = nullptr;   // [P+1] first sub-chunk of each part
+  int32_t* vert_begin = nullptr;  // [P+1] vertices of each part
   double* buf = nullptr;        // [4][n_sc] partial sums
+  // per-part results of a solve in one launch
+  double* rel = nullptr;
+  double* bn2 = nullptr;
+  int* outer = nullptr;
+  int* inner = nullptr;
+  int* stat = nullptr;
   int* active = nullptr;        // [P] parts the inner solve works on
   int* out_inner = nullptr;     // [P] inner iterations of the last CG launch
   double* norms = nullptr;      // [P] per-part sums of squares
@@ -139,11 +146,11 @@ struct PartsDev {
 
 struct Barrier {
   unsigned int count = 0;  // arrivals since the launch (zeroed before every launch)
-  int status = 0;          // 0 ok, 1 timeout
-  int pad[2] = {0, 0};
+  int status = 0;          // of the whole launch (first barrier): 0 ok, 1 timeout
+  int pad[30] = {};        // a line of its own
 };
 
-// Result of a whole solve run on the device (single mesh).
+// Result of a whole solve run on the device.
 struct SolveInfoDev {
   int outer;      // outer steps (max over parts)
   int inner;      // inner CG iterations (max over parts)
@@ -182,7 +189,7 @@ struct fvgb_mesh_s {
   double* dphi_tmp = nullptr;           // [N] FP64 scratch (residual r)
   double* dphi_tmp2 = nullptr;          // [N] FP64 scratch (rhs b)
   double* dzero = nullptr;              // [N] zeros
-  fvgb::Barrier* barrier = nullptr;
+  fvgb::Barrier* barrier = nullptr;     // [P + 1] the launch's, then one per part
   int* d_cg_info = nullptr;             // [4] iterations, status
   fvgb::SolveInfoDev* d_solve = nullptr;  // result of the last solve in one launch
   int* d_status = nullptr;              // latched asynchronous errors, cleared when reported:
@@ -398,9 +405,9 @@ cudaError_t launch_inner(fvgb_mesh_s* m, int bcset, const double* r, const fvgb_
   return launch_cg<T>(m, bcset, r, o->inner_rtol, o->maxit_inner, phi, s);
 }
 
-// A whole solve of the refinement loop with the CG inner solve in one cooperative launch, for
-// a single mesh: from b (and, when primed, the start's residual r) to phi; parts.norms,
-// parts.out_inner and *info are written. rel / outer / inner: optional per-part results.
+// A whole solve of the refinement loop with the CG inner solve in one cooperative launch: from
+// b (and, when primed, the start's residual r) to phi; *info (over all parts) and the per-part
+// rel / outer / inner are written.
 bool solve_one_ok(const fvgb_mesh_s* m, const fvgb_solve_opts* o);
 // check_latched: solve nothing when an earlier error is latched (info->latched then holds it).
 cudaError_t launch_solve_one(fvgb_mesh_s* m, int bcset, const double* b, double* phi, double* r, bool primed,

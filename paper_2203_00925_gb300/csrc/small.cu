@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(kSmallThreads) k_small_steps(SmallArgs<T> a) {
     if (threadIdx.x < 32) {
       if (threadIdx.x == 0) grid_arrive(a.bar);
       __syncwarp();
-      ok = grid_wait(a.bar, target, a.barrier_ns);
+      ok = grid_wait(a.bar, &a.bar->status, target, a.barrier_ns);
     }
     if (!__syncthreads_and(ok)) {             // latched: reported by fvgb_sync
       if (threadIdx.x == 0) atomicOr(a.status, 2);

@@ -50,24 +50,6 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
   return t;
 }
 
-// Block-wide FP64 sum in a fixed order for launches over many parts: a shuffle tree inside
-// each warp, then warp 0 sums the warp totals in warp order. Valid in thread 0. Measured
-// faster than block_sum on the 64-mesh ensemble, whose short inner solves leave most
-// blocks summing finished or tiny sub-chunks; block_sum is faster on a single mesh.
-__device__ __forceinline__ double block_sum_tree(double v, double* sh) {
-  __syncthreads();                      // the previous call's readers are done with sh
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  if (l == 0) sh[w] = v;
-  __syncthreads();
-  double t = 0.0;
-  if (threadIdx.x < 32) {
-    t = l < (int)(blockDim.x >> 5) ? sh[l] : 0.0;
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-  }
-  return t;
-}
-
 template <typename T>
 struct SolveArgs {
   int64_t N;
@@ -89,8 +71,8 @@ struct SolveArgs {
   const int32_t* sc_part;   // [n_sc]
   const int32_t* part_sc;   // [P+1]
   const int* active;        // [P] parts to solve
-  double* buf;              // [2][n_sc] partial sums, used in turn
-  Barrier* bar;
+  double* buf;              // [4][n_sc] partial sums, used in turn
+  Barrier* bar;             // [P + 1]: the launch's status, then the parts' barriers
   double inner_tol2;
   int maxit_inner;
   int* out_inner;           // [P] iterations per part
@@ -99,69 +81,36 @@ struct SolveArgs {
   unsigned long long barrier_ns;  // limit of a barrier wait
 };
 
-// One exchange of a launch over many parts: the grid's barrier behind the blocks' partial
-// sums (buf[sc], written by thread 0 of each block), then the per-part totals (shared memory
-// tot[p]), every part in sub-chunk order. A part of at most kSeqSubChunks sub-chunks is summed
-// by one thread, left to right; a longer one by one warp: lanes stride 32 over its sub-chunks,
-// then a shuffle tree. (A warp-wide FP64 add costs the same whatever its active lanes, so the
-// few adds of the short parts of an ensemble are cheaper in one thread than in a five-level
-// shuffle tree.) False when a wait ran out.
-constexpr int kSeqSubChunks = 8;
 constexpr int kLaneSlots = 5;        // partial sums a lane loads at once (160 blocks)
 
-template <typename T>
-__device__ bool exchange(const SolveArgs<T>& a, const double* buf, unsigned& target, bool arrive, double* tot,
-                         double* stage) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  bool ok = true;
-  target += gridDim.x;
-  if (warp == 0) {
-    if (lane == 0 && arrive) grid_arrive(a.bar);
-    __syncwarp();
-    ok = grid_wait(a.bar, target, a.barrier_ns);
-    if (ok)
-      for (int sc = lane; sc < a.n_sc; sc += 32) stage[sc] = __ldcg(buf + sc);
-  }
-  if (!__syncthreads_and(ok)) return false;
-  for (int p = threadIdx.x; p < a.n_part; p += blockDim.x) {
-    const int s0 = a.part_sc[p], s1 = a.part_sc[p + 1];
-    if (s1 - s0 > kSeqSubChunks) continue;
-    double t = 0.0;
-    for (int sc = s0; sc < s1; ++sc) t += stage[sc];
-    tot[p] = t;
-  }
-  for (int p = warp; p < a.n_part; p += nw) {
-    if (a.part_sc[p + 1] - a.part_sc[p] <= kSeqSubChunks) continue;
-    double t = 0.0;
-    for (int sc = a.part_sc[p] + lane; sc < a.part_sc[p + 1]; sc += 32) t += stage[sc];
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-    if (lane == 0) tot[p] = t;
-  }
-  __syncthreads();
-  return true;
-}
-
-// This block's rows in a single mesh, and its grid barriers.
+// A block's piece of a part, and the barrier of the blocks that share the part. The parts of an
+// ensemble never wait for one another: every part has its own blocks, counter, scalars and
+// stopping tests.
 struct OneBlock {
-  int sc0, sc1;
+  int part, sc, sc0, sc1;              // the part, this piece, the part's pieces
   int64_t lo, hi;
+  Barrier* bar;
+  int* status;
   bool arrive;                         // test hook: false leaves out this block's arrivals
   unsigned target;
 };
 template <typename T>
-__device__ OneBlock one_block(const SolveArgs<T>& a) {
+__device__ OneBlock one_block(const SolveArgs<T>& a, int sc) {
   OneBlock k;
-  k.sc0 = a.blk_sc[blockIdx.x];
-  k.sc1 = a.blk_sc[blockIdx.x + 1];
-  k.lo = a.sc_begin[k.sc0];
-  k.hi = k.sc1 > k.sc0 ? a.sc_begin[k.sc1] : k.lo;
+  k.sc = sc;
+  k.part = a.sc_part[sc];
+  k.sc0 = a.part_sc[k.part];
+  k.sc1 = a.part_sc[k.part + 1];
+  k.lo = a.sc_begin[sc];
+  k.hi = a.sc_begin[sc + 1];
+  k.bar = a.bar + 1 + k.part;
+  k.status = &a.bar->status;
   k.arrive = a.skip_block != (int)blockIdx.x;
   k.target = 0;
   return k;
 }
 
-// The same for a single mesh (at most one sub-chunk a block), with the block's sum before it
-// and the scalars after it: acc of every thread -> block sum (four warps, one per SM
+// One exchange of a part's blocks: acc of every thread -> block sum (four warps, one per SM
 // sub-partition, a quarter each: GB300 issues FP64 adds at a small fraction of the FP32 rate,
 // so the FP64 instructions on the critical path are few and spread) -> buf; warp 0 waits,
 // sums the partials from registers and hands the total to use(total) (every lane of warp 0);
@@ -171,7 +120,7 @@ __device__ __forceinline__ bool exchange_one(const SolveArgs<T>& a, double* buf,
                                              int* s_ok, F use) {
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
   const int quarter = blockDim.x >> 2;
-  k.target += gridDim.x;
+  k.target += k.sc1 - k.sc0;
   sh[threadIdx.x] = acc;
   __syncthreads();                   // and every row of the phase is written before the arrival
   if (w < 4) {
@@ -185,19 +134,19 @@ __device__ __forceinline__ bool exchange_one(const SolveArgs<T>& a, double* buf,
   if (w == 0) {
     if (l == 0) {
       const double* q = sh + blockDim.x;
-      if (k.sc1 > k.sc0) __stcg(buf + k.sc0, (q[0] + q[1]) + (q[2] + q[3]));
-      if (k.arrive) grid_arrive(a.bar);
+      __stcg(buf + k.sc, (q[0] + q[1]) + (q[2] + q[3]));
+      if (k.arrive) grid_arrive(k.bar);
     }
     __syncwarp();
-    const bool ok = grid_wait(a.bar, k.target, a.barrier_ns);
+    const bool ok = grid_wait(k.bar, k.status, k.target, a.barrier_ns);
     double t = 0.0;
     if (ok) {
       double v[kLaneSlots];
 #pragma unroll
-      for (int q = 0; q < kLaneSlots; ++q) v[q] = l + 32 * q < a.n_sc ? __ldcg(buf + l + 32 * q) : 0.0;
+      for (int q = 0; q < kLaneSlots; ++q) v[q] = k.sc0 + l + 32 * q < k.sc1 ? __ldcg(buf + k.sc0 + l + 32 * q) : 0.0;
 #pragma unroll
       for (int q = 0; q < kLaneSlots; ++q) t += v[q];
-      for (int sc = l + 32 * kLaneSlots; sc < a.n_sc; sc += 32) t += __ldcg(buf + sc);
+      for (int sc = k.sc0 + l + 32 * kLaneSlots; sc < k.sc1; sc += 32) t += __ldcg(buf + sc);
       for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
       use(t);
     }
@@ -401,7 +350,7 @@ __device__ __forceinline__ T cg_phase_pq(const SolveArgs<T>& a, int64_t lo, int6
   return acc;
 }
 
-// Shared memory of the single-mesh kernels.
+// Shared memory of the kernels.
 template <typename T>
 struct OneShared {
   double sh[kCgThreads + 4];
@@ -411,7 +360,7 @@ struct OneShared {
   int ok;
 };
 
-// CG on a single mesh: scalars in shared memory, one exchange per phase. Returns false when a
+// CG on one part: scalars in shared memory, one exchange per phase. Returns false when a
 // wait ran out; its: iterations.
 template <typename T, bool kStream>
 __device__ bool cg_one(const SolveArgs<T>& a, OneBlock& k, OneShared<T>& s, bool act, int& its) {
@@ -459,156 +408,32 @@ __device__ bool cg_one(const SolveArgs<T>& a, OneBlock& k, OneShared<T>& s, bool
   return ok;
 }
 
-// Many parts (an ensemble): per-part scalars and stopping tests.
-template <typename T, bool kStream>
-__device__ void cg_many(const SolveArgs<T>& a) {
-  __shared__ double sh[kCgThreads];
-  __shared__ double stage[kCgThreads];
-  __shared__ double tot[kMaxParts];
-  __shared__ double s_rr[kMaxParts], s_rr0[kMaxParts];
-  __shared__ T s_alpha[kMaxParts], s_beta[kMaxParts];
-  __shared__ int s_cg[kMaxParts];      // 0 running, 1 converged, 2 breakdown, 3 idle
-  __shared__ int s_inner[kMaxParts];
-  __shared__ int s_pend[kMaxParts];    // x += alpha p of the part's last phase 1 not yet applied
-  __shared__ int s_flag, s_status;
-  const int P = a.n_part;
-  const int sc0 = a.blk_sc[blockIdx.x], sc1 = a.blk_sc[blockIdx.x + 1];
-  const bool arrive = a.skip_block != (int)blockIdx.x;   // test hook
-  unsigned target = 0;
-  int total_its = 0;
-  if (threadIdx.x == 0) s_status = 0;
-  for (int p = threadIdx.x; p < P; p += blockDim.x) { s_inner[p] = 0; s_pend[p] = 0; }
-
-  // r = D^-1/2 rhs on active parts (0 elsewhere), p = q = x = 0; the first p/q phase
-  // (beta = 0) then gives p = r, q = S r
-  for (int sc = sc0; sc < sc1; ++sc) {
-    const bool act = a.active[a.sc_part[sc]] != 0;
-    T l0 = T(0);
-    for (int64_t i = a.sc_begin[sc] + threadIdx.x; i < a.sc_begin[sc + 1]; i += blockDim.x) {
-      const T ri = act ? (T)(a.r_in[i] * (double)__ldg(a.at_isd + i)) : T(0);
-      a.cr[i] = ri;
-      a.cp[i] = T(0);
-      a.cq[i] = T(0);
-      a.cx[i] = T(0);
-      l0 += ri * ri;
-    }
-    const double t0 = act ? block_sum_tree((double)l0, sh) : 0.0;
-    __syncthreads();                  // the block's rows are written before it arrives
-    if (threadIdx.x == 0) __stcg(a.buf + sc, t0);
-  }
-  if (!exchange<T>(a, a.buf, target, arrive, tot, stage)) goto done;
-  for (int p = threadIdx.x; p < P; p += blockDim.x) s_rr[p] = s_rr0[p] = tot[p];
-  for (int sc = sc0; sc < sc1; ++sc) {
-    const int p = a.sc_part[sc];
-    double t1 = 0.0;
-    if (a.active[p])
-      t1 = block_sum_tree((double)cg_phase_pq<T, kStream>(a, a.sc_begin[sc], a.sc_begin[sc + 1], T(0), T(0)), sh);
-    if (threadIdx.x == 0) __stcg(a.buf + a.n_sc + sc, t1);
-  }
-  if (!exchange<T>(a, a.buf + a.n_sc, target, arrive, tot, stage)) goto done;
-  if (threadIdx.x == 0) s_flag = 0;
-  __syncthreads();
-  for (int p = threadIdx.x; p < P; p += blockDim.x) {
-    const double rr0 = s_rr0[p], pq = tot[p];
-    int st = 3;
-    if (a.active[p]) {
-      if (!(rr0 > 0.0)) st = rr0 == 0.0 ? 3 : 2;
-      else st = (!(pq > 0.0) || !isfinite(pq)) ? 2 : 0;
-    }
-    s_cg[p] = st;
-    s_alpha[p] = st == 0 ? (T)(rr0 / pq) : T(0);
-    if (st == 0) atomicOr(&s_flag, 1);
-  }
-  __syncthreads();
-  for (int its = 0; s_flag != 0 && its < a.maxit_inner; ++its) {
-    double* buf = a.buf;
-    for (int sc = sc0; sc < sc1; ++sc) {
-      const int p = a.sc_part[sc];
-      double t = 0.0;
-      if (s_cg[p] == 0)               // uniform in the block
-        t = block_sum_tree((double)cg_phase_r<T>(a, a.sc_begin[sc], a.sc_begin[sc + 1], s_alpha[p]), sh);
-      if (threadIdx.x == 0) __stcg(buf + sc, t);
-    }
-    if (!exchange<T>(a, buf, target, arrive, tot, stage)) goto done;
-    ++total_its;
-    if (threadIdx.x == 0) s_flag = 0;
-    __syncthreads();
-    for (int p = threadIdx.x; p < P; p += blockDim.x) {
-      if (s_cg[p] != 0) continue;
-      s_pend[p] = 1;
-      s_inner[p] += 1;
-      const double rrn = tot[p];
-      if (!isfinite(rrn)) { s_cg[p] = 2; continue; }
-      if (rrn <= a.inner_tol2 * s_rr0[p]) { s_cg[p] = 1; continue; }
-      s_beta[p] = (T)(rrn / s_rr[p]);
-      s_rr[p] = rrn;
-      atomicOr(&s_flag, 1);
-    }
-    __syncthreads();
-    if (s_flag == 0) break;
-    buf = a.buf + a.n_sc;
-    for (int sc = sc0; sc < sc1; ++sc) {
-      const int p = a.sc_part[sc];
-      double t = 0.0;
-      if (s_cg[p] == 0)               // uniform in the block
-        t = block_sum_tree((double)cg_phase_pq<T, kStream>(a, a.sc_begin[sc], a.sc_begin[sc + 1], s_beta[p], s_alpha[p]), sh);
-      if (threadIdx.x == 0) __stcg(buf + sc, t);
-    }
-    if (!exchange<T>(a, buf, target, arrive, tot, stage)) goto done;
-    for (int p = threadIdx.x; p < P; p += blockDim.x) {
-      if (s_cg[p] != 0) continue;
-      s_pend[p] = 0;                  // phase 2 applied the pending x update
-      const double pq = tot[p];
-      if (!(pq > 0.0) || !isfinite(pq)) { s_cg[p] = 2; continue; }
-      s_alpha[p] = (T)(s_rr[p] / pq);
-    }
-    __syncthreads();
-  }
-  // own rows: the deferred x += alpha p of the parts whose last phase was a phase 1, and
-  // every row back to the unscaled correction
-  __syncthreads();
-  for (int sc = sc0; sc < sc1; ++sc) {
-    const int p = a.sc_part[sc];
-    cg_phase_x<T>(a, a.sc_begin[sc], a.sc_begin[sc + 1], s_pend[p] != 0, s_alpha[p]);
-  }
-  for (int p = threadIdx.x; p < P; p += blockDim.x)
-    if (s_cg[p] == 2) s_status = 6;
-done:
-  __syncthreads();
-  if (blockIdx.x == 0) {
-    for (int p = threadIdx.x; p < P; p += blockDim.x) a.out_inner[p] = s_inner[p];
-    if (threadIdx.x == 0) {
-      a.out_status[0] = s_status;
-      a.out_status[1] = total_its;
-    }
-  }
-}
-
 // One 512-thread block per SM (measured faster than two smaller-register blocks: fewer
-// exchanges and partial sums, more rows in flight per thread).
-template <typename T, bool kMany, bool kStream>
+// arrivals and partial sums, more rows in flight per thread).
+template <typename T, bool kStream>
 __global__ void __launch_bounds__(kCgThreads, kCgBlocksPerSm) k_cg(SolveArgs<T> a) {
-  if constexpr (kMany) {
-    cg_many<T, kStream>(a);
-  } else {
-    __shared__ OneShared<T> s;
-    OneBlock k = one_block(a);
+  __shared__ OneShared<T> s;
+  for (int sc = a.blk_sc[blockIdx.x]; sc < a.blk_sc[blockIdx.x + 1]; ++sc) {
+    OneBlock k = one_block(a, sc);
     int its = 0;
-    const bool ok = cg_one<T, kStream>(a, k, s, a.active[0] != 0, its);
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-      a.out_inner[0] = its;
-      a.out_status[0] = ok && s.state == 2 ? 6 : 0;
-      a.out_status[1] = its;
+    const bool ok = cg_one<T, kStream>(a, k, s, a.active[k.part] != 0, its);
+    if (k.sc == k.sc0 && threadIdx.x == 0) {      // out_status was zeroed with the barriers
+      a.out_inner[k.part] = its;
+      if (ok && s.state == 2) atomicMax(&a.out_status[0], 6);
+      atomicMax(&a.out_status[1], its);
     }
+    __syncthreads();
+    if (!ok) break;
   }
 }
 
-// ---- a whole solve in one launch (single mesh) -----------------------------------------------
+// ---- a whole solve in one launch -----------------------------------------------
 // The refinement loop of api.cu's solve_impl on the device: r = b - A phi on the full diamond
 // operator, its norm, the stopping test, then the CG above with the correction added to phi
 // in its last pass. An outer step as separate launches is six kernels and a host
 // synchronisation around the CG, some 60 us on 10,000 cells against 60 us of CG; here it is
-// three grid barriers. The operator is applied in two passes: vertex values, then per cell its
+// three grid barriers. In an ensemble every part runs its own loop on its own blocks, where
+// the launches' loop ran each inner solve to the slowest part's last iteration. The operator is applied in two passes: vertex values, then per cell its
 // faces' fluxes (each formed from both sides, the operations and their order those of k_face and
 // k_update, so the residual has the same bits).
 struct ResidualArgs {
@@ -630,18 +455,23 @@ struct ResidualArgs {
   int maxit_outer;
   int primed;                          // r holds b - A phi already
   const int* latched;                  // status word to check first, or null
-  SolveInfoDev* info;
-  double* rel;                         // optional per-part results
+  const int32_t* vert_begin;           // [P + 1] vertices of each part
+  SolveInfoDev* info;                  // over all parts
+  double* rel;                         // per part
+  double* bn2;
   int* outer;
   int* inner;
+  int* stat;
 };
 
 // an FP64 value other blocks wrote before the last grid barrier
 __device__ __forceinline__ double load_shared(const double* p) { return load_r(p); }
 
-__device__ __forceinline__ void residual_vertices(const ResidualArgs& g) {
+__device__ __forceinline__ void residual_vertices(const ResidualArgs& g, const OneBlock& k) {
   constexpr int U = 8;
-  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < g.V; v += (int64_t)gridDim.x * blockDim.x) {
+  const int64_t end = g.vert_begin[k.part + 1];
+  for (int64_t v = g.vert_begin[k.part] + (k.sc - k.sc0) * (int64_t)blockDim.x + threadIdx.x; v < end;
+       v += (k.sc1 - k.sc0) * (int64_t)blockDim.x) {
     const int64_t b0 = g.sptr[v >> 5];
     const int width = (int)((g.sptr[(v >> 5) + 1] - b0) >> 5);
     const int32_t* col = g.sidx + b0 + (v & 31);
@@ -716,24 +546,23 @@ __device__ __forceinline__ double residual_rows(const ResidualArgs& g, int64_t l
   return sum;
 }
 
-// grid barrier without sums; false when the wait ran out
+// barrier of the part's blocks without sums; false when the wait ran out
 template <typename T>
 __device__ bool one_barrier(const SolveArgs<T>& a, OneBlock& k) {
   bool ok = true;
-  k.target += gridDim.x;
+  k.target += k.sc1 - k.sc0;
   __syncthreads();
   if (threadIdx.x < 32) {
-    if (threadIdx.x == 0 && k.arrive) grid_arrive(a.bar);
+    if (threadIdx.x == 0 && k.arrive) grid_arrive(k.bar);
     __syncwarp();
-    ok = grid_wait(a.bar, k.target, a.barrier_ns);
+    ok = grid_wait(k.bar, k.status, k.target, a.barrier_ns);
   }
   return __syncthreads_and(ok) != 0;
 }
 
-template <typename T, int D>
-__global__ void __launch_bounds__(kCgThreads, kCgBlocksPerSm) k_solve_one(SolveArgs<T> a, ResidualArgs g) {
-  __shared__ OneShared<T> s;
-  OneBlock k = one_block(a);
+// the refinement loop of one part
+template <typename T, int D, bool kStream>
+__device__ SolveInfoDev solve_part(const SolveArgs<T>& a, const ResidualArgs& g, OneBlock& k, OneShared<T>& s) {
   SolveInfoDev out{0, 0, 0, 0, 0.0, 0.0};
   double* const buf0 = a.buf + 2 * (size_t)a.n_sc;   // the CG uses the first two
   double* const buf1 = buf0 + a.n_sc;
@@ -764,7 +593,7 @@ __global__ void __launch_bounds__(kCgThreads, kCgBlocksPerSm) k_solve_one(SolveA
       for (int64_t i = k.lo + threadIdx.x; i < k.hi; i += blockDim.x) sum += g.r[i] * g.r[i];
     } else {
       if (outer > 0 && !(ok = one_barrier(a, k))) break;      // phi of every block
-      residual_vertices(g);
+      residual_vertices(g, k);
       if (!(ok = one_barrier(a, k))) break;                    // vertex values of every block
       sum = residual_rows<D>(g, k.lo, k.hi);
     }
@@ -776,36 +605,56 @@ __global__ void __launch_bounds__(kCgThreads, kCgBlocksPerSm) k_solve_one(SolveA
     if (!(rel > g.rtol)) break;
     if (outer >= g.maxit_outer) { out.status = 5; break; }
     int its = 0;
-    ok = cg_one<T, false>(a, k, s, true, its);
+    ok = cg_one<T, kStream>(a, k, s, true, its);
     out.inner += its;
     if (ok && s.state == 2) { out.outer = outer + 1; out.status = 6; break; }
   }
   if (!ok) out.status = 7;
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    *g.info = out;
-    a.out_inner[0] = out.inner;
-    if (g.rel) {
-      g.rel[0] = out.rel;
-      g.outer[0] = out.outer;
-      g.inner[0] = out.inner;
+  return out;
+}
+
+template <typename T, int D, bool kStream>
+__global__ void __launch_bounds__(kCgThreads, kCgBlocksPerSm) k_solve(SolveArgs<T> a, ResidualArgs g) {
+  __shared__ OneShared<T> s;
+  for (int sc = a.blk_sc[blockIdx.x]; sc < a.blk_sc[blockIdx.x + 1]; ++sc) {
+    OneBlock k = one_block(a, sc);
+    const SolveInfoDev out = solve_part<T, D, kStream>(a, g, k, s);
+    if (k.sc == k.sc0 && threadIdx.x == 0) {
+      g.rel[k.part] = out.rel;
+      g.bn2[k.part] = out.bn2;
+      g.outer[k.part] = out.outer;
+      g.inner[k.part] = out.inner;
+      g.stat[k.part] = out.status;
+      __threadfence();
+      // the last part to finish sums up over all, in part order
+      if (atomicAdd(&a.bar->count, 1u) == (unsigned)a.n_part - 1) {
+        __threadfence();
+        SolveInfoDev all{0, 0, 0, out.latched, 0.0, 0.0};
+        for (int p = 0; p < a.n_part; ++p) {
+          all.outer = max(all.outer, __ldcg(g.outer + p));
+          all.inner = max(all.inner, __ldcg(g.inner + p));
+          all.status = max(all.status, __ldcg(g.stat + p));
+          all.rel = fmax(all.rel, __ldcg(g.rel + p));
+          all.bn2 += __ldcg(g.bn2 + p);
+        }
+        *g.info = all;
+      }
     }
+    __syncthreads();
   }
 }
 
-// The variant for a mesh of N cells in n_part parts: kStream in FP32 once an iteration's
-// operator and vectors (48 bytes a cell) are beyond L2.
+// kStream in FP32 once an iteration's operator and vectors (48 bytes a cell) are beyond L2.
 template <typename T>
-const void* cg_kernel(int64_t N, int n_part, int64_t l2_bytes) {
-  if constexpr (sizeof(T) == 4) {
-    if (48 * N > l2_bytes)
-      return n_part > 1 ? (const void*)k_cg<T, true, true> : (const void*)k_cg<T, false, true>;
-  }
-  return n_part > 1 ? (const void*)k_cg<T, true, false> : (const void*)k_cg<T, false, false>;
-}
+bool cg_streams(const fvgb_mesh_s* m) { return sizeof(T) == 4 && 48 * m->topo.N > m->l2_bytes; }
 
 // a kernel, not a memset: the same engine as its neighbours in the stream or graph
-__global__ void k_barrier_reset(Barrier* bar) {
-  if (threadIdx.x == 0) *bar = Barrier{};
+__global__ void k_barrier_reset(Barrier* bar, int n, int* cg_info) {
+  for (int p = threadIdx.x; p < n; p += blockDim.x) {
+    bar[p].count = 0;
+    bar[p].status = 0;
+  }
+  if (threadIdx.x < 2) cg_info[threadIdx.x] = 0;
 }
 
 // Per part the sum of its sub-chunks' partial sums, in order.
@@ -853,23 +702,18 @@ __global__ void __launch_bounds__(kCgThreads) k_part_dots_partial(const double* 
 }  // namespace
 
 cudaError_t launch_barrier_reset(fvgb_mesh_s* m, cudaStream_t s) {
-  k_barrier_reset<<<1, 32, 0, s>>>(m->barrier);
+  k_barrier_reset<<<1, 32, 0, s>>>(m->barrier, m->parts.n_part + 1, m->d_cg_info);
   count_launch();
   return cudaGetLastError();
 }
 
 int solve_grid_size(fvgb_mesh_s* m) {
-  const void* kernels[] = {(const void*)k_cg<float, false, false>, (const void*)k_cg<float, true, false>,
-                           (const void*)k_cg<float, false, true>, (const void*)k_cg<float, true, true>,
-                           (const void*)k_cg<double, false, false>, (const void*)k_cg<double, true, false>};
+  const void* kernels[] = {(const void*)k_cg<float, false>, (const void*)k_cg<float, true>,
+                           (const void*)k_cg<double, false>,
+                           (const void*)k_solve<float, 2, false>, (const void*)k_solve<float, 3, false>,
+                           (const void*)k_solve<float, 2, true>, (const void*)k_solve<float, 3, true>,
+                           (const void*)k_solve<double, 2, false>, (const void*)k_solve<double, 3, false>};
   int per_sm = kCgBlocksPerSm;
-  const void* whole[] = {(const void*)k_solve_one<float, 2>, (const void*)k_solve_one<float, 3>,
-                         (const void*)k_solve_one<double, 2>, (const void*)k_solve_one<double, 3>};
-  for (const void* k : whole) {
-    int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, kCgThreads, 0) != cudaSuccess) return 0;
-    per_sm = n < per_sm ? n : per_sm;
-  }
   for (const void* k : kernels) {
     int n = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, kCgThreads, 0) != cudaSuccess) return 0;
@@ -919,7 +763,10 @@ cudaError_t launch_whole(fvgb_mesh_s* m, int bcset, ResidualArgs& g, const doubl
   cudaError_t e = launch_barrier_reset(m, s);
   if (e != cudaSuccess) return e;
   void* args[] = {&a, &g};
-  const void* k = m->topo.dim == 3 ? (const void*)k_solve_one<T, 3> : (const void*)k_solve_one<T, 2>;
+  const void* k = m->topo.dim == 3 ? (const void*)k_solve<T, 3, false> : (const void*)k_solve<T, 2, false>;
+  if constexpr (sizeof(T) == 4) {
+    if (cg_streams<T>(m)) k = m->topo.dim == 3 ? (const void*)k_solve<T, 3, true> : (const void*)k_solve<T, 2, true>;
+  }
   count_launch();
   return cudaLaunchCooperativeKernel(k, dim3(m->solve_grid), dim3(kCgThreads), args, 0, s);
 }
@@ -929,13 +776,15 @@ template <typename T>
 cudaError_t launch_cg(fvgb_mesh_s* m, int bcset, const double* r, double inner_rtol, int maxit, double* phi,
                       cudaStream_t s) {
   SolveArgs<T> a = solve_args<T>(m, bcset, r, inner_rtol, maxit, phi);
-  if (a.n_sc > kCgThreads) return cudaErrorInvalidConfiguration;   // their staging
   cudaError_t e = launch_barrier_reset(m, s);
   if (e != cudaSuccess) return e;
   void* args[] = {&a};
   count_launch();
-  return cudaLaunchCooperativeKernel(cg_kernel<T>(a.N, a.n_part, m->l2_bytes), dim3(m->solve_grid), dim3(kCgThreads),
-                                     args, 0, s);
+  const void* k = (const void*)k_cg<T, false>;
+  if constexpr (sizeof(T) == 4) {
+    if (cg_streams<T>(m)) k = (const void*)k_cg<T, true>;
+  }
+  return cudaLaunchCooperativeKernel(k, dim3(m->solve_grid), dim3(kCgThreads), args, 0, s);
 }
 
 // The whole solve in one launch up to kSolveOneMax cells. A solve to 1e-8 against separate
@@ -945,7 +794,7 @@ cudaError_t launch_cg(fvgb_mesh_s* m, int bcset, const double* r, double inner_r
 constexpr int64_t kSolveOneMax = 600000;
 
 bool solve_one_ok(const fvgb_mesh_s* m, const fvgb_solve_opts* o) {
-  return m->parts.n_part == 1 && o->inner == 0 && !m->time_cg && m->topo.N <= kSolveOneMax;
+  return o->inner == 0 && !m->time_cg && (m->parts.n_part > 1 || m->topo.N <= kSolveOneMax);
 }
 
 cudaError_t launch_solve_one(fvgb_mesh_s* m, int bcset, const double* b, double* phi, double* r, bool primed,
@@ -964,7 +813,9 @@ cudaError_t launch_solve_one(fvgb_mesh_s* m, int bcset, const double* b, double*
   g.primed = primed ? 1 : 0;
   g.latched = check_latched ? m->d_status : nullptr;
   g.info = info;
+  g.vert_begin = m->parts.vert_begin;
   g.rel = rel; g.outer = outer; g.inner = inner;
+  g.bn2 = m->parts.bn2; g.stat = m->parts.stat;
   const bool fp32 = o->prec == FVGB_FP32 || o->prec == FVGB_MIXED;
   return fp32 ? launch_whole<float>(m, bcset, g, r, o, s) : launch_whole<double>(m, bcset, g, r, o, s);
 }
