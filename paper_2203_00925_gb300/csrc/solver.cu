@@ -221,29 +221,36 @@ __host__ __device__ constexpr int unroll_rows() { return sizeof(T) == 4 ? 2 : 1;
 template <typename T>
 __host__ __device__ constexpr int unroll_rows_r() { return sizeof(T) == 4 ? 8 : 4; }
 
+// A thread's rows are lo + threadIdx.x + 512 k in every phase, so its first rows of a phase can
+// be loaded before the exchange that the phase waits for: only neighbours' r come from other
+// blocks.
+
 // CG phase 1 on rows [lo, hi): r -= alpha q; returns the thread's sum of r^2. (The matching
 // x += alpha p is deferred to the next phase 2, which reads p anyway, or to the final pass:
 // the same additions in the same order, without streaming x and p through this phase.)
 template <typename T>
-__device__ __forceinline__ T cg_phase_r(const SolveArgs<T>& a, int64_t lo, int64_t hi, T alpha) {
-  constexpr int U = unroll_rows_r<T>();
-  T* R = a.cr + lo;
-  const T* __restrict__ Q = a.cq + lo;
-  const int n = (int)(hi - lo), bd = blockDim.x;
-  T acc = T(0), r[U], q[U];
-  auto load = [&](int b) {
+struct CgRowsR {
+  static constexpr int U = unroll_rows_r<T>();
+  T r[U], q[U];
+  __device__ __forceinline__ void load(const SolveArgs<T>& a, int64_t lo, int n, int b) {
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int i = b + u * bd;
-      if (i < n) { r[u] = R[i]; q[u] = Q[i]; }
+      const int i = b + u * kCgThreads;
+      if (i < n) { r[u] = a.cr[lo + i]; q[u] = a.cq[lo + i]; }
     }
-  };
-  load(threadIdx.x);
+  }
+};
+template <typename T>
+__device__ __forceinline__ T cg_phase_r(const SolveArgs<T>& a, int64_t lo, int64_t hi, T alpha, CgRowsR<T>& w) {
+  constexpr int U = CgRowsR<T>::U;
+  T* R = a.cr + lo;
+  const int n = (int)(hi - lo), bd = kCgThreads;
+  T acc = T(0);
   for (int b = threadIdx.x; b < n; b += U * bd) {
     T rn[U];
 #pragma unroll
-    for (int u = 0; u < U; ++u) rn[u] = r[u] - alpha * q[u];
-    load(b + U * bd);
+    for (int u = 0; u < U; ++u) rn[u] = w.r[u] - alpha * w.q[u];
+    w.load(a, lo, n, b + U * bd);
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int i = b + u * bd;
@@ -271,41 +278,40 @@ __device__ __forceinline__ void cg_phase_x(const SolveArgs<T>& a, int64_t lo, in
 // CG phase 2 on rows [lo, hi): x += alpha p (the previous phase 1's update, with the old p),
 // p = r + beta p, q = S r + beta q (= S p, S = D^-1/2 A_T D^-1/2 with unit diagonal);
 // returns the thread's sum of p.q.
-template <typename T, int U>
+template <typename T, bool kStream>
 struct CgRows {
+  static constexpr int U = unroll_rows<T>();
   T r[U], p[U], q[U], x[U];
   int4 nb[U];
   Coef4<T> c[U];
+  __device__ __forceinline__ void load(const SolveArgs<T>& a, int64_t lo, int n, int b) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int i = b + u * kCgThreads;
+      if (i < n) {
+        nb[u] = load_op<kStream>(reinterpret_cast<const int4*>(a.at_nbr) + lo + i);
+        c[u].template load<kStream>(a.at_scoef + 4 * lo, i);
+        r[u] = load_r(a.cr + lo + i);
+        p[u] = a.cp[lo + i];
+        q[u] = a.cq[lo + i];
+        x[u] = kStream ? __ldcs(a.cx + lo + i) : a.cx[lo + i];
+      }
+    }
+  }
 };
 
 template <typename T, bool kStream>
-__device__ __forceinline__ T cg_phase_pq(const SolveArgs<T>& a, int64_t lo, int64_t hi, T beta, T alpha) {
-  constexpr int U = unroll_rows<T>();
-  T* __restrict__ P = a.cp + lo;
-  T* __restrict__ Q = a.cq + lo;
-  T* __restrict__ X = a.cx + lo;
+__device__ __forceinline__ T cg_phase_pq(const SolveArgs<T>& a, int64_t lo, int64_t hi, T beta, T alpha,
+                                         CgRows<T, kStream>& w0) {
+  constexpr int U = CgRows<T, kStream>::U;
+  T* P = a.cp + lo;
+  T* Q = a.cq + lo;
+  T* X = a.cx + lo;
   const T* R0 = a.cr;
-  const T* R = a.cr + lo;
-  const int4* __restrict__ NB = reinterpret_cast<const int4*>(a.at_nbr) + lo;
-  const T* __restrict__ C = a.at_scoef + 4 * lo;
-  const int n = (int)(hi - lo), bd = blockDim.x;
+  const int n = (int)(hi - lo), bd = kCgThreads;
   T acc = T(0);
-  auto load = [&](CgRows<T, U>& w, int b) {
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int i = b + u * bd;
-      if (i < n) {
-        w.nb[u] = load_op<kStream>(NB + i);
-        w.c[u].template load<kStream>(C, i);
-        w.r[u] = load_r(R + i);
-        w.p[u] = P[i];
-        w.q[u] = Q[i];
-        w.x[u] = kStream ? __ldcs(X + i) : X[i];
-      }
-    }
-  };
   // rows w of trip b; the next trip's go to nx behind this trip's gathers
-  auto work = [&](const CgRows<T, U>& w, CgRows<T, U>& nx, int b) {
+  auto work = [&](const CgRows<T, kStream>& w, CgRows<T, kStream>& nx, int b) {
     T g[U][4];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
@@ -316,7 +322,7 @@ __device__ __forceinline__ T cg_phase_pq(const SolveArgs<T>& a, int64_t lo, int6
         g[u][3] = load_r(R0 + w.nb[u].w);
       }
     }
-    load(nx, b + U * bd);
+    nx.load(a, lo, n, b + U * bd);
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int i = b + u * bd;
@@ -337,9 +343,8 @@ __device__ __forceinline__ T cg_phase_pq(const SolveArgs<T>& a, int64_t lo, int6
       }
     }
   };
-  CgRows<T, U> w0, w1;
+  CgRows<T, kStream> w1;
   int b = threadIdx.x;
-  load(w0, b);
   while (b < n) {
     work(w0, w1, b);
     b += U * bd;
@@ -371,6 +376,7 @@ __device__ bool cg_one(const SolveArgs<T>& a, OneBlock& k, OneShared<T>& s, bool
   bool pending = false, ok;
   double rr = 0.0, rr0 = 0.0;          // warp 0's
   T acc = T(0);
+  const int n = (int)(hi - lo);
   // r = D^-1/2 rhs, p = q = x = 0; the first p/q phase (beta = 0) then gives p = r, q = S r
   for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) {
     const T ri = act ? (T)(a.r_in[i] * (double)__ldg(a.at_isd + i)) : T(0);
@@ -380,22 +386,27 @@ __device__ bool cg_one(const SolveArgs<T>& a, OneBlock& k, OneShared<T>& s, bool
     a.cx[i] = T(0);
     acc += ri * ri;
   }
+  CgRows<T, kStream> w;
+  CgRowsR<T> wr;
+  w.load(a, lo, n, threadIdx.x);
   ok = exchange_one(a, buf0, k, (double)acc, s.sh, &s.ok, [&](double t) {
     rr = rr0 = t;
     s.state = !act || t == 0.0 ? 3 : (t > 0.0 ? 0 : 2);
     s.alpha = s.beta = T(0);
   });
   while (ok && s.state == 0) {
-    acc = cg_phase_pq<T, kStream>(a, lo, hi, s.beta, s.alpha);
+    acc = cg_phase_pq<T, kStream>(a, lo, hi, s.beta, s.alpha, w);
     pending = false;                   // x += alpha p of the last r phase is applied
+    wr.load(a, lo, n, threadIdx.x);
     ok = exchange_one(a, buf1, k, (double)acc, s.sh, &s.ok, [&](double pq) {
       if (!(pq > 0.0) || !isfinite(pq)) s.state = 2;
       else s.alpha = (T)(rr / pq);
     });
     if (!ok || s.state != 0 || its >= a.maxit_inner) break;
-    acc = cg_phase_r<T>(a, lo, hi, s.alpha);
+    acc = cg_phase_r<T>(a, lo, hi, s.alpha, wr);
     pending = true;
     ++its;
+    w.load(a, lo, n, threadIdx.x);
     ok = exchange_one(a, buf0, k, (double)acc, s.sh, &s.ok, [&](double rrn) {
       if (!isfinite(rrn)) s.state = 2;
       else if (rrn <= a.inner_tol2 * rr0) s.state = 1;
