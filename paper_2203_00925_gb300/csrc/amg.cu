@@ -27,7 +27,7 @@ struct CsrDev {
   int64_t* ptr = nullptr;
   int32_t* idx = nullptr;
   T* val = nullptr;
-  int lanes = 1;            // threads per row: 1, 4, 8 or 32 (from the mean row length)
+  int lanes = 1;            // threads per row (lanes_of)
 };
 
 template <typename T>
@@ -64,25 +64,19 @@ inline unsigned blocks_for(int64_t n, int per_block) {
   return (unsigned)((n + per_block - 1) / per_block);
 }
 
-template <typename T>
-__global__ void k_amg_jacobi0(int64_t n, const T* __restrict__ dinv, const T* __restrict__ b,
-                              T* __restrict__ x, T w) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i < n) x[i] = w * dinv[i] * b[i];
-}
-
-// mode 0: y = M v; 1: y += M v; 2: y = b - M v (residual); 3: y = x + w dinv (b - M x).
+// mode 0: y = M v, and into x0 (if given) the first smoothing step of the level it goes to,
+// x0 = w dinv y (its own launch took 2 to 5 us a level, most of that latency); 1: y += M v; 2: y = b - M v (residual); 3: y = x + w dinv (b - M x).
 // LANES consecutive threads share a row: lane l sums entries l, l + LANES, ..., then a
 // shuffle tree over the group (fixed order).
 template <typename T, int LANES>
 __global__ void __launch_bounds__(kAmgThreads)
 k_amg_csr(int64_t n, const int64_t* __restrict__ ptr, const int32_t* __restrict__ idx,
           const T* __restrict__ val, const T* __restrict__ v, const T* __restrict__ b,
-          const T* __restrict__ dinv, T w, int mode, T* __restrict__ y) {
+          const T* __restrict__ dinv, T w, int mode, T* __restrict__ y, T* __restrict__ x0) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t i = t / LANES;
   const int lane = (int)(t % LANES);
-  const bool valid = i < n;
+  const bool valid = i < n, first = valid && lane == 0;
   T s = T(0);
   if (valid)
     for (int64_t a = ptr[i] + lane; a < ptr[i + 1]; a += LANES) s += val[a] * v[idx[a]];
@@ -91,9 +85,11 @@ k_amg_csr(int64_t n, const int64_t* __restrict__ ptr, const int32_t* __restrict_
 #pragma unroll
     for (int o = LANES / 2; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o, LANES);
   }
-  if (!valid || lane != 0) return;
-  if (mode == 0) y[i] = s;
-  else if (mode == 1) y[i] += s;
+  if (!first) return;
+  if (mode == 0) {
+    y[i] = s;
+    if (x0) x0[i] = w * dinv[i] * s;
+  } else if (mode == 1) y[i] += s;
   else if (mode == 2) y[i] = b[i] - s;
   else y[i] = v[i] + w * dinv[i] * (b[i] - s);
 }
@@ -180,18 +176,34 @@ __global__ void k_amg_info(int P, const int* __restrict__ active, int cycles, in
 }
 
 template <typename T>
-cudaError_t csr_launch(const CsrDev<T>& M, const T* v, const T* b, const T* dinv, T w, int mode, T* y,
+cudaError_t csr_launch(const CsrDev<T>& M, const T* v, const T* b, const T* dinv, T w, int mode, T* y, T* x0,
                        cudaStream_t s) {
   if (M.n == 0) return cudaSuccess;
   const unsigned g = blocks_for(M.n * M.lanes, kAmgThreads);
+  auto go = [&](auto lanes) {
+    k_amg_csr<T, decltype(lanes)::value><<<g, kAmgThreads, 0, s>>>(M.n, M.ptr, M.idx, M.val, v, b, dinv, w, mode, y, x0);
+  };
   switch (M.lanes) {
-    case 32: k_amg_csr<T, 32><<<g, kAmgThreads, 0, s>>>(M.n, M.ptr, M.idx, M.val, v, b, dinv, w, mode, y); break;
-    case 8: k_amg_csr<T, 8><<<g, kAmgThreads, 0, s>>>(M.n, M.ptr, M.idx, M.val, v, b, dinv, w, mode, y); break;
-    case 4: k_amg_csr<T, 4><<<g, kAmgThreads, 0, s>>>(M.n, M.ptr, M.idx, M.val, v, b, dinv, w, mode, y); break;
-    default: k_amg_csr<T, 1><<<g, kAmgThreads, 0, s>>>(M.n, M.ptr, M.idx, M.val, v, b, dinv, w, mode, y); break;
+    case 32: go(std::integral_constant<int, 32>{}); break;
+    case 16: go(std::integral_constant<int, 16>{}); break;
+    case 8: go(std::integral_constant<int, 8>{}); break;
+    case 4: go(std::integral_constant<int, 4>{}); break;
+    case 2: go(std::integral_constant<int, 2>{}); break;
+    default: go(std::integral_constant<int, 1>{}); break;
   }
   count_launch();
   return cudaGetLastError();
+}
+
+// Threads of a row from the matrix's mean row length. A level that fills the chip (some 300,000
+// resident threads) takes the fewest that leave a thread four to ten entries, a smaller one more,
+// since its rows are waited for one after another. The small levels' rule throughout against
+// this one: 6M cells 18.1 -> 17.3 ms a streamer step; the large levels' throughout: 83,000 cells
+// 2.98 ms a solve against 2.65.
+int lanes_of(int64_t rows, double mean) {
+  const int few = mean <= 6.0 ? 1 : mean <= 16.0 ? 2 : mean <= 40.0 ? 4 : mean <= 64.0 ? 8 : mean <= 128.0 ? 16 : 32;
+  if (rows * few >= 300000) return few;
+  return mean <= 6.0 ? 1 : mean <= 24.0 ? 4 : mean <= 64.0 ? 8 : 32;
 }
 
 template <typename T>
@@ -199,8 +211,7 @@ cudaError_t upload_csr(fvgb_mesh_s* m, const HostCsr& h, CsrDev<T>& d, cudaStrea
   d.n = h.n;
   d.m = h.m;
   d.nnz = (int64_t)h.idx.size();
-  const double mean = h.n > 0 ? (double)d.nnz / (double)h.n : 0.0;
-  d.lanes = mean <= 6.0 ? 1 : mean <= 24.0 ? 4 : mean <= 64.0 ? 8 : 32;
+  d.lanes = lanes_of(h.n, h.n > 0 ? (double)d.nnz / (double)h.n : 0.0);
   cudaError_t e;
   if ((e = dupload(m, &d.ptr, h.ptr, s))) return e;
   if ((e = dupload(m, &d.idx, h.idx, s))) return e;
@@ -242,7 +253,17 @@ fvgb_status amg_upload(fvgb_mesh m, const AmgHost& H, AmgDev<T>& a, cudaStream_t
   return FVGB_OK;
 }
 
-// One V-cycle on level l >= 1: b -> out (zero initial guess).
+// The right-hand side and the first smoothing step of level l + 1 from level l's residual
+template <typename T>
+cudaError_t restrict_to_next(AmgDev<T>& a, int l, T w, cudaStream_t s) {
+  AmgLevelDev<T>& L = a.lv[l];
+  if (l + 1 == (int)a.lv.size()) return csr_launch<T>(L.R, L.r, nullptr, nullptr, w, 0, a.cb, nullptr, s);
+  AmgLevelDev<T>& C = a.lv[l + 1];
+  return csr_launch<T>(L.R, L.r, nullptr, C.dinv, w, 0, C.b, C.x, s);
+}
+
+// One V-cycle on level l >= 1 (or, on a mesh of the dense size, l = 0): b -> out; L.x holds the
+// first smoothing step from zero.
 template <typename T>
 cudaError_t vcycle(AmgDev<T>& a, int l, const T* b, T* out, cudaStream_t s) {
   const T w = T(2.0 / 3.0);
@@ -256,14 +277,11 @@ cudaError_t vcycle(AmgDev<T>& a, int l, const T* b, T* out, cudaStream_t s) {
   T* nb = last ? a.cb : a.lv[l + 1].b;
   T* nx = last ? a.cx : a.lv[l + 1].xo;
   cudaError_t e;
-  k_amg_jacobi0<T><<<blocks_for(L.A.n, kAmgThreads), kAmgThreads, 0, s>>>(L.A.n, L.dinv, b, L.x, w);
-  count_launch();
-  if ((e = cudaGetLastError())) return e;
-  if ((e = csr_launch(L.A, L.x, b, L.dinv, w, 2, L.r, s))) return e;          // r = b - A x
-  if ((e = csr_launch(L.R, L.r, (const T*)nullptr, L.dinv, w, 0, nb, s))) return e;   // b' = R r
+  if ((e = csr_launch<T>(L.A, L.x, b, L.dinv, w, 2, L.r, nullptr, s))) return e;       // r = b - A x
+  if ((e = restrict_to_next(a, l, w, s))) return e;                                    // b' = R r, x' = w D'^-1 b'
   if ((e = vcycle(a, l + 1, nb, nx, s))) return e;
-  if ((e = csr_launch(L.P, nx, (const T*)nullptr, L.dinv, w, 1, L.x, s))) return e;   // x += P x'
-  return csr_launch(L.A, L.x, b, L.dinv, w, 3, out, s);                        // smoothing
+  if ((e = csr_launch<T>(L.P, nx, nullptr, nullptr, w, 1, L.x, nullptr, s))) return e;   // x += P x'
+  return csr_launch<T>(L.A, L.x, b, L.dinv, w, 3, out, nullptr, s);                    // smoothing
 }
 
 }  // namespace
@@ -351,9 +369,9 @@ cudaError_t launch_amg_inner(fvgb_mesh_s* m, int bcset, const double* r, int cyc
     for (int c = 0; c < cycles; ++c) {
       if (c > 0 && (e = fine(std::integral_constant<int, 1>{}, L.xo, L.x))) return e;          // smoothing
       if ((e = fine(std::integral_constant<int, 0>{}, L.x, L.r))) return e;                    // r = b - A x
-      if ((e = csr_launch(L.R, L.r, (const T*)nullptr, L.dinv, om, 0, nb, s))) return e;      // b' = R r
+      if ((e = restrict_to_next(a, 0, om, s))) return e;                                       // b' = R r
       if ((e = vcycle(a, 1, nb, nx, s))) return e;
-      if ((e = csr_launch(L.P, nx, (const T*)nullptr, L.dinv, om, 1, L.x, s))) return e;      // x += P x'
+      if ((e = csr_launch<T>(L.P, nx, nullptr, nullptr, om, 1, L.x, nullptr, s))) return e;    // x += P x'
       if (c + 1 < cycles) e = fine(std::integral_constant<int, 1>{}, L.x, L.xo);               // smoothing
       else e = fine(std::integral_constant<int, 2>{}, L.x, (T*)nullptr);
       if (e) return e;
