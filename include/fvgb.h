@@ -298,7 +298,10 @@ typedef struct {
  *  f_dev    [n_cell] double (NULL = 0)
  *  phi_dev  [n_cell] double, in: initial guess, out: solution
  *  info     host, may be NULL
- * The call synchronises the stream once per outer step (to read the FP64 residual).
+ * With a CG inner solve an ensemble, and a single mesh of up to 600,000 cells, solves in one
+ * launch (the outer loop on the device) and the call synchronises the stream once, at its end;
+ * otherwise (a larger mesh, inner > 0, or fvgb_stats_enable on) it does so once per outer step,
+ * to read the FP64 residual.
  * Returns FVGB_ENOCONV (with info filled and phi the last iterate) if rtol is not met
  * within maxit_outer steps, FVGB_ENONFINITE on NaN/Inf, FVGB_ETIMEOUT if a grid-wide
  * barrier of the persistent CG kernel gave up. */
@@ -509,8 +512,9 @@ fvgb_status fvgb_mpnn_train_step(fvgb_mpnn net, const double* dq_dev, const doub
                                  void* stream);
 
 /* Synchronise the stream and report the latched asynchronous status of the mesh (see the
- * conventions above), then clear it: FVGB_ETIMEOUT when a bounded wait on the device ran out, FVGB_ENONFINITE when a transport update wrote a non-finite value since
- * the last report, FVGB_OK otherwise. */
+ * conventions above), then clear it: FVGB_ETIMEOUT when a bounded wait on the device ran out,
+ * FVGB_ENONFINITE when a transport update wrote a non-finite value since the last report,
+ * FVGB_OK otherwise. */
 fvgb_status fvgb_sync(fvgb_mesh m, void* stream);
 
 /* Test hook of the bounded grid barrier of the persistent CG kernel (no counterpart in the

@@ -88,7 +88,7 @@ struct TopoDev {
   float4* tile_xa = nullptr;     // [N]
   float2* tile_xb = nullptr;     // [N]
   // FP64 meshes (k_gradient_fixed): integer centres, and per tile and cell what its
-  // fixed-point sums need (see build_fixed_tiles)
+  // fixed-point sums need (see build_fixed_start and build_fixed_sums)
   longlong4_16a* xfix = nullptr; // [N] {x, y, z, 0} in units of 2^-fix_scale
   GradTileFix* tile_fix = nullptr;  // [n_tile]
   int64_t* tile_dsum = nullptr;  // [3][N] sum of the cell's shifted neighbour differences

@@ -214,7 +214,8 @@ struct Coef4<double> {
 // one's, so that the loads of one trip are always in flight: two FP32 rows of 48 bytes or one
 // FP64 row of 80 for each of 512 threads. 6M cells FP64 168 -> 146 us an iteration, 750,000
 // cells 23.1 -> 20.7 us (more rows a trip without the overlap were no faster, and more rows
-// with it spill).
+// with it spill). A phase's first rows are loaded before the exchange in front of it: 10,000
+// cells FP64 7.4 -> 7.0, 750,000 FP64 20.8 -> 19.9, FP32 11.5 -> 10.8 us an iteration.
 template <typename T>
 __host__ __device__ constexpr int unroll_rows() { return sizeof(T) == 4 ? 2 : 1; }
 // the r phase holds two values a row
@@ -444,9 +445,10 @@ __global__ void __launch_bounds__(kCgThreads, kCgBlocksPerSm) k_cg(SolveArgs<T> 
 // in its last pass. An outer step as separate launches is six kernels and a host
 // synchronisation around the CG, some 60 us on 10,000 cells against 60 us of CG; here it is
 // three grid barriers. In an ensemble every part runs its own loop on its own blocks, where
-// the launches' loop ran each inner solve to the slowest part's last iteration. The operator is applied in two passes: vertex values, then per cell its
-// faces' fluxes (each formed from both sides, the operations and their order those of k_face and
-// k_update, so the residual has the same bits).
+// the launches' loop ran each inner solve to the slowest part's last iteration (16 meshes of 20k
+// to 200k cells, mixed: 23.4 -> 10.1 ms a step). The operator is applied in two passes: vertex
+// values, then per cell its faces' fluxes (each formed from both sides, the operations and their
+// order those of k_face and k_update, so the residual has the same bits).
 struct ResidualArgs {
   int64_t N, F, Fi, V;
   const int64_t* sptr;
@@ -799,7 +801,7 @@ cudaError_t launch_cg(fvgb_mesh_s* m, int bcset, const double* r, double inner_r
 }
 
 // The whole solve in one launch up to kSolveOneMax cells. A solve to 1e-8 against separate
-// launches: 10,368 cells FP64 3.46 -> 2.38 ms, 384,000 13.4 -> 12.3 (mixed 9.7 -> 8.8); 750,000
+// launches: 10,368 cells FP64 3.46 -> 2.26 ms, 384,000 13.4 -> 11.9 (mixed 9.7 -> 8.8); 750,000
 // equal; 1.3M 38.8 -> 43.1: one 512-thread block an SM streams the operator's passes slower than
 // their own kernels. (CUDA-event timing of the CG wants its own launches.)
 constexpr int64_t kSolveOneMax = 600000;
