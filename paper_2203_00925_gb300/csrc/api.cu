@@ -114,9 +114,10 @@ void order_rows_for_banks(int16_t* const* row, const int* width) {
 // Halo lists of the shared-memory gradient (see TopoDev): per tile its own rows, then every
 // other cell met in the rows' padded node-neighbour lists (sorted); lidx[pos] is the position
 // of sidx[pos] in its row's tile list. Returns the longest list.
-// Tiles are the row ranges [start[t], start[t + 1]) (at most kGradTile rows each).
-int build_grad_tiles(int64_t N, const std::vector<int64_t>& start, const std::vector<int64_t>& sptr,
-                     const std::vector<int32_t>& sidx, std::vector<int32_t>& tptr, std::vector<int32_t>& tidx,
+// Tiles are the row ranges [start[t], start[t + 1]) (at most kGradTile rows each); those of FP64
+// sums (fix, where given) stage nothing and get no list.
+int build_grad_tiles(int64_t N, const std::vector<int64_t>& start, const std::vector<GradTileFix>& fix,
+                     const std::vector<int64_t>& sptr, const std::vector<int32_t>& sidx, std::vector<int32_t>& tptr, std::vector<int32_t>& tidx,
                      std::vector<int16_t>& lidx) {
   const int64_t ntile = (int64_t)start.size() - 1;
   std::vector<std::vector<int32_t>> lists(ntile);
@@ -128,6 +129,7 @@ int build_grad_tiles(int64_t N, const std::vector<int64_t>& start, const std::ve
 #pragma omp for schedule(dynamic, 64)
     for (int64_t t = 0; t < ntile; ++t) {
       const int64_t r0 = start[t], r1 = start[t + 1];
+      if (!fix.empty() && fix[t].bits == 0) continue;
       std::vector<int32_t>& L = lists[t];
       for (int64_t r = r0; r < r1; ++r) { stamp[r] = (int32_t)t; L.push_back((int32_t)r); }
       const size_t own = L.size();
@@ -162,20 +164,27 @@ int build_grad_tiles(int64_t N, const std::vector<int64_t>& start, const std::ve
   return max_len;
 }
 
-// What the FP64 gradient's fixed-point sums (k_gradient_fixed) need beside the halo lists.
-// Tiles do not cross parts, so that a mesh gives the same bits alone and in an ensemble.
-//  - centres as integers in units of 2^-scale (|x| 2^scale < 2^61: exact for every coordinate
-//    of at least 2^-9 of the largest);
-//  - tiles: up to kGradTile consecutive rows, ended early where the next row would stretch
-//    the halo to more than kFixedSpread times the smallest neighbourhood (a jump of the Morton
-//    curve, a graded mesh): the tile's unit would be coarse for those cells;
+// What the FP64 gradient's fixed-point sums (k_gradient_fixed) need beside the halo lists. All of
+// it is per part and per coordinate: flat cells keep the bits of their short direction, and a
+// part's tiles do not depend on the parts beside it (nor do tiles cross parts; only a halo too
+// long for shared memory, in any part, takes the whole mesh to k_gradient).
+//  - centres as integers in units of 2^-scale (|x| 2^scale < 2^61, x the part's coordinate:
+//    exact for every value of at least 2^-9 of the largest);
+//  - a row may take fixed-point sums when its own neighbourhood loses nothing by that: in every
+//    coordinate it extends over 2^52 units, or its and its neighbours' centres are exact;
+//  - tiles: up to kGradTile consecutive such rows, ended early where in some coordinate the next
+//    row would stretch the halo to more than kFixedSpread times the smallest neighbourhood (a
+//    jump of the Morton curve, a graded mesh): the tile's unit would be coarse for those cells.
+//    From a row that may not, or where the next kGradTile rows would make tiles of fewer than
+//    kFixedRows on average, a whole tile takes FP64 sums, in the order of k_gradient;
 //  - per tile bits = 62 - ceil(log2(w + 1)), w the longest neighbour list of its part, so
 //    that a sum over a list stays below 2^62 (0, FP64 sums, in a part of less than one tile
-//    and with lists above 511), and the right shifts (negative: left) that bring its centre
-//    differences below 2^bits;
-//  - per cell D = sum_j (y_j - y_i) of those shifted differences over its neighbours, and the
-//    padding entries of its list.
-constexpr double kFixedSpread = 8.0;
+//    and with lists above 511), and the left shifts that bring its centre differences to 63
+//    magnitude bits;
+//  - per cell D = sum_j (y_j - y_i) of those shifted differences over its neighbours, in units
+//    of 2^(62 - bits), and the padding entries of its list.
+constexpr double kFixedSpread = 12.0;
+constexpr int kFixedRows = 32;
 
 struct FixedHost {
   std::vector<longlong4_16a> xfix;
@@ -183,55 +192,98 @@ struct FixedHost {
   std::vector<GradTileFix> tile;
   std::vector<int64_t> dsum;
   std::vector<int16_t> pad;
-  int scale = 0;
 };
 
-// largest component of x_j - x_i
-long long fixed_distance(const longlong4_16a& p, const longlong4_16a& q) {
+struct Extent3 { long long v[3]; };
+
+// |x_j - x_i| per coordinate
+Extent3 fixed_distance(const longlong4_16a& p, const longlong4_16a& q) {
   auto mag = [](long long v) { return v < 0 ? -v : v; };
-  return std::max(mag(p.x - q.x), std::max(mag(p.y - q.y), mag(p.z - q.z)));
+  return Extent3{{mag(p.x - q.x), mag(p.y - q.y), mag(p.z - q.z)}};
 }
 
 // integer centres and tiles
 void build_fixed_start(const HostMesh& h, FixedHost& o) {
   const int64_t N = h.N;
   const std::vector<double>& cen = h.cen;
-  double top = 0.0;
-  for (double c : cen) top = std::max(top, std::fabs(c));
-  int e = 0;
-  std::frexp(top, &e);                       // top < 2^e
-  o.scale = 61 - e;
-  const bool usable = top > 0.0 && std::isfinite(top) && o.scale > -200 && o.scale < 260;
   o.xfix.resize(N);
-  std::vector<long long> near(N, 0);         // extent of each neighbourhood
-#pragma omp parallel for
-  for (int64_t i = 0; i < N; ++i) {
-    auto fix = [&](double c) { return usable ? std::llrint(std::ldexp(c, o.scale)) : 0ll; };
-    o.xfix[i] = longlong4_16a{fix(cen[i]), fix(cen[N + i]), fix(cen[2 * N + i]), 0};
-  }
-#pragma omp parallel for
-  for (int64_t i = 0; i < N; ++i)
-    for (int32_t q = h.nptr[i]; q < h.nptr[i + 1]; ++q)
-      near[i] = std::max(near[i], fixed_distance(o.xfix[h.nidx[q]], o.xfix[i]));
+  std::vector<Extent3> near(N);              // extent of each neighbourhood
+  std::vector<uint8_t> exact(N), may(N);     // bit a: coordinate a of the centre is exact
   for (size_t p = 0; p + 1 < h.part_cell_begin.size(); ++p) {
     const int64_t lo = h.part_cell_begin[p], hi = h.part_cell_begin[p + 1];
+    int16_t scale[3];
+    bool usable = true;
+    for (int a = 0; a < 3; ++a) {
+      double top = 0.0;
+      bool finite = true;
+      for (int64_t i = lo; i < hi; ++i) {
+        top = std::max(top, std::fabs(cen[a * N + i]));
+        finite = finite && std::isfinite(cen[a * N + i]);
+      }
+      int e = 0;
+      if (finite) std::frexp(top, &e);       // top < 2^e
+      scale[a] = (int16_t)(top > 0.0 ? 61 - e : 0);
+      usable = usable && finite && scale[a] > -200 && scale[a] < 260;
+    }
+#pragma omp parallel for
+    for (int64_t i = lo; i < hi; ++i) {
+      long long v[3] = {0, 0, 0};
+      exact[i] = 0;
+      for (int a = 0; usable && a < 3; ++a) {
+        const double x = std::ldexp(cen[a * N + i], scale[a]);
+        v[a] = std::llrint(x);
+        exact[i] |= (uint8_t)((double)v[a] == x ? 1 << a : 0);
+      }
+      o.xfix[i] = longlong4_16a{v[0], v[1], v[2], 0};
+    }
     int64_t widest = 1;
     for (int64_t i = lo; i < hi; ++i) widest = std::max<int64_t>(widest, h.nptr[i + 1] - h.nptr[i]);
     int w = 0;
     while ((int64_t(1) << w) < widest + 1) ++w;
     const int bits = usable && hi - lo >= kGradTile && w <= 9 ? 62 - w : 0;
-    for (int64_t r = lo; r < hi;) {
-      long long reach = 0, least = near[r];
-      int64_t end = r;
-      for (; end < hi && end < r + kGradTile; ++end) {
-        const long long to = std::max(reach, fixed_distance(o.xfix[end], o.xfix[r]) + near[end]);
-        const long long small = std::min(least, near[end]);
-        if (bits > 0 && end > r && (double)to > kFixedSpread * (double)small) break;
-        reach = to;
-        least = small;
+#pragma omp parallel for
+    for (int64_t i = lo; i < hi; ++i) {
+      Extent3 ext{{0, 0, 0}};
+      uint8_t all = exact[i];
+      for (int32_t q = h.nptr[i]; q < h.nptr[i + 1]; ++q) {
+        const Extent3 d = fixed_distance(o.xfix[h.nidx[q]], o.xfix[i]);
+        for (int a = 0; a < 3; ++a) ext.v[a] = std::max(ext.v[a], d.v[a]);
+        all &= exact[h.nidx[q]];
       }
+      near[i] = ext;
+      may[i] = bits > 0;
+      for (int a = 0; a < 3; ++a) may[i] = may[i] && (((all >> a) & 1) != 0 || ext.v[a] >= 1ll << 52);
+    }
+    // the tile of fixed-point sums from row r ends before row ...
+    auto tile_end = [&](int64_t r) {
+      Extent3 reach{{0, 0, 0}}, least = near[r];
+      int64_t end = r;
+      for (; end < hi && end < r + kGradTile && may[end]; ++end) {
+        const Extent3 d = fixed_distance(o.xfix[end], o.xfix[r]);
+        bool stop = false;
+        for (int a = 0; a < 3; ++a) {
+          reach.v[a] = std::max(reach.v[a], d.v[a] + near[end].v[a]);
+          least.v[a] = std::min(least.v[a], near[end].v[a]);
+          stop = stop || (double)reach.v[a] > kFixedSpread * (double)least.v[a];
+        }
+        if (stop && end > r) break;
+      }
+      return end;
+    };
+    for (int64_t r = lo; r < hi;) {
+      int64_t end = tile_end(r);
+      bool fixed = end > r;
+      const int64_t whole = std::min<int64_t>(hi, r + kGradTile);
+      int64_t q = end;
+      for (int n = 1; fixed && q < whole; ++n) {          // the tiles that would follow
+        fixed = n < kGradTile / kFixedRows;
+        q = std::max(tile_end(q), q + 1);
+      }
+      if (!fixed) end = whole;
+      GradTileFix t{(int32_t)r, (int16_t)(end - r), (int16_t)(fixed ? bits : 0), {}, {},
+                    {scale[0], scale[1], scale[2]}, {}};      // units: see build_fixed_sums
       o.start.push_back(r);
-      o.tile.push_back(GradTileFix{(int32_t)r, (int32_t)(end - r), (int16_t)bits, 0, 0, 0});
+      o.tile.push_back(t);
       r = end;
     }
   }
@@ -253,30 +305,36 @@ void build_fixed_sums(const HostMesh& h, const std::vector<int64_t>& sptr, const
       o.pad[i] = (int16_t)std::min<int64_t>(INT16_MAX, (sptr[i / 32 + 1] - sptr[i / 32]) / 32 - (h.nptr[i + 1] - h.nptr[i]));
     if (bits == 0) continue;
     const longlong4_16a at = o.xfix[r0];
-    long long most = 1, widest = 1;
-    for (int32_t k = tptr[t]; k < tptr[t + 1]; ++k) most = std::max(most, fixed_distance(o.xfix[tidx[k]], at));
-    for (int64_t i = r0; i < r1; ++i)
-      for (int32_t q = h.nptr[i]; q < h.nptr[i + 1]; ++q)
-        widest = std::max(widest, fixed_distance(o.xfix[h.nidx[q]], o.xfix[i]));
-    auto shift_for = [&](long long top) {
-      int sh = 0;
-      while (top < (1ll << (bits - 1 + sh))) --sh;     // room to the left
-      while (bits + sh < 62 && top >= (1ll << (bits + sh))) ++sh;  // or cut to the right
-      return sh;
+    Extent3 most{{1, 1, 1}}, widest{{1, 1, 1}};
+    auto widen = [](Extent3& e, const Extent3& d) {
+      for (int a = 0; a < 3; ++a) e.v[a] = std::max(e.v[a], d.v[a]);
     };
-    const int sh = shift_for(most);
-    tile.shift = (int16_t)sh;
-    tile.own_shift = (int16_t)shift_for(widest);
-    auto cut = [&](long long v) { return sh >= 0 ? v >> sh : (long long)((unsigned long long)v << -sh); };
+    for (int32_t k = tptr[t]; k < tptr[t + 1]; ++k) widen(most, fixed_distance(o.xfix[tidx[k]], at));
+    for (int64_t i = r0; i < r1; ++i)
+      for (int32_t q = h.nptr[i]; q < h.nptr[i + 1]; ++q) widen(widest, fixed_distance(o.xfix[h.nidx[q]], o.xfix[i]));
+    auto left_for = [](long long top) {        // top 2^left in [2^62, 2^63)
+      int l = 0;
+      while (top < (1ll << (62 - l))) ++l;
+      return l;
+    };
+    for (int a = 0; a < 3; ++a) {
+      const int l = left_for(std::max(most.v[a], widest.v[a])), own = left_for(widest.v[a]), scale = tile.unit[a];
+      tile.left[a] = (int8_t)l;
+      tile.own_left[a] = (int8_t)own;
+      tile.unit[a] = (int16_t)(63 - bits - l - scale);
+      tile.own_unit[a] = (int16_t)(63 - bits - own - scale);
+    }
     for (int64_t i = r0; i < r1; ++i) {
       const longlong4_16a& x = o.xfix[i];
-      const long long yi[3] = {cut(x.x - at.x), cut(x.y - at.y), cut(x.z - at.z)};
+      __int128 sum[3] = {0, 0, 0};
       for (int32_t q = h.nptr[i]; q < h.nptr[i + 1]; ++q) {
         const longlong4_16a& y = o.xfix[h.nidx[q]];
-        o.dsum[i] += cut(y.x - at.x) - yi[0];
-        o.dsum[N + i] += cut(y.y - at.y) - yi[1];
-        o.dsum[2 * N + i] += cut(y.z - at.z) - yi[2];
+        sum[0] += y.x - x.x;
+        sum[1] += y.y - x.y;
+        sum[2] += y.z - x.z;
       }
+      for (int a = 0; a < 3; ++a)              // |sum| 2^left < 2^63 (2^(62 - bits) - 1)
+        o.dsum[a * N + i] = (int64_t)(((sum[a] << tile.left[a]) + (((__int128)1 << (62 - bits)) >> 1)) >> (62 - bits));
     }
   }
 }
@@ -993,17 +1051,17 @@ static fvgb_status upload_impl(int32_t dim, int64_t n_vert, const double* xyz, i
       for (int64_t r = 0; r < h.N; r += kGradTile) fx.start.push_back(r);
       fx.start.push_back(h.N);
     }
-    // tiles much shorter than their room (a mesh in no local order) gain nothing
-    bool tiled = (int64_t)fx.start.size() - 1 <= h.N / 32 + n_part;
-    const int mx = tiled ? build_grad_tiles(h.N, fx.start, sptr, sidx, tptr, tidx, lidx) : 0;
+    // tiles of FP64 sums take what k_gradient takes (750,000 cells 731 and 732 us): one other pays
+    bool tiled = prec != FVGB_FP64;
+    for (const GradTileFix& q : fx.tile) tiled = tiled || q.bits > 0;
+    const int mx = tiled ? build_grad_tiles(h.N, fx.start, fx.tile, sptr, sidx, tptr, tidx, lidx) : 0;
     tiled = tiled && mx <= kGradTileMaxHalo;
     if (tiled && prec == FVGB_FP64) {
       build_fixed_sums(h, sptr, tptr, tidx, fx);
       t.n_tile = (int)fx.tile.size();
-      t.fix_scale = fx.scale;
-      t.fix_bits = fx.tile[0].bits;
+      for (const GradTileFix& q : fx.tile) t.fix_bits = std::max<int>(t.fix_bits, q.bits);
       for (const GradTileFix& q : fx.tile)
-        if (q.bits != t.fix_bits) t.fix_bits = 0;
+        if (q.bits != 0 && q.bits != t.fix_bits) t.fix_bits = 0;
       if ((e = dupload(m, &t.tile_pad, fx.pad, s))) return fail(e, "upload");
       if ((e = dupload(m, &t.xfix, fx.xfix, s))) return fail(e, "upload");
       if ((e = dupload(m, &t.tile_fix, fx.tile, s))) return fail(e, "upload");

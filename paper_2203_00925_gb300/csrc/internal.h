@@ -12,13 +12,14 @@
 
 namespace fvgb {
 
-// Tile of the FP64 gradient's fixed-point sums (k_gradient_fixed).
+// Tile of the FP64 gradient's fixed-point sums (k_gradient_fixed); [3]: per coordinate.
 struct GradTileFix {
-  int32_t row0, rows;
-  int16_t bits;       // magnitude bits of its integers (0: FP64 sums)
-  int16_t shift;      // right shift of centre differences from its first cell
-  int16_t own_shift;  // right shift of centre differences from a cell to its neighbours
-  int16_t spare;
+  int32_t row0;
+  int16_t rows;
+  int16_t bits;                  // magnitude bits of u's integers and of a product (0: FP64 sums)
+  int8_t left[3], own_left[3];   // left shifts that bring centre differences, from its first cell
+                                 // and from a cell to its neighbours, to 63 magnitude bits
+  int16_t unit[3], own_unit[3];  // exponents of a product's units, less that of u
 };
 
 // Sliced-ELL (SELL-32) list: rows grouped in slices of 32 consecutive rows; slice s
@@ -89,12 +90,11 @@ struct TopoDev {
   float2* tile_xb = nullptr;     // [N]
   // FP64 meshes (k_gradient_fixed): integer centres, and per tile and cell what its
   // fixed-point sums need (see build_fixed_start and build_fixed_sums)
-  longlong4_16a* xfix = nullptr; // [N] {x, y, z, 0} in units of 2^-fix_scale
+  longlong4_16a* xfix = nullptr; // [N] {x, y, z, 0} in the units of the cell's part
   GradTileFix* tile_fix = nullptr;  // [n_tile]
-  int64_t* tile_dsum = nullptr;  // [3][N] sum of the cell's shifted neighbour differences
+  int64_t* tile_dsum = nullptr;  // [3][N] sum of the cell's shifted neighbour differences / 2^(62 - bits)
   int16_t* tile_pad = nullptr;   // [N] padding entries of the cell's list (the cell itself)
-  int fix_scale = 0;             // see xfix
-  int fix_bits = 0;              // the tiles' bits where all have the same, else 0
+  int fix_bits = 0;              // the bits of the fixed-point tiles where all have the same, else 0
   int n_tile = 0;
 };
 

@@ -286,18 +286,22 @@ k_gradient_tiled(int64_t N, int64_t F, int64_t Fi, const int64_t* __restrict__ s
 //   y_j = x_j - x_o,  v_j = u_j - u_o,  z_j = y_j v_j   (once per record of the halo list)
 //   J_i = sum_j (y_j - y_i)(v_j - v_i) = sum_j z_j - y_i sum_j v_j - v_i D_i,
 // D_i = sum_j (y_j - y_i) being geometry (tile_dsum). y is the difference of integer centres,
-// v the FP64 difference converted with the tile's largest exponent, z the 128-bit product cut
-// back; all keep ``bits`` (53..61) magnitude bits relative to the tile's range, the sums are
-// exact in 64 bits and the last line is formed in 128. Per neighbour entry that leaves four
+// moved left per coordinate to 63 magnitude bits of the tile's range, v the FP64 difference
+// converted with the tile's largest exponent, z the 128-bit product cut back; v and z keep
+// ``bits`` (53..61) magnitude bits relative to the tile's range, the sums are exact in 64 bits
+// and the last line is formed in 128. Per neighbour entry that leaves four
 // 64-bit additions and two 16-byte shared-memory reads (the records, in two arrays so that the
 // lists' bank-aware order serves both).
 // The unit is relative to the tile's range R of v. A cell whose own neighbours differ by less
 // than R / 16 (a steep field in the tile) sums its own products (x_j - x_i)(u_j - u_i) instead,
 // also as integers but with the cell's own unit (own_scale_sum). Two threads share a cell's
-// entries. Where u is not finite or beyond 2^+-600, and in parts of less than a tile, the sum
-// stays in FP64, in the order of k_gradient. 750,000 cells: 732 us with FP64 sums, 181 us now
-// (integer issue and shared memory); the error against exact values went from 5.8e-16 to 4.5e-16
-// of the largest.
+// entries. Where u is not finite or beyond 2^+-600, and in tiles whose integers would lose bits
+// of the centres (build_fixed_start), the sum stays in FP64, in the order of k_gradient.
+// 750,000 cells: 732 us with FP64 sums (tiles of FP64 sums take the same), 186 us now (integer
+// issue and shared memory; 182 with one shift for the three coordinates, which lost the short
+// direction of flat cells); the error against exact values went from 5.8e-16 to 4.4e-16 of the
+// largest, and on cells flattened 10^2 to 10^6 : 1, on boundary layers and beside parts 10^9
+// times as large it is the direct sum's, 5 to 9e-16 of each component.
 constexpr int kFixTopMin = 400, kFixTopMax = 1600;   // biased exponents the scaled sums stay normal for
 
 __device__ __forceinline__ int exp_bits(long long v) { return (int)((unsigned long long)v >> 52) & 0x7ff; }
@@ -316,13 +320,10 @@ __device__ __forceinline__ long long to_fixed(long long a, int top, int bits) {
   return a < 0 ? -(long long)mag : (long long)mag;
 }
 
-// floor(y v / 2^bits) as one high product: the operands are shifted up by 64 - bits in all,
-// y here and v by the caller (v_up). The missing half unit of every product is added to the
+// floor(y v / 2^63) as one high product. The missing half unit of every product is added to the
 // sums (half the number of terms).
-__device__ __forceinline__ int y_up(int bits) { return (64 - bits) / 2; }
-__device__ __forceinline__ int v_up(int bits) { return 64 - bits - y_up(bits); }
-__device__ __forceinline__ long long fixed_mul(long long y, long long v_shifted, int bits) {
-  return __mul64hi((long long)((unsigned long long)y << y_up(bits)), v_shifted);
+__device__ __forceinline__ long long fixed_mul(long long y, long long v) {
+  return __mul64hi(y, (long long)((unsigned long long)v << 1));
 }
 
 // v 2^e as FP64, rounded to nearest even (the result is in the normal range), without the
@@ -342,14 +343,24 @@ __device__ __forceinline__ double from_fixed(long long v, int e) {
 // J of one cell in FP64, neighbours' values and centres from memory
 __device__ __noinline__ void direct_sum(int64_t N, int64_t i, int width, const int32_t* __restrict__ col,
                                         const double* __restrict__ u, const double* __restrict__ cen, double* J) {
+  constexpr int U = 4;                  // neighbours in flight
   const double ui = u[i], x = cen[i], y = cen[N + i], z = cen[2 * N + i];
   double j0 = 0.0, j1 = 0.0, j2 = 0.0;
-  for (int c = 0; c < width; ++c) {
-    const int64_t j = col[32 * c];
-    const double du = u[j] - ui;
-    j0 += (cen[j] - x) * du;
-    j1 += (cen[N + j] - y) * du;
-    j2 += (cen[2 * N + j] - z) * du;
+  for (int c = 0; c < width; c += U) {
+    int64_t j[U];
+    double uj[U], xj[U], yj[U], zj[U];
+#pragma unroll
+    for (int q = 0; q < U; ++q) j[q] = c + q < width ? col[32 * (c + q)] : i;
+#pragma unroll
+    for (int q = 0; q < U; ++q) { uj[q] = u[j[q]]; xj[q] = cen[j[q]]; yj[q] = cen[N + j[q]]; zj[q] = cen[2 * N + j[q]]; }
+#pragma unroll
+    for (int q = 0; q < U; ++q) {
+      if (c + q >= width) break;
+      const double du = uj[q] - ui;
+      j0 += (xj[q] - x) * du;
+      j1 += (yj[q] - y) * du;
+      j2 += (zj[q] - z) * du;
+    }
   }
   J[0] = j0; J[1] = j1; J[2] = j2;
 }
@@ -375,9 +386,10 @@ __device__ __forceinline__ int own_top(int c, int end, double ui, const int32_t*
 template <int BITS>
 __device__ __noinline__ void own_scale_sum(int64_t i, int c, int end, double ui, const int32_t* __restrict__ col,
                                            const longlong4_16a* __restrict__ xfix, const double* __restrict__ u,
-                                           int tile_bits, int shift, int top, long long* s) {
+                                           const GradTileFix* __restrict__ tile, int top, long long* s) {
   constexpr int U = 4;
-  const int bits = BITS > 0 ? BITS : tile_bits;
+  const int bits = BITS > 0 ? BITS : tile->bits;
+  const int l0 = tile->own_left[0], l1 = tile->own_left[1], l2 = tile->own_left[2];
   const longlong2* X = reinterpret_cast<const longlong2*>(xfix);
   const longlong2 xi = X[2 * i];
   const long long zi = X[2 * i + 1].x;
@@ -397,11 +409,10 @@ __device__ __noinline__ void own_scale_sum(int64_t i, int c, int end, double ui,
     }
 #pragma unroll
     for (int q = 0; q < U; ++q) {
-      const long long v = (long long)((unsigned long long)to_fixed(__double_as_longlong(uj[q] - ui), top, bits) << v_up(bits));
-      const long long d[3] = {a[q].x - xi.x, a[q].y - xi.y, az[q] - zi};
-      s0 += fixed_mul(shift >= 0 ? d[0] >> shift : d[0] << -shift, v, bits);
-      s1 += fixed_mul(shift >= 0 ? d[1] >> shift : d[1] << -shift, v, bits);
-      s2 += fixed_mul(shift >= 0 ? d[2] >> shift : d[2] << -shift, v, bits);
+      const long long v = to_fixed(__double_as_longlong(uj[q] - ui), top, bits);
+      s0 += fixed_mul((a[q].x - xi.x) << l0, v);
+      s1 += fixed_mul((a[q].y - xi.y) << l1, v);
+      s2 += fixed_mul((az[q] - zi) << l2, v);
     }
   }
   s[0] = s0; s[1] = s1; s[2] = s2;
@@ -420,7 +431,7 @@ k_gradient_fixed(int64_t N, int64_t F, int64_t Fi, const int64_t* __restrict__ s
                  const int32_t* __restrict__ sidx, const uint32_t* __restrict__ lidx,
                  const int32_t* __restrict__ tptr, const int32_t* __restrict__ tidx,
                  const GradTileFix* __restrict__ tfix, const longlong4_16a* __restrict__ xfix,
-                 const int64_t* __restrict__ dsum, const int16_t* __restrict__ pad, int scale, int max_halo,
+                 const int64_t* __restrict__ dsum, const int16_t* __restrict__ pad, int max_halo,
                  const double* __restrict__ u, const double* __restrict__ cen,
                  const double* __restrict__ xf, const double* __restrict__ minv,
                  const int32_t* __restrict__ gptr, const int32_t* __restrict__ gface,
@@ -431,9 +442,11 @@ k_gradient_fixed(int64_t N, int64_t F, int64_t Fi, const int64_t* __restrict__ s
   __shared__ int s_top[kFixThreads / 32];
   __shared__ longlong2 s_sum[2][kGradTile];   // the second halves' sums
   __shared__ int2 s_range[kGradTile];
-  const GradTileFix td = tfix[blockIdx.x];
+  const GradTileFix* const tile = tfix + blockIdx.x;
+  const GradTileFix td = *tile;
   const int64_t r0 = td.row0;
-  const int bits = BITS > 0 ? BITS : td.bits, shift = td.shift;
+  const bool fixed = td.bits > 0;
+  const int bits = BITS > 0 ? BITS : td.bits;
   const int row = threadIdx.x & (kGradTile - 1), half = threadIdx.x / kGradTile;
   const bool own = row < td.rows;
   const int64_t i = own ? r0 + row : r0;
@@ -442,9 +455,9 @@ k_gradient_fixed(int64_t N, int64_t F, int64_t Fi, const int64_t* __restrict__ s
   const int32_t* gcol = sidx + b0 + (i & 31);
   double J[3] = {0.0, 0.0, 0.0};
   // how the cell sums: 0 done, 1 its own unit, 2 FP64
-  int todo = bits == 0 ? 2 : 1;
+  int todo = fixed ? 1 : 2;
   int otop = 0;                         // known exponent of the cell's own differences
-  if (bits > 0) {                       // uniform over the block
+  if (fixed) {                          // uniform over the block
     const int32_t h0 = tptr[blockIdx.x], nh = tptr[blockIdx.x + 1] - h0;
     const int32_t* halo = tidx + h0;
     const uint32_t* col = lidx + (b0 >> 1) + (i & 31);    // two entries a word, width even
@@ -475,7 +488,7 @@ k_gradient_fixed(int64_t N, int64_t F, int64_t Fi, const int64_t* __restrict__ s
         const long long du = __double_as_longlong(uj[q] - uo);
         long long y[3] = {a[q].x - oa.x, a[q].y - oa.y, az[q] - oz};
 #pragma unroll
-        for (int c = 0; c < 3; ++c) y[c] = shift >= 0 ? y[c] >> shift : y[c] << -shift;
+        for (int c = 0; c < 3; ++c) y[c] <<= td.left[c];
         if (k < kGradTile) { yi[0] = y[0]; yi[1] = y[1]; yi[2] = y[2]; }   // the thread's own cell
         ra[k] = make_longlong2(du, y[0]);
         rb[k] = make_longlong2(y[1], y[2]);
@@ -494,9 +507,9 @@ k_gradient_fixed(int64_t N, int64_t F, int64_t Fi, const int64_t* __restrict__ s
     } else {
       for (int k = threadIdx.x; k < nh; k += kFixThreads) {   // the entries this thread staged
         const longlong2 a = ra[k], b = rb[k];
-        const long long v = to_fixed(a.x, top, bits), vu = (long long)((unsigned long long)v << v_up(bits));
-        ra[k] = make_longlong2(v, fixed_mul(a.y, vu, bits));
-        rb[k] = make_longlong2(fixed_mul(b.x, vu, bits), fixed_mul(b.y, vu, bits));
+        const long long v = to_fixed(a.x, top, bits);
+        ra[k] = make_longlong2(v, fixed_mul(a.y, v));
+        rb[k] = make_longlong2(fixed_mul(b.x, v), fixed_mul(b.y, v));
       }
       __syncthreads();
       const longlong2 ai = ra[own ? row : 0], bi = rb[own ? row : 0];
@@ -542,8 +555,8 @@ k_gradient_fixed(int64_t N, int64_t F, int64_t Fi, const int64_t* __restrict__ s
           const long long Z[3] = {Z0 + half_units, Z1 + half_units, Z2 + half_units};
 #pragma unroll
           for (int k = 0; k < 3; ++k) {
-            const __int128 t = (__int128)yi[k] * V + (__int128)vi * dsum[k * N + i] + ((__int128)1 << (bits - 1));
-            J[k] = from_fixed(Z[k] - (long long)(t >> bits), shift - scale + top - 1022);
+            const __int128 t = (__int128)yi[k] * V + (((__int128)vi * dsum[k * N + i]) << (62 - bits)) + ((__int128)1 << 62);
+            J[k] = from_fixed(Z[k] - (long long)(t >> 63), td.unit[k] + top - 1022);
           }
         } else if (m >= 2) {
           // (m - 1) 2^32 < range of the u_j < (m + 1) 2^32 units: the largest |u_j - u_i| has
@@ -569,7 +582,7 @@ k_gradient_fixed(int64_t N, int64_t F, int64_t Fi, const int64_t* __restrict__ s
     top = max(tops[row], tops[row + kGradTile]);
     const bool usable = top >= kFixTopMin && top <= kFixTopMax;
     long long s[3] = {0, 0, 0};
-    if (mine && usable) own_scale_sum<BITS>(i, c0, c1, ui, gcol, xfix, u, bits, td.own_shift, top, s);
+    if (mine && usable) own_scale_sum<BITS>(i, c0, c1, ui, gcol, xfix, u, tile, top, s);
     if (half == 1) {
       s_sum[0][row] = make_longlong2(s[0], s[1]);
       s_sum[1][row].x = s[2];
@@ -583,7 +596,7 @@ k_gradient_fixed(int64_t N, int64_t F, int64_t Fi, const int64_t* __restrict__ s
         const long long half_units = (width - pad[i]) >> 1;
         const long long t[3] = {s_sum[0][row].x, s_sum[0][row].y, s_sum[1][row].x};
 #pragma unroll
-        for (int k = 0; k < 3; ++k) J[k] = from_fixed(s[k] + t[k] + half_units, td.own_shift - scale + top - 1022);
+        for (int k = 0; k < 3; ++k) J[k] = from_fixed(s[k] + t[k] + half_units, td.own_unit[k] + top - 1022);
       } else {
         todo = 2;
       }
@@ -1306,7 +1319,7 @@ cudaError_t launch_gradient(fvgb_mesh_s* m, int bcset, const T* u, T* grad, cuda
         auto* k = t.fix_bits == kFixBitsUsual ? k_gradient_fixed<kFixBitsUsual> : k_gradient_fixed<0>;
         k<<<(unsigned)t.n_tile, kFixThreads, 2 * t.tile_max * sizeof(longlong2), s>>>(
             t.N, t.F, t.Fi, t.nsell.ptr, t.nsell.idx, t.tile_lidx, t.tile_ptr, t.tile_idx, t.tile_fix, t.xfix,
-            t.tile_dsum, t.tile_pad, t.fix_scale, t.tile_max, (const double*)u, (const double*)g.cen,
+            t.tile_dsum, t.tile_pad, t.tile_max, (const double*)u, (const double*)g.cen,
             (const double*)g.xf, (const double*)b.minv, b.gptr, b.gface, (const double*)b.bval, (double*)grad);
         count_launch();
         return cudaGetLastError();
