@@ -28,6 +28,7 @@ struct GraphState {
   void* E = nullptr;
   fvgb_streamer_params params{};
   std::vector<fvgb_spot> spots;   // copy of the captured step's plasma spots
+  bool whole = false;             // the solve is one launch, without a loop node
   // device state
   double* bn2 = nullptr;        // [P]
   double* rel = nullptr;        // [P]
@@ -133,6 +134,7 @@ bool same_params(const fvgb_streamer_params& a, const fvgb_streamer_params& b) {
          a.bcset_ne == b.bcset_ne && a.bcset_phi == b.bcset_phi && a.solve.rtol == b.solve.rtol &&
          a.solve.inner_rtol == b.solve.inner_rtol && a.solve.maxit_inner == b.solve.maxit_inner &&
          a.solve.maxit_outer == b.solve.maxit_outer && a.solve.prec == b.solve.prec &&
+         a.solve.inner == b.solve.inner &&
          a.warm == b.warm && a.extrapolate == b.extrapolate && a.recon == b.recon &&
          a.stages == b.stages;
 }
@@ -257,6 +259,7 @@ fvgb_status build_graph(fvgb_mesh m, GraphState& g, const fvgb_streamer_params* 
   g.exec = exec;
   g.ne = ne; g.ni = ni; g.phi = phi; g.E = E; g.params = *p;
   g.spots.assign(p->spots, p->spots + p->n_spot);
+  g.whole = whole;
   g.params.spots = nullptr;
   g.k_pre = k1 - k0;
   g.k_post = k2 - k1;
@@ -308,7 +311,8 @@ fvgb_status streamer_graph_steps(fvgb_mesh m, const fvgb_streamer_params* p, voi
     g->ctl = (int*)c;
   }
   GraphState& g = *m->graph;
-  if (!g.exec || g.ne != ne || g.ni != ni || g.phi != phi || g.E != E || !same_params(g.params, *p) || !same_spots(g.spots, *p)) {
+  if (!g.exec || g.ne != ne || g.ni != ni || g.phi != phi || g.E != E || !same_params(g.params, *p) || !same_spots(g.spots, *p) ||
+      g.whole != solve_one_ok(m, &p->solve)) {
     FVGB_TRY(cudaStreamSynchronize(s), "synchronize");
     if (fvgb_status st = build_graph(m, g, p, ne, ni, phi, E)) return st;
   }
