@@ -168,11 +168,12 @@ __global__ void k_amg_add(int64_t n, const T* __restrict__ a, double* __restrict
   if (i < n) phi[i] += (double)a[i];
 }
 
-// inner-solve bookkeeping read by the outer loop: cycles per active part, status ok
+// inner-solve bookkeeping read by the outer loop: cycles per active part, status ok, and no
+// barrier timed out (the word holds what the last cooperative launch left, in whatever call)
 __global__ void k_amg_info(int P, const int* __restrict__ active, int cycles, int* __restrict__ out_inner,
-                           int* __restrict__ cg_info) {
+                           int* __restrict__ cg_info, Barrier* __restrict__ bar) {
   for (int p = threadIdx.x; p < P; p += blockDim.x) out_inner[p] = active[p] ? cycles : 0;
-  if (threadIdx.x == 0) { cg_info[0] = 0; cg_info[1] = cycles; }
+  if (threadIdx.x == 0) { cg_info[0] = 0; cg_info[1] = cycles; bar->status = 0; }
 }
 
 template <typename T>
@@ -377,7 +378,7 @@ cudaError_t launch_amg_inner(fvgb_mesh_s* m, int bcset, const double* r, int cyc
       if (e) return e;
     }
   }
-  k_amg_info<<<1, 128, 0, s>>>(pd.n_part, pd.active, cycles, pd.out_inner, m->d_cg_info);
+  k_amg_info<<<1, 128, 0, s>>>(pd.n_part, pd.active, cycles, pd.out_inner, m->d_cg_info, m->barrier);
   count_launch();
   return cudaGetLastError();
 }
