@@ -403,7 +403,7 @@ def fvgb_sync(m, stream=None):
 
 
 def fvgb_test_barrier(m, skip_block=-1, timeout_ms=0.0):
-    """Test hook of the CG kernel's bounded grid barrier (see include/fvgb.h)."""
+    """Test hook of the bounded grid barriers (see include/fvgb.h)."""
     return _check(lib.fvgb_test_barrier(m, int(skip_block), float(timeout_ms)), "fvgb_test_barrier")
 
 

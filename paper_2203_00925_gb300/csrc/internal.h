@@ -194,9 +194,10 @@ struct fvgb_mesh_s {
   fvgb::SolveInfoDev* d_solve = nullptr;  // result of the last solve in one launch
   int* d_status = nullptr;              // latched asynchronous errors, cleared when reported:
                                         // bit 0 (1) non-finite transport output, bit 1 (2) a
-                                        // tensor-core wait of the network kernels timed out
+                                        // bounded wait timed out: the network kernels' for the
+                                        // tensor cores, the one-launch steps' for one another
   double* d_time = nullptr;             // start time of the current streamer step
-  int test_skip_block = -1;             // test hook of the CG barrier (fvgb_test_barrier)
+  int test_skip_block = -1;             // test hook of the grid barriers (fvgb_test_barrier)
   unsigned long long test_barrier_ns = 0;  // barrier wait limit (0: the default 1 s)
   int solve_grid = 0;                   // cooperative grid of the Poisson kernel
   bool small_ok = false;                // time steps can run as one launch (small.cu)

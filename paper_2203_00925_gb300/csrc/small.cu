@@ -74,7 +74,8 @@ struct SmallArgs {
   T adt[kSmallStages];
   int star_max;
   Barrier* bar;
-  unsigned long long barrier_ns;
+  int skip_block;                 // test hook: this block never arrives at a barrier (-1: none)
+  unsigned long long barrier_ns;  // limit of a barrier wait
   int* status;
 };
 
@@ -210,7 +211,7 @@ __global__ void __launch_bounds__(kSmallThreads) k_small_steps(SmallArgs<T> a) {
     __syncthreads();
     bool ok = true;
     if (threadIdx.x < 32) {
-      if (threadIdx.x == 0) grid_arrive(a.bar);
+      if (threadIdx.x == 0 && a.skip_block != (int)blockIdx.x) grid_arrive(a.bar);
       __syncwarp();
       ok = grid_wait(a.bar, &a.bar->status, target, a.barrier_ns);
     }
@@ -292,7 +293,8 @@ cudaError_t launch_small_steps(fvgb_mesh_s* m, const fvgb_tcoef* tc, T* u, doubl
   for (int q = 0; q < nstage; ++q) a.adt[q] = (T)(alpha[q] * dt);
   a.star_max = t.star_max;
   a.bar = m->barrier;
-  a.barrier_ns = kBarrierTimeoutNs;
+  a.skip_block = m->test_skip_block;
+  a.barrier_ns = m->test_barrier_ns > 0 ? m->test_barrier_ns : kBarrierTimeoutNs;
   a.status = m->d_status;
   const int threads = small_threads<T>(m);
   cudaError_t e = launch_barrier_reset(m, s);

@@ -87,3 +87,36 @@ def test_multigrid_after_a_timeout(dev, launches):
         capi.fvgb_test_barrier(dm.handle, -1, 0.0)
         assert call(2) == capi.FVGB_OK
     dm.free()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_timeout_of_the_one_launch_steps(dev, prec):
+    """The steps of a small mesh latch the timeout; fvgb_sync or the next solve reports it once."""
+    capi, device = dev
+    m = jittered_square(20)
+    dm = device.DeviceMesh(m, [{1: ("wall", 0.0), 2: ("neumann", 0.0), 3: ("dirichlet", 0.3), 4: ("wall", 0.0)}], prec=prec)
+    tc = capi.tcoef(vel_const=(1.0, -0.5), diff=0.1)
+    u0 = dm.to_device(1.0 + m.xyz[m.cells].mean(axis=1)[:, 0])
+    f = torch.ones(dm.n_cell, dtype=torch.float64, device="cuda")
+    phi = torch.zeros_like(f)
+    want = u0.clone()
+    capi.fvgb_fv_step(dm.handle, tc, want, 1e-5, 3)
+    capi.fvgb_sync(dm.handle)
+
+    def late():
+        capi.fvgb_test_barrier(dm.handle, 2, 5.0)
+        capi.fvgb_fv_step(dm.handle, tc, u0.clone(), 1e-5, 3)
+        capi.fvgb_test_barrier(dm.handle, -1, 0.0)
+
+    late()
+    assert _status(capi, capi.fvgb_sync, dm.handle) == capi.FVGB_ETIMEOUT
+    assert _status(capi, capi.fvgb_sync, dm.handle) == capi.FVGB_OK
+    late()
+    opts = capi.solve_opts(rtol=1e-8)
+    assert _status(capi, capi.fvgb_poisson_solve, dm.handle, 0, f, phi, opts) == capi.FVGB_ETIMEOUT
+    assert _status(capi, capi.fvgb_poisson_solve, dm.handle, 0, f, phi.zero_(), opts) == capi.FVGB_OK
+    got = u0.clone()
+    capi.fvgb_fv_step(dm.handle, tc, got, 1e-5, 3)
+    assert _status(capi, capi.fvgb_sync, dm.handle) == capi.FVGB_OK
+    assert torch.equal(got, want)
+    dm.free()
