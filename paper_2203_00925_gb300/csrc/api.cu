@@ -591,18 +591,17 @@ fvgb_status poisson_rhs_impl(fvgb_mesh m, int bcset, const double* f, double* b,
   return FVGB_OK;
 }
 
-namespace {
-// The latched status of an earlier call, met by a solve: cleared and reported.
 fvgb_status report_latched(fvgb_mesh m, int latched, cudaStream_t s) {
   FVGB_TRY(cudaMemsetAsync(m->d_status, 0, sizeof(int), s), "memset");
   if (latched & 2) {
     set_error("a bounded wait on the device (tensor cores, grid barrier) timed out (latched status)");
     return FVGB_ETIMEOUT;
   }
-  set_error("an earlier transport call produced a non-finite value (latched status)");
+  set_error("a transport call produced a non-finite value (latched status)");
   return FVGB_ENONFINITE;
 }
 
+namespace {
 // The refinement loop as one launch (solver.cu), with one host synchronisation for its result.
 fvgb_status solve_one(fvgb_mesh m, int bcset, const double* b, double* r, double* phi, bool primed,
                       const fvgb_solve_opts* o, fvgb_solve_info* info, cudaStream_t s) {

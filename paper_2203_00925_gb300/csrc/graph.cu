@@ -353,11 +353,7 @@ fvgb_status streamer_graph_steps(fvgb_mesh m, const fvgb_streamer_params* p, voi
       set_error("streamer step " + std::to_string(n) + ": Poisson solve failed (status " + std::to_string(d.status) + ")");
     }
   }
-  if (first == FVGB_OK && *hlatch != 0) {
-    FVGB_TRY(cudaMemsetAsync(m->d_status, 0, sizeof(int), s), "memset");
-    set_error("a transport update of a graph step produced a non-finite value (latched status)");
-    first = FVGB_ENONFINITE;
-  }
+  if (first == FVGB_OK && *hlatch != 0) first = report_latched(m, *hlatch, s);
   return first;
 }
 

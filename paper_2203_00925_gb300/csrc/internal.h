@@ -259,6 +259,8 @@ inline void count_launch(int n = 1) { g_kernel_launches.fetch_add(n, std::memory
 
 void set_error(const std::string& msg);
 fvgb_status cuda_status(cudaError_t e, const char* what);
+// clear the latched status, met by a solve or at the end of a captured step, and report it
+fvgb_status report_latched(fvgb_mesh m, int latched, cudaStream_t s);
 
 // ops.cu -------------------------------------------------------------------------------
 cudaError_t prepare_gradient_fixed();   // allow its shared memory (longest halo list)

@@ -120,3 +120,23 @@ def test_timeout_of_the_one_launch_steps(dev, prec):
     assert _status(capi, capi.fvgb_sync, dm.handle) == capi.FVGB_OK
     assert torch.equal(got, want)
     dm.free()
+
+
+def test_captured_step_reports_a_latched_timeout(dev):
+    """A latched word met at the end of a captured step is reported as what it is."""
+    capi, device = dev
+    dm, _, step = _mesh(capi, device, "mixed")
+    u = dm.to_device(np.ones(dm.n_cell))
+    tc = capi.tcoef(vel_const=(1.0, -0.5, 0.2), diff=0.1)
+    assert step(0) == capi.FVGB_OK
+    for bad, want in ((None, capi.FVGB_ETIMEOUT), (float("nan"), capi.FVGB_ENONFINITE)):
+        if bad is None:
+            capi.fvgb_test_barrier(dm.handle, 2, 5.0)
+            capi.fvgb_fv_step(dm.handle, tc, u, 1e-6, 2)
+            capi.fvgb_test_barrier(dm.handle, -1, 0.0)
+        else:
+            u[7] = bad
+            capi.fvgb_fv_step(dm.handle, tc, u, 1e-6, 2)
+        assert step(0) == want
+        assert step(0) == capi.FVGB_OK
+    dm.free()
