@@ -183,7 +183,7 @@ int build_grad_tiles(int64_t N, const std::vector<int64_t>& start, const std::ve
 //    magnitude bits;
 //  - per cell D = sum_j (y_j - y_i) of those shifted differences over its neighbours, in units
 //    of 2^(62 - bits), and the padding entries of its list.
-constexpr double kFixedSpread = 12.0;
+constexpr double kFixedSpread = 8.0;
 constexpr int kFixedRows = 32;
 
 struct FixedHost {
