@@ -1339,26 +1339,26 @@ void infer_decode(MpnnNet* n, int set, double* pred, cudaStream_t s) {
   }
 }
 
-// The second evaluation's work on the network's own stream, between two events of s: it is
-// behind what s holds when it forks, and s waits for it when it joins (a capture of s takes
-// both in).
-cudaError_t fork_side(MpnnNet* n, cudaStream_t s) {
-  cudaError_t e = cudaEventRecord(n->fork, s);
-  return e == cudaSuccess ? cudaStreamWaitEvent(n->side, n->fork, 0) : e;
-}
-cudaError_t join_side(MpnnNet* n, cudaStream_t s) {
-  cudaError_t e = cudaEventRecord(n->join, n->side);
-  return e == cudaSuccess ? cudaStreamWaitEvent(s, n->join, 0) : e;
+// first(s) and, beside it, second(the network's own stream), between two events of s: the second
+// is behind what s holds, and s waits for it (a capture of s takes both in). An error of either
+// comes back behind the join: what the second has launched reads the caller's arrays, and a
+// capture of s could not end without it.
+template <typename A, typename B>
+cudaError_t side_by_side(MpnnNet* n, cudaStream_t s, A first, B second) {
+  cudaError_t e;
+  if ((e = cudaEventRecord(n->fork, s))) return e;
+  if ((e = cudaStreamWaitEvent(n->side, n->fork, 0))) return e;
+  const cudaError_t a = first(s), b = second(n->side);
+  if ((e = cudaEventRecord(n->join, n->side))) return e;
+  if ((e = cudaStreamWaitEvent(s, n->join, 0))) return e;
+  return a != cudaSuccess ? a : b;
 }
 
 // prediction dphi = V s2 (N(f) - N(f0 = 0))
 cudaError_t predict(MpnnNet* n, const double* dq, const double* phi, double* dphi, cudaStream_t s) {
   cudaError_t e;
-  if ((e = fork_side(n, s))) return e;
-  infer_layers(n, 0, dq, phi, s);
-  infer_layers(n, 1, dq, phi, n->side);
-  infer_decode(n, 0, dphi, s);
-  if ((e = join_side(n, s))) return e;
+  if ((e = side_by_side(n, s, [&](cudaStream_t q) { infer_layers(n, 0, dq, phi, q); infer_decode(n, 0, dphi, q); return cudaGetLastError(); },
+                        [&](cudaStream_t q) { infer_layers(n, 1, dq, phi, q); return cudaGetLastError(); }))) return e;
   infer_decode(n, 1, dphi, s);
   return cudaGetLastError();
 }
@@ -1430,19 +1430,15 @@ cudaError_t loss_grad(MpnnNet* n, const double* dq, const double* phi, const dou
   const int64_t N = n->N;
   const int G = kGradBlocks;
   if ((e = cudaMemsetAsync(n->part, 0, (size_t)2 * G * kNParams * sizeof(float), s))) return e;
-  if ((e = fork_side(n, s))) return e;
-  if ((e = forward(n, 0, dq, phi, false, s))) return e;
-  if ((e = forward(n, 1, dq, phi, true, n->side))) return e;
-  if ((e = join_side(n, s))) return e;
+  if ((e = side_by_side(n, s, [&](cudaStream_t q) { return forward(n, 0, dq, phi, false, q); },
+                        [&](cudaStream_t q) { return forward(n, 1, dq, phi, true, q); }))) return e;
   k_head_train<<<G, 256, 0, s>>>(N, n->H[0][kLayers], n->H[1][kLayers], n->theta, n->V * n->s2, target,
                                  n->dout, n->dpart);
   k_reduce_loss<<<1, 32, 0, s>>>(G, n->dpart, n->dloss);
   k_decode_grad<<<G, kRowGroups * kHid, 0, s>>>(N, n->H[0][kLayers], n->H[1][kLayers], n->dout, n->part);
   count_launch(3);
-  if ((e = fork_side(n, s))) return e;
-  backward_set(n, 0, 1.0f, 0, s);
-  backward_set(n, 1, -1.0f, G, n->side);
-  if ((e = join_side(n, s))) return e;
+  if ((e = side_by_side(n, s, [&](cudaStream_t q) { backward_set(n, 0, 1.0f, 0, q); return cudaGetLastError(); },
+                        [&](cudaStream_t q) { backward_set(n, 1, -1.0f, G, q); return cudaGetLastError(); }))) return e;
   k_reduce_grad<<<grid_n(kNParams), 256, 0, s>>>(2 * G, n->part, n->grad);
   count_launch();
   return cudaGetLastError();
