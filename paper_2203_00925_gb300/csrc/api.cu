@@ -411,33 +411,106 @@ cudaError_t alloc_work(fvgb_mesh_s* m, Work<T>& w) {
   return cudaSuccess;
 }
 
-// Sub-chunks of the persistent solve. Blocks are given to the parts one by one, always to the
-// part with the most cells a block, and a part's blocks share its cells equally; a single
-// mesh: block b owns rows [b N / G, (b+1) N / G). With more parts than blocks a block takes
-// whole parts.
+// Which blocks of the persistent solve work on which part. A CG solve of n cells on k blocks is
+// taken to need n^(1/dim) iterations of fixed + n / k rows' time (measured on ensembles of 2, 8
+// and 128 equal cubes of 100 to 1.5M cells: 8 us, two exchanges and the share of the outer
+// steps, and 1.5 ns a row of a block in FP32, 3.5 in FP64). Parts that one block solves within
+// the time of the whole share blocks, whole parts in turn; the others get blocks of their own,
+// and no part waits for another. The time of the whole is the smallest for which the blocks are
+// enough; blocks left over go to the slowest part, one by one.
+// Solves to 1e-8, mixed (FP64), in ms: one mesh of 1M cells and 100 of 1,000, blocks by cells alone
+// with at least one for every part 73 (171), equal rows to every block 73 (115), this 42 (77);
+// 3M and 127 of 1,000 476 (1,193), 192 (332), 130 (276); 16 of 20,000 to 200,000 23 (44), 61 (93),
+// 20 (37); 16 of 162,000 51 (107) either way.
+constexpr double kFixedRows32 = 5500.0, kFixedRows64 = 2300.0;
+
+struct PartBlocks {
+  std::vector<int> own;                      // per part: blocks of its own (0: in a shared one)
+  std::vector<std::vector<int>> shared;      // per shared block: its parts
+};
+
+PartBlocks share_blocks(const std::vector<int64_t>& begin, int G, int dim, double fixed) {
+  const int P = (int)begin.size() - 1;
+  std::vector<double> n(P), iterations(P);
+  std::vector<int> order(P);
+  for (int p = 0; p < P; ++p) {
+    n[p] = (double)(begin[p + 1] - begin[p]);
+    iterations[p] = std::pow(n[p], 1.0 / dim);
+    order[p] = p;
+  }
+  auto time = [&](int p, int k) { return iterations[p] * (fixed + n[p] / k); };
+  std::stable_sort(order.begin(), order.end(), [&](int p, int q) { return n[p] > n[q]; });
+  // blocks for a given time of the whole, first fit by decreasing size; false when G are too few
+  auto fits = [&](double whole, PartBlocks& out) {
+    out.own.assign(P, 0);
+    out.shared.clear();
+    std::vector<double> load;
+    int64_t used = 0;
+    for (int p : order) {
+      const double t = time(p, 1), room = whole / iterations[p] - fixed;
+      if (t > whole) {
+        const double k = room > 0.0 ? std::ceil(n[p] / room) : 2.0 * G;
+        if (used + k > G) return false;
+        out.own[p] = (int)k;
+        used += out.own[p];
+        continue;
+      }
+      size_t s = 0;
+      while (s < load.size() && load[s] + t > whole) ++s;
+      if (s == load.size()) {
+        if (used + 1 > G) return false;
+        ++used;
+        load.push_back(0.0);
+        out.shared.emplace_back();
+      }
+      load[s] += t;
+      out.shared[s].push_back(p);
+    }
+    return true;
+  };
+  PartBlocks best, trial;
+  double lo = 0.0, hi = 0.0;
+  for (int p = 0; p < P; ++p) hi += time(p, 1);
+  hi *= 1.0 + 1e-9;
+  fits(hi, best);                            // everything in one block
+  for (int it = 0; it < 60; ++it) {
+    const double mid = 0.5 * (lo + hi);
+    if (fits(mid, trial)) { hi = mid; best = trial; } else { lo = mid; }
+  }
+  for (auto it = best.shared.begin(); it != best.shared.end();) {   // alone in its block: its own
+    if (it->size() == 1) { best.own[(*it)[0]] = 1; it = best.shared.erase(it); } else { ++it; }
+  }
+  int used = (int)best.shared.size();
+  std::priority_queue<std::pair<double, int>> slowest;
+  for (int p = 0; p < P; ++p) {
+    used += best.own[p];
+    if (best.own[p] > 0) slowest.push({time(p, best.own[p]), -p});
+  }
+  for (; used < G && !slowest.empty(); ++used) {
+    const int p = -slowest.top().second;
+    slowest.pop();
+    slowest.push({time(p, ++best.own[p]), -p});
+  }
+  return best;
+}
+
+// Sub-chunks of the persistent solve: a part's blocks share its cells equally (a single mesh:
+// block b owns rows [b N / G, (b+1) N / G)), a part in a shared block is one sub-chunk.
 cudaError_t setup_parts(fvgb_mesh_s* m, const std::vector<int64_t>& part_begin, const HostMesh& h, cudaStream_t s) {
   const int64_t N = m->topo.N;
   const int G = m->solve_grid;
   const int P = (int)part_begin.size() - 1;
   m->part_cell_begin = part_begin;
-  std::vector<int> blocks(P, 1);
-  {
-    std::priority_queue<std::pair<double, int>> most;
-    for (int p = 0; p < P; ++p) most.push({(double)(part_begin[p + 1] - part_begin[p]), -p});
-    for (int left = G - P; left > 0; --left) {
-      const int p = -most.top().second;
-      most.pop();
-      blocks[p] += 1;
-      most.push({(double)(part_begin[p + 1] - part_begin[p]) / blocks[p], -p});
-    }
-  }
-  std::vector<int32_t> blk_sc(G + 1, 0), sc_part, part_sc(P + 1, 0), vert_begin(P + 1, 0);
+  const PartBlocks blocks = share_blocks(part_begin, G, h.dim, is_fp32(m) ? kFixedRows32 : kFixedRows64);
+  std::vector<int32_t> blk_work, sc_part, part_sc(P + 1, 0), vert_begin(P + 1, 0);
   std::vector<int64_t> sc_begin;
+  std::vector<WorkPiece> work;
   for (int p = 0; p < P; ++p) {
     const int64_t lo = part_begin[p], n = part_begin[p + 1] - lo;
+    const int pieces = std::max(1, blocks.own[p]);
     part_sc[p] = (int32_t)sc_part.size();
-    for (int b = 0; b < blocks[p]; ++b) {
-      sc_begin.push_back(lo + (int64_t)b * n / blocks[p]);
+    for (int b = 0; b < pieces; ++b) {
+      sc_begin.push_back(lo + (int64_t)b * n / pieces);
       sc_part.push_back(p);
     }
     // vertices are numbered in the order of the cells that touch them first: a part's are one range
@@ -448,12 +521,25 @@ cudaError_t setup_parts(fvgb_mesh_s* m, const std::vector<int64_t>& part_begin, 
   const int n_sc = (int)sc_part.size();
   part_sc[P] = n_sc;
   vert_begin[P] = (int32_t)h.V;
-  for (int b = 0; b <= G; ++b) blk_sc[b] = (int32_t)((int64_t)b * n_sc / G);
+  auto piece = [&](int p, int sc) {
+    work.push_back(WorkPiece{(int32_t)p, (int32_t)sc, part_sc[p], part_sc[p + 1], sc_begin[sc], sc_begin[sc + 1]});
+  };
+  for (int sc = 0; sc < n_sc; ++sc)
+    if (blocks.own[sc_part[sc]] > 0) {
+      blk_work.push_back((int32_t)work.size());
+      piece(sc_part[sc], sc);
+    }
+  for (const std::vector<int>& parts : blocks.shared) {
+    blk_work.push_back((int32_t)work.size());
+    for (int p : parts) piece(p, part_sc[p]);
+  }
+  blk_work.resize(G + 1, (int32_t)work.size());        // (blocks without work)
   PartsDev& pd = m->parts;
   pd.n_part = P;
   pd.n_sc = n_sc;
   cudaError_t e;
-  if ((e = dupload(m, &pd.blk_sc, blk_sc, s))) return e;
+  if ((e = dupload(m, &pd.blk_work, blk_work, s))) return e;
+  if ((e = dupload(m, &pd.work, work, s))) return e;
   if ((e = dupload(m, &pd.sc_begin, sc_begin, s))) return e;
   if ((e = dupload(m, &pd.sc_part, sc_part, s))) return e;
   if ((e = dupload(m, &pd.part_sc, part_sc, s))) return e;

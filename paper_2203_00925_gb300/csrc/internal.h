@@ -119,13 +119,20 @@ struct Work {
   T* cg_x = nullptr;
 };
 
+// A sub-chunk as its block sees it: the part, its place among the part's sub-chunks [sc0, sc1), rows.
+struct WorkPiece {
+  int32_t part, sc, sc0, sc1;
+  int64_t lo, hi;
+};
+
 // Parts of a mesh (an ensemble of independent meshes packed into one index space) and
-// the sub-chunks of the persistent solve: every block owns one, an equal piece of one part
-// (with more parts than blocks: whole parts in turn).
+// the sub-chunks of the persistent solve: a block owns one, an equal piece of one part, or solves
+// several small parts in turn (share_blocks).
 struct PartsDev {
   int n_part = 1;
   int n_sc = 0;
-  int32_t* blk_sc = nullptr;    // [G+1] first sub-chunk of each block
+  int32_t* blk_work = nullptr;  // [G+1] first entry of each block in work
+  WorkPiece* work = nullptr;    // [n_sc] the blocks' sub-chunks
   int64_t* sc_begin = nullptr;  // [n_sc+1] first row of each sub-chunk
   int32_t* sc_part = nullptr;   // [n_sc] part of each sub-chunk
   int32_t* part_sc = nullptr;   // [P+1] first sub-chunk of each part
