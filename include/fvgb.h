@@ -298,10 +298,11 @@ typedef struct {
  *  f_dev    [n_cell] double (NULL = 0)
  *  phi_dev  [n_cell] double, in: initial guess, out: solution
  *  info     host, may be NULL
- * With a CG inner solve an ensemble, and a single mesh of up to 600,000 cells, solves in one
- * launch (the outer loop on the device) and the call synchronises the stream once, at its end;
- * otherwise (a larger mesh, inner > 0, or fvgb_stats_enable on) it does so once per outer step,
- * to read the FP64 residual.
+ * With a CG inner solve a single mesh of up to 600,000 cells, and an ensemble (with an FP64 inner
+ * solve: of up to 1,000,000 cells a part on average), solves in one launch (the outer loop on the
+ * device) and the call synchronises the stream once, at its end; otherwise (larger, inner > 0, or
+ * fvgb_stats_enable on, which times the inner solves in launches of their own) it does so once
+ * per outer step, to read the FP64 residual.
  * Returns FVGB_ENOCONV (with info filled and phi the last iterate) if rtol is not met
  * within maxit_outer steps, FVGB_ENONFINITE on NaN/Inf, FVGB_ETIMEOUT if a grid-wide
  * barrier of the persistent CG kernel gave up. */
@@ -408,7 +409,8 @@ fvgb_status fvgb_integral(fvgb_mesh m, const void* u_dev, double* out_host, void
 
 /* Counters for measurement (no counterpart in the paper's method).
  *  kernel_launches  kernels launched by the library since the last reset (all meshes)
- *  cg_launches      inner CG kernels launched for this mesh
+ *  cg_launches      inner solves for this mesh (the largest part's, in an ensemble solved in one
+ *                   launch): launches of their own, or within the one launch of a solve
  *  cg_iterations    CG iterations they ran
  *  cg_ms            summed device time of those kernels, measured with CUDA events on the
  *                   launching stream when timing was enabled (0 otherwise)

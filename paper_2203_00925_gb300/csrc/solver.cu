@@ -800,14 +800,20 @@ cudaError_t launch_cg(fvgb_mesh_s* m, int bcset, const double* r, double inner_r
   return cudaLaunchCooperativeKernel(k, dim3(m->solve_grid), dim3(kCgThreads), args, 0, s);
 }
 
-// The whole solve in one launch up to kSolveOneMax cells. A solve to 1e-8 against separate
-// launches: 10,368 cells FP64 3.46 -> 2.26 ms, 384,000 13.4 -> 11.9 (mixed 9.7 -> 8.8); 750,000
-// equal; 1.3M 38.8 -> 43.1: one 512-thread block an SM streams the operator's passes slower than
-// their own kernels. (CUDA-event timing of the CG wants its own launches.)
-constexpr int64_t kSolveOneMax = 600000;
+// The whole solve in one launch. A single mesh up to kSolveOneMax cells; a solve to 1e-8 against
+// separate launches: 10,368 cells FP64 3.46 -> 2.26 ms, 384,000 13.4 -> 11.9 (mixed 9.7 -> 8.8);
+// 750,000 equal; 1.3M 38.8 -> 43.1: one 512-thread block an SM streams the operator's passes slower
+// than their own kernels. An ensemble gains more, since no part waits for another's inner solve
+// (mixed / FP64, ms: 16 x 162,000 74 -> 52 / 164 -> 109, 8 x 750,000 213 -> 175 / 430 -> 394,
+// 2 x 750,000 52 -> 44 / 107 -> 101; 2 x 3M mixed 227 -> 226), but in FP64, bound by its issue,
+// not with few parts of more than kSolveOneMean64 cells (2 x 1.3M 181 -> 207, 4 x 1.3M 389 -> 409,
+// 2 x 3M 456 -> 513). (CUDA-event timing of the CG wants its own launches.)
+constexpr int64_t kSolveOneMax = 600000, kSolveOneMean64 = 1000000;
 
 bool solve_one_ok(const fvgb_mesh_s* m, const fvgb_solve_opts* o) {
-  return o->inner == 0 && !m->time_cg && (m->parts.n_part > 1 || m->topo.N <= kSolveOneMax);
+  if (o->inner != 0 || m->time_cg) return false;
+  const int64_t N = m->topo.N, P = m->parts.n_part;
+  return P == 1 ? N <= kSolveOneMax : o->prec != FVGB_FP64 || N <= kSolveOneMean64 * P;
 }
 
 cudaError_t launch_solve_one(fvgb_mesh_s* m, int bcset, const double* b, double* phi, double* r, bool primed,

@@ -75,3 +75,24 @@ def test_parts_that_share_blocks(dev, name, prec):
             assert e.value.status == capi.FVGB_ETIMEOUT
             capi.fvgb_test_barrier(dm.handle, -1, 0.0)
     dm.free()
+
+
+@pytest.mark.parametrize("n,prec,one", [(707, "fp64", True), (708, "fp64", False), (708, "mixed", True)])
+def test_line_of_the_one_launch_solve(dev, n, prec, one):
+    """FP64 ensembles of more than 1,000,000 cells a part on average run separate launches; the
+    launches are counted: some ten a solve, or several an outer step."""
+    capi, device = dev
+    m = jittered_square(n)
+    dm = device.DeviceMesh([m, m], [[BC2], [BC2]], prec=prec, ensemble=True)
+    f = dm.to_device(np.tile(np.cos(3 * m.xyz[m.cells].mean(axis=1)[:, 0]), 2), torch.float64)
+    phi, b, y = (torch.zeros(dm.n_cell, dtype=torch.float64, device="cuda") for _ in range(3))
+    capi.fvgb_stats_get(dm.handle, reset=True)
+    _, info = capi.fvgb_poisson_solve(dm.handle, 0, f, phi, capi.solve_opts(
+        rtol=1e-4, prec=capi.FVGB_FP64 if prec == "fp64" else capi.FVGB_FP32))
+    launches = capi.fvgb_stats_get(dm.handle, reset=True)["kernel_launches"]
+    assert info.outer_its >= 2 and (launches <= 10) == one and (launches >= 4 * info.outer_its) != one
+    capi.fvgb_poisson_rhs(dm.handle, 0, f, b)
+    capi.fvgb_poisson_apply(dm.handle, 0, phi, y)
+    for half in (slice(0, dm.n_cell // 2), slice(dm.n_cell // 2, None)):
+        assert torch.linalg.norm((b - y)[half]) <= 1.0001e-4 * torch.linalg.norm(b[half])
+    dm.free()
