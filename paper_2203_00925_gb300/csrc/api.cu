@@ -616,7 +616,7 @@ fvgb_status step_T(fvgb_mesh m, const fvgb_tcoef* tc, T* u, double dt, int nstep
                    const double* alpha, int nstage, T* ni_out, cudaStream_t s) {
   Work<T>& w = work_of<T>(m);
   const bool diff = tc->diff != 0.0;
-  if (!tc->recon && !ni_out && step_small_ok<T>(m, (int64_t)nsteps * nstage))
+  if (!tc->recon && !ni_out && step_small_ok(m, (int64_t)nsteps * nstage))
     return cuda_status(launch_small_steps<T>(m, tc, u, dt, nsteps, alpha, nstage, s), "step kernel");
   for (int n = 0; n < nsteps; ++n) {
     const T* in = u;

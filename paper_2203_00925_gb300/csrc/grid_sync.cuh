@@ -48,4 +48,17 @@ __device__ __forceinline__ bool grid_wait(const Barrier* bar, int* status, unsig
   }
 }
 
+// A value that other blocks wrote before the last grid barrier: a plain load that may hit L1 (an
+// acquire in every barrier orders it behind the other blocks' stores), never moved across one.
+__device__ __forceinline__ float load_synced(const float* p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ double load_synced(const double* p) {
+  double v;
+  asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p) : "memory");
+  return v;
+}
+
 }  // namespace fvgb

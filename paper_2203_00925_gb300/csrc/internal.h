@@ -386,7 +386,6 @@ fvgb_status streamer_transport(fvgb_mesh m, const fvgb_streamer_params* p, void*
 
 // small.cu: all steps and stages of a call on a small mesh in one launch
 cudaError_t prepare_small(fvgb_mesh_s* m);
-template <typename T>
 bool step_small_ok(const fvgb_mesh_s* m, int64_t stages);
 template <typename T>
 cudaError_t launch_small_steps(fvgb_mesh_s* m, const fvgb_tcoef* tc, T* u, double dt, int nsteps,

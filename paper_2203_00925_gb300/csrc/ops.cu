@@ -13,6 +13,7 @@
 #include <cmath>
 
 #include "internal.h"
+#include "rounded.cuh"
 
 namespace fvgb {
 namespace {
@@ -40,18 +41,6 @@ __device__ __forceinline__ float cdiff(const float* a, const float* alo, int64_t
                                        const float* b, const float* blo, int64_t ib) {
   return (a[ia] - b[ib]) + (alo[ia] - blo[ib]);
 }
-
-// Explicitly rounded operations: the face flux is written with them so that its rounding
-// sequence (which products are fused) is fixed by the source, not by how the compiler
-// schedules a particular instantiation; every launch shape then gives the same bits.
-__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
-__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
-__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
-__device__ __forceinline__ float sub_rn(float a, float b) { return __fsub_rn(a, b); }
-__device__ __forceinline__ double sub_rn(double a, double b) { return __dsub_rn(a, b); }
-__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
 
 // Tests on the bits. A comparison in FP64 takes the FP64 pipe as long as an addition (64 cycles
 // a warp), and these are asked of every face or cell.

@@ -18,6 +18,7 @@
 
 #include "grid_sync.cuh"
 #include "internal.h"
+#include "rounded.cuh"
 
 namespace fvgb {
 namespace {
@@ -26,30 +27,9 @@ constexpr int kSmallThreads = 512;
 constexpr int kSmallCells = kSmallThreads / 4;   // cells of a block
 constexpr int kSmallStages = 8;                  // stages of a step (fvgb_fv_step's limit)
 
-__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
-__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
-__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
-__device__ __forceinline__ float sub_rn(float a, float b) { return __fsub_rn(a, b); }
-__device__ __forceinline__ double sub_rn(double a, double b) { return __dsub_rn(a, b); }
-__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
-
-// u of any cell: written by other blocks before the last grid barrier
-__device__ __forceinline__ float load_u(const float* p) {
-  float v;
-  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ double load_u(const double* p) {
-  double v;
-  asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p) : "memory");
-  return v;
-}
-
 template <typename T>
 struct SmallArgs {
-  int64_t N, F, Fi, V;
+  int64_t N, F, Fi;
   const int32_t* cell_face;
   const int32_t* fL;
   const int32_t* fR;
@@ -157,7 +137,7 @@ __global__ void __launch_bounds__(kSmallThreads) k_small_steps(SmallArgs<T> a) {
   for (int s = 0, stage = 0; s < total; ++s) {
     T* out = s + 1 == total ? a.u : a.w[s & 1];
     // gathers: the star of the vertex (four in flight) and the face's other cell
-    const T uo = kind == kInterior ? load_u(in + other) : T(0);
+    const T uo = kind == kInterior ? load_synced(in + other) : T(0);
     T uv = T(0);
     {
       int c = 0;
@@ -165,14 +145,14 @@ __global__ void __launch_bounds__(kSmallThreads) k_small_steps(SmallArgs<T> a) {
         T g[4], w[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          g[q] = load_u(in + sj[(c + q) * blockDim.x + threadIdx.x]);
+          g[q] = load_synced(in + sj[(c + q) * blockDim.x + threadIdx.x]);
           w[q] = sw[(c + q) * blockDim.x + threadIdx.x];
         }
 #pragma unroll
         for (int q = 0; q < 4; ++q) uv = fma_rn(w[q], g[q], uv);
       }
       for (; c < width; ++c)
-        uv = fma_rn(sw[c * blockDim.x + threadIdx.x], load_u(in + sj[c * blockDim.x + threadIdx.x]), uv);
+        uv = fma_rn(sw[c * blockDim.x + threadIdx.x], load_synced(in + sj[c * blockDim.x + threadIdx.x]), uv);
       if (fixed) uv = vfix;
     }
     const T va = __shfl_sync(0xffffffffu, uv, lanes[0], 4), vb = __shfl_sync(0xffffffffu, uv, lanes[1], 4),
@@ -228,7 +208,6 @@ size_t small_smem(const fvgb_mesh_s* m, int threads) {
   return (size_t)m->topo.star_max * threads * (sizeof(T) + sizeof(int32_t));
 }
 
-template <typename T>
 int small_threads(const fvgb_mesh_s* m) {
   const int64_t G = m->num_sms;
   const int64_t cells = (m->topo.N + G - 1) / G;
@@ -247,7 +226,6 @@ const void* small_kernel(const fvgb_mesh_s* m) {
 // registers), and stars that fit shared memory. The line is what a block can hold, not where the
 // two meet: 19,208 triangles take 5.0 us a step in one launch (FP32 2.3), 19,602 take 12.4 in
 // three kernels a stage (FP32 12.4).
-template <typename T>
 bool step_small_ok(const fvgb_mesh_s* m, int64_t stages) {
   return m->small_ok && stages >= 2 && stages < (int64_t(1) << 22);
 }
@@ -256,7 +234,7 @@ bool step_small_ok(const fvgb_mesh_s* m, int64_t stages) {
 cudaError_t prepare_small(fvgb_mesh_s* m) {
   m->small_ok = false;
   const bool fp32 = is_fp32(m);
-  const int threads = fp32 ? small_threads<float>(m) : small_threads<double>(m);
+  const int threads = small_threads(m);
   if (threads > kSmallThreads) return cudaSuccess;
   const size_t smem = fp32 ? small_smem<float>(m, threads) : small_smem<double>(m, threads);
   int limit = 0;
@@ -278,7 +256,7 @@ cudaError_t launch_small_steps(fvgb_mesh_s* m, const fvgb_tcoef* tc, T* u, doubl
   Work<T>& w = work_of<T>(m);
   const BCDev<T>& b = g.bc[tc->bcset];
   SmallArgs<T> a;
-  a.N = t.N; a.F = t.F; a.Fi = t.Fi; a.V = t.V;
+  a.N = t.N; a.F = t.F; a.Fi = t.Fi;
   a.cell_face = t.cell_face; a.fL = t.fL; a.fR = t.fR; a.fvert = t.fvert; a.cverts = t.cverts;
   a.sptr = t.vsell.ptr; a.sidx = t.vsell.idx;
   a.alpha = g.valpha; a.vdir = b.vdir; a.S = g.S; a.coef = g.coef;
@@ -296,7 +274,7 @@ cudaError_t launch_small_steps(fvgb_mesh_s* m, const fvgb_tcoef* tc, T* u, doubl
   a.skip_block = m->test_skip_block;
   a.barrier_ns = m->test_barrier_ns > 0 ? m->test_barrier_ns : kBarrierTimeoutNs;
   a.status = m->d_status;
-  const int threads = small_threads<T>(m);
+  const int threads = small_threads(m);
   cudaError_t e = launch_barrier_reset(m, s);
   if (e != cudaSuccess) return e;
   void* args[] = {&a};
@@ -305,8 +283,6 @@ cudaError_t launch_small_steps(fvgb_mesh_s* m, const fvgb_tcoef* tc, T* u, doubl
                                      dim3(threads), args, small_smem<T>(m, threads), s);
 }
 
-template bool step_small_ok<float>(const fvgb_mesh_s*, int64_t);
-template bool step_small_ok<double>(const fvgb_mesh_s*, int64_t);
 template cudaError_t launch_small_steps<float>(fvgb_mesh_s*, const fvgb_tcoef*, float*, double, int, const double*, int, cudaStream_t);
 template cudaError_t launch_small_steps<double>(fvgb_mesh_s*, const fvgb_tcoef*, double*, double, int, const double*, int, cudaStream_t);
 

@@ -53,7 +53,6 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
 
 template <typename T>
 struct SolveArgs {
-  int64_t N;
   // two-point operator scaled to unit diagonal, D^-1/2 A_T D^-1/2, in T, cell-major [N][4]
   const int32_t* at_nbr;
   const T* at_scoef;
@@ -172,20 +171,9 @@ __device__ __forceinline__ int4 load_op(const int4* p) {
                : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p), "l"(pol));
   return v;
 }
-// r, own rows and neighbours': a plain load that may hit L1 (an acquire in every grid barrier
-// orders it behind the other blocks' stores). Neighbours are mostly rows of the same warps, so
-// L1 takes most of the gathers' traffic: 6M cells FP32 68.5 -> 64.5 us, 750,000 cells 13.4 ->
-// 11.8 us an iteration against loads that pass L1 by.
-__device__ __forceinline__ float load_r(const float* p) {
-  float v;
-  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ double load_r(const double* p) {
-  double v;
-  asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p) : "memory");
-  return v;
-}
+// r, own rows and neighbours', comes through load_synced: neighbours are mostly rows of the same
+// warps, so L1 takes most of the gathers' traffic: 6M cells FP32 68.5 -> 64.5 us, 750,000 cells
+// 13.4 -> 11.8 us an iteration against loads that pass L1 by.
 
 // Four operator coefficients of one row, loaded with vector loads.
 template <typename T>
@@ -292,7 +280,7 @@ struct CgRows {
       if (i < n) {
         nb[u] = load_op<kStream>(reinterpret_cast<const int4*>(a.at_nbr) + lo + i);
         c[u].template load<kStream>(a.at_scoef + 4 * lo, i);
-        r[u] = load_r(a.cr + lo + i);
+        r[u] = load_synced(a.cr + lo + i);
         p[u] = a.cp[lo + i];
         q[u] = a.cq[lo + i];
         x[u] = kStream ? __ldcs(a.cx + lo + i) : a.cx[lo + i];
@@ -317,10 +305,10 @@ __device__ __forceinline__ T cg_phase_pq(const SolveArgs<T>& a, int64_t lo, int6
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       if (b + u * bd < n) {
-        g[u][0] = load_r(R0 + w.nb[u].x);
-        g[u][1] = load_r(R0 + w.nb[u].y);
-        g[u][2] = load_r(R0 + w.nb[u].z);
-        g[u][3] = load_r(R0 + w.nb[u].w);
+        g[u][0] = load_synced(R0 + w.nb[u].x);
+        g[u][1] = load_synced(R0 + w.nb[u].y);
+        g[u][2] = load_synced(R0 + w.nb[u].z);
+        g[u][3] = load_synced(R0 + w.nb[u].w);
       }
     }
     nx.load(a, lo, n, b + U * bd);
@@ -452,7 +440,7 @@ __global__ void __launch_bounds__(kCgThreads, kCgBlocksPerSm) k_cg(SolveArgs<T> 
 // values, then per cell its faces' fluxes (each formed from both sides, the operations and their
 // order those of k_face and k_update, so the residual has the same bits).
 struct ResidualArgs {
-  int64_t N, F, Fi, V;
+  int64_t N, F, Fi;
   const int64_t* sptr;
   const int32_t* sidx;
   const double* alpha;
@@ -479,9 +467,6 @@ struct ResidualArgs {
   int* stat;
 };
 
-// an FP64 value other blocks wrote before the last grid barrier
-__device__ __forceinline__ double load_shared(const double* p) { return load_r(p); }
-
 __device__ __forceinline__ void residual_vertices(const ResidualArgs& g, const OneBlock& k) {
   constexpr int U = 8;
   const int64_t end = g.vert_begin[k.part + 1];
@@ -500,7 +485,7 @@ __device__ __forceinline__ void residual_vertices(const ResidualArgs& g, const O
 #pragma unroll
       for (int q = 0; q < U; ++q) {
         w[q] = j[q] >= 0 ? __ldg(wcol + 32 * (c + q)) : 0.0;
-        x[q] = j[q] >= 0 ? load_shared(g.phi + j[q]) : 0.0;
+        x[q] = j[q] >= 0 ? load_synced(g.phi + j[q]) : 0.0;
       }
 #pragma unroll
       for (int q = 0; q < U; ++q)
@@ -523,13 +508,13 @@ __device__ __forceinline__ double residual_rows(const ResidualArgs& g, int64_t l
     for (int k = 0; k <= D; ++k) e[k] = g.cell_face[k * g.N + i];
     const int4 nb4 = __ldg(g.nbr + i);
     const int nb[4] = {nb4.x, nb4.y, nb4.z, nb4.w};
-    const double me = load_shared(g.phi + i);
+    const double me = load_synced(g.phi + i);
 #pragma unroll
     for (int k = 0; k <= D; ++k) {
       const int64_t f = e[k] >= 0 ? e[k] : ~e[k];
       bnd[k] = f >= g.Fi;
       on[k] = !bnd[k] || g.bkind[f - g.Fi] == FVGB_BC_DIRICHLET;
-      o[k] = bnd[k] ? 0.0 : load_shared(g.phi + nb[k]);
+      o[k] = bnd[k] ? 0.0 : load_synced(g.phi + nb[k]);
 #pragma unroll
       for (int q = 0; q < D; ++q) {
         c[k][q] = __ldg(g.coef + q * g.F + f);
@@ -539,7 +524,7 @@ __device__ __forceinline__ double residual_rows(const ResidualArgs& g, int64_t l
 #pragma unroll
     for (int k = 0; k <= D; ++k)
 #pragma unroll
-      for (int q = 0; q < D; ++q) uvx[k][q] = on[k] ? load_shared(g.uv + vx[k][q]) : 0.0;
+      for (int q = 0; q < D; ++q) uvx[k][q] = on[k] ? load_synced(g.uv + vx[k][q]) : 0.0;
     double acc = 0.0;
 #pragma unroll
     for (int k = 0; k <= D; ++k) {
@@ -750,7 +735,6 @@ SolveArgs<T> solve_args(fvgb_mesh_s* m, int bcset, const double* r, double inner
   GeoDev<T>& g = geo_of<T>(m);
   Work<T>& w = work_of<T>(m);
   SolveArgs<T> a;
-  a.N = m->topo.N;
   a.at_nbr = g.bc[bcset].at_nbr; a.at_scoef = g.bc[bcset].at_scoef; a.at_isd = g.bc[bcset].at_isd;
   a.r_in = r;
   a.phi = phi;
@@ -822,7 +806,7 @@ cudaError_t launch_solve_one(fvgb_mesh_s* m, int bcset, const double* b, double*
   const TopoDev& t = m->topo;
   const BCDev<double>& bc = m->g64.bc[bcset];
   ResidualArgs g;
-  g.N = t.N; g.F = t.F; g.Fi = t.Fi; g.V = t.V;
+  g.N = t.N; g.F = t.F; g.Fi = t.Fi;
   g.sptr = t.vsell.ptr; g.sidx = t.vsell.idx;
   g.alpha = m->g64.valpha; g.vdir = bc.vdir;
   g.cell_face = t.cell_face; g.nbr = reinterpret_cast<const int4*>(bc.at_nbr);
