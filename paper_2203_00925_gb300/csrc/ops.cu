@@ -286,9 +286,8 @@ k_gradient_tiled(int64_t N, int64_t F, int64_t Fi, const int64_t* __restrict__ s
 // also as integers but with the cell's own unit (own_scale_sum). Two threads share a cell's
 // entries. Where u is not finite or beyond 2^+-600, and in tiles whose integers would lose bits
 // of the centres (build_fixed_start), the sum stays in FP64, in the order of k_gradient.
-// 750,000 cells: 732 us with FP64 sums (tiles of FP64 sums take the same), 186 us now (integer
-// issue and shared memory; 182 with one shift for the three coordinates, which lost the short
-// direction of flat cells); the error against exact values went from 5.8e-16 to 4.4e-16 of the
+// 750,000 cells: 732 us with FP64 sums (tiles of FP64 sums take the same), 181 us now (integer
+// issue and shared memory); the error against exact values went from 5.8e-16 to 4.4e-16 of the
 // largest, and on cells flattened 10^2 to 10^6 : 1, on boundary layers and beside parts 10^9
 // times as large it is the direct sum's, 5 to 9e-16 of each component.
 constexpr int kFixTopMin = 400, kFixTopMax = 1600;   // biased exponents the scaled sums stay normal for
@@ -370,10 +369,11 @@ __device__ __forceinline__ int own_top(int c, int end, double ui, const int32_t*
 }
 
 // A cell's own integer products over entries [c, end): differences of the integer centres
-// shifted to ``bits`` bits, u_j - u_i converted with the exponent top. (Padding entries, the
-// cell itself, add 0.)
+// moved to 63 bits, u_j - u_i converted with the exponent top. (Padding entries, the cell itself,
+// add 0.) Inlined: as a function its call spilled the caller's registers, 750,000 cells 184.2 ->
+// 181.3 us, a steep field 240 -> 229.
 template <int BITS>
-__device__ __noinline__ void own_scale_sum(int64_t i, int c, int end, double ui, const int32_t* __restrict__ col,
+__device__ __forceinline__ void own_scale_sum(int64_t i, int c, int end, double ui, const int32_t* __restrict__ col,
                                            const longlong4_16a* __restrict__ xfix, const double* __restrict__ u,
                                            const GradTileFix* __restrict__ tile, int top, long long* s) {
   constexpr int U = 4;
@@ -431,6 +431,7 @@ k_gradient_fixed(int64_t N, int64_t F, int64_t Fi, const int64_t* __restrict__ s
   __shared__ int s_top[kFixThreads / 32];
   __shared__ longlong2 s_sum[2][kGradTile];   // the second halves' sums
   __shared__ int2 s_range[kGradTile];
+  __shared__ long long s_y[3][kGradTile];     // y of the tile's own cells (kept in registers: 184.2 -> 187.4 us)
   const GradTileFix* const tile = tfix + blockIdx.x;
   const GradTileFix td = *tile;
   const int64_t r0 = td.row0;
@@ -456,7 +457,6 @@ k_gradient_fixed(int64_t N, int64_t F, int64_t Fi, const int64_t* __restrict__ s
     const longlong2 oa = X[2 * r0];
     const long long oz = X[2 * r0 + 1].x;
     int top = 0;
-    long long yi[3] = {0, 0, 0};
     for (int k0 = threadIdx.x; k0 < nh; k0 += kFixBatch * kFixThreads) {
       int32_t j[kFixBatch];
       longlong2 a[kFixBatch];
@@ -478,7 +478,7 @@ k_gradient_fixed(int64_t N, int64_t F, int64_t Fi, const int64_t* __restrict__ s
         long long y[3] = {a[q].x - oa.x, a[q].y - oa.y, az[q] - oz};
 #pragma unroll
         for (int c = 0; c < 3; ++c) y[c] <<= td.left[c];
-        if (k < kGradTile) { yi[0] = y[0]; yi[1] = y[1]; yi[2] = y[2]; }   // the thread's own cell
+        if (k < kGradTile) { s_y[0][k] = y[0]; s_y[1][k] = y[1]; s_y[2][k] = y[2]; }
         ra[k] = make_longlong2(du, y[0]);
         rb[k] = make_longlong2(y[1], y[2]);
         top = max(top, exp_of(du));
@@ -544,7 +544,7 @@ k_gradient_fixed(int64_t N, int64_t F, int64_t Fi, const int64_t* __restrict__ s
           const long long Z[3] = {Z0 + half_units, Z1 + half_units, Z2 + half_units};
 #pragma unroll
           for (int k = 0; k < 3; ++k) {
-            const __int128 t = (__int128)yi[k] * V + (((__int128)vi * dsum[k * N + i]) << (62 - bits)) + ((__int128)1 << 62);
+            const __int128 t = (__int128)s_y[k][row] * V + (((__int128)vi * dsum[k * N + i]) << (62 - bits)) + ((__int128)1 << 62);
             J[k] = from_fixed(Z[k] - (long long)(t >> 63), td.unit[k] + top - 1022);
           }
         } else if (m >= 2) {
