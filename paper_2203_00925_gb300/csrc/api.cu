@@ -412,16 +412,18 @@ cudaError_t alloc_work(fvgb_mesh_s* m, Work<T>& w) {
 }
 
 // Which blocks of the persistent solve work on which part. A CG solve of n cells on k blocks is
-// taken to need n^(1/dim) iterations of fixed + n / k rows' time (measured on ensembles of 2, 8
-// and 128 equal cubes of 100 to 1.5M cells: 8 us, two exchanges and the share of the outer
-// steps, and 1.5 ns a row of a block in FP32, 3.5 in FP64). Parts that one block solves within
+// taken to need n^(0.6 / dim) iterations of fixed + n / k rows' time (measured on ensembles of 2,
+// 8 and 128 equal cubes of 100 to 1.5M cells: 8 us, two exchanges and the share of the outer
+// steps, and 1.5 ns a row of a block in FP32, 3.5 in FP64; iterations grow as n^0.33 from a zero
+// start and as n^0.2 over the steps of 64 streamers). Parts that one block solves within
 // the time of the whole share blocks, whole parts in turn; the others get blocks of their own,
 // and no part waits for another. The time of the whole is the smallest for which the blocks are
 // enough; blocks left over go to the slowest part, one by one.
-// Solves to 1e-8, mixed (FP64), in ms: one mesh of 1M cells and 100 of 1,000, blocks by cells alone
-// with at least one for every part 73 (171), equal rows to every block 73 (115), this 42 (77);
-// 3M and 127 of 1,000 476 (1,193), 192 (332), 130 (276); 16 of 20,000 to 200,000 23 (44), 61 (93),
-// 20 (37); 16 of 162,000 51 (107) either way.
+// ms mixed (FP64) of solves to 1e-8 with blocks by cells alone and one at least for every part,
+// with equal rows to every block, and this: 1M cells and 100 parts of 1,000 73 (171), 73 (115),
+// 41 (80); 3M and 127 of 1,000 476 (1,193), 192 (332), 115 (272); 16 of 20,000 to 200,000 23
+// (44), 61 (93), 21 (40); 16 of 162,000 51 (107), 115 (210), 51 (108). A step of 64 streamers of
+// 20,000 to 1M cells 85, 145, 83 (with n^(1 / dim) iterations 95).
 constexpr double kFixedRows32 = 5500.0, kFixedRows64 = 2300.0;
 
 struct PartBlocks {
@@ -435,7 +437,7 @@ PartBlocks share_blocks(const std::vector<int64_t>& begin, int G, int dim, doubl
   std::vector<int> order(P);
   for (int p = 0; p < P; ++p) {
     n[p] = (double)(begin[p + 1] - begin[p]);
-    iterations[p] = std::pow(n[p], 1.0 / dim);
+    iterations[p] = std::pow(n[p], 0.6 / dim);
     order[p] = p;
   }
   auto time = [&](int p, int k) { return iterations[p] * (fixed + n[p] / k); };
