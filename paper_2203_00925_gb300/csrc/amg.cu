@@ -65,7 +65,8 @@ inline unsigned blocks_for(int64_t n, int per_block) {
 }
 
 // mode 0: y = M v, and into x0 (if given) the first smoothing step of the level it goes to,
-// x0 = w dinv y (its own launch took 2 to 5 us a level, most of that latency); 1: y += M v; 2: y = b - M v (residual); 3: y = x + w dinv (b - M x).
+// x0 = w dinv y (its own launch took 2 to 5 us a level, most of that latency); 1: y += M v;
+// 2: y = b - M v (residual); 3: y = x + w dinv (b - M x).
 // LANES consecutive threads share a row: lane l sums entries l, l + LANES, ..., then a
 // shuffle tree over the group (fixed order).
 template <typename T, int LANES>

@@ -436,7 +436,7 @@ __global__ void __launch_bounds__(kCgThreads, kCgBlocksPerSm) k_cg(SolveArgs<T> 
 // synchronisation around the CG, some 60 us on 10,000 cells against 60 us of CG; here it is
 // three grid barriers. In an ensemble every part runs its own loop on its own blocks, where
 // the launches' loop ran each inner solve to the slowest part's last iteration (16 meshes of 20k
-// to 200k cells, mixed: 23.4 -> 10.1 ms a step). The operator is applied in two passes: vertex
+// to 200k cells, mixed: 22.8 -> 9.2 ms a step). The operator is applied in two passes: vertex
 // values, then per cell its faces' fluxes (each formed from both sides, the operations and their
 // order those of k_face and k_update, so the residual has the same bits).
 struct ResidualArgs {
