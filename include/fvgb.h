@@ -521,9 +521,10 @@ fvgb_status fvgb_sync(fvgb_mesh m, void* stream);
 
 /* Test hook of the bounded grid barriers of the persistent CG kernel and of the one-launch
  * steps of a small mesh (no counterpart in the paper; for tests of the timeout path only).
- * skip_block >= 0 makes that block of the kernel's grid never arrive at a barrier, so that the
- * other blocks' waits run out and the solve returns FVGB_ETIMEOUT (the steps latch it);
- * timeout_ms > 0 replaces the 1 s wait limit. skip_block = -1
+ * skip_block >= 0 makes that block of the solver's grid never arrive at a barrier (the steps
+ * wait for one arrival more than there are blocks), so that the waits run out and the solve
+ * returns FVGB_ETIMEOUT (the steps latch it); timeout_ms > 0 replaces the 1 s wait limit.
+ * skip_block = -1
  * and timeout_ms = 0 restore normal operation. A captured step graph is dropped.
  * Errors: FVGB_EINVAL for skip_block outside [-1, grid) or timeout_ms outside [0, 1000]. */
 fvgb_status fvgb_test_barrier(fvgb_mesh m, int32_t skip_block, double timeout_ms);

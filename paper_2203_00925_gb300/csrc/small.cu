@@ -54,7 +54,7 @@ struct SmallArgs {
   T adt[kSmallStages];
   int star_max;
   Barrier* bar;
-  int skip_block;                 // test hook: this block never arrives at a barrier (-1: none)
+  unsigned arrivals;              // that a barrier waits for: the blocks (test hook: one more)
   unsigned long long barrier_ns;  // limit of a barrier wait
   int* status;
 };
@@ -187,11 +187,11 @@ __global__ void __launch_bounds__(kSmallThreads) k_small_steps(SmallArgs<T> a) {
     }
     in = out;
     if (s + 1 == total) break;
-    target += gridDim.x;
+    target += a.arrivals;
     __syncthreads();
     bool ok = true;
     if (threadIdx.x < 32) {
-      if (threadIdx.x == 0 && a.skip_block != (int)blockIdx.x) grid_arrive(a.bar);
+      if (threadIdx.x == 0) grid_arrive(a.bar);
       __syncwarp();
       ok = grid_wait(a.bar, &a.bar->status, target, a.barrier_ns);
     }
@@ -271,7 +271,8 @@ cudaError_t launch_small_steps(fvgb_mesh_s* m, const fvgb_tcoef* tc, T* u, doubl
   for (int q = 0; q < nstage; ++q) a.adt[q] = (T)(alpha[q] * dt);
   a.star_max = t.star_max;
   a.bar = m->barrier;
-  a.skip_block = m->test_skip_block;
+  const unsigned grid = (unsigned)std::min<int64_t>(m->num_sms, t.N);
+  a.arrivals = grid + (m->test_skip_block >= 0 ? 1 : 0);
   a.barrier_ns = m->test_barrier_ns > 0 ? m->test_barrier_ns : kBarrierTimeoutNs;
   a.status = m->d_status;
   const int threads = small_threads(m);
@@ -279,8 +280,7 @@ cudaError_t launch_small_steps(fvgb_mesh_s* m, const fvgb_tcoef* tc, T* u, doubl
   if (e != cudaSuccess) return e;
   void* args[] = {&a};
   count_launch();
-  return cudaLaunchCooperativeKernel(small_kernel<T>(m), dim3((unsigned)std::min<int64_t>(m->num_sms, t.N)),
-                                     dim3(threads), args, small_smem<T>(m, threads), s);
+  return cudaLaunchCooperativeKernel(small_kernel<T>(m), dim3(grid), dim3(threads), args, small_smem<T>(m, threads), s);
 }
 
 template cudaError_t launch_small_steps<float>(fvgb_mesh_s*, const fvgb_tcoef*, float*, double, int, const double*, int, cudaStream_t);
