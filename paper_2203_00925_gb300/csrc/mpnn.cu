@@ -1357,8 +1357,13 @@ cudaError_t side_by_side(MpnnNet* n, cudaStream_t s, A first, B second) {
 // prediction dphi = V s2 (N(f) - N(f0 = 0))
 cudaError_t predict(MpnnNet* n, const double* dq, const double* phi, double* dphi, cudaStream_t s) {
   cudaError_t e;
-  if ((e = side_by_side(n, s, [&](cudaStream_t q) { infer_layers(n, 0, dq, phi, q); infer_decode(n, 0, dphi, q); return cudaGetLastError(); },
-                        [&](cudaStream_t q) { infer_layers(n, 1, dq, phi, q); return cudaGetLastError(); }))) return e;
+  // the first one's last layer is launched behind the second one's layers, so that these start early
+  if ((e = side_by_side(n, s, [&](cudaStream_t q) { infer_layers(n, 0, dq, phi, q); return cudaGetLastError(); },
+                        [&](cudaStream_t q) {
+                          infer_layers(n, 1, dq, phi, q);
+                          infer_decode(n, 0, dphi, s);
+                          return cudaGetLastError();
+                        }))) return e;
   infer_decode(n, 1, dphi, s);
   return cudaGetLastError();
 }
